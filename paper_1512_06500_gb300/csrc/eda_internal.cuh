@@ -124,7 +124,7 @@ constexpr int kCholBlock = 64;
 size_t chol_inv_blocked_doubles(int m);
 int chol_inv_blocked(int m, double* G, int ldg, double* Rinv, int ldr, double rank_tol, int* status, double* work,
                      double* partial, size_t pcap, cudaStream_t s);
-// chol_inv_small (one CTA) up to b = 90, chol_inv_blocked beyond (Rinv with ld b); no lost list, no pivot floor.
+// chol_inv_small (one CTA) up to b = 96, chol_inv_blocked beyond (Rinv with ld b); no lost list, no pivot floor.
 int chol_inv_auto(int b, double* G, int ldg, double* Rinv, double rank_tol, int* status, double* work, double* partial,
                   size_t pcap, cudaStream_t s);
 // Copy / scale / symmetrise helpers.

@@ -317,76 +317,159 @@ __global__ void k_gemm_small(bool ta, bool tb, int m, int p, int kk, double alph
     C[(int64_t)j * ldc + i] = v;
 }
 
-// Single-CTA right-looking upper Cholesky G = R^T R with rank detection, then R^{-1}.
-// The same factorisation for b <= 32 by one warp with the matrix in shared memory: lane c owns
-// column c; one reciprocal per pivot; warp-level synchronisation only. Rank decisions (threshold,
-// lost list in pivot order, status bits) are those of k_chol_inv.
-__global__ void __launch_bounds__(32) k_chol_inv_warp(int b, double* G, int ldg, double* Rinv, double rank_tol,
-                                                      double piv_min2, int* status, int* lost) {
-    __shared__ double sg[32][33];   // sg[c][r] = G[r, c]
-    __shared__ double sx[32][33];   // sx[c][i] = Rinv[i, c]
-    __shared__ double inv[32];
-    const int lane = threadIdx.x;
-    const bool live = lane < b;
-    if (live)
-        for (int r = 0; r <= lane; ++r) sg[lane][r] = G[(int64_t)lane * ldg + r];
-    double dg = live ? G[(int64_t)lane * ldg + lane] : 0.0;
-    const bool bad = live && !isfinite(dg);
-    double mx = fabs(dg);
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, ST_NONFINITE);
-    const double thr = fmax(rank_tol * mx, piv_min2);
-    int nlost = 0;
-    __syncwarp();
-    for (int j = 0; j < b; ++j) {
-        const double g = sg[j][j];
-        const bool lost_j = !(g > thr) || mx == 0.0;
-        const double piv = lost_j ? 0.0 : sqrt(g);
-        const double ip = lost_j ? 0.0 : 1.0 / piv;
-        __syncwarp();   // every lane has read the pivot before lane 0 overwrites it
-        if (lane == 0) {
-            if (lost_j) {
-                if (lost) lost[nlost] = j;
-                atomicOr(status, ST_RANKLOSS);
-            }
-            sg[j][j] = piv;
-            inv[j] = ip;
-        }
-        nlost += lost_j ? 1 : 0;
-        // row j of R (entries (j, c) for c > j), then the trailing update of column c
-        if (live && lane > j) sg[lane][j] *= ip;
-        __syncwarp();
-        if (live && lane > j) {
-            const double rjc = sg[lane][j];
-            for (int c1 = j + 1; c1 <= lane; ++c1) sg[lane][c1] -= sg[c1][j] * rjc;
-        }
-        __syncwarp();
-    }
-    // Rinv = R^{-1} (upper triangular): lane c solves R x = e_c from the bottom up
-    if (live) {
-        const int c = lane;
-        for (int i = b - 1; i > c; --i) sx[c][i] = 0.0;
-        for (int i = c; i >= 0; --i) {
-            double a0 = (i == c) ? 1.0 : 0.0, a1 = 0.0;
-            int l = i + 1;
-            for (; l + 1 <= c; l += 2) {
-                a0 -= sg[l][i] * sx[c][l];
-                a1 -= sg[l + 1][i] * sx[c][l + 1];
-            }
-            if (l <= c) a0 -= sg[l][i] * sx[c][l];
-            sx[c][i] = (a0 + a1) * inv[i];
-        }
-    }
-    __syncwarp();
-    if (live) {
-        for (int r = 0; r < b; ++r) {
-            G[(int64_t)lane * ldg + r] = (r <= lane) ? sg[lane][r] : 0.0;
-            Rinv[(int64_t)lane * b + r] = sx[lane][r];
-        }
-    }
-    if (lane == 0 && lost) lost[b] = nlost;
+// 1 / x for a positive normal x: the hardware's 20-bit approximation (PTX rcp.approx.ftz.f64) and two
+// Newton-Raphson steps r <- r + r (1 - x r), each doubling the correct bits. The IEEE division is used where
+// x or 1 / x leaves the approximation's range.
+__device__ __forceinline__ double newton_rcp(double x) {
+    const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+    if (ex < 24 || ex > 2022) return 1.0 / x;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
 }
 
+// Upper Cholesky G = R^T R with rank detection and X = R^{-1}, one CTA of eight warps, b <= 32 NC; the pivot
+// order, threshold, lost list and status bits are those of k_chol_inv. The kernel is a chain of b pivots on an
+// FP64 pipe that holds a warp instruction for about 64 cycles, so the work is arranged to keep FP64
+// instructions off that chain:
+//  - G and the inverse are eliminated together as [G | I] -> [R | R^{-T}]: row i keeps G's entries c >= i and the
+//    inverse's entries c < i (its unit diagonal is implicit), one b x b square in registers, warp w owning rows
+//    w, w + 8, ... and lane l columns l, l + 32, ... There is no back substitution after the factorisation.
+//  - rows stay unscaled (G[i, :] -= (u_i / g_j) u for the pivot row u): one reciprocal per pivot, no square root;
+//    the square roots and the scaling follow at the end, for all rows at once.
+//  - the owner of row j + 1 updates that row first, publishes it and its reciprocal, and updates its other rows
+//    while the other warps update theirs: one barrier per pivot, the pivot row double-buffered.
+// GB300, one launch: b = 16 12 us and b = 32 22 us (30 and 76 us by one warp with a back substitution), b = 64 88 us
+// (220 us with three barriers, a division and a square root per pivot).
+template <int NC>
+__global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg, double* Rinv, double rank_tol,
+                                                       double piv_min2, int* status, int* lost) {
+    constexpr int NR = 4 * NC;               // rows per warp
+    __shared__ double urow[2][32 * NC];      // the pivot row: G's part c >= j, the inverse's part c < j
+    __shared__ double ginv[2];               // 1 / pivot, 0 where the pivot is lost
+    __shared__ double gpiv[32 * NC];         // pivots (0 where lost)
+    __shared__ double rdiag[32 * NC];        // 1 / sqrt(pivot)
+    __shared__ double s_thr;
+    __shared__ int s_nlost;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double a[NR][NC];
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+        const int i = w + 8 * q;
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+            const int c = lane + 32 * h;
+            a[q][h] = (i < b && c < b && c >= i) ? G[(int64_t)c * ldg + i] : 0.0;
+        }
+    }
+    if (w == 0) {
+        double mx = 0.0;
+        bool bad = false;
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+            const int c = lane + 32 * h;
+            const double g = c < b ? G[(int64_t)c * ldg + c] : 0.0;
+            bad |= !isfinite(g);
+            mx = fmax(mx, fabs(g));
+        }
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, ST_NONFINITE);
+        // a zero diagonal loses every pivot
+        if (lane == 0) {
+            s_thr = mx == 0.0 ? INFINITY : fmax(rank_tol * mx, piv_min2);
+            s_nlost = 0;
+        }
+    }
+    __syncthreads();
+    const double thr = s_thr;
+    // row i (register row v, owned by this warp) becomes pivot row i: publish it with its reciprocal
+    auto publish = [&](int i, const double (&v)[NC]) {
+        double g = v[0];
+#pragma unroll
+        for (int h = 1; h < NC; ++h)
+            if (h == (i >> 5)) g = v[h];
+        g = __shfl_sync(0xffffffffu, g, i & 31);
+        const bool lost_i = !(g > thr);
+#pragma unroll
+        for (int h = 0; h < NC; ++h) urow[i & 1][lane + 32 * h] = v[h];
+        if (lane == 0) {
+            ginv[i & 1] = lost_i ? 0.0 : newton_rcp(g);
+            gpiv[i] = lost_i ? 0.0 : g;
+            if (lost_i) {
+                if (lost) lost[s_nlost] = i;
+                ++s_nlost;
+                atomicOr(status, ST_RANKLOSS);
+            }
+        }
+    };
+    if (w == 0) publish(0, a[0]);
+    __syncthreads();
+    for (int j = 0; j + 1 < b; ++j) {
+        const double gi = ginv[j & 1];
+        const double* u = urow[j & 1];
+        double uc[NC], f[NC];
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+            const int c = lane + 32 * h;
+            uc[h] = c == j ? 1.0 : u[c];     // column j of the inverse's part: its unit diagonal
+            f[h] = u[c] * gi;                // u_i / g_j for row i = c
+        }
+        // rows i > j: columns c <= j (inverse) and c >= i (G)
+        auto update = [&](int i, double (&v)[NC]) {
+            double fi = f[0];
+#pragma unroll
+            for (int h = 1; h < NC; ++h)
+                if (h == (i >> 5)) fi = f[h];
+            fi = __shfl_sync(0xffffffffu, fi, i & 31);
+#pragma unroll
+            for (int h = 0; h < NC; ++h) {
+                // a 32-column slice strictly between the two parts holds nothing (uniform over the warp)
+                if (32 * h > j && 32 * h + 31 < i) continue;
+                const int c = lane + 32 * h;
+                const double x = fma(-fi, uc[h], v[h]);
+                if (c <= j || c >= i) v[h] = x;
+            }
+        };
+        const int nx = j + 1;
+        if ((nx & 7) == w) {
+#pragma unroll
+            for (int q = 0; q < NR; ++q)
+                if (w + 8 * q == nx) {
+                    update(nx, a[q]);
+                    publish(nx, a[q]);
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+            const int i = w + 8 * q;
+            if (i > nx && i < b) update(i, a[q]);
+        }
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < b; i += blockDim.x) {
+        const double g = gpiv[i];
+        rdiag[i] = g > 0.0 ? 1.0 / sqrt(g) : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+        const int i = w + 8 * q;
+        if (i >= b) break;
+        const double sc = rdiag[i];
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+            const int c = lane + 32 * h;
+            if (c >= b) continue;
+            const double v = sc > 0.0 ? a[q][h] * sc : 0.0;   // a lost row of R, and of R^{-T}, is zero
+            G[(int64_t)c * ldg + i] = c >= i ? v : 0.0;
+            Rinv[(int64_t)i * b + c] = c < i ? v : (c == i ? sc : 0.0);
+        }
+    }
+    if (threadIdx.x == 0 && lost) lost[b] = s_nlost;
+}
+
+// The same by one CTA in global memory, for any b: two divisions a column and a back substitution.
 __global__ void k_chol_inv(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2, int* status,
                            int* lost) {
     __shared__ double maxdiag;
@@ -457,82 +540,8 @@ __global__ void k_chol_inv(int b, double* G, int ldg, double* Rinv, double rank_
     if (threadIdx.x == 0 && lost) lost[b] = nlost;
 }
 
-// The factorisation of k_chol_inv for 32 < b <= kCholSmemMax with G and R^{-1} held in shared memory
-// (the same pivot order, rank threshold, lost list and status bits): one reciprocal per pivot
-// scales its row of R, and the back substitution for R^{-1} multiplies by the stored reciprocal
-// pivots and splits each inner product over two accumulators, halving its dependent FMA chain.
-constexpr int kCholSmemMax = 90;
-
-__global__ void __launch_bounds__(256) k_chol_inv_smem(int b, double* G, int ldg, double* Rinv, double rank_tol,
-                                                       double piv_min2, int* status, int* lost) {
-    extern __shared__ double smc[];
-    double* sg = smc;              // sg[c * b + r] = G[r, c]
-    double* sx = smc + b * b;      // sx[c * b + i] = Rinv[i, c]
-    __shared__ double inv[kCholSmemMax];
-    __shared__ double maxdiag;
-    __shared__ int nlost;
-    for (int e = threadIdx.x; e < b * b; e += blockDim.x) sg[e] = G[(int64_t)(e / b) * ldg + e % b];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double mx = 0.0;
-        bool bad = false;
-        for (int j = 0; j < b; ++j) {
-            const double g = sg[j * b + j];
-            if (!isfinite(g)) bad = true;
-            mx = fmax(mx, fabs(g));
-        }
-        maxdiag = mx;
-        nlost = 0;
-        if (bad) atomicOr(status, ST_NONFINITE);
-    }
-    __syncthreads();
-    const double thr = fmax(rank_tol * maxdiag, piv_min2);
-    for (int j = 0; j < b; ++j) {
-        if (threadIdx.x == 0) {
-            const double g = sg[j * b + j];
-            double piv = 0.0;
-            if (!(g > thr) || maxdiag == 0.0) {
-                if (lost) lost[nlost] = j;
-                nlost++;
-                atomicOr(status, ST_RANKLOSS);
-            } else {
-                piv = sqrt(g);
-            }
-            sg[j * b + j] = piv;
-            inv[j] = piv > 0.0 ? 1.0 / piv : 0.0;
-        }
-        __syncthreads();
-        const double ip = inv[j];
-        for (int c = j + 1 + threadIdx.x; c < b; c += blockDim.x) sg[c * b + j] *= ip;
-        __syncthreads();
-        const int rem = b - j - 1;
-        for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-            const int c1 = j + 1 + e % rem, c2 = j + 1 + e / rem;
-            if (c1 <= c2) sg[c2 * b + c1] -= sg[c1 * b + j] * sg[c2 * b + j];
-        }
-        __syncthreads();
-    }
-    for (int c = threadIdx.x; c < b; c += blockDim.x) {
-        for (int i = b - 1; i > c; --i) sx[c * b + i] = 0.0;
-        for (int i = c; i >= 0; --i) {
-            double a0 = (i == c) ? 1.0 : 0.0, a1 = 0.0;
-            int l = i + 1;
-            for (; l + 1 <= c; l += 2) {
-                a0 -= sg[l * b + i] * sx[c * b + l];
-                a1 -= sg[(l + 1) * b + i] * sx[c * b + l + 1];
-            }
-            if (l <= c) a0 -= sg[l * b + i] * sx[c * b + l];
-            sx[c * b + i] = (a0 + a1) * inv[i];
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-        const int r = e % b, c = e / b;
-        G[(int64_t)c * ldg + r] = (r > c) ? 0.0 : sg[e];
-        Rinv[e] = sx[e];
-    }
-    if (threadIdx.x == 0 && lost) lost[b] = nlost;
-}
+// the register-resident factorisation up to this size (three 32-column slices a lane)
+constexpr int kCholPairMax = 96;
 
 template <class Ti, class To>
 __global__ void k_copy(int64_t rows, int cols, const Ti* __restrict__ A, int64_t lda, To* __restrict__ B,
@@ -799,20 +808,14 @@ int gemm_small_f64(bool ta, bool tb, int m, int p, int kk, double alpha, const d
 
 int chol_inv_small(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2, int* status, int* lost,
                    cudaStream_t s) {
-    if (b <= 32) {
-        k_chol_inv_warp<<<1, 32, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
-    } else if (b <= kCholSmemMax) {
-        static std::once_flag once;
-        static cudaError_t attr_rc = cudaSuccess;
-        std::call_once(once, [] {
-            attr_rc = cudaFuncSetAttribute(k_chol_inv_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(2 * sizeof(double) * kCholSmemMax * kCholSmemMax));
-        });
-        EDA_CUDA_TRY(attr_rc);
-        k_chol_inv_smem<<<1, 256, 2 * sizeof(double) * b * b, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
-    } else {
+    if (b <= 32)
+        k_chol_inv_pair<1><<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
+    else if (b <= 64)
+        k_chol_inv_pair<2><<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
+    else if (b <= kCholPairMax)
+        k_chol_inv_pair<3><<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
+    else
         k_chol_inv<<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
-    }
     EDA_LAUNCHED();
     return EDA_OK;
 }
@@ -880,7 +883,7 @@ int chol_inv_blocked(int m, double* G, int ldg, double* Rinv, int ldr, double ra
 
 int chol_inv_auto(int b, double* G, int ldg, double* Rinv, double rank_tol, int* status, double* work, double* partial,
                   size_t pcap, cudaStream_t s) {
-    if (b <= 90) return chol_inv_small(b, G, ldg, Rinv, rank_tol, 0.0, status, nullptr, s);
+    if (b <= kCholPairMax) return chol_inv_small(b, G, ldg, Rinv, rank_tol, 0.0, status, nullptr, s);
     return chol_inv_blocked(b, G, ldg, Rinv, b, rank_tol, status, work, partial, pcap, s);
 }
 

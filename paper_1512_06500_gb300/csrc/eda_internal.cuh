@@ -160,6 +160,8 @@ int col_norms(int64_t rows, int cols, const T* A, int64_t lda, double* out, cuda
 // ---------------------------------------------------------------- symmetric eigensolver
 struct SymEigWork {
     double* A;        // n x n copy (destroyed)
+    double* X;        // n x n exchange buffer of the cooperative reduction (carved from xn columns on)
+    int xn = 0;       // matrix order X holds (0: none)
     double* dgl;      // n diagonal
     double* eoff;     // n off-diagonal
     double* tau;      // n Householder scalars

@@ -5,13 +5,12 @@
 // Route: Householder reduction to tridiagonal form (from n = 288 a cooperative grid with the columns
 // resident in its CTAs' shared memory; below that, or when the GPU is shared, one thread-block cluster;
 // beyond what shared memory holds, a cooperative grid streaming the matrix through L2; all with bounded
-// barriers) -> eigenvalues by 33-way
+// waits) -> eigenvalues by 33-way
 // multisection on Sturm counts (one warp per eigenvalue) -> eigenvectors of the tridiagonal
 // by inverse iteration with partial pivoting (one thread per eigenvector) -> modified
 // Gram-Schmidt inside tight clusters (one warp per cluster) -> back-transformation with the
 // stored reflectors. Callers add a Newton-Schulz step for orthogonality across near clusters.
 #include "eda_internal.cuh"
-#include "grid_bar.cuh"
 
 #include <cooperative_groups.h>
 
@@ -165,317 +164,323 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag(int n, double* A, doubl
     }
 }
 
-constexpr int CT_THREADS = 128;
+// Householder tridiagonalisation with one exchange between CTAs per column, on a cooperative grid (CL = false) or
+// in one thread-block cluster (CL = true). Column r of the symmetric matrix is owned by CTA r % G and stays in its
+// shared memory (in a cluster, for large n, in a global slab of that CTA).
+//
+// Every CTA holds the current column x = A[c.., c] and forms its reflector itself: v = x - beta e_{c+1} (rows
+// c + 1.., unscaled), H = I - tau v v^T with tau = 1 / (beta (beta - alpha)). What the CTAs exchange for column c is
+// p = tau A v, each entry from the owner of its row, and the next column A[.., c + 1] before its update, from its owner.
+// From these every CTA forms, with the same operations in the same order,
+//     K = (tau / 2) v^T p,  w = p - K v,  x' = A[.., c + 1] - v w_{c+1} - w v_{c+1},  ||x'||
+// and then updates its own columns (A <- A - v w^T - w v^T) and multiplies them by x' in the same pass; the reflector's
+// scalars beta', tau' are formed by one warp beside that pass and applied afterwards, A v' = A x' - beta' A e_{c+2}.
+//
+// What bounds it: per column one exchange and a chain of FP64 instructions (each holds a sub-partition's pipe for about
+// 64 cycles whatever the number of lanes), so the design spends CTA-wide redundant work to have one exchange instead of
+// two, keeps square root and reciprocal beside the pass, and reduces with one warp per sub-partition.
+//   Grid: the exchanged values are written once to their own place (row c of two n x n buffers, filled before the launch
+// with a bit pattern that no result has) and polled there by the reader: no barrier, flag or fence is on the path, each
+// value vouches for itself. The polls are bounded (ST_TIMEOUT); a thread that gave up once does not wait again.
+//   Cluster: entries in the owners' shared memory, read through distributed shared memory after one cluster barrier;
+// p is double-buffered, and a column is never written again once it is next.
+// GB300, against two barriers (or cluster barriers) per column and the reflector formed by its owner alone: grid n = 700
+// 7.66 -> 4.62 ms, n = 668 7.13 -> 4.30 ms; cluster n = 144 0.95 -> 0.51 ms, n = 100 0.55 -> 0.33 ms.
+constexpr int TD_WARPS = 8;                             // warps that share the owned columns; one more forms the scalars
+constexpr int TD_THREADS = 32 * TD_WARPS + 32;
+constexpr int TD_RED = 128;                             // threads (one warp per sub-partition) of the vector work
 
-// Reflector of column j (entries a[i], i > j) formed by the CTA that owns the column and
-// published in its shared memory: vpub[i] for i > j, vpub[n] = tau, vpub[n + 1] = beta.
-__device__ void make_reflector(int j, int n, const double* a, double* vpub, double* HV, double* eoff, double* tau,
-                               double* red) {
-    const int tid = threadIdx.x, bd = blockDim.x;
-    const int i0 = j + 1;
-    double ss = 0.0;
-    for (int i = i0 + 1 + tid; i < n; i += bd) ss = fma(a[i], a[i], ss);
-    ss = block_sum(ss, red);
-    const double alpha = a[i0];
-    double beta, tj, scal;
-    if (ss == 0.0) {
-        beta = alpha;
-        tj = 0.0;
-        scal = 0.0;
-    } else {
-        // beta = -sign(alpha) ||x||, tau = (beta - alpha) / beta, scal = 1 / (alpha - beta)
-        const double nrm2 = fma(alpha, alpha, ss);
-        const double rn = rsqrt(nrm2);
-        const double sg = (alpha >= 0.0) ? 1.0 : -1.0;
-        beta = -sg * nrm2 * rn;
-        tj = fma(sg * alpha, rn, 1.0);
-        scal = 1.0 / (alpha - beta);
-    }
-    for (int i = tid; i < n; i += bd) {
-        const double val = (i < i0) ? 0.0 : ((i == i0) ? 1.0 : a[i] * scal);
-        if (i >= i0) vpub[i] = val;
-        HV[(int64_t)j * n + i] = val;
-    }
-    if (tid == 0) {
-        vpub[n] = tj;
-        vpub[n + 1] = beta;
-        eoff[j] = beta;
-        tau[j] = tj;
-    }
+// Warps per owned column in the pass over the columns: enough tasks to even out the sub-partitions.
+__host__ __device__ inline int td_split(int ncl) { return ncl >= TD_WARPS ? 1 : (ncl > 4 ? 4 : 2); }
+__host__ __device__ inline int td_dots(int ncl) { return ncl * 32 * td_split(ncl); }
+constexpr unsigned long long TD_EMPTY = ~0ull;          // "not written yet": a NaN with this payload is never stored
+
+__device__ __forceinline__ unsigned long long td_ld(const double* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void td_st(double* p, double x) {
+    unsigned long long v = (unsigned long long)__double_as_longlong(x);
+    if (v == TD_EMPTY) v = 0x7FF8000000000000ull;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// 1 / x for a positive normal x: PTX rcp.approx.ftz.f64 (20 bits) and two Newton-Raphson steps; the IEEE division where x
+// or 1 / x leaves the approximation's range.
+__device__ __forceinline__ double td_rcp(double x) {
+    const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+    if (ex < 24 || ex > 2022) return 1.0 / x;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
 }
 
-// Householder tridiagonalisation on one thread-block cluster (C <= 16 CTAs). Column c of the
-// symmetric matrix is owned by CTA c % C and kept in its shared memory (or, for large n, in a
-// global slab of that CTA). Per column j: after a cluster barrier every CTA reads the reflector
-// that the owner of column j published, forms its partial p over the columns it owns; after a
-// second barrier every CTA sums the partials of all CTAs (distributed shared memory, fixed
-// pairwise order), forms w and updates its columns. The owner of column j + 1 updates that
-// column first and publishes reflector j + 1 while the other CTAs are still updating
-// (look-ahead), so the reflector's FP64 latency chain is off the critical path.
-template <int C>
-__global__ void __launch_bounds__(CT_THREADS) k_tridiag_cluster(int n, const double* __restrict__ Ain, int lda,
-                                                                double* Aglob, int in_smem, double* HV, double* dgl,
-                                                                double* eoff, double* tau) {
+// sqrt(x), x >= 0: PTX rsqrt.approx.ftz.f64 and two Goldschmidt steps on g ~ sqrt(x), h ~ 1 / (2 sqrt(x))
+// (r = 1/2 - g h, g <- g + g r, h <- h + h r); the library's square root outside the approximation's range.
+__device__ __forceinline__ double td_sqrt(double x) {
+    const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+    if (ex < 24 || ex > 2022) return sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = x * y, h = 0.5 * y;
+    double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    r = fma(-g, h, 0.5);
+    return fma(g, r, g);
+}
+
+template <bool CL>
+__global__ void __launch_bounds__(TD_THREADS) k_tridiag_x(int n, const double* __restrict__ Ain, int lda, double* Aglob,
+                                                          int in_smem, double* pbuf, double* cbuf, double* HV, double* dgl,
+                                                          double* eoff, double* tau, long long spin, int* status) {
     namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
     extern __shared__ double sm[];
-    __shared__ double red[32];
-    const int ncl = (n + C - 1) / C;
-    double* vbuf = sm;                 // n: reflector (local copy)
-    double* vpub = sm + n;             // n + 2: reflector published by the owner, then tau, beta
-    double* ppart = sm + 2 * n + 2;    // n: this CTA's partial p
-    double* pw = sm + 3 * n + 2;       // n: full p, then w
-    double* Aloc = in_smem ? (sm + 4 * n + 2) : (Aglob + (size_t)rank * ncl * n);
-    const int tid = threadIdx.x, bd = blockDim.x;
-
-    for (int q = 0; q < ncl; ++q) {
-        const int c = q * C + rank;
-        if (c >= n) break;
-        for (int i = tid; i < n; i += bd)
-            Aloc[(size_t)q * n + i] = 0.5 * (Ain[(int64_t)c * lda + i] + Ain[(int64_t)i * lda + c]);
-    }
-    __syncthreads();
-    if (n >= 3 && rank == 0) make_reflector(0, n, Aloc, vpub, HV, eoff, tau, red);
-
-    for (int j = 0; j + 2 < n; ++j) {
-        const int i0 = j + 1;
-        const int owner = j % C;
-        const int next = j + 1;
-        const bool own_next = (next + 2 < n) && (next % C == rank);
-        cluster.sync();                                   // reflector j published
-        const double* rv = cluster.map_shared_rank(vpub, owner);
-        const double tj = rv[n];
-        if (tj == 0.0) {                                  // same decision in every CTA
-            __syncthreads();
-            if (own_next) make_reflector(next, n, Aloc + (size_t)(next / C) * n, vpub, HV, eoff, tau, red);
-            continue;
-        }
-        for (int i = i0 + tid; i < n; i += bd) vbuf[i] = rv[i];
-        __syncthreads();
-        const int q0 = (i0 - rank + C - 1) / C;           // first owned column >= i0
-        for (int i = i0 + tid; i < n; i += bd) {
-            double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
-            int q = q0;
-            for (; q + 3 < ncl; q += 4) {
-                const int c0 = q * C + rank;
-                if (c0 + 3 * C >= n) break;
-                const double* a = Aloc + (size_t)q * n + i;
-                acc0 = fma(a[0], vbuf[c0], acc0);
-                acc1 = fma(a[n], vbuf[c0 + C], acc1);
-                acc2 = fma(a[2 * n], vbuf[c0 + 2 * C], acc2);
-                acc3 = fma(a[3 * n], vbuf[c0 + 3 * C], acc3);
-            }
-            for (; q < ncl; ++q) {
-                const int c = q * C + rank;
-                if (c >= n) break;
-                acc0 = fma(Aloc[(size_t)q * n + i], vbuf[c], acc0);
-            }
-            ppart[i] = (acc0 + acc1) + (acc2 + acc3);
-        }
-        cluster.sync();                                   // partial products published
-        for (int i = i0 + tid; i < n; i += bd) {
-            double t[C];
-#pragma unroll
-            for (int r = 0; r < C; ++r) t[r] = cluster.map_shared_rank(ppart, r)[i];
-#pragma unroll
-            for (int wd = 1; wd < C; wd <<= 1)
-#pragma unroll
-                for (int r = 0; r + wd < C; r += 2 * wd) t[r] += t[r + wd];
-            pw[i] = tj * t[0];
-        }
-        __syncthreads();
-        double pv = 0.0;
-        for (int i = i0 + tid; i < n; i += bd) pv = fma(pw[i], vbuf[i], pv);
-        pv = block_sum(pv, red);
-        const double kk = 0.5 * tj * pv;
-        for (int i = i0 + tid; i < n; i += bd) pw[i] = fma(-kk, vbuf[i], pw[i]);
-        __syncthreads();
-        if (own_next) {
-            double* col = Aloc + (size_t)(next / C) * n;
-            const double vc = vbuf[next], wc = pw[next];
-            for (int i = i0 + tid; i < n; i += bd) col[i] -= fma(vbuf[i], wc, pw[i] * vc);
-            __syncthreads();
-            make_reflector(next, n, col, vpub, HV, eoff, tau, red);
-        }
-        {
-            const int qskip = own_next ? next / C : -1;
-            int qend = ncl;
-            while (qend > q0 && (qend - 1) * C + rank >= n) --qend;
-            for (int i = i0 + tid; i < n; i += bd) {
-                const double vi = vbuf[i], wi = pw[i];
-                int q = q0;
-                for (; q + 3 < qend; q += 4) {
-                    double* c0 = Aloc + (size_t)q * n + i;
-                    const int cc = q * C + rank;
-                    const double a0 = c0[0], a1 = c0[n], a2 = c0[2 * n], a3 = c0[3 * n];
-                    const double r0 = a0 - fma(vi, pw[cc], wi * vbuf[cc]);
-                    const double r1 = a1 - fma(vi, pw[cc + C], wi * vbuf[cc + C]);
-                    const double r2 = a2 - fma(vi, pw[cc + 2 * C], wi * vbuf[cc + 2 * C]);
-                    const double r3 = a3 - fma(vi, pw[cc + 3 * C], wi * vbuf[cc + 3 * C]);
-                    if (q != qskip) c0[0] = r0;
-                    if (q + 1 != qskip) c0[n] = r1;
-                    if (q + 2 != qskip) c0[2 * n] = r2;
-                    if (q + 3 != qskip) c0[3 * n] = r3;
-                }
-                for (; q < qend; ++q) {
-                    if (q == qskip) continue;
-                    const int cc = q * C + rank;
-                    double* c0 = Aloc + (size_t)q * n + i;
-                    c0[0] -= fma(vi, pw[cc], wi * vbuf[cc]);
-                }
-            }
-        }
-        __syncthreads();
-    }
-    for (int q = 0; q < ncl; ++q) {
-        const int c = q * C + rank;
-        if (c >= n) break;
-        if (tid == 0) {
-            dgl[c] = Aloc[(size_t)q * n + c];
-            if (c == n - 2) eoff[c] = Aloc[(size_t)q * n + c + 1];
-        }
-    }
-    if (rank == 0) {
-        for (int jj = (n >= 2 ? n - 2 : 0); jj < n; ++jj) {
-            if (tid == 0) tau[jj] = 0.0;
-            for (int i = tid; i < n; i += bd) HV[(int64_t)jj * n + i] = 0.0;
-        }
-        if (tid == 0) eoff[n - 1] = 0.0;
-    }
-    cluster.sync();   // no CTA leaves while another may still read its shared memory
-}
-
-// Householder tridiagonalisation on a cooperative grid of G CTAs with the matrix resident in shared
-// memory: column c is owned by CTA c % G (slot c / G, n doubles). Per column j, after the grid barrier
-// that publishes reflector j (global memory, read through L2): every CTA copies it into shared memory,
-// forms p[r] = tau v^T A[:, r] for its own columns r and its share of p^T v (its columns in increasing
-// order), publishes both; after a second barrier every CTA reads p and the G shares (summed in CTA
-// order: the same value everywhere), forms w = p - (tau / 2)(p^T v) v and updates its columns
-// (A -= v w^T + w v^T). The owner of column j + 1 updates that column first and publishes reflector
-// j + 1 while the others update theirs (look-ahead). Two bounded grid barriers per column on the
-// monotonic arrival counter; the columns never leave shared memory.
-__global__ void __launch_bounds__(TRI_THREADS) k_tridiag_res(int n, const double* __restrict__ Ain, int lda,
-                                                             double* vglob, double* pglob, double* pshare, double* HV,
-                                                             double* dgl, double* eoff, double* tau, GridBarWords bw,
-                                                             int* status) {
-    extern __shared__ double sm[];
-    __shared__ double red[32];
-    __shared__ double s_pv;
+    __shared__ double red[2][TD_RED / 32];   // partial sums of v^T p and of ||x'||^2
+    __shared__ double s_pc, s_alpha;         // p_c; x'_{c+1}
+    __shared__ double s_beta, s_tau, s_htau, s_v1;   // the current reflector: beta, tau, tau / 2, v_{c+1}
     const int G = gridDim.x, cta = blockIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int NW = TD_WARPS;
     const int ncl = (n + G - 1) / G;
-    double* vs = sm;             // n: reflector j
-    double* ws = sm + n;         // n: p, then w
-    double* Aloc = sm + 2 * n;   // ncl x n: the owned columns
-    double* shs = Aloc + (size_t)ncl * n;   // G: the CTAs' shares of p^T v
-    const int tid = threadIdx.x, bd = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = bd >> 5;
-    const unsigned base = gb_base(bw);
-    unsigned nb = 0;
+    double* vs = sm;                     // n: reflector of the previous column (entries below its first)
+    double* xs = sm + n;                 // n: the current column
+    double* ws = sm + 2 * n;             // n: p, then w
+    const int split = td_split(ncl);
+    double* sdot = sm + 3 * n;             // ncl x (32 split): the lanes' partial sums of A x
+    double* pin = sdot + td_dots(ncl);     // cluster: 2 x n, p of this column and of the next (written by all CTAs)
+    double* Aloc = CL ? (in_smem ? pin + 2 * n : Aglob + (size_t)cta * ncl * n) : pin;
 
     for (int q = 0; q < ncl; ++q) {
-        const int c = q * G + cta;
-        if (c >= n) break;
-        for (int i = tid; i < n; i += bd)
-            Aloc[(size_t)q * n + i] = 0.5 * (Ain[(int64_t)c * lda + i] + Ain[(int64_t)i * lda + c]);
+        const int r = q * G + cta;
+        if (r >= n) break;
+        for (int i = tid; i < n; i += TD_THREADS)
+            Aloc[(size_t)q * n + i] = 0.5 * (Ain[(int64_t)r * lda + i] + Ain[(int64_t)i * lda + r]);
     }
+    for (int i = tid; i < n; i += TD_THREADS) {
+        vs[i] = 0.0;
+        ws[i] = 0.0;
+        xs[i] = 0.5 * (Ain[i] + Ain[(int64_t)i * lda]);
+    }
+    if (tid == 0) s_tau = s_htau = s_v1 = 0.0;
     __syncthreads();
-    if (n >= 3 && cta == 0) make_reflector(0, n, Aloc, vglob, HV, eoff, tau, red);
-    gb_sync(bw, base, ++nb, status);
 
-    for (int j = 0; j + 2 < n; ++j) {
-        const int i0 = j + 1;
-        const int next = j + 1;
-        const bool own_next = (next + 2 < n) && (next % G == cta);
-        const int q0 = (i0 - cta + G - 1) / G;   // first owned slot with a column >= i0
-        const double tj = __ldcg(vglob + n);
-        if (tj == 0.0) {
-            // no reflection at this column: every CTA has read tau before the owner of j + 1 overwrites it
-            gb_sync(bw, base, ++nb, status);
-            if (own_next) make_reflector(next, n, Aloc + (size_t)(next / G) * n, vglob, HV, eoff, tau, red);
-            gb_sync(bw, base, ++nb, status);
-            continue;
+    for (int c = 0; c + 1 < n; ++c) {
+        double ss = 0.0;
+        if (c > 0) {
+            // ---- p (warps 0-3) and the raw column c (warps 4-7) into ws and xs; v^T p ----
+            const bool first = tid < TD_RED;   // the last warp (the scalars') takes no part
+            double acc = 0.0;
+            double* dst = first ? ws : xs;
+            const double vc = s_v1;
+            auto take = [&](int i, double x) {
+                dst[i] = x;
+                if (first) {
+                    acc = fma(i == c ? vc : vs[i], x, acc);
+                    if (i == c) s_pc = x;
+                }
+            };
+            if (CL) {
+                cg::cluster_group cluster = cg::this_cluster();
+                const int oc = c & (G - 1);   // a cluster's size is a power of two
+                const double* own = in_smem ? cluster.map_shared_rank(Aloc, oc) : Aglob + (size_t)oc * ncl * n;
+                const double* col = own + (size_t)(c / G) * n;
+                const double* src = first ? pin + ((c - 1) & 1) * n : col;
+                if (warp < NW)
+                    for (int i = c + (tid & (TD_RED - 1)); i < n; i += TD_RED) take(i, src[i]);
+            } else if (warp < NW) {
+                const double* src = (first ? pbuf : cbuf) + (size_t)(c - 1) * n;
+                // one lane waits for its value before the warp reads all of them: the polls of every lane of every CTA
+                // would slow down the writes that they wait for
+                if (lane == 0 && c + tid % TD_RED < n) {
+                    long long polls = 0;
+                    while (td_ld(src + c + tid % TD_RED) == TD_EMPTY && spin >= 0 && ++polls <= spin) {
+                    }
+                }
+                __syncwarp();
+                for (int i0 = c + (tid & (TD_RED - 1)); i0 < n; i0 += 4 * TD_RED) {
+                    unsigned long long u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) u[k] = i0 + k * TD_RED < n ? td_ld(src + i0 + k * TD_RED) : 0ull;
+                    long long polls = 0;
+                    while (u[0] == TD_EMPTY || u[1] == TD_EMPTY || u[2] == TD_EMPTY || u[3] == TD_EMPTY) {
+                        if (++polls > spin) {
+                            if (spin >= 0) atomicOr(status, ST_TIMEOUT);
+                            spin = -1;   // this thread does not wait again
+                            break;
+                        }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (u[k] == TD_EMPTY) u[k] = td_ld(src + i0 + k * TD_RED);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (i0 + k * TD_RED < n) take(i0 + k * TD_RED, __longlong_as_double((long long)u[k]));
+                }
+            }
+            if (first) {
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0) red[0][warp] = acc;
+            }
+            __syncthreads();
+            // ---- w and the finished column x' ----
+            if (first) {
+                const double K = s_htau * ((red[0][0] + red[0][1]) + (red[0][2] + red[0][3]));
+                const double wc = fma(-K, vc, s_pc);
+                for (int i = c + tid; i < n; i += TD_RED) {
+                    const double vi = i == c ? vc : vs[i];
+                    const double wi = fma(-K, vi, ws[i]);
+                    const double xi = fma(-wi, vc, fma(-vi, wc, xs[i]));
+                    ws[i] = wi;
+                    xs[i] = xi;
+                    if (i >= c + 2) ss = fma(xi, xi, ss);
+                    if (i == c + 1) s_alpha = xi;
+                    if (i == c && cta == 0) dgl[c] = xi;
+                }
+            } else if (warp < NW && cta == (c - 1) % G) {
+                // the previous reflector, for the back-transformation
+                for (int i = tid - TD_RED; i < n; i += TD_RED)
+                    HV[(int64_t)(c - 1) * n + i] = i < c ? 0.0 : (i == c ? vc : vs[i]);
+            }
+        } else if (tid < TD_RED) {
+            for (int i = tid; i < n; i += TD_RED) {
+                const double xi = xs[i];
+                if (i >= 2) ss = fma(xi, xi, ss);
+                if (i == 1) s_alpha = xi;
+                if (i == 0 && cta == 0) dgl[0] = xi;
+            }
         }
-        for (int i = i0 + tid; i < n; i += bd) vs[i] = __ldcg(vglob + i);
+        if (tid < TD_RED) {
+            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            if (lane == 0) red[1][warp] = ss;
+        }
         __syncthreads();
-        // p over the owned columns, one warp per column (lane-strided dot, fixed shuffle tree)
-        for (int q = q0 + warp; q < ncl; q += nw) {
+        if (c + 2 == n) break;
+        // ---- the reflector's scalars (one warp) beside the update of the owned columns and their products with x' ----
+        if (warp == NW) {
+            const double alpha = s_alpha;
+            const double sig = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
+            double beta = alpha, t = 0.0, v1 = 0.0;
+            if (__double_as_longlong(sig) != 0) {   // tests on the bits: a comparison would take the FP64 pipe
+                const double ab = td_sqrt(fma(alpha, alpha, sig));
+                const double av = fabs(alpha) + ab;   // |alpha - beta|: beta has the other sign
+                t = td_rcp(ab * av);
+                const int sg = __double2hiint(alpha) & 0x80000000;
+                beta = __hiloint2double(__double2hiint(ab) | (sg ^ 0x80000000), __double2loint(ab));
+                v1 = __hiloint2double(__double2hiint(av) | sg, __double2loint(av));
+            }
+            if (lane == 0) {
+                s_beta = beta;
+                s_tau = t;
+                s_htau = 0.5 * t;
+                s_v1 = v1;
+                if (cta == 0) {
+                    eoff[c] = beta;
+                    tau[c] = t;
+                }
+            }
+        }
+        const int i0 = c + 1;
+        const int q0 = (i0 - cta + G - 1) / G;   // first owned slot with a column >= i0
+        // few tasks: none on the scalar warp's sub-partition (warps 0 and 4)
+        const int ntask = (ncl - q0) * split;
+        const bool apart = ntask <= 2 * (NW - 2);
+        const int tw = apart ? ((warp & 3) == 0 ? ntask : (warp < 4 ? warp - 1 : warp - 2)) : warp;
+        for (int task = tw; warp < NW && task < ntask; task += apart ? NW - 2 : NW) {
+            const int q = q0 + task / split, part = task % split;
             const int r = q * G + cta;
             if (r >= n) break;
-            const double* col = Aloc + (size_t)q * n;
-            double a0 = 0.0, a1 = 0.0;
-            int c = i0 + lane;
-            for (; c + 32 < n; c += 64) {
-                a0 = fma(col[c], vs[c], a0);
-                a1 = fma(col[c + 32], vs[c + 32], a1);
-            }
-            if (c < n) a0 = fma(col[c], vs[c], a0);
-            double acc = a0 + a1;
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) {
-                const double p = tj * acc;
-                pglob[r] = p;
-                ws[r] = p;
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double sh = 0.0;
-            for (int q = q0; q < ncl; ++q) {
-                const int r = q * G + cta;
-                if (r >= n) break;
-                sh = fma(ws[r], vs[r], sh);
-            }
-            pshare[cta] = sh;
-        }
-        gb_sync(bw, base, ++nb, status);
-        // w = p - (tau / 2)(p^T v) v
-        for (int i = i0 + tid; i < n; i += bd) ws[i] = __ldcg(pglob + i);
-        for (int g = tid; g < G; g += bd) shs[g] = __ldcg(pshare + g);
-        __syncthreads();
-        if (warp == 0) {
-            // the G shares in a fixed order (lane-strided runs, then a shuffle tree): the same value in every CTA
-            double pv = 0.0;
-            for (int g = lane; g < G; g += 32) pv += shs[g];
-            for (int o = 16; o > 0; o >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, o);
-            if (lane == 0) s_pv = pv;
-        }
-        __syncthreads();
-        const double kk = 0.5 * tj * s_pv;
-        for (int i = i0 + tid; i < n; i += bd) ws[i] = fma(-kk, vs[i], ws[i]);
-        __syncthreads();
-        if (own_next) {
-            double* col = Aloc + (size_t)(next / G) * n;
-            const double vc = vs[next], wc = ws[next];
-            for (int i = i0 + tid; i < n; i += bd) col[i] -= fma(vs[i], wc, ws[i] * vc);
-            __syncthreads();
-            make_reflector(next, n, col, vglob, HV, eoff, tau, red);
-        }
-        for (int q = q0; q < ncl; ++q) {
-            const int c = q * G + cta;
-            if (c >= n) break;
-            if (own_next && c == next) continue;
             double* col = Aloc + (size_t)q * n;
-            const double vc = vs[c], wc = ws[c];
-            for (int i = i0 + tid; i < n; i += bd) col[i] -= fma(vs[i], wc, ws[i] * vc);
+            const double vr = vs[r], wr = ws[r];
+            double* pub = (!CL && r == i0) ? cbuf + (size_t)c * n : nullptr;   // the next column: publish it on the way
+            double acc0 = 0.0, acc1 = 0.0;
+            int i = i0 + 32 * part + lane;
+            const int st = 32 * split;
+            for (; i + st < n; i += 2 * st) {
+                const double a0 = fma(-ws[i], vr, fma(-vs[i], wr, col[i]));
+                const double a1 = fma(-ws[i + st], vr, fma(-vs[i + st], wr, col[i + st]));
+                col[i] = a0;
+                col[i + st] = a1;
+                if (pub) {
+                    td_st(pub + i, a0);
+                    td_st(pub + i + st, a1);
+                }
+                acc0 = fma(a0, xs[i], acc0);
+                acc1 = fma(a1, xs[i + st], acc1);
+            }
+            if (i < n) {
+                const double a0 = fma(-ws[i], vr, fma(-vs[i], wr, col[i]));
+                col[i] = a0;
+                if (pub) td_st(pub + i, a0);
+                acc0 = fma(a0, xs[i], acc0);
+            }
+            sdot[(q * split + part) * 32 + lane] = acc0 + acc1;
         }
-        gb_sync(bw, base, ++nb, status);
+        // ---- p = tau (A x' - beta A e_{c+1}) of the owned rows: the lanes' sums by 8 threads a column, or by a warp,
+        //      while the scalar warp still works (a barrier of the other warps alone), then the scalars ----
+        const int tpc = split == 1 ? 8 : 32;           // threads per column
+        const int g = tid & (tpc - 1), cps = (32 * NW) / tpc;
+        constexpr int MAXP = 16;                       // rounds held in registers: up to 512 columns a CTA (n = 1024, two CTAs)
+        double ax[MAXP], a0[MAXP];
+        if (warp < NW) {
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory");
+#pragma unroll
+            for (int u = 0; u < MAXP; ++u) {
+                ax[u] = a0[u] = 0.0;
+                const int q = q0 + u * cps + tid / tpc;
+                if (q0 + u * cps + (32 * warp) / tpc >= ncl) break;   // none of this warp's columns (uniform)
+                if (q < ncl) {
+                    const double* d = sdot + (size_t)q * split * 32 + g;
+                    if (split == 1) ax[u] = (d[0] + d[8]) + (d[16] + d[24]);
+                    else if (split == 2) ax[u] = d[0] + d[32];
+                    else ax[u] = (d[0] + d[32]) + (d[64] + d[96]);
+                    a0[u] = Aloc[(size_t)q * n + i0];
+                }
+                for (int o = tpc >> 1; o > 0; o >>= 1) ax[u] += __shfl_xor_sync(0xffffffffu, ax[u], o);
+            }
+        }
+        __syncthreads();
+        if (warp < NW) {
+            const double tj = s_tau, bj = s_beta;
+#pragma unroll
+            for (int u = 0; u < MAXP; ++u) {
+                const int q = q0 + u * cps + tid / tpc;
+                if (q0 + u * cps + (32 * warp) / tpc >= ncl) break;
+                const int r = q * G + cta;
+                if (q >= ncl || r >= n) continue;
+                const double p = tj * fma(-bj, a0[u], ax[u]);
+                if (CL) {
+                    double* mine = pin + (c & 1) * n + r;
+                    for (int k = g; k < G; k += tpc) *cg::this_cluster().map_shared_rank(mine, k) = p;
+                } else if (g == 0) {
+                    td_st(pbuf + (size_t)c * n + r, p);
+                }
+            }
+        }
+        double* sw = vs;   // x' becomes the reflector (its first entry is s_v1)
+        vs = xs;
+        xs = sw;
+        if (CL) cg::this_cluster().sync();
     }
-    for (int q = 0; q < ncl; ++q) {
-        const int c = q * G + cta;
-        if (c >= n) break;
-        if (tid == 0) {
-            dgl[c] = Aloc[(size_t)q * n + c];
-            if (c == n - 2) eoff[c] = Aloc[(size_t)q * n + c + 1];
+    if (n >= 2) {
+        // column n - 2 is x'; the last diagonal entry is the owner's, updated by the last reflector
+        if (cta == 0 && tid == 0) eoff[n - 2] = xs[n - 1];
+        if (cta == (n - 1) % G && tid == 0) {
+            const double a = Aloc[(size_t)((n - 1) / G) * n + n - 1];
+            dgl[n - 1] = fma(-2.0 * vs[n - 1], ws[n - 1], a);
         }
+    } else if (cta == 0 && tid == 0) {
+        dgl[0] = xs[0];
     }
     if (cta == 0) {
         for (int jj = (n >= 2 ? n - 2 : 0); jj < n; ++jj) {
             if (tid == 0) tau[jj] = 0.0;
-            for (int i = tid; i < n; i += bd) HV[(int64_t)jj * n + i] = 0.0;
+            for (int i = tid; i < n; i += TD_THREADS) HV[(int64_t)jj * n + i] = 0.0;
         }
         if (tid == 0) eoff[n - 1] = 0.0;
     }
-    gb_finish(bw, base, nb);
+    if (CL) cg::this_cluster().sync();   // no CTA leaves while another may still read its shared memory
 }
 
 // Number of eigenvalues below x of the tridiagonal with diagonal d and squared off-diagonal e2, in
@@ -1114,11 +1119,16 @@ int symeig_orth_clusters(int n, int nv, const double* w, double* Z, int ldz, Sym
                          int maxc, cudaStream_t s);
 int symeig_backtransform(int n, int nv, double* Z, int ldz, SymEigWork* ws, cudaStream_t s);
 
+// the cooperative grid from here when its columns fit: at n = 288 a column step takes about 5 us on either path, beyond it
+// the columns of 16 CTAs grow with n while those of the grid's up to 152 stay few
+constexpr int kResMinN = 288;
+
 size_t symeig_work_bytes(int n, int nv) {
     const size_t nn = (size_t)n * n;
     size_t b = 0;
     auto add = [&](size_t cnt) { b += ((cnt * sizeof(double) + 255) / 256) * 256; };
-    add(nn + 16 * (size_t)n);   // A (the cluster path keeps up to n + 16 columns of n)
+    add(nn + 16 * (size_t)n);   // A (the cluster path keeps up to n + 16 columns of n; the grid path its exchange of p)
+    add(n >= kResMinN ? nn : 0);   // X (the grid path's exchange of columns)
     add(nn);            // HV
     add(n);             // d
     add(n);             // e
@@ -1131,6 +1141,7 @@ size_t symeig_work_bytes(int n, int nv) {
 int symeig_work_carve(Arena& a, int n, int nv, GridBarrier bar, SymEigWork* w) {
     const size_t nn = (size_t)n * n;
     w->A = a.take<double>(nn + 16 * (size_t)n);
+    w->X = a.take<double>(n >= kResMinN ? nn : 0);
     w->partial = a.take<double>(nn);      // HV
     w->dgl = a.take<double>(n);
     w->eoff = a.take<double>(n);
@@ -1139,13 +1150,13 @@ int symeig_work_carve(Arena& a, int n, int nv, GridBarrier bar, SymEigWork* w) {
     w->lu = a.take<double>(6 * (size_t)n * std::max(nv, 1));
     w->bar = bar;
     w->max_ctas = 0;
-    if (!w->A || !w->partial || !w->dgl || !w->eoff || !w->tau || !w->vbuf || !w->lu) return EDA_ERR_OOM;
+    if (!w->A || !w->partial || !w->dgl || !w->eoff || !w->tau || !w->vbuf || !w->lu || !w->X) return EDA_ERR_OOM;
+    w->xn = n >= kResMinN ? n : 0;
     return EDA_OK;
 }
 
 constexpr int kClusterMaxN = 512;        // the cluster path up to here; a cooperative grid beyond
 constexpr int kClusterMaxNShared = 1024; // limit of the cluster path when the GPU is shared (see below)
-constexpr int kResMinN = 288;            // the resident-column cooperative grid from here (when it fits)
 
 // Host threads that run many problems side by side (the batched solver) set this: a cooperative
 // grid with a software grid barrier needs all its CTAs resident at once, which concurrent kernels
@@ -1154,25 +1165,24 @@ constexpr int kResMinN = 288;            // the resident-column cooperative grid
 // kClusterMaxNShared.
 thread_local bool tl_shared_gpu = false;
 
-// Launch k_tridiag_cluster<C> on one cluster of C CTAs (a power of two, 16 only when the device
-// accepts that non-portable cluster size with the needed shared memory).
-template <int C>
-int launch_tridiag_cluster(int n, const double* A, int lda, SymEigWork* ws, cudaStream_t s, bool probe_only,
-                           bool* fits) {
-    auto kern = k_tridiag_cluster<C>;
+// Launch k_tridiag_x on one cluster of C CTAs (a power of two, 16 only when the device accepts that non-portable
+// cluster size with the needed shared memory).
+int launch_tridiag_cluster(int C, int n, const double* A, int lda, SymEigWork* ws, int* status, cudaStream_t s,
+                           bool probe_only, bool* fits) {
+    auto kern = k_tridiag_x<true>;
     static std::mutex mu;                 // the function attributes below are shared by all threads
     static size_t smem_set = 0;
     static bool attrs = false;
     const int ncl = (n + C - 1) / C;
-    const size_t vec_bytes = (4 * (size_t)n + 2) * sizeof(double);
+    const size_t vec_bytes = (5 * (size_t)n + td_dots(ncl)) * sizeof(double);
     const size_t a_bytes = (size_t)ncl * n * sizeof(double);
-    const int in_smem = (vec_bytes + a_bytes <= 200 * 1024) ? 1 : 0;
+    const int in_smem = (vec_bytes + a_bytes <= 220 * 1024) ? 1 : 0;
     const size_t smem = vec_bytes + (in_smem ? a_bytes : 0);
     {
         std::lock_guard<std::mutex> lk(mu);
         if (!attrs) {
             attrs = true;
-            if (C > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             cudaGetLastError();
         }
         if (smem > smem_set) {
@@ -1188,7 +1198,7 @@ int launch_tridiag_cluster(int n, const double* A, int lda, SymEigWork* ws, cuda
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(CT_THREADS);
+    cfg.blockDim = dim3(TD_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -1200,85 +1210,71 @@ int launch_tridiag_cluster(int n, const double* A, int lda, SymEigWork* ws, cuda
         return EDA_OK;
     }
     ProfScope prof("tridiag", s, 4.0 / 3.0 * (double)n * n * n);
-    EDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, n, A, lda, ws->A, in_smem, ws->partial, ws->dgl, ws->eoff, ws->tau));
+    EDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, n, A, lda, ws->A, in_smem, (double*)nullptr, (double*)nullptr, ws->partial,
+                                    ws->dgl, ws->eoff, ws->tau, 0LL, status));
     launch_counter()++;
     return EDA_OK;
 }
 
-int launch_tridiag_c(int C, int n, const double* A, int lda, SymEigWork* ws, cudaStream_t s, bool probe_only,
-                     bool* fits) {
-    switch (C) {
-        case 16: return launch_tridiag_cluster<16>(n, A, lda, ws, s, probe_only, fits);
-        case 8: return launch_tridiag_cluster<8>(n, A, lda, ws, s, probe_only, fits);
-        case 4: return launch_tridiag_cluster<4>(n, A, lda, ws, s, probe_only, fits);
-        case 2: return launch_tridiag_cluster<2>(n, A, lda, ws, s, probe_only, fits);
-        default: return launch_tridiag_cluster<1>(n, A, lda, ws, s, probe_only, fits);
-    }
-}
-
-int tridiag_cluster(int n, const double* A, int lda, SymEigWork* ws, cudaStream_t s) {
+int tridiag_cluster(int n, const double* A, int lda, SymEigWork* ws, int* status, cudaStream_t s) {
     static int chosen_C[kClusterMaxNShared + 1] = {};   // cluster size that passed the occupancy check, per n
     static std::mutex mu;
     std::unique_lock<std::mutex> lk(mu);
     if (!chosen_C[n]) {
-        // about 12 or more columns per CTA: fewer FP64 instructions per warp and column step (each
-        // holds a sub-partition's FP64 pipe for ~64 cycles) outweigh the wider cluster barrier
-        int want = 2;
-        if (n > 32) {
-            want = 1;
-            while (want < 16 && want * 2 * 12 <= n) want *= 2;
-        }
-        // clusters of at least two CTAs: the kernel's one-CTA instance loses accuracy on small n and is
-        // not used
+        // eight columns or more per CTA, one for each warp of the pass (4, 6 and 12 measured within 3 %, n = 48 .. 200)
+        int want = 1;
+        while (want < 16 && want * 2 * 8 <= n) want *= 2;
         int C = std::max(2, want);
         for (; C > 2; C /= 2) {
             bool fits = false;
-            EDA_TRY(launch_tridiag_c(C, n, A, lda, ws, s, true, &fits));
+            EDA_TRY(launch_tridiag_cluster(C, n, A, lda, ws, status, s, true, &fits));
             if (fits) break;
         }
         chosen_C[n] = C;
     }
     const int C = chosen_C[n];
     lk.unlock();
-    return launch_tridiag_c(C, n, A, lda, ws, s, false, nullptr);
+    return launch_tridiag_cluster(C, n, A, lda, ws, status, s, false, nullptr);
 }
 
-// The resident-column grid (k_tridiag_res): about four columns per CTA, at most one CTA per SM, when the
-// owned columns and two work vectors fit in 200 KB of shared memory. INVALID_ARG: does not apply.
+// k_tridiag_x on a cooperative grid: about four columns per CTA, at most one CTA per SM, when the owned columns and
+// three work vectors fit in 220 KB of shared memory. INVALID_ARG: does not apply.
 int tridiag_res(int n, const double* A, int lda, double* HV, SymEigWork* ws, int* status, int sms, cudaStream_t s) {
     const int G = std::max(1, std::min(sms, (n + 3) / 4));
     const int ncl = (n + G - 1) / G;
-    const size_t smem = ((size_t)(ncl + 2) * n + G) * sizeof(double);
-    if (smem > 200 * 1024 || 2 * (size_t)n + 2 + G > 4 * (size_t)n) return EDA_ERR_INVALID_ARG;
+    const size_t smem = ((size_t)(ncl + 3) * n + td_dots(ncl)) * sizeof(double);
+    if (smem > 220 * 1024 || ws->xn < n) return EDA_ERR_INVALID_ARG;
+    auto kern = k_tridiag_x<false>;
     {
         static std::mutex mu;
         static size_t set = 0;
         std::lock_guard<std::mutex> lk(mu);
         if (smem > set && smem > 40 * 1024) {
-            EDA_CUDA_TRY(cudaFuncSetAttribute(k_tridiag_res, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            EDA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)std::max<size_t>(smem, 48 * 1024)));
             set = std::max<size_t>(smem, 48 * 1024);
         }
     }
     int per_sm = 0;
-    EDA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_res, TRI_THREADS, smem));
+    EDA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TD_THREADS, smem));
     if (per_sm < 1 || G > per_sm * sms) return EDA_ERR_INVALID_ARG;
-    // both barrier words to zero: the launch starts its arrival count from 0
-    EDA_CUDA_TRY(cudaMemsetAsync(ws->bar.count, 0, 256, s));
+    // both exchange buffers to the "not written yet" pattern
+    EDA_CUDA_TRY(cudaMemsetAsync(ws->A, 0xFF, (size_t)n * n * sizeof(double), s));
+    EDA_CUDA_TRY(cudaMemsetAsync(ws->X, 0xFF, (size_t)n * n * sizeof(double), s));
     ProfScope prof("tridiag", s, 4.0 / 3.0 * (double)n * n * n);
-    int nn = n, ld = lda;
+    int nn = n, ld = lda, insm = 1;
     const double* a0 = A;
-    double* vg = ws->vbuf;
-    double* pg = ws->vbuf + n + 2;
-    double* ps = ws->vbuf + 2 * n + 2;
+    double* ag = nullptr;
+    double* pb = ws->A;
+    double* cb = ws->X;
     double* a1 = HV;
     double* a2 = ws->dgl;
     double* a3 = ws->eoff;
     double* a4 = ws->tau;
-    GridBarWords bw{ws->bar.count, ws->bar.gen, ws->bar.spin_limit};
+    long long spin = ws->bar.spin_limit;
     int* st = status;
-    void* args[] = {&nn, &a0, &ld, &vg, &pg, &ps, &a1, &a2, &a3, &a4, &bw, &st};
-    EDA_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_tridiag_res, dim3(G), dim3(TRI_THREADS), args, smem, s));
+    void* args[] = {&nn, &a0, &ld, &ag, &insm, &pb, &cb, &a1, &a2, &a3, &a4, &spin, &st};
+    EDA_CUDA_TRY(cudaLaunchCooperativeKernel((void*)kern, dim3(G), dim3(TD_THREADS), args, smem, s));
     launch_counter()++;
     return EDA_OK;
 }
@@ -1313,7 +1309,7 @@ int symeig_values(int n, const double* A, int lda, int il, int iu, double* w, Sy
     } else if (res != EDA_ERR_INVALID_ARG) {
         return res;
     } else if (n <= (tl_shared_gpu ? kClusterMaxNShared : kClusterMaxN)) {
-        EDA_TRY(tridiag_cluster(n, A, lda, ws, s));
+        EDA_TRY(tridiag_cluster(n, A, lda, ws, status, s));
     } else {
     int per_sm = 0;
     EDA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag, TRI_THREADS, smem));

@@ -40,3 +40,37 @@ def test_solve_block_width_edges(eda, b):
     assert np.abs(V.T @ V - np.eye(p.k - 1)).max() <= 1e-13
     assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
     assert O.sin_angle(ref["V"], V) <= 1e-8
+
+
+# matrix orders around the eigensolver's rules (cluster sizes double from 24 columns on, the cooperative grid starts at
+# 288, one exchange chunk holds 512 rows, the columns of 608 and more no longer come four to a CTA) and its smallest
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 23, 24, 25, 48, 97, 192, 257, 287, 288, 289, 511, 513, 609, 700])
+def test_gram_eigenvalue_orders(eda, n):
+    rng = np.random.default_rng(n)
+    d = 720
+    k = max(1, n // 6)
+    lab = rng.permutation(np.arange(n) % k).astype(np.int32)
+    X = rng.random((n, d))
+    with eda.build(_dev(X), _dev(lab), k, eda.config(tau=5.0)) as h:
+        f = h.factors()
+        c2 = h.c2
+    G = f["GW"].cpu().numpy()
+    ev, Q = np.linalg.eigh(G)
+    # Householder reduction and bisection are backward stable: errors of order n eps ||G||
+    assert np.abs(f["evals_w"].cpu().numpy() - ev).max() <= 4 * n * np.finfo(float).eps * ev[-1]
+    z = -0.5 * c2 * np.maximum(ev, 0.0)
+    phi = np.where(z == 0.0, 1.0, np.expm1(z) / np.where(z == 0.0, 1.0, z))
+    K = (Q * (-0.5 * c2 * phi)) @ Q.T
+    assert np.abs(f["KW"].cpu().numpy() - K).max() <= 1e-11 * np.abs(K).max()
+
+
+# the same reduction with the columns in a global slab: the largest Gram of a batch, whose kernels share the GPU
+def test_batched_large_gram(eda):
+    ps = [synth.gaussian_clusters(d=900, k=9, n_per_class=nj, seed=40 + nj) for nj in (72, 30, 20)]
+    probs = [dict(X=_dev(p.X), labels=_dev(p.labels), k=p.k, t=p.k - 1, tol=1e-11) for p in ps]
+    res, code = eda.solve_batched(probs, eda.config(block_b=8, tau=8.0), workers=3)
+    assert code == 0
+    for p, r in zip(ps, res):
+        ref = O.eda(p.X, p.labels, p.k, p.k - 1, c2=r["info"]["c2"], tier="projected")
+        assert np.max(np.abs(r["lam"].cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
+        assert O.sin_angle(ref["V"], r["V"].cpu().numpy().T) <= 1e-8

@@ -282,6 +282,10 @@ int eda_get_dims(eda_handle h, int64_t* d, int64_t* n, int32_t* k, double* c2,
                  double* lmax_w, double* lmax_b);
 
 void eda_destroy(eda_handle h);
+/* Device memory, streams and pinned pages of destroyed handles are kept for the next ones (at most a sixteenth
+ * of the device's memory; less-used blocks are released as newer ones come in, all of them when an
+ * allocation fails). This call gives everything that is kept for the current device back to the driver. */
+int eda_release_cached(void);
 const char* eda_strerror(int status);
 /* The last CUDA error code seen by any call of this thread (0 = none), and its name with the
  * library source location that saw it (a static per-thread string). */

@@ -174,8 +174,7 @@ int arn_ritz(eda_ctx* h, int m, int ldh, int t, int b, ArnWs& w, std::vector<dou
     EDA_LAUNCHED();
     k_arn_relres<<<ceil_div(t, 128), 128, 0, s>>>(t, w.n1, w.n2, w.sn, w.theta, w.relres);
     EDA_LAUNCHED();
-    EDA_CUDA_TRY(cudaMemcpyAsync(relres_h.data(), w.relres, t * sizeof(double), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(relres_h.data(), w.relres, t * sizeof(double), s));
     return EDA_OK;
 }
 
@@ -204,8 +203,7 @@ int arn_true_residuals(eda_ctx* h, int m, int t, int b, ArnWs& w, std::vector<do
     EDA_CUDA_TRY(cudaMemsetAsync(w.n2, 0, t * sizeof(double), s));
     k_arn_relres<<<ceil_div(t, 128), 128, 0, s>>>(t, w.n1, w.n2, w.sn, w.theta, w.relres);
     EDA_LAUNCHED();
-    EDA_CUDA_TRY(cudaMemcpyAsync(relres_h.data(), w.relres, t * sizeof(double), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(relres_h.data(), w.relres, t * sizeof(double), s));
     return EDA_OK;
 }
 
@@ -222,7 +220,7 @@ int ensure_n_operators(eda_ctx* h, cudaStream_t s) {
     }
     const size_t nn = a256((size_t)n * n * 8);
     void* p = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&p, 2 * nn + a256(6 * (size_t)n * n * 8)));
+    EDA_TRY(dev_alloc(&p, 2 * nn + a256(6 * (size_t)n * n * 8)));
     h->nblock = p;
     h->KWm = static_cast<double*>(p);
     h->KWp = reinterpret_cast<double*>(static_cast<char*>(p) + nn);
@@ -274,9 +272,9 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
     if (m_max < t + b || m_max < 2 * b || m_max > (1 << 16)) return EDA_ERR_INVALID_ARG;
     EDA_TRY(ensure_n_operators(h, s));
 
-    cudaEvent_t ev0, ev1;
-    EDA_CUDA_TRY(cudaEventCreate(&ev0));
-    EDA_CUDA_TRY(cudaEventCreate(&ev1));
+    HostHold hold;
+    EDA_TRY(hold.open());
+    const cudaEvent_t ev0 = hold.kit->timer[0], ev1 = hold.kit->timer[1];
     EDA_CUDA_TRY(cudaEventRecord(ev0, s));
 
     ArnWs w{};
@@ -463,20 +461,13 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
         if (cudaMemcpyAsync(lambda, w.lamd, t * sizeof(double), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             rc = EDA_ERR_CUDA;
     } while (false);
-    if (rc != EDA_OK && rc != EDA_ERR_NOT_CONVERGED) {
-        cudaEventDestroy(ev0);
-        cudaEventDestroy(ev1);
-        return rc;
-    }
+    if (rc != EDA_OK && rc != EDA_ERR_NOT_CONVERGED) return rc;
     EDA_CUDA_TRY(cudaEventRecord(ev1, s));
     EDA_CUDA_TRY(cudaEventSynchronize(ev1));
     float ms = 0.f;
     EDA_CUDA_TRY(cudaEventElapsedTime(&ms, ev0, ev1));
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
     int stw = 0;
-    EDA_CUDA_TRY(cudaMemcpyAsync(&stw, h->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(&stw, h->status, sizeof(int), s));
     if (stw & ST_TIMEOUT) return EDA_ERR_TIMEOUT;
     if (stw & ST_NONFINITE) return EDA_ERR_NONFINITE;
     if (info) {

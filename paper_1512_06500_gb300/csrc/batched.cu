@@ -3,8 +3,8 @@
 //
 // Problems are ordered by an estimated cost, largest first, and taken from one shared queue by
 // `workers` host threads. Each worker owns a non-blocking CUDA stream and drives its problems through
-// eda_build, block-size tuning, eda_solve; the handles are destroyed after all workers have joined
-// (a cudaFree waits for the whole device). The per-problem kernels are small and latency-bound
+// eda_build, block-size tuning, eda_solve; a finished problem's memory goes back to the process's cache, from which
+// the worker's next problem takes it (devpool.cu), so a batch holds one handle per worker. The per-problem kernels are small and latency-bound
 // (cluster eigensolves on 2-16 SMs, Krylov sweeps over a few MB), so running many problems side by
 // side is what fills the GPU. The Krylov loop keeps its host decisions (rank loss, convergence
 // checks), which is why concurrency comes from streams and host workers rather than from one
@@ -54,16 +54,20 @@ int tune_block(eda_handle h, int t, cudaStream_t s, int* b_out) {
     const bool f32io = prec == EDA_F32 || prec == EDA_BF16;   // the FP64 solvers (also EDA_F64_TC) take FP64 blocks
     const size_t esz = f32io ? 4 : 8;
     void* buf = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&buf, 2 * (size_t)h->d * bmax * esz));
+    EDA_TRY(dev_alloc(&buf, 2 * (size_t)h->d * bmax * esz));
+    HostHold hold;
+    if (int rc = hold.open()) {
+        dev_free(buf);
+        return rc;
+    }
     char* X = static_cast<char*>(buf);
     char* Y = X + (size_t)h->d * bmax * esz;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    const cudaEvent_t e0 = hold.kit->timer[0], e1 = hold.kit->timer[1];
     int rc = EDA_OK;
     double best = INFINITY;
     int best_b = 8;
     do {
-        if (cudaMemsetAsync(buf, 0, 2 * (size_t)h->d * bmax * esz, s) != cudaSuccess ||
-            cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+        if (cudaMemsetAsync(buf, 0, 2 * (size_t)h->d * bmax * esz, s) != cudaSuccess) {
             rc = EDA_ERR_CUDA;
             break;
         }
@@ -89,10 +93,8 @@ int tune_block(eda_handle h, int t, cudaStream_t s, int* b_out) {
             }
         }
     } while (false);
-    if (e0) cudaEventDestroy(e0);
-    if (e1) cudaEventDestroy(e1);
     cudaStreamSynchronize(s);
-    cudaFree(buf);
+    dev_free(buf);
     if (rc != EDA_OK) return rc;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -128,8 +130,9 @@ extern "C" int eda_solve_batched(eda_problem* probs, int32_t nprob, const eda_co
     int dev = 0;
     EDA_CUDA_TRY(cudaGetDevice(&dev));
     cudaStream_t caller = static_cast<cudaStream_t>(stream);
-    cudaEvent_t start = nullptr;
-    EDA_CUDA_TRY(cudaEventCreateWithFlags(&start, cudaEventDisableTiming));
+    HostHold hold;
+    EDA_TRY(hold.open());
+    const cudaEvent_t start = hold.kit->order[0];
     EDA_CUDA_TRY(cudaEventRecord(start, caller));
 
     std::vector<int> order(nprob);
@@ -137,22 +140,18 @@ extern "C" int eda_solve_batched(eda_problem* probs, int32_t nprob, const eda_co
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return est_cost(probs[a]) > est_cost(probs[b]); });
     const int W = std::max(1, std::min<int>(workers > 0 ? workers : 16, nprob));
-    std::vector<eda_handle> handles(nprob, nullptr);
-    std::vector<cudaStream_t> streams(W, nullptr);
-    std::vector<cudaEvent_t> done(W, nullptr);
+    std::vector<HostKit*> kits(W, nullptr);   // each worker's stream and its last event
     std::atomic<int> next{0};
     std::vector<int> worker_rc(W, EDA_OK);
 
     auto work = [&](int w) {
         symeig_set_shared_gpu(true);   // no grid-wide barriers while other problems run beside this one
-        if (cudaSetDevice(dev) != cudaSuccess ||
-            cudaStreamCreateWithFlags(&streams[w], cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&done[w], cudaEventDisableTiming) != cudaSuccess ||
-            cudaStreamWaitEvent(streams[w], start, 0) != cudaSuccess) {
+        if (cudaSetDevice(dev) != cudaSuccess || host_kit_take(&kits[w]) != EDA_OK ||
+            cudaStreamWaitEvent(kits[w]->s, start, 0) != cudaSuccess) {
             worker_rc[w] = EDA_ERR_CUDA;
             return;
         }
-        cudaStream_t s = streams[w];
+        const cudaStream_t s = kits[w]->s;
         for (int q = next++; q < nprob; q = next++) {
             eda_problem& p = probs[order[q]];
             eda_config pc = c;
@@ -162,7 +161,6 @@ extern "C" int eda_solve_batched(eda_problem* probs, int32_t nprob, const eda_co
             pc.tc_fused = -1;
             eda_handle h = nullptr;
             int rc = eda_build(p.X, p.x_dtype, p.d, p.n, p.ldx, p.labels, p.k, &pc, s, &h);
-            handles[order[q]] = h;
             if (rc == EDA_OK && autotune && p.block_b <= 0) {
                 int b = 8;
                 rc = tune_block(h, p.t, s, &b);
@@ -173,8 +171,10 @@ extern "C" int eda_solve_batched(eda_problem* probs, int32_t nprob, const eda_co
                 rc = eda_solve(h, p.t, p.tol, nullptr, 0, p.V, p.lambda, nullptr, &p.info, s);
             }
             p.status = rc;
+            // the problem ran on this stream alone: once it is idle the handle's memory serves the next problem
+            if (h) destroy_handle(h, cudaStreamSynchronize(s) == cudaSuccess);
         }
-        cudaEventRecord(done[w], s);
+        cudaEventRecord(kits[w]->order[0], s);
     };
     std::vector<std::thread> pool;
     pool.reserve(W);
@@ -184,18 +184,12 @@ extern "C" int eda_solve_batched(eda_problem* probs, int32_t nprob, const eda_co
     int rc = EDA_OK;
     for (int w = 0; w < W; ++w) {
         if (worker_rc[w] != EDA_OK && rc == EDA_OK) rc = worker_rc[w];
-        if (done[w]) cudaStreamWaitEvent(caller, done[w], 0);
+        if (kits[w] && worker_rc[w] == EDA_OK) cudaStreamWaitEvent(caller, kits[w]->order[0], 0);
     }
     for (int w = 0; w < W; ++w) {
-        if (streams[w]) cudaStreamSynchronize(streams[w]);
+        if (kits[w]) cudaStreamSynchronize(kits[w]->s);
     }
-    for (eda_handle h : handles)
-        if (h) eda_destroy(h);
-    for (int w = 0; w < W; ++w) {
-        if (done[w]) cudaEventDestroy(done[w]);
-        if (streams[w]) cudaStreamDestroy(streams[w]);
-    }
-    cudaEventDestroy(start);
+    for (int w = 0; w < W; ++w) host_kit_give(kits[w]);
     for (int i = 0; i < nprob && rc == EDA_OK; ++i) {
         const int st = probs[order[i]].status;
         if (st != EDA_OK && st != EDA_ERR_NOT_CONVERGED) rc = st;

@@ -151,8 +151,7 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
 
     // kept columns of Z: all but the last column of each class in H_W and the last column of H_B
     std::vector<int32_t> offs(k + 1);
-    EDA_CUDA_TRY(cudaMemcpyAsync(offs.data(), h->offsets, (k + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(offs.data(), h->offsets, (k + 1) * sizeof(int32_t), s));
     std::vector<int> keep;
     keep.reserve(r);
     for (int j = 0; j < k; ++j)
@@ -204,9 +203,9 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
     EDA_TRY(symeig_work_carve(a, r, t, h->bar, &w.eig));
     if (!w.keep) return EDA_ERR_OOM;
 
-    cudaEvent_t ev0, ev1;
-    EDA_CUDA_TRY(cudaEventCreate(&ev0));
-    EDA_CUDA_TRY(cudaEventCreate(&ev1));
+    HostHold hold;
+    EDA_TRY(hold.open());
+    const cudaEvent_t ev0 = hold.kit->timer[0], ev1 = hold.kit->timer[1];
     int rc = EDA_OK;
     do {
         if (cudaEventRecord(ev0, s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
@@ -276,15 +275,12 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
             cudaEventElapsedTime(&ms, ev0, ev1) != cudaSuccess)
             rc = EDA_ERR_CUDA;
     }
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
     if (rc != EDA_OK) {
         cudaStreamSynchronize(s);
         return rc;
     }
     int st = 0;
-    EDA_CUDA_TRY(cudaMemcpyAsync(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(&st, h->status, sizeof(int), s));
     if (st & ST_TIMEOUT) return EDA_ERR_TIMEOUT;
     if (st & ST_NONFINITE) return EDA_ERR_NONFINITE;
     if (st & ST_RANKLOSS) return EDA_ERR_BREAKDOWN;   // dependent samples: Z' is rank deficient

@@ -28,16 +28,27 @@ void note_cuda_error(cudaError_t e, const char* file, int line) {
 int ensure_workspace(eda_ctx* h, size_t bytes) {
     if (h->ws_bytes >= bytes) return EDA_OK;
     if (h->ws) {
-        EDA_CUDA_TRY(cudaFree(h->ws));
+        void* old = h->ws;
         h->ws = nullptr;
         h->ws_bytes = 0;
+        EDA_TRY(dev_free_idle(old));   // calls on other streams may still use it
     }
     void* p = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&p, bytes));
+    EDA_TRY(dev_alloc(&p, bytes));
     h->ws = p;
     h->ws_bytes = bytes;
     return EDA_OK;
 }
+
+void destroy_handle(eda_ctx* h, bool idle) {
+    for (void* p : {h->ws, h->kblock, h->xblock, h->ozblock, h->ozsmall, h->nblock, h->block32, h->fblock, h->block}) {
+        if (!p) continue;
+        if (idle) dev_free(p);
+        else cudaFree(p);
+    }
+    delete h;
+}
+
 std::atomic<uint64_t>& launch_counter() { return g_launches; }
 
 // Solve-side entry points implemented in lanczos.cu.
@@ -68,7 +79,7 @@ int ensure_cross_gram(eda_ctx* h, double* part, size_t pcap, cudaStream_t s) {
     const int n = (int)h->n, k = h->k;
     const size_t xb = ((size_t)n * k * 8 + 255) & ~size_t(255);
     void* xp = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&xp, 2 * xb));
+    EDA_TRY(dev_alloc(&xp, 2 * xb));
     h->xblock = xp;
     h->GWB = static_cast<double*>(xp);
     h->GBW = reinterpret_cast<double*>(static_cast<char*>(xp) + xb);
@@ -93,9 +104,7 @@ int tc_operands(eda_ctx* h, cudaStream_t s);
 int tc_grams(eda_ctx* h, cudaStream_t s);
 
 int read_status(eda_ctx* h, cudaStream_t s, int* out) {
-    EDA_CUDA_TRY(cudaMemcpyAsync(out, h->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
-    return EDA_OK;
+    return read_back(out, h->status, sizeof(int), s);
 }
 
 int status_to_code(int st) {
@@ -106,7 +115,7 @@ int status_to_code(int st) {
 }
 
 // Allocate the handle's device block: factors, Grams, eigenpairs, operators, status, barrier.
-int alloc_handle(eda_ctx* h, bool with_labels) {
+int alloc_handle(eda_ctx* h, bool with_labels, cudaStream_t s) {
     const size_t d = h->d, n = h->n, k = h->k;
     const size_t N = std::max(n, k);
     size_t bytes = 0;
@@ -149,7 +158,7 @@ int alloc_handle(eda_ctx* h, bool with_labels) {
     add(4096);
     h->block_bytes = bytes + 4096;
     void* p = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&p, h->block_bytes));
+    EDA_TRY(dev_alloc(&p, h->block_bytes));
     h->block = p;
     Arena a{static_cast<char*>(p), h->block_bytes, 0};
     h->HW = a.take<double>(d * (n + k));
@@ -174,8 +183,9 @@ int alloc_handle(eda_ctx* h, bool with_labels) {
     h->bar = GridBarrier{bar, bar + 32, h->cfg.wait_limit > 0 ? (long long)h->cfg.wait_limit : kGridSpinDefault};
     h->build_arena_off = a.used;
     if (!h->KB || !bar) return EDA_ERR_OOM;
-    EDA_CUDA_TRY(cudaMemset(h->status, 0, 256));
-    EDA_CUDA_TRY(cudaMemset(bar, 0, 256));
+    // on the caller's stream: the block may hold an earlier handle's words
+    EDA_CUDA_TRY(cudaMemsetAsync(h->status, 0, 256, s));
+    EDA_CUDA_TRY(cudaMemsetAsync(bar, 0, 256, s));
     return EDA_OK;
 }
 
@@ -213,8 +223,7 @@ int gram_eigen(eda_ctx* h, int m, double* G, double* evals, double* evecs, Arena
     EDA_TRY(symeig_work_carve(scratch, m, m, h->bar, &ws));
     EDA_TRY(symeig_values(m, G, m, 0, m - 1, evals, &ws, h->status, s));
     std::vector<double> w(m);
-    EDA_CUDA_TRY(cudaMemcpyAsync(w.data(), evals, m * sizeof(double), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(w.data(), evals, m * sizeof(double), s));
     int st = 0;
     EDA_TRY(read_status(h, s, &st));
     if (int c = status_to_code(st)) return c;
@@ -225,6 +234,32 @@ int gram_eigen(eda_ctx* h, int m, double* G, double* evals, double* evecs, Arena
     h->nsig_first = first;   // only meaningful for the last call; the callers store their own copy
     return EDA_OK;
 }
+
+// A second stream for the independent halves of the build (the two Grams), joined back into the
+// caller's stream when it goes out of scope.
+struct AuxStream {
+    cudaStream_t main = nullptr, aux = nullptr;
+    HostHold hold;
+    int open(cudaStream_t s) {
+        EDA_TRY(hold.open());
+        main = s;
+        aux = hold.kit->s;
+        return EDA_OK;
+    }
+    int fork() {
+        EDA_CUDA_TRY(cudaEventRecord(hold.kit->order[0], main));
+        EDA_CUDA_TRY(cudaStreamWaitEvent(aux, hold.kit->order[0], 0));
+        return EDA_OK;
+    }
+    int join() {
+        EDA_CUDA_TRY(cudaEventRecord(hold.kit->order[1], aux));
+        EDA_CUDA_TRY(cudaStreamWaitEvent(main, hold.kit->order[1], 0));
+        return EDA_OK;
+    }
+    ~AuxStream() {
+        if (aux && join() != EDA_OK) cudaStreamSynchronize(aux);
+    }
+};
 
 // Both Gram eigensolves side by side on two streams (each runs in one thread-block cluster, so
 // together they still leave most SMs idle): eigenvalues of G_W on s and of G_B on a second stream,
@@ -241,18 +276,13 @@ int gram_eigen_pair(eda_ctx* h, Arena& scratch, double* partW, size_t pcapW, int
     double* tmpW = scratch.take<double>(3 * (size_t)n * n + 64);
     double* tmpB = scratch.take<double>(3 * (size_t)k * k + 64);
     if (!partB || !tmpW || !tmpB) return EDA_ERR_OOM;
-    cudaStream_t s2 = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    AuxStream pair;   // joins s when it goes out of scope
+    EDA_TRY(pair.open(s));
+    EDA_TRY(pair.fork());
+    const cudaStream_t s2 = pair.aux;
     int rc = EDA_OK;
     std::vector<double> ww(n), wb(k);
     do {
-        if (cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&join, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventRecord(fork, s) != cudaSuccess || cudaStreamWaitEvent(s2, fork, 0) != cudaSuccess) {
-            rc = EDA_ERR_CUDA;
-            break;
-        }
         // two reductions in flight at once: both on the cluster path (a cooperative grid needs every SM it
         // spans, and the two would share the handle's grid-barrier words)
         const bool prev_shared = symeig_set_shared_gpu(true);
@@ -260,12 +290,8 @@ int gram_eigen_pair(eda_ctx* h, Arena& scratch, double* partW, size_t pcapW, int
         if (rc == EDA_OK) rc = symeig_values(k, h->GB, k, 0, k - 1, h->evals_b, &wsB, h->status, s2);
         symeig_set_shared_gpu(prev_shared);
         if (rc != EDA_OK) break;
-        if (cudaMemcpyAsync(ww.data(), h->evals_w, n * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(wb.data(), h->evals_b, k * sizeof(double), cudaMemcpyDeviceToHost, s2) != cudaSuccess ||
-            cudaStreamSynchronize(s2) != cudaSuccess) {
-            rc = EDA_ERR_CUDA;
-            break;
-        }
+        if ((rc = read_back(wb.data(), h->evals_b, k * sizeof(double), s2)) != EDA_OK) break;
+        if ((rc = read_back(ww.data(), h->evals_w, n * sizeof(double), s)) != EDA_OK) break;
         int st = 0;
         if ((rc = read_status(h, s, &st)) != EDA_OK) break;
         if ((rc = status_to_code(st)) != EDA_OK) break;
@@ -276,51 +302,9 @@ int gram_eigen_pair(eda_ctx* h, Arena& scratch, double* partW, size_t pcapW, int
                                     first_b, s2)) != EDA_OK)
             break;
     } while (false);
-    if (s2) {
-        if (join && cudaEventRecord(join, s2) == cudaSuccess) cudaStreamWaitEvent(s, join, 0);
-        else cudaStreamSynchronize(s2);
-        cudaStreamDestroy(s2);   // released once its queued work has finished
-    }
-    if (fork) cudaEventDestroy(fork);
-    if (join) cudaEventDestroy(join);
     return rc;
 }
 
-
-// A second stream for the independent halves of the build (the two Grams), joined back into the
-// caller's stream when it goes out of scope.
-struct AuxStream {
-    cudaStream_t main = nullptr, aux = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    int open(cudaStream_t s) {
-        main = s;
-        if (cudaStreamCreateWithFlags(&aux, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming) != cudaSuccess)
-            return EDA_ERR_CUDA;
-        return EDA_OK;
-    }
-    int fork() {
-        EDA_CUDA_TRY(cudaEventRecord(ev_fork, main));
-        EDA_CUDA_TRY(cudaStreamWaitEvent(aux, ev_fork, 0));
-        return EDA_OK;
-    }
-    int join() {
-        EDA_CUDA_TRY(cudaEventRecord(ev_join, aux));
-        EDA_CUDA_TRY(cudaStreamWaitEvent(main, ev_join, 0));
-        return EDA_OK;
-    }
-    ~AuxStream() {
-        if (aux) {
-            if (!ev_join || cudaEventRecord(ev_join, aux) != cudaSuccess ||
-                cudaStreamWaitEvent(main, ev_join, 0) != cudaSuccess)
-                cudaStreamSynchronize(aux);
-            cudaStreamDestroy(aux);   // released once its queued work has finished
-        }
-        if (ev_fork) cudaEventDestroy(ev_fork);
-        if (ev_join) cudaEventDestroy(ev_join);
-    }
-};
 
 // lambda_max of a Gram from its Lanczos run (theta_1, theta_2, |z_m|, beta_m), or -1 when theta_1 is not
 // accepted. The residual r = beta_m |z_m| of the top Ritz pair bounds the distance from theta_1 to an
@@ -349,8 +333,7 @@ int gram_lmax_one(eda_ctx* h, int m, const double* G, double* w, Arena& scratch,
     if (!out) return EDA_ERR_OOM;
     EDA_TRY(lanczos_top(m, G, m, std::min(m, kLanczosStepsLarge), h->cfg.seed, &ws, out, s));
     double o[4];
-    EDA_CUDA_TRY(cudaMemcpyAsync(o, out, sizeof(o), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(o, out, sizeof(o), s));
     double l = lmax_accepted(o);
     const double r = o[2] * o[3];
     if (l < 0.0 && std::isfinite(o[0]) && std::isfinite(r) && o[0] + r < below) {
@@ -361,8 +344,7 @@ int gram_lmax_one(eda_ctx* h, int m, const double* G, double* w, Arena& scratch,
     if (l < 0.0) {
         EDA_TRY(symeig_values(m, G, m, m - 1, m - 1, w, &ws, h->status, s));
         double top = 0.0;
-        EDA_CUDA_TRY(cudaMemcpyAsync(&top, w, sizeof(double), cudaMemcpyDeviceToHost, s));
-        EDA_CUDA_TRY(cudaStreamSynchronize(s));
+        EDA_TRY(read_back(&top, w, sizeof(double), s));
         int st = 0;
         EDA_TRY(read_status(h, s, &st));
         if (int c = status_to_code(st)) return c;
@@ -388,8 +370,7 @@ int gram_lmax_pair(eda_ctx* h, Arena& scratch, AuxStream& aux, cudaStream_t s) {
     EDA_TRY(lanczos_top(k, h->GB, k, std::min(k, kLanczosSteps), h->cfg.seed, &wsB, out + 4, aux.aux));
     EDA_TRY(aux.join());
     double o[8];
-    EDA_CUDA_TRY(cudaMemcpyAsync(o, out, sizeof(o), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(o, out, sizeof(o), s));
     double lw = lmax_accepted(o), lb = lmax_accepted(o + 4);
     for (int g = 0; g < 2; ++g) {
         double& l = g == 0 ? lw : lb;
@@ -398,8 +379,7 @@ int gram_lmax_pair(eda_ctx* h, Arena& scratch, AuxStream& aux, cudaStream_t s) {
         double* w = g == 0 ? h->evals_w : h->evals_b;
         EDA_TRY(symeig_values(m, g == 0 ? h->GW : h->GB, m, m - 1, m - 1, w, g == 0 ? &wsW : &wsB, h->status, s));
         double top = 0.0;
-        EDA_CUDA_TRY(cudaMemcpyAsync(&top, w, sizeof(double), cudaMemcpyDeviceToHost, s));
-        EDA_CUDA_TRY(cudaStreamSynchronize(s));
+        EDA_TRY(read_back(&top, w, sizeof(double), s));
         int st = 0;
         EDA_TRY(read_status(h, s, &st));
         if (int c = status_to_code(st)) return c;
@@ -442,7 +422,7 @@ int finish_build(eda_ctx* h, cudaStream_t s) {
     if (h->cfg.prec == EDA_F32) {
         const size_t bw = align256((size_t)d * n * sizeof(float)), bb = align256((size_t)d * k * sizeof(float));
         void* p = nullptr;
-        EDA_CUDA_TRY(cudaMalloc(&p, bw + bb));
+        EDA_TRY(dev_alloc(&p, bw + bb));
         h->block32 = p;
         h->HW32 = static_cast<float*>(p);
         h->HB32 = reinterpret_cast<float*>(static_cast<char*>(p) + bw);
@@ -474,7 +454,7 @@ int finish_build(eda_ctx* h, cudaStream_t s) {
         // four n x n split operands: the squaring's two factors, then K_W and G_W for the solves
         const size_t b1 = align256(oz_operand_bytes(n, n));
         void* p = nullptr;
-        EDA_CUDA_TRY(cudaMalloc(&p, 4 * b1));
+        EDA_TRY(dev_alloc(&p, 4 * b1));
         h->ozsmall = p;
     }
     if (tc) {
@@ -595,7 +575,7 @@ int finish_build(eda_ctx* h, cudaStream_t s) {
         size_t tot = 0;
         for (size_t v : sz) tot += v;
         void* p = nullptr;
-        EDA_CUDA_TRY(cudaMalloc(&p, tot));
+        EDA_TRY(dev_alloc(&p, tot));
         h->block32 = p;
         EDA_CUDA_TRY(cudaMemsetAsync(p, 0, tot, s));
         char* c = static_cast<char*>(p);
@@ -618,7 +598,7 @@ int finish_build(eda_ctx* h, cudaStream_t s) {
             const size_t fz[4] = {align256((size_t)tc_fused_elems(d, n) * 2), align256((size_t)tc_fused_elems(d, k) * 2),
                                   align256(tc_fused_partial_floats(d, std::max(n, k)) * 4), 256};
             void* fp = nullptr;
-            EDA_CUDA_TRY(cudaMalloc(&fp, fz[0] + fz[1] + fz[2] + fz[3]));
+            EDA_TRY(dev_alloc(&fp, fz[0] + fz[1] + fz[2] + fz[3]));
             h->fblock = fp;
             char* fc = static_cast<char*>(fp);
             EDA_CUDA_TRY(cudaMemsetAsync(fc + fz[0] + fz[1] + fz[2], 0, fz[3], s));   // grid-barrier words
@@ -644,7 +624,7 @@ int tc_operands(eda_ctx* h, cudaStream_t s) {
     const size_t bT = align256(oz_operand_bytes(nk, d)), bN = align256(oz_operand_bytes(d, nk));
     const size_t bS = align256(oz_narrow_bytes(std::max<int64_t>(d, nk), sm_count(), nk));
     void* p = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&p, bT + bN + bS));
+    EDA_TRY(dev_alloc(&p, bT + bN + bS));
     h->ozblock = p;
     char* c = static_cast<char*>(p);
     EDA_TRY(oz_operand_make(h->HW, d, nk, d, true, c, &h->ozT, h->status, s));
@@ -661,16 +641,14 @@ int tc_grams(eda_ctx* h, cudaStream_t s) {
     const int64_t d = h->d;
     const int n = (int)h->n, k = h->k, nk = n + k;
     ProfScope prof("gram", s, (double)d * nk * (nk + 1.0), 8.0 * (double)d * nk);
-    double* GZ = nullptr;
-    EDA_CUDA_TRY(cudaMalloc(&GZ, (size_t)nk * nk * 8));
+    void* gz = nullptr;
+    EDA_TRY(dev_alloc(&gz, (size_t)nk * nk * 8));
+    double* GZ = static_cast<double*>(gz);
     int rc = oz_gemm_tiled(h->ozT, h->ozT, 1.0, 0.0, nullptr, 0, GZ, nk, true, h->status, s);
     if (rc == EDA_OK && !h->GWB) {
         const size_t xb = ((size_t)n * k * 8 + 255) & ~size_t(255);
         void* xp = nullptr;
-        if (cudaMalloc(&xp, 2 * xb) != cudaSuccess) {
-            cudaGetLastError();
-            rc = EDA_ERR_OOM;
-        } else {
+        if ((rc = dev_alloc(&xp, 2 * xb)) == EDA_OK) {
             h->xblock = xp;
             h->GWB = static_cast<double*>(xp);
             h->GBW = reinterpret_cast<double*>(static_cast<char*>(xp) + xb);
@@ -681,7 +659,7 @@ int tc_grams(eda_ctx* h, cudaStream_t s) {
     if (rc == EDA_OK) rc = copy_mat_f64(n, k, GZ + (size_t)n * nk, nk, h->GWB, n, s);
     if (rc == EDA_OK) rc = copy_mat_f64(k, n, GZ + n, nk, h->GBW, k, s);
     cudaStreamSynchronize(s);   // GZ is released below
-    cudaFree(GZ);
+    dev_free(GZ);
     return rc;
 }
 
@@ -728,7 +706,7 @@ int eda_build(const void* X, int32_t x_dtype, int64_t d, int64_t n, int64_t ldx,
     h->n = n;
     h->k = k;
     h->cfg = c;
-    int rc = alloc_handle(h, true);
+    int rc = alloc_handle(h, true, s);
     if (rc == EDA_OK) rc = segment_labels(labels, (int)n, k, h->counts, h->offsets, h->perm, h->status, s);
     if (rc == EDA_OK) {
         int st = 0;
@@ -766,7 +744,7 @@ int eda_build_from_factors(const double* HW, int64_t n, const double* HB, int64_
     h->n = n;
     h->k = (int32_t)kb;
     h->cfg = c;
-    int rc = alloc_handle(h, false);
+    int rc = alloc_handle(h, false, s);
     if (rc == EDA_OK) rc = copy_mat_f64(d, (int)n, HW, d, h->HW, d, s);
     if (rc == EDA_OK) rc = copy_mat_f64(d, (int)kb, HB, d, h->HB, d, s);
     if (rc == EDA_OK) rc = check_finite_f64(d, (int)n, h->HW, d, h->status, s);
@@ -841,7 +819,7 @@ int eda_apply_exp(eda_handle h, int32_t op, double alpha, const void* X, void* Y
         EDA_TRY(ensure_eigen(h, s));
         if (!h->kblock) {
             void* kb = nullptr;
-            EDA_CUDA_TRY(cudaMalloc(&kb, 2 * align256((size_t)N * N * 8)));
+            EDA_TRY(dev_alloc(&kb, 2 * align256((size_t)N * N * 8)));
             h->kblock = kb;
             h->Kalpha = static_cast<double*>(kb);
             h->Kalpha_tmp = reinterpret_cast<double*>(static_cast<char*>(kb) + align256((size_t)N * N * 8));
@@ -937,17 +915,8 @@ int eda_get_dims(eda_handle h, int64_t* d, int64_t* n, int32_t* k, double* c2, d
 }
 
 void eda_destroy(eda_handle h) {
-    if (!h) return;
-    if (h->ws) cudaFree(h->ws);
-    if (h->kblock) cudaFree(h->kblock);
-    if (h->xblock) cudaFree(h->xblock);
-    if (h->ozblock) cudaFree(h->ozblock);
-    if (h->ozsmall) cudaFree(h->ozsmall);
-    if (h->nblock) cudaFree(h->nblock);
-    if (h->block32) cudaFree(h->block32);
-    if (h->fblock) cudaFree(h->fblock);
-    if (h->block) cudaFree(h->block);
-    delete h;
+    // as cudaFree would: calls on any stream may still use the blocks (after a failed device nothing is kept)
+    if (h) eda::destroy_handle(h, cudaDeviceSynchronize() == cudaSuccess);
 }
 
 const char* eda_strerror(int status) {

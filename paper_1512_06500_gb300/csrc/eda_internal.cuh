@@ -82,6 +82,38 @@ struct Arena {
     void reset() { used = 0; }
 };
 
+// ---------------------------------------------------------------- memory, streams and events kept between handles
+// Device memory from the process's cache or cudaMalloc. EDA_ERR_OOM / EDA_ERR_CUDA on failure.
+int dev_alloc(void** p, size_t bytes);
+// Give back a block of dev_alloc that the GPU has finished with (the caller has synchronised the stream or the device; any
+// stream may get it next). dev_free_idle waits for the device first, as cudaFree does.
+void dev_free(void* p);
+int dev_free_idle(void* p);
+// Identity of the current context (0: none, or not offered by the driver).
+unsigned long long current_ctx_id();
+// A non-blocking stream, two events for ordering, two for timing and a pinned page, kept between calls.
+constexpr size_t kHostPage = 64 * 1024;
+struct HostKit {
+    cudaStream_t s = nullptr;
+    cudaEvent_t order[2] = {nullptr, nullptr};
+    cudaEvent_t timer[2] = {nullptr, nullptr};
+    void* page = nullptr;
+    unsigned long long ctx = 0;
+};
+int host_kit_take(HostKit** k);
+void host_kit_give(HostKit* k);      // its stream's work is ordered before whatever uses it next
+void host_kit_destroy(HostKit* k);
+struct HostHold {
+    HostKit* kit = nullptr;
+    int open() { return host_kit_take(&kit); }
+    HostHold() = default;
+    HostHold(const HostHold&) = delete;
+    HostHold& operator=(const HostHold&) = delete;
+    ~HostHold() { host_kit_give(kit); }
+};
+// Copy `bytes` from the device once the work queued on s is done, and wait for it (through a pinned page when it fits).
+int read_back(void* host, const void* dev, size_t bytes, cudaStream_t s);
+
 // Grid barrier state in device memory (zeroed at allocation) and the number of polls a wait makes
 // before it gives up (ST_TIMEOUT).
 constexpr long long kGridSpinDefault = 20000000;   // about 1-2 s of polling
@@ -421,6 +453,8 @@ struct eda_ctx {
 };
 
 namespace eda {
+// Give back a handle's memory and the handle; idle: the GPU has finished with it.
+void destroy_handle(eda_ctx* h, bool idle);
 // Grow the handle's solve workspace to at least `bytes` (contents are not preserved).
 int ensure_workspace(eda_ctx* h, size_t bytes);
 // The two sweeps over Z = [H_W H_B] of a composed product (FP64, or the tensor-core FP64 products when the

@@ -1494,8 +1494,7 @@ int symeig_orth_clusters(int n, int nv, const double* w, double* Z, int ldz, Sym
     EDA_LAUNCHED();
     if (maxc == INT_MAX || nv < maxc) return EDA_OK;
     std::vector<double> wh(nv);
-    EDA_CUDA_TRY(cudaMemcpyAsync(wh.data(), w, nv * sizeof(double), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(wh.data(), w, nv * sizeof(double), s));
     double mx = 0.0;
     for (int i = 0; i < nv; ++i) mx = std::fmax(mx, std::fabs(wh[i]));
     const double tol = cluster_rel * mx;

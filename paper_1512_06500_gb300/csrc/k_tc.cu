@@ -519,13 +519,11 @@ int tc_factor_make(const double* H, int64_t d, int m, const double* K, __nv_bflo
     // H K (tiled like the sweep-2 operand) as sweep-2 products: A = tiled bf16(H) by rows, B = 32-column
     // slices of K as bf16 pairs. Temporaries are freed before returning (the stream is synchronised).
     const int64_t tot2 = tc_tiles_sweep2(d, m);
-    __nv_bfloat16* Hr = nullptr;
     const size_t hbytes = ((size_t)tot2 * 2 + 255) / 256 * 256;
     const size_t kbytes = (size_t)ldm * 32 * 2;
-    if (cudaMalloc(&Hr, hbytes + 2 * kbytes) != cudaSuccess) {
-        cudaGetLastError();
-        return EDA_ERR_OOM;
-    }
+    void* tmp = nullptr;
+    EDA_TRY(dev_alloc(&tmp, hbytes + 2 * kbytes));
+    __nv_bfloat16* Hr = static_cast<__nv_bfloat16*>(tmp);
     __nv_bfloat16* Khi = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(Hr) + hbytes);
     __nv_bfloat16* Klo = Khi + (size_t)ldm * 32;
     int rc = EDA_OK;
@@ -547,7 +545,7 @@ int tc_factor_make(const double* H, int64_t d, int m, const double* K, __nv_bflo
         if (rc == EDA_OK && cudaStreamSynchronize(s) != cudaSuccess) rc = EDA_ERR_CUDA;
     } while (false);
     if (rc != EDA_OK) cudaStreamSynchronize(s);
-    cudaFree(Hr);
+    dev_free(tmp);
     return rc;
 }
 

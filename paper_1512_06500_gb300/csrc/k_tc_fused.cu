@@ -481,13 +481,10 @@ int tc_fused_make(const double* H, int64_t d, int m, const double* K, double alp
     // sigma K = R^T R, B = H R^T (FP64), then the bf16 tiled image; temporaries freed before returning
     const size_t mm = (size_t)m * m;
     const size_t pcap = std::max<size_t>(mm, 1u << 16);
-    double* tmp = nullptr;
     const size_t bytes = (3 * mm + (size_t)d * m + chol_inv_blocked_doubles(m) + pcap) * 8 + 1024;
-    if (cudaMalloc(&tmp, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return EDA_ERR_OOM;
-    }
-    double* R = tmp;
+    void* tmp = nullptr;
+    EDA_TRY(dev_alloc(&tmp, bytes));
+    double* R = static_cast<double*>(tmp);
     double* Ri = R + mm;
     double* RT = Ri + mm;
     double* Bf = RT + mm;
@@ -509,7 +506,7 @@ int tc_fused_make(const double* H, int64_t d, int m, const double* K, double alp
         if (cudaStreamSynchronize(s) != cudaSuccess) rc = EDA_ERR_CUDA;
     } while (false);
     if (rc != EDA_OK) cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    dev_free(tmp);
     if (rc != EDA_OK) return rc;
     f->F = img;
     f->fsign = (float)sigma;

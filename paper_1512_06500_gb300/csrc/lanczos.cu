@@ -283,8 +283,7 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
     EDA_TRY(oz_basis_grow<T>(w, d, 0, b, h->status, s));
     {
         int lostc = 0;
-        EDA_CUDA_TRY(cudaMemcpyAsync(&lostc, w.lost + b, sizeof(int), cudaMemcpyDeviceToHost, s));
-        EDA_CUDA_TRY(cudaStreamSynchronize(s));
+        EDA_TRY(read_back(&lostc, w.lost + b, sizeof(int), s));
         if (lostc) return EDA_ERR_BREAKDOWN;   // the start block itself is rank deficient
     }
 
@@ -314,16 +313,14 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
         EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 1) * sizeof(int), s));
         EDA_TRY(cholqr_pass<T>(d, b, w.W, d, w.R1, w.R1i, w.W1, piv_min2, h->status, w.lost, w, s));
         int lostc = 0;
-        EDA_CUDA_TRY(cudaMemcpyAsync(&lostc, w.lost + b, sizeof(int), cudaMemcpyDeviceToHost, s));
-        EDA_CUDA_TRY(cudaStreamSynchronize(s));
+        EDA_TRY(read_back(&lostc, w.lost + b, sizeof(int), s));
         const bool room = cols + b <= m_max;
         if (room) {
             if (lostc > 0) {
                 // replace the lost columns by fresh random directions orthogonal to the basis
                 st.refills += lostc;
                 std::vector<int> lost_h(b + 1);
-                EDA_CUDA_TRY(cudaMemcpyAsync(lost_h.data(), w.lost, (b + 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
-                EDA_CUDA_TRY(cudaStreamSynchronize(s));
+                EDA_TRY(read_back(lost_h.data(), w.lost, (b + 1) * sizeof(int), s));
                 for (int q = 0; q < lostc; ++q)
                     EDA_TRY(fill_gaussian<T>(d, 1, w.W1 + (size_t)lost_h[q] * d, d, h->cfg.seed,
                                              1000 + (uint64_t)st.iters * 64 + q, s));
@@ -362,9 +359,7 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
                                                                      w.relres);
                     EDA_LAUNCHED();
                 }
-                EDA_CUDA_TRY(
-                    cudaMemcpyAsync(st.relres.data(), w.relres, t * sizeof(double), cudaMemcpyDeviceToHost, s));
-                EDA_CUDA_TRY(cudaStreamSynchronize(s));
+                EDA_TRY(read_back(st.relres.data(), w.relres, t * sizeof(double), s));
                 st.max_rel = 0.0;
                 st.conv_count = 0;
                 for (int i = 0; i < t; ++i) {
@@ -566,8 +561,7 @@ int ritz_residuals(int64_t d, int t, SolveWs<T>& w, std::vector<double>& relres_
     EDA_TRY(col_norms_f64(d, t, w.R, d, w.relres, s));
     k_divide<<<ceil_div(t, 128), 128, 0, s>>>(t, w.relres, w.theta);
     EDA_LAUNCHED();
-    EDA_CUDA_TRY(cudaMemcpyAsync(relres_h.data(), w.relres, t * sizeof(double), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(relres_h.data(), w.relres, t * sizeof(double), s));
     *max_rel = 0.0;
     for (int i = 0; i < t; ++i) *max_rel = std::max(*max_rel, relres_h[i]);
     return EDA_OK;
@@ -655,9 +649,9 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
     const int N = std::max(n, k);
     const int tw = std::max(t, b);   // width of the final blocks
 
-    cudaEvent_t ev0, ev1;
-    EDA_CUDA_TRY(cudaEventCreate(&ev0));
-    EDA_CUDA_TRY(cudaEventCreate(&ev1));
+    HostHold hold;
+    EDA_TRY(hold.open());
+    const cudaEvent_t ev0 = hold.kit->timer[0], ev1 = hold.kit->timer[1];
     EDA_CUDA_TRY(cudaEventRecord(ev0, s));
 
     // ---- workspace ----
@@ -779,8 +773,7 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
         for (int i = 0; i < t; ++i) st.conv_count += relres_h[i] <= tol;
     }
     int stw = 0;
-    EDA_CUDA_TRY(cudaMemcpyAsync(&stw, h->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(&stw, h->status, sizeof(int), s));
     if (stw & ST_TIMEOUT) return EDA_ERR_TIMEOUT;
     if (stw & ST_NONFINITE) return EDA_ERR_NONFINITE;
 
@@ -839,9 +832,8 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
         EDA_LAUNCHED();
         EDA_TRY(col_norms_f64(d, t, MY, d, w.relres, s));
         std::vector<double> rn(t), lam_h(t);
-        EDA_CUDA_TRY(cudaMemcpyAsync(rn.data(), w.relres, t * 8, cudaMemcpyDeviceToHost, s));
-        EDA_CUDA_TRY(cudaMemcpyAsync(lam_h.data(), w.lamd, t * 8, cudaMemcpyDeviceToHost, s));
-        EDA_CUDA_TRY(cudaStreamSynchronize(s));
+        EDA_TRY(read_back(rn.data(), w.relres, t * 8, s));
+        EDA_TRY(read_back(lam_h.data(), w.lamd, t * 8, s));
         true_max = 0.0;
         for (int i = 0; i < t; ++i) true_max = std::max(true_max, rn[i] / std::fabs(lam_h[i]));
         // the estimates must not claim more than an independent FP64 evaluation confirms
@@ -851,10 +843,7 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
     EDA_CUDA_TRY(cudaEventSynchronize(ev1));
     float ms = 0.f;
     EDA_CUDA_TRY(cudaEventElapsedTime(&ms, ev0, ev1));
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
-    EDA_CUDA_TRY(cudaMemcpyAsync(&stw, h->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    EDA_CUDA_TRY(cudaStreamSynchronize(s));
+    EDA_TRY(read_back(&stw, h->status, sizeof(int), s));
     if (stw & ST_TIMEOUT) return EDA_ERR_TIMEOUT;
     if (stw & ST_NONFINITE) return EDA_ERR_NONFINITE;
     if (info) {

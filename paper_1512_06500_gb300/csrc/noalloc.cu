@@ -30,35 +30,6 @@ struct ScratchSlot {
 ScratchSlot g_scratch[kMaxDevices];
 std::mutex g_scratch_mu;
 
-using CtxGetCurrentFn = CUresult (*)(CUcontext*);
-using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
-
-// Identity of the calling thread's current context (0 when there is none or the driver does not
-// offer context identities, in which case nothing is cached and every call looks the address up).
-unsigned long long current_ctx_id() {
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<CtxGetCurrentFn>(p);
-        p = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<CtxGetIdFn>(p);
-        cudaGetLastError();
-    });
-    if (!get_current || !get_id) return 0;
-    CUcontext ctx = nullptr;
-    unsigned long long id = 0;
-    if (get_current(&ctx) != CUDA_SUCCESS || ctx == nullptr) return 0;
-    if (get_id(ctx, &id) != CUDA_SUCCESS) return 0;
-    return id;
-}
-
 int scratch_address(double** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -69,7 +40,7 @@ int scratch_address(double** out) {
     if (dev < 0 || dev >= kMaxDevices) return EDA_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(g_scratch_mu);
     ScratchSlot& slot = g_scratch[dev];
-    const unsigned long long id = current_ctx_id();
+    const unsigned long long id = eda::current_ctx_id();
     if (id != 0 && slot.ctx_id == id && slot.addr) {
         *out = slot.addr;
         return EDA_OK;
@@ -81,7 +52,7 @@ int scratch_address(double** out) {
         return EDA_ERR_CUDA;
     }
     slot.addr = static_cast<double*>(p);
-    slot.ctx_id = current_ctx_id();   // the lookup has made the device's primary context current
+    slot.ctx_id = eda::current_ctx_id();   // the lookup has made the device's primary context current
     *out = slot.addr;
     return EDA_OK;
 }

@@ -35,6 +35,7 @@ EXPORTS = [
     "eda_last_cuda_error", "eda_last_cuda_error_string", "eda_kernel_launches",
     "eda_profile_enable", "eda_profile_reset", "eda_profile_read", "eda_profile_work",
     "eda_lowrank_exp_apply_noalloc", "eda_solve_batched", "eda_solve_arnoldi", "eda_solve_direct",
+    "eda_release_cached",
 ]
 
 
@@ -104,6 +105,7 @@ def load(path: str | None = None):
         "eda_get_factors": ([vp] + [vp] * 10 + [vp], ctypes.c_int),
         "eda_get_dims": ([vp, P(i64), P(i64), P(i32), P(f64), P(f64), P(f64)], ctypes.c_int),
         "eda_destroy": ([vp], None),
+        "eda_release_cached": ([], ctypes.c_int),
         "eda_strerror": ([ctypes.c_int], ctypes.c_char_p),
         "eda_last_cuda_error": ([], ctypes.c_int),
         "eda_last_cuda_error_string": ([], ctypes.c_char_p),
@@ -167,6 +169,11 @@ def config(**kw) -> Config:
 
 def kernel_launches() -> int:
     return int(load().eda_kernel_launches())
+
+
+def release_cached():
+    """Give the device memory kept for later handles back to the driver."""
+    _check(load().eda_release_cached(), "eda_release_cached")
 
 
 def profile_enable(on=True):

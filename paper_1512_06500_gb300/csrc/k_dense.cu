@@ -18,7 +18,8 @@ constexpr int TN_THREADS = 256;
 // Tile (bx, by) with bx >= by of the lower triangle of a T x T tile grid from its index
 // q = bx (bx + 1) / 2 + by (row by row).
 __device__ __forceinline__ void tri_tile(int q, int& bx, int& by) {
-    int x = (int)((sqrt(8.0 * q + 1.0) - 1.0) * 0.5);
+    // single precision, corrected below: an FP64 square root takes the FP64 pipe for longer than some callers' products
+    int x = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
     while ((x + 1) * (x + 2) / 2 <= q) ++x;
     while (x * (x + 1) / 2 > q) --x;
     bx = x;
@@ -115,6 +116,96 @@ __global__ void __launch_bounds__(TN_THREADS) k_gemm_tn_partial(int64_t d, int m
             const int j = j0 + ty + b * (TP / TPT);
             if (i < m && j < p) out[(int64_t)j * m + i] = acc[a][b];
         }
+}
+
+// The symmetric product A^T A of a narrow block (m <= 32 columns: the CholQR Grams), partial sums by CTA in the layout of
+// k_gemm_tn_partial. The FP64 pipe bounds it, so only the m (m + 1) / 2 entries of the lower triangle are computed: the
+// items (row phase r < R, entry e of the triangle) are dealt to the lanes of each warp, ACC or fewer accumulators a lane, and
+// a step of a warp takes R rows of the block, so that almost every lane of every FP64 instruction works (m = 8: 9 instructions
+// for 8 rows; the 32 x 32 tiles of the general kernel take 32 a row). Rows come through shared memory, the next chunk
+// read into registers meanwhile; the warps' sums are added in order at the end.
+// GB300: d = 16384, m = 16 59 -> 17.8 us; d = 65536, m = 32 111 -> 90 us (69 us at the FP64 rate); d = 256, m = 1 .. 7
+// 19 -> 8 us. Two CTAs per SM (a few accumulators spill at m > 16: 104 us with one).
+constexpr int SN_THREADS = 256;
+constexpr int SN_MAXM = 32;
+template <int ACC, int CH, int MC, class T>
+__global__ void __launch_bounds__(SN_THREADS, 2) k_syrk_narrow(int64_t d, int m, const T* __restrict__ A, int64_t lda,
+                                                            int64_t rows_per_split, int R, T* __restrict__ partial) {
+    constexpr int LD = MC | 1;   // odd: the columns of a row and the rows of a column fall into different banks
+    __shared__ T As[CH][LD];
+    __shared__ T tot[32 * ACC];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int tri = m * (m + 1) / 2, items = R * tri;
+    const int64_t r_begin = (int64_t)blockIdx.x * rows_per_split, r_end = min(d, r_begin + rows_per_split);
+    // this lane's items: offsets of the two factors within a step's rows
+    int off[ACC];
+    T acc[ACC];
+#pragma unroll
+    for (int k = 0; k < ACC; ++k) {
+        const int it = lane + 32 * k;
+        const int r = it < items ? it / tri : 0, e = it < items ? it % tri : 0;
+        int i, j;
+        tri_tile(e, i, j);
+        off[k] = (r * LD + i) << 16 | (r * LD + j);
+        acc[k] = T(0);
+    }
+    constexpr int PA = CH * MC / SN_THREADS;
+    T ra[PA];
+    auto fetch = [&](int64_t r0) {
+#pragma unroll
+        for (int q = 0; q < PA; ++q) {
+            const int e = tid + q * SN_THREADS;
+            const int64_t r = r0 + e % CH;
+            const int c = e / CH;
+            ra[q] = (r < r_end && c < m) ? A[(int64_t)c * lda + r] : T(0);
+        }
+    };
+    if (r_begin < r_end) fetch(r_begin);
+    for (int64_t r0 = r_begin; r0 < r_end; r0 += CH) {
+#pragma unroll
+        for (int q = 0; q < PA; ++q) {
+            const int e = tid + q * SN_THREADS;
+            As[e % CH][e / CH] = ra[q];
+        }
+        __syncthreads();
+        if (r0 + CH < r_end) fetch(r0 + CH);
+        // the warp's steps of R rows (rows at or beyond r_end are zero; R divides CH)
+        const int live = (int)min((int64_t)CH, r_end - r0);
+        for (int rr = w * R; rr < live; rr += (SN_THREADS / 32) * R) {
+            const T* base = &As[rr][0];
+            // groups of four: their eight loads are in flight together (lanes beyond the items repeat item 0)
+#pragma unroll
+            for (int k0 = 0; k0 < ACC; k0 += 4) {
+                if (32 * k0 >= items) break;
+                T x[4], y[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k0 + u < ACC) {
+                        x[u] = base[off[k0 + u] >> 16];
+                        y[u] = base[off[k0 + u] & 0xffff];
+                    }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k0 + u < ACC) acc[k0 + u] = fma(x[u], y[u], acc[k0 + u]);
+            }
+        }
+        __syncthreads();
+    }
+    for (int v = 0; v < SN_THREADS / 32; ++v) {
+        if (w == v) {
+#pragma unroll
+            for (int k = 0; k < ACC; ++k) tot[lane + 32 * k] = v == 0 ? acc[k] : tot[lane + 32 * k] + acc[k];
+        }
+        __syncthreads();
+    }
+    T* out = partial + (int64_t)blockIdx.x * m * m;
+    for (int e = tid; e < tri; e += SN_THREADS) {
+        int i, j;
+        tri_tile(e, i, j);
+        T v = tot[e];
+        for (int r = 1; r < R; ++r) v += tot[r * tri + e];
+        out[(int64_t)j * m + i] = v;
+    }
 }
 
 // C[i, j] = alpha * sum_s partial[s][j][i] + beta * C[i, j]. Small split counts: one thread per
@@ -622,6 +713,31 @@ int gemm_tn_impl(int64_t d, int m, int p, double alpha, const T* A, int64_t lda,
     const double flops = sym ? (double)d * m * (m + 1.0) : 2.0 * (double)d * m * p;
     const double bytes = (double)sizeof(T) * (double)d * (sym ? m : (double)m + p) + 8.0 * m * p;
     ProfScope prof(std::is_same<T, double>::value ? "tn_f64" : "tn_f32", s, flops, bytes);
+    if (sym && m <= SN_MAXM && d > 0) {
+        // narrow blocks: one triangle of entries dealt to the lanes. Rows evenly over up to two CTAs per SM (a CTA with a
+        // chunk more than the others would set the time), at least 64 a CTA
+        int64_t G = std::max<int64_t>(1, std::min<int64_t>(2 * nsm, d / 64));
+        while (G > 1 && (size_t)G * m * m > partial_cap) --G;
+        if ((size_t)G * m * m > partial_cap) return EDA_ERR_INVALID_ARG;
+        const int64_t rw = (d + G - 1) / G;
+        G = (d + rw - 1) / rw;
+        const int tri = m * (m + 1) / 2;
+        const int cap = 32 * (m <= 8 ? 9 : (m <= 16 ? 17 : 33));
+        int R = 32;
+        while (R * tri > cap) R >>= 1;
+        if (m <= 8) k_syrk_narrow<9, 256, 8, T><<<(unsigned)G, SN_THREADS, 0, s>>>(d, m, A, lda, rw, R, partial);
+        else if (m <= 16) k_syrk_narrow<17, 128, 16, T><<<(unsigned)G, SN_THREADS, 0, s>>>(d, m, A, lda, rw, R, partial);
+        else k_syrk_narrow<33, 64, 32, T><<<(unsigned)G, SN_THREADS, 0, s>>>(d, m, A, lda, rw, R, partial);
+        EDA_LAUNCHED();
+        const int64_t out = (int64_t)m * m;
+        if (G >= 16)
+            k_gemm_tn_reduce_warp<T><<<ceil_div(out * 32, 256), 256, 0, s>>>(m, m, (int)G, partial, alpha, beta, C, ldc,
+                                                                            true);
+        else
+            k_gemm_tn_reduce<T><<<ceil_div(out, 256), 256, 0, s>>>(m, m, (int)G, partial, alpha, beta, C, ldc, true);
+        EDA_LAUNCHED();
+        return EDA_OK;
+    }
     // Split count: the kernel is FP64- or bandwidth-bound per SM, so an SM holding one CTA more than
     // the others sets the time. Among counts giving 1.8 to 4 CTAs per SM (after rounding the split
     // rows to TN_KB), take the one that fills the SMs most evenly, tiles * splits over

@@ -74,3 +74,30 @@ def test_batched_large_gram(eda):
         ref = O.eda(p.X, p.labels, p.k, p.k - 1, c2=r["info"]["c2"], tier="projected")
         assert np.max(np.abs(r["lam"].cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
         assert O.sin_angle(ref["V"], r["V"].cpu().numpy().T) <= 1e-8
+
+
+# narrow symmetric products: widths around the three instances (8, 16, 32 columns) and the powers of two of the row phases,
+# lengths around one CTA's rows and chunks, in FP64 (Grams) and single precision (the solver's block Grams)
+@pytest.mark.parametrize("d,k", [(5, 2), (63, 3), (64, 4), (65, 5), (129, 8), (255, 9), (256, 16), (257, 17), (1000, 23),
+                                 (4097, 31), (20011, 32), (20011, 33)])
+def test_narrow_gram(eda, d, k):
+    p = synth.gaussian_clusters(d=d, k=k, n_per_class=2, seed=d + k)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(tau=5.0)) as h:
+        f = h.factors()
+    for H, G in ((f["HB"], f["GB"]), (f["HW"], f["GW"])):
+        H = H.cpu().numpy()
+        G = G.cpu().numpy()
+        assert np.array_equal(G, G.T)
+        # a dot product of length d: |error| <= d eps sum |a||b|
+        assert np.all(np.abs(G - H @ H.T) <= d * np.finfo(float).eps * (np.abs(H) @ np.abs(H).T) + 1e-300)
+
+
+@pytest.mark.parametrize("b", [3, 8, 13, 16, 29, 32])
+def test_narrow_block_single_precision(eda, b):
+    p = synth.gaussian_clusters(d=1500, k=20, n_per_class=4, seed=b)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(prec=eda.EDA_F32, block_b=b, tau=6.0)) as h:
+        V, lam, _, info, code = h.solve(p.k - 1, 1e-9)
+        assert code == 0, info
+        ref = O.eda(p.X, p.labels, p.k, p.k - 1, c2=h.c2, tier="projected")
+    assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-9
+    assert O.sin_angle(ref["V"], V.cpu().numpy().T) <= 1e-6

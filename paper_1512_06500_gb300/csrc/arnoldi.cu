@@ -369,22 +369,18 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
             if ((rc = cgs2_f64(d, cols, b, w.V, w.W, C1, C2, w, s)) != EDA_OK) break;
             k_arn_set_hcol<<<ceil_div(cols * b, 256), 256, 0, s>>>(w.H, m_max, cols, j0, b, C1, C2);
             launch_counter()++;
-            if (cudaMemsetAsync(w.lost, 0, (b + 1) * sizeof(int), s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
+            if (cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
             // W1 = W R1^{-1} (the remainder W itself stays for the residuals)
             if ((rc = cholqr_once(d, b, w.W, w.W1, w.R1, w.R1i, piv_min2, h->status, w.lost, w, s)) != EDA_OK) break;
-            int lostc = 0;
-            if (cudaMemcpyAsync(&lostc, w.lost + b, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                cudaStreamSynchronize(s) != cudaSuccess) {
-                rc = EDA_ERR_CUDA;
-                break;
-            }
+            int lw[2] = {0, 0};   // lost and nearly lost columns
+            if ((rc = read_back(lw, w.lost + b, sizeof(lw), s)) != EDA_OK) break;
+            const int lostc = lw[0];
             const bool room = cols + b <= m_max;
             if (room) {
                 if (lostc > 0) {
                     refills += lostc;
                     std::vector<int> lost_h(b + 1);
-                    cudaMemcpyAsync(lost_h.data(), w.lost, (b + 1) * sizeof(int), cudaMemcpyDeviceToHost, s);
-                    cudaStreamSynchronize(s);
+                    if ((rc = read_back(lost_h.data(), w.lost, (b + 1) * sizeof(int), s)) != EDA_OK) break;
                     for (int q = 0; q < lostc && rc == EDA_OK; ++q)
                         rc = fill_gaussian_f64(d, 1, w.W1 + (size_t)lost_h[q] * d, d, h->cfg.seed,
                                                1000 + (uint64_t)iters * 64 + q, s);
@@ -394,7 +390,20 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
                     if (rc != EDA_OK) break;
                 }
                 double* Vn = w.V + (size_t)cols * d;
-                if (cudaMemsetAsync(w.lost, 0, (b + 1) * sizeof(int), s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
+                // columns whose pivot was nearly lost are rounding errors of W magnified up to 1e8 times, no longer
+                // orthogonal to the basis: twice W1 against the basis again, the first time normalised in between (its
+                // R folded into R1)
+                for (int round = 0; lw[1] > 0 && round < 2 && rc == EDA_OK; ++round) {
+                    double* C3 = w.C + 2 * (size_t)m_max * b;
+                    if ((rc = cgs2_f64(d, cols, b, w.V, w.W1, C3, C3 + (size_t)m_max * b, w, s)) != EDA_OK || round == 1)
+                        break;
+                    if ((rc = cholqr_once(d, b, w.W1, Vn, w.R2, w.R2i, 0.0, h->status, w.lost, w, s)) != EDA_OK) break;
+                    if ((rc = copy_mat_f64(d, b, Vn, d, w.W1, d, s)) != EDA_OK) break;
+                    if ((rc = gemm_small_f64(false, false, b, b, b, 1.0, w.R2, b, w.R1, b, 0.0, w.Bm, b, s)) != EDA_OK) break;
+                    rc = copy_mat_f64(b, b, w.Bm, b, w.R1, b, s);
+                }
+                if (rc != EDA_OK) break;
+                if (cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
                 if ((rc = cholqr_once(d, b, w.W1, Vn, w.R2, w.R2i, 0.0, h->status, w.lost, w, s)) != EDA_OK) break;
                 if ((rc = gemm_small_f64(false, false, b, b, b, 1.0, w.R2, b, w.R1, b, 0.0, w.Bm, b, s)) != EDA_OK)
                     break;

@@ -145,7 +145,8 @@ int gemm_small_f64(bool ta, bool tb, int m, int p, int kk, double alpha, const d
 // In-place upper Cholesky of a b x b SPD matrix G = R^T R (R stored in the upper triangle, the
 // strict lower triangle zeroed) and Rinv = R^{-1} (b x b, ld b). A pivot (squared) at or below
 // max(rank_tol * max diag, piv_min2) marks rank loss: that row of R and of Rinv is set to zero
-// and ST_RANKLOSS is or-ed into *status; lost pivots are listed in lost[0..], lost[b] = count.
+// and ST_RANKLOSS is or-ed into *status; lost pivots are listed in lost[0..], lost[b] = count, and
+// lost[b + 1] counts the kept pivots below 1e-10 of their column's squared norm.
 int chol_inv_small(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2,
                    int* status, int* lost, cudaStream_t s);
 // The same factorisation for any m, blocked: one-CTA factorisations of kCholBlock x kCholBlock diagonal

@@ -431,8 +431,11 @@ __device__ __forceinline__ double newton_rcp(double x) {
 //    the square roots and the scaling follow at the end, for all rows at once.
 //  - the owner of row j + 1 updates that row first, publishes it and its reciprocal, and updates its other rows
 //    while the other warps update theirs: one barrier per pivot, the pivot row double-buffered.
+// A kept pivot far below its column's own squared norm (kCholWeak) is counted in lost[b + 1]: that column of X = A R^{-1}
+// is A's rounding errors magnified, and no longer orthogonal to what A's columns were orthogonal to.
 // GB300, one launch: b = 16 12 us and b = 32 22 us (30 and 76 us by one warp with a back substitution), b = 64 88 us
 // (220 us with three barriers, a division and a square root per pivot).
+constexpr double kCholWeak = 1e-10;
 template <int NC>
 __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg, double* Rinv, double rank_tol,
                                                        double piv_min2, int* status, int* lost) {
@@ -441,8 +444,9 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
     __shared__ double ginv[2];               // 1 / pivot, 0 where the pivot is lost
     __shared__ double gpiv[32 * NC];         // pivots (0 where lost)
     __shared__ double rdiag[32 * NC];        // 1 / sqrt(pivot)
+    __shared__ double diag0[32 * NC];        // the squared column norms (G's diagonal)
     __shared__ double s_thr;
-    __shared__ int s_nlost;
+    __shared__ int s_nlost, s_nweak;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double a[NR][NC];
 #pragma unroll
@@ -461,6 +465,7 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
         for (int h = 0; h < NC; ++h) {
             const int c = lane + 32 * h;
             const double g = c < b ? G[(int64_t)c * ldg + c] : 0.0;
+            diag0[c] = g;
             bad |= !isfinite(g);
             mx = fmax(mx, fabs(g));
         }
@@ -470,6 +475,7 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
         if (lane == 0) {
             s_thr = mx == 0.0 ? INFINITY : fmax(rank_tol * mx, piv_min2);
             s_nlost = 0;
+            s_nweak = 0;
         }
     }
     __syncthreads();
@@ -541,6 +547,7 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
     for (int i = threadIdx.x; i < b; i += blockDim.x) {
         const double g = gpiv[i];
         rdiag[i] = g > 0.0 ? 1.0 / sqrt(g) : 0.0;
+        if (g > 0.0 && g < kCholWeak * diag0[i]) atomicAdd(&s_nweak, 1);
     }
     __syncthreads();
 #pragma unroll
@@ -557,7 +564,10 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
             Rinv[(int64_t)i * b + c] = c < i ? v : (c == i ? sc : 0.0);
         }
     }
-    if (threadIdx.x == 0 && lost) lost[b] = s_nlost;
+    if (threadIdx.x == 0 && lost) {
+        lost[b] = s_nlost;
+        lost[b + 1] = s_nweak;
+    }
 }
 
 // The same by one CTA in global memory, for any b: two divisions a column and a back substitution.
@@ -628,7 +638,19 @@ __global__ void k_chol_inv(int b, double* G, int ldg, double* Rinv, double rank_
             Rinv[(int64_t)c * b + i] = v;
         }
     }
-    if (threadIdx.x == 0 && lost) lost[b] = nlost;
+    if (!lost) return;
+    if (threadIdx.x == 0) lost[b] = nlost;
+    __shared__ int nweak;
+    if (threadIdx.x == 0) nweak = 0;
+    __syncthreads();
+    for (int c = threadIdx.x; c < b; c += blockDim.x) {
+        double sum = 0.0;   // the column's squared norm, from its column of R
+        for (int r = 0; r <= c; ++r) sum = fma(G[(int64_t)c * ldg + r], G[(int64_t)c * ldg + r], sum);
+        const double p = G[(int64_t)c * ldg + c];
+        if (p > 0.0 && p * p < kCholWeak * sum) atomicAdd(&nweak, 1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) lost[b + 1] = nweak;
 }
 
 // the register-resident factorisation up to this size (three 32-column slices a lane)

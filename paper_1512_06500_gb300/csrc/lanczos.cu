@@ -247,6 +247,22 @@ int m_apply_f32(eda_ctx* h, int b, const float* X, int64_t ldx, float* Y, int64_
 
 namespace {
 
+// W1 = W R1^{-1} has columns whose pivot was nearly lost (lost[b + 1] of chol_inv_small): rounding errors of W magnified
+// up to 1e8 times, no longer orthogonal to the basis. Twice: W1 against the basis again, then (the first time) normalised
+// by another CholQR pass, its R folded into R1. C: 2 cols x b; tmpX: d x b.
+template <class T>
+int strengthen(eda_ctx* h, int64_t d, int cols, int b, T* tmpX, double* C, SolveWs<T>& w, cudaStream_t s) {
+    for (int round = 0; round < 2; ++round) {
+        EDA_TRY(cgs2<T>(d, cols, b, w.V, w.W1, d, C, C + (size_t)cols * b, w, s, h));
+        if (round == 1) break;
+        EDA_TRY(cholqr_pass<T>(d, b, w.W1, d, w.R2, w.R2i, tmpX, 0.0, h->status, w.lost, w, s));
+        EDA_TRY((copy_mat<T, T>(d, b, tmpX, d, w.W1, d, s)));
+        EDA_TRY(gemm_small_f64(false, false, b, b, b, 1.0, w.R2, b, w.R1, b, 0.0, w.Bm, b, s));
+        EDA_TRY(copy_mat_f64(b, b, w.Bm, b, w.R1, b, s));
+    }
+    return EDA_OK;
+}
+
 struct LanczosStats {
     int iters = 0, mapplies = 0, checks = 0, refills = 0, rr_cols = 0, conv_count = 0;
     bool converged = false;
@@ -310,10 +326,11 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
         k_set_col_block<<<ceil_div(cols * b, 256), 256, 0, s>>>(w.Tm, m_max, cols, j0, b, C1, C2);
         EDA_LAUNCHED();
         // CholQR2 of W with rank detection: W = V_{j+1} B_{j+1}
-        EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 1) * sizeof(int), s));
+        EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s));
         EDA_TRY(cholqr_pass<T>(d, b, w.W, d, w.R1, w.R1i, w.W1, piv_min2, h->status, w.lost, w, s));
-        int lostc = 0;
-        EDA_TRY(read_back(&lostc, w.lost + b, sizeof(int), s));
+        int lw[2] = {0, 0};   // lost and nearly lost columns
+        EDA_TRY(read_back(lw, w.lost + b, sizeof(lw), s));
+        const int lostc = lw[0];
         const bool room = cols + b <= m_max;
         if (room) {
             if (lostc > 0) {
@@ -329,7 +346,9 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
                 EDA_TRY(cgs2<T>(d, cols, b, w.V, w.W1, d, C3, C3 + (size_t)m_max * b, w, s, h));
             }
             T* Vn = w.V + (size_t)cols * d;
-            EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 1) * sizeof(int), s));
+            if (lw[1] > 0 && std::is_same<T, double>::value)
+                EDA_TRY(strengthen<T>(h, d, cols, b, Vn, w.C + (size_t)m_max * tw * 2, w, s));
+            EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s));
             EDA_TRY(cholqr_pass<T>(d, b, w.W1, d, w.R2, w.R2i, Vn, 0.0, h->status, w.lost, w, s));
             EDA_TRY(oz_basis_grow<T>(w, d, cols, cols + b, h->status, s));
             EDA_TRY(gemm_small_f64(false, false, b, b, b, 1.0, w.R2, b, w.R1, b, 0.0, w.Bm, b, s));   // B = R2 R1

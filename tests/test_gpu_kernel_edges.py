@@ -101,3 +101,19 @@ def test_narrow_block_single_precision(eda, b):
         ref = O.eda(p.X, p.labels, p.k, p.k - 1, c2=h.c2, tier="projected")
     assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-9
     assert O.sin_angle(ref["V"], V.cpu().numpy().T) <= 1e-6
+
+
+# blocks whose Gram loses a column to rounding without its pivot being recognised as lost: the new direction has to come out
+# orthogonal to the basis all the same, whichever side of the threshold the rounding falls
+@pytest.mark.parametrize("prec_name", ["f64", "tc"])
+@pytest.mark.parametrize("seed,b", [(55, 3), (55, 4), (55, 5), (55, 7), (58, 3), (59, 3), (61, 5)])
+def test_nearly_dependent_blocks(eda, seed, b, prec_name):
+    p = synth.gaussian_clusters(d=333, k=7, n_per_class=[2, 3, 5, 1, 4, 3, 2], seed=seed)
+    prec = eda.EDA_F64 if prec_name == "f64" else eda.EDA_F64_TC
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(prec=prec, block_b=b, tau=8.0, tc_min_mi=-1)) as h:
+        ref = O.eda(p.X, p.labels, p.k, 6, c2=h.c2, tier="projected")
+        for V, lam, code in ((lambda r: (r[0], r[1], r[3]))(h.solve_arnoldi(6, 1e-12)),
+                             (lambda r: (r[0], r[1], r[4]))(h.solve(6, 1e-12))):
+            assert code == 0
+            assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
+            assert O.sin_angle(ref["V"], V.cpu().numpy().T) <= 1e-8

@@ -552,7 +552,6 @@ __global__ void __launch_bounds__(64) k_bisect(int n, const double* __restrict__
     float* e232 = d32 + n;                                 // n
     __shared__ double s_tnorm;
     __shared__ unsigned s_ball[2];
-    __shared__ int s_cnt[2];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     // ||T||_inf by warp 0
     if (threadIdx.x < 32) {
@@ -597,17 +596,27 @@ __global__ void __launch_bounds__(64) k_bisect(int n, const double* __restrict__
         }
     }
     double dlo = (double)lo - 1e-5, dhi = (double)hi + 1e-5;
-    // confirm the bracket in double precision (warp 0 at dlo, warp 1 at dhi); fall back to the full
-    // interval if it fails
+    // first double-precision round: 64 shifts from dlo to dhi, both included (lane l of warp 0 at shift 2 l, of warp 1 at
+    // 2 l + 1), so that it confirms the bracket and divides it; the full interval when the bracket fails
     {
-        if (lane == 0) s_cnt[wp] = sturm_count1_f64(n, d64, e264, wp == 0 ? dlo : dhi);
+        const double step = (dhi - dlo) / 63.0;
+        const int c = sturm_count1_f64(n, d64, e264, dlo + (2 * lane + wp) * step);
+        const unsigned b = __ballot_sync(0xffffffffu, c > idx);
+        if (lane == 0) s_ball[wp] = b;
         __syncthreads();
-        const int clo = s_cnt[0], chi = s_cnt[1];
-        if (!(clo <= idx && chi > idx)) {
+        const unsigned b0 = s_ball[0], b1 = s_ball[1];
+        __syncthreads();
+        if ((b0 & 1u) || !(b1 >> 31)) {
             dlo = -1.0 - 1e-12;
             dhi = 1.0 + 1e-12;
+        } else {
+            // the first shift with more than idx eigenvalues below it
+            const int l = __ffs(b0 | b1) - 1;
+            const int k = ((b0 >> l) & 1u) ? 2 * l : 2 * l + 1;
+            const double base = dlo;
+            dlo = base + (k - 1) * step;
+            dhi = base + k * step;
         }
-        __syncthreads();
     }
     for (int round = 0; round < 24; ++round) {
         const double width = dhi - dlo;
@@ -650,147 +659,188 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 
 // Inverse iteration, one thread per eigenvector; factor arrays laid out [array][i][q] so that
 // the threads of a warp touch consecutive addresses. Gaussian elimination with partial pivoting
-// of T - lambda I takes one reciprocal per row (of the pivot); the two triangular solves carry
-// the running entries in registers. Every pass over the stored arrays reads IV_U rows at a time
-// into registers before it uses them, so one memory latency is paid per IV_U rows instead of per
-// row (the loads of a pass never depend on its stores: row i + 1 is read before row i is written,
-// and the values read are the ones the previous pass left).
-// Output: Zt[i][q] (n x nv, row stride nv).
-constexpr int IV_U = 16;
+// of T - lambda I, two triangular solves a pass, two passes from a counter-based random start.
+//
+// What bounds it is the chain of FP64 instructions of a thread (each about 64 cycles, whatever the number of warps), so a
+// row takes as few as it can: 8 in the elimination (one Newton reciprocal per pivot), 1 or 2 in the forward and 3 in the
+// backward solve, 2 for the norm; comparisons, maxima and the start vector use the bits, the scale between the passes is
+// a power of two, the normalisation is left to the transposition. The rows of a pass are read IV_U at a time, the next
+// group while the current one is used; the interchanges are one bit a row. GB300: n = 288, nv = 199 450 -> 225 us;
+// n = nv = 698 and 100 together 1.77 -> 0.97 ms; n = 144, nv = 99 305 -> 175 us.
+constexpr int IV_U = 8;
 
-__global__ void k_invit(int n, int nv, const double* __restrict__ dgl, const double* __restrict__ eoff,
-                        const double* __restrict__ lam, double* lu, double* Zt, uint64_t seed) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ bool abs_less(double a, double b) {   // |a| < |b|
+    return (__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) < (__double_as_longlong(b) & 0x7FFFFFFFFFFFFFFFll);
+}
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
+// 1 / x for any sign: td_rcp on |x| with the sign put back
+__device__ __forceinline__ double signed_rcp(double x) {
+    const double r = td_rcp(fabs(x));
+    return __hiloint2double(__double2hiint(r) | (__double2hiint(x) & 0x80000000), __double2loint(r));
+}
+
+__global__ void __launch_bounds__(32) k_invit(int n, int nv, const double* __restrict__ dgl,
+                                              const double* __restrict__ eoff, const double* __restrict__ lam, double* lu,
+                                              double* Zt, uint64_t seed) {
+    const int lane = threadIdx.x;
+    // ||T||_inf, by the whole warp
+    double tn = 0.0;
+    for (int i = lane; i < n; i += 32) {
+        const double r = fabs(dgl[i]) + ((i > 0) ? fabs(eoff[i - 1]) : 0.0) + ((i + 1 < n) ? fabs(eoff[i]) : 0.0);
+        tn = fmax(tn, r);
+    }
+    for (int o = 16; o > 0; o >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    const int q = blockIdx.x * blockDim.x + lane;
     if (q >= nv) return;
     const int64_t S = nv;
     double* DL = lu;                           // multipliers
     double* RD = lu + (int64_t)n * S;          // reciprocal pivots
     double* DU = lu + 2 * (int64_t)n * S;      // first superdiagonal of U
     double* DU2 = lu + 3 * (int64_t)n * S;     // second superdiagonal of U
-    double* PIV = lu + 4 * (int64_t)n * S;     // 1.0 where rows i and i+1 were interchanged
+    unsigned* PIV = reinterpret_cast<unsigned*>(lu + 4 * (int64_t)n * S);   // bit i % 32 of word i / 32: rows i, i + 1 swapped
     double* x = Zt;
     const double l = lam[q];
-    double tnorm = 0.0;
-    for (int i = 0; i < n; ++i)
-        tnorm = fmax(tnorm, fabs(dgl[i]) + ((i > 0) ? fabs(eoff[i - 1]) : 0.0) + ((i + 1 < n) ? fabs(eoff[i]) : 0.0));
-    const double tiny = fmax(DBL_EPSILON * tnorm, DBL_MIN);
+    const double tiny = fmax(DBL_EPSILON * tn, DBL_MIN);
     double dcur = dgl[0] - l;
     double ucur = (n > 1) ? eoff[0] : 0.0;
+    unsigned bits = 0;
     for (int i = 0; i + 1 < n; ++i) {
         const double sub = eoff[i];                    // T[i+1, i]
         const double dnext = dgl[i + 1] - l;
         const double unext = (i + 2 < n) ? eoff[i + 1] : 0.0;
-        const bool swap = fabs(dcur) < fabs(sub);
-        const double piv = swap ? sub : ((dcur == 0.0) ? tiny : dcur);
-        const double r = 1.0 / piv;
+        const bool swap = abs_less(dcur, sub);
+        const double piv = swap ? sub : (is_zero(dcur) ? tiny : dcur);
+        const double r = signed_rcp(piv);
         const double f = (swap ? dcur : sub) * r;
         RD[i * S + q] = r;
         DL[i * S + q] = f;
         DU[i * S + q] = swap ? dnext : ucur;
         DU2[i * S + q] = swap ? unext : 0.0;
-        PIV[i * S + q] = swap ? 1.0 : 0.0;
-        const double nd = swap ? (ucur - f * dnext) : (dnext - f * ucur);
+        if (swap) bits |= 1u << (i & 31);
+        if ((i & 31) == 31 || i + 2 == n) {
+            PIV[(i >> 5) * S + q] = bits;
+            bits = 0;
+        }
+        const double hi = swap ? ucur : dnext, lo = swap ? dnext : ucur;
+        dcur = fma(-f, lo, hi);
         ucur = swap ? -f * unext : unext;
-        dcur = nd;
     }
-    RD[(int64_t)(n - 1) * S + q] = 1.0 / ((dcur == 0.0) ? tiny : dcur);
-    // random start in [-1, 1]
-    for (int i = 0; i < n; ++i) {
+    RD[(int64_t)(n - 1) * S + q] = signed_rcp(is_zero(dcur) ? tiny : dcur);
+    // start vector, uniform in [-1, 1): 52 bits of the hash as the fraction of a number in [1, 2)
+    auto start = [&](int i) {
         const uint64_t h = mix64(seed ^ mix64(((uint64_t)q << 32) + (uint64_t)i + 0x5851F42D4C957F2Dull));
-        x[i * S + q] = 2.0 * ((h >> 11) * (1.0 / 9007199254740992.0)) - 1.0;
-    }
-    double sc = 1.0;   // scale of the previous pass, applied to x as it is read
+        return fma(2.0, __longlong_as_double((long long)((h >> 12) | 0x3FF0000000000000ull)), -3.0);
+    };
+    double sc = 1.0;   // power-of-two scale of the previous pass, applied to x as it is read
     for (int it = 0; it < 2; ++it) {
         // forward: L^{-1} P b, the running entry carried in a register
-        double carry = x[q];
+        auto in = [&](int i) { return it == 0 ? start(i) : x[(int64_t)i * S + q]; };
+        double carry = in(0);
         if (it > 0) carry *= sc;
-        for (int i0 = 0; i0 + 1 < n; i0 += IV_U) {
-            double f[IV_U], nx[IV_U], pv[IV_U];
+        double f[IV_U], nx[IV_U];
+        auto load = [&](int i0, double (&ff)[IV_U], double (&xx)[IV_U]) {
 #pragma unroll
             for (int u = 0; u < IV_U; ++u) {
                 const int i = i0 + u;
                 if (i + 1 < n) {
-                    f[u] = DL[i * S + q];
-                    pv[u] = PIV[i * S + q];
-                    nx[u] = x[(i + 1) * S + q];
-                    if (it > 0) nx[u] *= sc;
+                    ff[u] = DL[(int64_t)i * S + q];
+                    xx[u] = in(i + 1);
+                }
+            }
+        };
+        load(0, f, nx);
+        unsigned pv = 0;
+        for (int i0 = 0; i0 + 1 < n; i0 += IV_U) {
+            double fn[IV_U], xn[IV_U];
+            if ((i0 & 31) == 0) pv = PIV[(i0 >> 5) * S + q];
+            if (i0 + IV_U + 1 < n) load(i0 + IV_U, fn, xn);
+#pragma unroll
+            for (int u = 0; u < IV_U; ++u) {
+                const int i = i0 + u;
+                if (i + 1 < n) {
+                    const double b = it > 0 ? nx[u] * sc : nx[u];
+                    const bool swap = (pv >> (i & 31)) & 1u;
+                    const double keep = swap ? b : carry;      // this row of the permuted right-hand side
+                    const double other = swap ? carry : b;
+                    x[(int64_t)i * S + q] = keep;
+                    carry = fma(-f[u], keep, other);
                 }
             }
 #pragma unroll
             for (int u = 0; u < IV_U; ++u) {
-                const int i = i0 + u;
-                if (i + 1 < n) {
-                    if (pv[u] != 0.0) {
-                        x[i * S + q] = nx[u];
-                        carry = carry - f[u] * nx[u];
-                    } else {
-                        x[i * S + q] = carry;
-                        carry = nx[u] - f[u] * carry;
-                    }
-                }
+                f[u] = fn[u];
+                nx[u] = xn[u];
             }
         }
         x[(int64_t)(n - 1) * S + q] = carry;
         // back: U^{-1}, carrying the two previous solution entries
-        double v1 = 0.0, v2 = 0.0, mx = 0.0;
-        for (int i0 = n - 1; i0 >= 0; i0 -= IV_U) {
-            double xv[IV_U], du[IV_U], du2[IV_U], rd[IV_U];
+        double v1 = 0.0, v2 = 0.0;
+        int mx = 0;   // largest biased exponent
+        double xv[IV_U], du[IV_U], du2[IV_U], rd[IV_U];
+        auto loadb = [&](int i0, double (&a)[IV_U], double (&b)[IV_U], double (&c)[IV_U], double (&d)[IV_U]) {
 #pragma unroll
             for (int u = 0; u < IV_U; ++u) {
                 const int i = i0 - u;
                 if (i >= 0) {
-                    xv[u] = x[i * S + q];
-                    du[u] = (i + 1 < n) ? DU[i * S + q] : 0.0;
-                    du2[u] = (i + 2 < n) ? DU2[i * S + q] : 0.0;
-                    rd[u] = RD[i * S + q];
+                    a[u] = x[(int64_t)i * S + q];
+                    b[u] = (i + 1 < n) ? DU[(int64_t)i * S + q] : 0.0;
+                    c[u] = (i + 2 < n) ? DU2[(int64_t)i * S + q] : 0.0;
+                    d[u] = RD[(int64_t)i * S + q];
                 }
             }
+        };
+        loadb(n - 1, xv, du, du2, rd);
+        for (int i0 = n - 1; i0 >= 0; i0 -= IV_U) {
+            double xn[IV_U], dn[IV_U], d2n[IV_U], rn[IV_U];
+            if (i0 - IV_U >= 0) loadb(i0 - IV_U, xn, dn, d2n, rn);
 #pragma unroll
             for (int u = 0; u < IV_U; ++u) {
                 const int i = i0 - u;
                 if (i >= 0) {
-                    double v = xv[u];
-                    if (i + 1 < n) v -= du[u] * v1;
-                    if (i + 2 < n) v -= du2[u] * v2;
-                    v *= rd[u];
-                    x[i * S + q] = v;
-                    mx = fmax(mx, fabs(v));
+                    const double v = fma(-du2[u], v2, fma(-du[u], v1, xv[u])) * rd[u];
+                    x[(int64_t)i * S + q] = v;
+                    mx = max(mx, (__double2hiint(v) >> 20) & 0x7ff);
                     v2 = v1;
                     v1 = v;
                 }
             }
+#pragma unroll
+            for (int u = 0; u < IV_U; ++u) {
+                xv[u] = xn[u];
+                du[u] = dn[u];
+                du2[u] = d2n[u];
+                rd[u] = rn[u];
+            }
         }
-        sc = (mx > 0.0 && isfinite(mx)) ? 1.0 / mx : 0.0;
+        // 2^-(exponent of the largest entry); a zero or non-finite vector comes out zero
+        sc = (mx > 0 && mx < 0x7ff) ? __hiloint2double(max(1, min(0x7fe, 2046 - mx)) << 20, 0) : 0.0;
     }
-    // the last pass's scale, then the norm and the normalisation
+    // norm of the scaled vector; the normalisation factor goes where the pivots were
     double nrm = 0.0;
-    for (int i0 = 0; i0 < n; i0 += IV_U) {
-        double xv[IV_U];
+    for (int i0 = 0; i0 < n; i0 += 2 * IV_U) {
+        double xv[2 * IV_U];
 #pragma unroll
-        for (int u = 0; u < IV_U; ++u)
-            if (i0 + u < n) xv[u] = x[(i0 + u) * S + q] * sc;
+        for (int u = 0; u < 2 * IV_U; ++u) xv[u] = i0 + u < n ? x[(int64_t)(i0 + u) * S + q] : 0.0;
 #pragma unroll
-        for (int u = 0; u < IV_U; ++u)
-            if (i0 + u < n) nrm = fma(xv[u], xv[u], nrm);
+        for (int u = 0; u < 2 * IV_U; ++u) {
+            const double t = xv[u] * sc;
+            nrm = fma(t, t, nrm);
+        }
     }
-    const double sn = (nrm > 0.0) ? 1.0 / sqrt(nrm) : 0.0;
-    for (int i0 = 0; i0 < n; i0 += IV_U) {
-        double xv[IV_U];
-#pragma unroll
-        for (int u = 0; u < IV_U; ++u)
-            if (i0 + u < n) xv[u] = x[(i0 + u) * S + q];
-#pragma unroll
-        for (int u = 0; u < IV_U; ++u)
-            if (i0 + u < n) x[(i0 + u) * S + q] = (xv[u] * sc) * sn;
-    }
+    RD[q] = (nrm > 0.0) ? sc / sqrt(nrm) : 0.0;
 }
 
-// Zt (row-major n x nv) -> Z (column-major, ldz)
-__global__ void k_transpose_out(int n, int nv, const double* Zt, double* Z, int ldz) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)n * nv) return;
-    const int i = (int)(e % n), q = (int)(e / n);
-    Z[(int64_t)q * ldz + i] = Zt[(int64_t)i * nv + q];
+// Zt (row-major n x nv) times its column factors -> Z (column-major, ldz), by 32 x 32 tiles through shared memory
+__global__ void __launch_bounds__(256) k_transpose_out(int n, int nv, const double* __restrict__ Zt,
+                                                       const double* __restrict__ fac, double* __restrict__ Z, int ldz) {
+    __shared__ double t[32][33];
+    const int q0 = blockIdx.y * 32, i0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double f = q0 + lane < nv ? fac[q0 + lane] : 0.0;
+    for (int r = w; r < 32; r += 8)
+        if (i0 + r < n && q0 + lane < nv) t[r][lane] = Zt[(int64_t)(i0 + r) * nv + q0 + lane] * f;
+    __syncthreads();
+    for (int c = w; c < 32; c += 8)
+        if (q0 + c < nv && i0 + lane < n) Z[(int64_t)(q0 + c) * ldz + i0 + lane] = t[lane][c];
 }
 
 // Z <- H_0 H_1 ... H_{n-3} Z, one warp per column of Z; reflector j is read from HV (row j,
@@ -1096,11 +1146,13 @@ __global__ void __launch_bounds__(LZG_THREADS) k_lz_update(int n, int j, double*
 
 // (theta_1, theta_2, |z_m|, beta_m) of the Lanczos tridiagonal: its two largest eigenvalues, the last
 // entry of the unit eigenvector of theta_1, and the residual norm after the last step.
-__global__ void k_lanczos_pack(int m, const double* w, const double* z, const double* eoff, double* out) {
+// (z: the inverse-iteration vector before its normalisation by *fac).
+__global__ void k_lanczos_pack(int m, const double* w, const double* z, const double* fac, const double* eoff,
+                               double* out) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     out[0] = w[m >= 2 ? 1 : 0];
     out[1] = (m >= 2) ? w[0] : -DBL_MAX;
-    out[2] = fabs(z[m - 1]);
+    out[2] = fabs(z[m - 1] * fac[0]);
     out[3] = eoff[m - 1];
 }
 
@@ -1368,7 +1420,8 @@ int invit_vectors(int n, int nv, const double* w, double* Z, int ldz, SymEigWork
         k_invit<<<ceil_div(nv, 32), 32, 0, s>>>(n, nv, ws->dgl, ws->eoff, w, lu, Zt, seed);
         EDA_LAUNCHED();
     }
-    k_transpose_out<<<ceil_div((int64_t)n * nv, 256), 256, 0, s>>>(n, nv, Zt, Z, ldz);
+    // the normalisation factors: row 0 of the reciprocal pivots
+    k_transpose_out<<<dim3(ceil_div(n, 32), ceil_div(nv, 32)), 256, 0, s>>>(n, nv, Zt, lu + (size_t)n * nv, Z, ldz);
     EDA_LAUNCHED();
     return EDA_OK;
 }
@@ -1586,7 +1639,7 @@ int lanczos_top(int n, const double* A, int lda, int m, uint64_t seed, SymEigWor
         EDA_LAUNCHED();
         k_invit<<<1, 32, 0, s>>>(m, 1, ws->dgl, ws->eoff, w + nv - 1, ws->lu, zt, seed);   // st is dead here
         EDA_LAUNCHED();
-        k_lanczos_pack<<<1, 32, 0, s>>>(m, w, zt, ws->eoff, out);
+        k_lanczos_pack<<<1, 32, 0, s>>>(m, w, zt, ws->lu + m, ws->eoff, out);
         EDA_LAUNCHED();
         return EDA_OK;
     }
@@ -1623,7 +1676,7 @@ int lanczos_top(int n, const double* A, int lda, int m, uint64_t seed, SymEigWor
     EDA_LAUNCHED();
     k_invit<<<1, 32, 0, s>>>(m, 1, ws->dgl, ws->eoff, w + nv - 1, ws->lu, zt, seed);
     EDA_LAUNCHED();
-    k_lanczos_pack<<<1, 32, 0, s>>>(m, w, zt, ws->eoff, out);
+    k_lanczos_pack<<<1, 32, 0, s>>>(m, w, zt, ws->lu + m, ws->eoff, out);
     EDA_LAUNCHED();
     return EDA_OK;
 }

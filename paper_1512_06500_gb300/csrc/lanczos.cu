@@ -396,8 +396,17 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
                                h->cfg.seed + 7, last ? 1e-7 : 0.0, s));
             EDA_TRY(estimate());
             if (!last && st.conv_count == t) {
-                EDA_TRY(symeig_vectors(cols, t, w.theta, w.S, cols, &w.eig, h->cfg.seed + 7, 1e-7, s));
-                EDA_TRY(estimate());
+                // without a cluster the vectors at hand are those that a second pass would give
+                std::vector<double> th(t);
+                EDA_TRY(read_back(th.data(), w.theta, t * sizeof(double), s));
+                double mx = 0.0;
+                for (double v : th) mx = std::fmax(mx, std::fabs(v));
+                bool cluster = false;
+                for (int i = 1; i < t; ++i) cluster |= th[i] - th[i - 1] <= 1e-7 * mx;
+                if (cluster) {
+                    EDA_TRY(symeig_vectors(cols, t, w.theta, w.S, cols, &w.eig, h->cfg.seed + 7, 1e-7, s));
+                    EDA_TRY(estimate());
+                }
             }
             if (st.conv_count == t) st.converged = true;
             // no usable rate (no progress since the last check): wait a quarter of the basis width (the

@@ -103,12 +103,9 @@ struct DirectWs {
 // from the handle's split when it has one, else as the FP64 product M^T X.
 int sym_nn(eda_ctx* h, const OzOperand* oz, const double* M, int n, int p, const double* X, int ldx, bool acc,
            double* D, int ldd, DirectWs& w, cudaStream_t s) {
-    if (oz) {
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(*oz, h->oznb, std::min(32, p - c0), X + (size_t)c0 * ldx, ldx, 1.0, acc ? 1.0 : 0.0,
-                            acc ? D + (size_t)c0 * ldd : nullptr, ldd, D + (size_t)c0 * ldd, ldd, h->status, s));
-        return EDA_OK;
-    }
+    if (oz)
+        return oz_gemm_wide(*oz, h->oznb, h->ozwide, p, X, ldx, 1.0, acc ? 1.0 : 0.0, acc ? D : nullptr, ldd, D, ldd,
+                            h->status, s);
     return gemm_tn_f64(n, n, p, 1.0, M, n, X, ldx, acc ? 1.0 : 0.0, D, ldd, w.part, w.pcap, s);
 }
 
@@ -132,12 +129,8 @@ int apply_c(eda_ctx* h, int p, double* PQ, double* U, DirectWs& w, cudaStream_t 
 // OUT (d x p) = Z U for U ((n + k) x p, ld nk): one sweep over Z (tensor-core FP64 when the handle has Z split).
 int z_times(eda_ctx* h, int p, const double* U, double* OUT, cudaStream_t s) {
     const int nk = (int)h->n + h->k;
-    if (h->cfg.prec == EDA_F64_TC && h->ozblock) {
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(h->ozN, h->oznb, std::min(32, p - c0), U + (size_t)c0 * nk, nk, 1.0, 0.0, nullptr, 0,
-                            OUT + (size_t)c0 * h->d, h->d, h->status, s));
-        return EDA_OK;
-    }
+    if (h->cfg.prec == EDA_F64_TC && h->ozblock)
+        return oz_gemm_wide(h->ozN, h->oznb, h->ozwide, p, U, nk, 1.0, 0.0, nullptr, 0, OUT, h->d, h->status, s);
     return gemm_nn_f64(h->d, nk, p, 1.0, h->HW, h->d, U, nk, 0.0, nullptr, 0, OUT, h->d, s);
 }
 

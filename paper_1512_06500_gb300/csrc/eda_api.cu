@@ -41,7 +41,8 @@ int ensure_workspace(eda_ctx* h, size_t bytes) {
 }
 
 void destroy_handle(eda_ctx* h, bool idle) {
-    for (void* p : {h->ws, h->kblock, h->xblock, h->ozblock, h->ozsmall, h->nblock, h->block32, h->fblock, h->block}) {
+    for (void* p : {h->ws, h->kblock, h->xblock, h->ozblock, h->ozsmall, h->nblock, h->block32, h->fblock, h->block,
+                    h->ozwide.mem}) {
         if (!p) continue;
         if (idle) dev_free(p);
         else cudaFree(p);

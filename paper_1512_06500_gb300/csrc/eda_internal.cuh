@@ -384,6 +384,18 @@ int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double b
                   double* D, int64_t ldd, bool upper, int* status, cudaStream_t s, double* part = nullptr,
                   size_t pcap = 0);
 
+// Device scratch of a handle for the split of a wide right-hand side.
+struct OzScratch {
+    void* mem = nullptr;
+    size_t bytes = 0;
+    int ensure(size_t need);
+};
+// D (M x p, ldd) = alpha op(A) B + beta C0 for any p: oz_gemm up to 32 columns; beyond, B (K x p, ldb) is split once as a
+// tiled operand and all its 32-column blocks run in one launch, in which the blocks of one band of A share A's tiles
+// through L2 (column by column of blocks, each launch reads all of A from HBM again).
+int oz_gemm_wide(const OzOperand& A, OzNarrow& nb, OzScratch& sc, int p, const double* B, int64_t ldb, double alpha,
+                 double beta, const double* C0, int64_t ldc0, double* D, int64_t ldd, int* status, cudaStream_t s);
+
 // K(alpha) = alpha phi(alpha G) from G itself by scaling and squaring (dense products only), given
 // lmax >= the largest eigenvalue of G. work: 6 m^2 doubles. With oz the m x m products run on the
 // tensor cores: abuf and bbuf hold oz_operand_bytes(m, m) bytes each (the two factors' splits).
@@ -439,6 +451,7 @@ struct eda_ctx {
     void* ozblock = nullptr;
     eda::OzOperand ozT, ozN;
     eda::OzNarrow oznb;
+    eda::OzScratch ozwide;                 // split of a right-hand side of more than 32 columns (grown on demand)
     // prec = EDA_F64_TC and n >= kOzSmallMinN: the left-factor split of the scaling and squaring that
     // forms K_W (and, for the nonsymmetric form, K(-c^2) and K(+c^2)), then K_W and G_W split for
     // their products with the n x p coordinates inside the composed M-apply and the recovery

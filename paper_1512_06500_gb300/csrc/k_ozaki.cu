@@ -61,12 +61,15 @@ __device__ __forceinline__ OzRing& oz_ring(unsigned char* raw) {
     return *reinterpret_cast<OzRing*>(raw + ((1024u - mis) & 1023u));
 }
 
-// B from a pre-tiled split operand (BT mode): its planes at tiles + q * slice, the same K tiling as A; the
-// product's 32-column block z (blockIdx.z) is the quarter z % 4 of B's 128-row band z / 4, one contiguous
-// 4 KB image per plane and stage. upper: skip the blocks wholly below the diagonal (z 32 + 32 <= band 128).
+// B from a pre-tiled split operand (BT mode): its planes at tiles + q * slice, kbs tiles along K per band; the
+// product's 32-column block x (blockIdx.x mod nblk) is the quarter x % 4 of B's 128-row band x / 4, one contiguous
+// 4 KB image per plane and stage, and the band of A is blockIdx.x / nblk: the CTAs that run together share few bands of A,
+// whose tiles they then find in L2. upper: skip the blocks wholly below the diagonal (x 32 + 32 <= band 128).
 struct OzBTiles {
     const __nv_bfloat16* tiles = nullptr;
     int64_t slice = 0;
+    int kbs = 0;
+    int nblk = 1;   // 32-column blocks
     int upper = 0;
 };
 
@@ -74,7 +77,7 @@ struct OzBTiles {
 // the split-th slice of D at D + split * split_stride. A: digit planes at At + q * aslice, pre-tiled
 // (128-row bands, kbs tiles of 64 along K per band), row scales expA. B: digit planes read through tmB
 // (inner = K, outer = 7 x 32 rows: plane q is rows 32 q .. 32 q + 31), or in BT mode from bt (N rows, the
-// CTA's 32 of them chosen by blockIdx.z), row scales expB. K stages [split * kps, min(kst, (split + 1) * kps)).
+// CTA's 32 of them chosen by blockIdx.x mod nblk), row scales expB. K stages [split * kps, min(kst, (split + 1) * kps)).
 template <bool BT>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(const __nv_bfloat16* __restrict__ At, int64_t aslice, int kbs, const __grid_constant__ CUtensorMap tmB,
@@ -84,8 +87,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     extern __shared__ unsigned char smraw[];
     OzRing& sm = oz_ring(smraw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int band = blockIdx.x, split = blockIdx.y;
-    const int blk = BT ? (int)blockIdx.z : 0;
+    const int band = BT ? (int)blockIdx.x / bt.nblk : (int)blockIdx.x, split = blockIdx.y;
+    const int blk = BT ? (int)blockIdx.x % bt.nblk : 0;
     if (BT) {
         if (bt.upper && blk * OZ_N + OZ_N <= band * TC_M) return;   // the whole CTA: a uniform exit
         expB += blk * OZ_N;
@@ -134,7 +137,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             mbar_expect_tx(&sm.fullB[bslot], bbytes);
             if (BT) {
                 const __nv_bfloat16* src =
-                    bt.tiles + ((((int64_t)(blk >> 2)) * kbs + kstage) << 13) + (int64_t)(blk & 3) * (OZ_N * TC_KS);
+                    bt.tiles + ((((int64_t)(blk >> 2)) * bt.kbs + kstage) << 13) + (int64_t)(blk & 3) * (OZ_N * TC_KS);
 #pragma unroll
                 for (int q = 0; q < OZ_S; ++q)
                     bulk_load(sm.B[bslot][q], src + q * bt.slice, OZ_N * TC_KS * 2, &sm.fullB[bslot]);
@@ -722,21 +725,32 @@ __global__ void k_oz_mirror_lower(int n, double* D, int64_t ldd) {
 
 int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double beta, const double* C0, int64_t ldc0,
                   double* D, int64_t ldd, bool upper, int* status, cudaStream_t s, double* part, size_t pcap) {
-    if (A.K != B.K || A.kbs != B.kbs || A.M < 1 || B.M < 1) return EDA_ERR_INVALID_ARG;
+    if (A.K != B.K || A.M < 1 || B.M < 1) return EDA_ERR_INVALID_ARG;
     if (upper && (A.tiles != B.tiles || beta != 0.0)) return EDA_ERR_INVALID_ARG;
     EDA_TRY(oz_attr());
-    const int kst = A.kbs;
+    const int kst = ceil_div(A.K, TC_KS);   // an operand with room for more (a growing basis) has more tiles a band
     const int nblk = ceil_div(B.M, OZ_N);
-    // K splits only when the (band, block) grid leaves SMs idle and a partial buffer is given
+    // K splits (when a partial buffer is given): the count of 1 .. 8, or up to one wave of CTAs, that fills the SMs best at one
+    // CTA each; a larger count only for 4 % more (each adds a pass over the result)
     int splits = 1;
     if (part && !upper) {
-        splits = std::max(1, std::min(kst / 8, sm_count() / std::max(1, A.mtiles * nblk)));
-        while (splits > 1 && (size_t)splits * A.M * B.M > pcap) --splits;
+        const int nsm = sm_count(), tiles = std::max(1, A.mtiles * nblk);
+        double best = 0.0;
+        for (int c = 1; c <= std::min(kst / 8, std::max(8, nsm / tiles)); ++c) {
+            if ((size_t)c * A.M * B.M > pcap) break;
+            const double fill = (double)tiles * c / ((double)nsm * ((tiles * c + nsm - 1) / nsm));
+            if (fill > best + 0.04) {
+                best = fill;
+                splits = c;
+            }
+        }
     }
     const int kps = ceil_div(kst, splits);
     splits = ceil_div(kst, kps);
-    const dim3 grid((unsigned)A.mtiles, (unsigned)splits, (unsigned)nblk);
+    const dim3 grid((unsigned)nblk * (unsigned)A.mtiles, (unsigned)splits);
     OzBTiles bt;
+    bt.kbs = B.kbs;
+    bt.nblk = nblk;
     bt.tiles = B.tiles;
     bt.slice = B.slice;
     bt.upper = upper ? 1 : 0;
@@ -768,6 +782,26 @@ int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double b
         k_oz_mirror_lower<<<ceil_div((int64_t)A.M * A.M, 256), 256, 0, s>>>((int)A.M, D, ldd);
         EDA_LAUNCHED();
     }
+    return EDA_OK;
+}
+
+int oz_gemm_wide(const OzOperand& A, OzNarrow& nb, OzScratch& sc, int p, const double* B, int64_t ldb, double alpha,
+                 double beta, const double* C0, int64_t ldc0, double* D, int64_t ldd, int* status, cudaStream_t s) {
+    if (p <= OZ_N) return oz_gemm(A, nb, p, B, ldb, alpha, beta, C0, ldc0, D, ldd, status, s);
+    EDA_TRY(sc.ensure(oz_operand_bytes(p, A.K)));
+    OzOperand op;
+    EDA_TRY(oz_operand_make(B, ldb, p, A.K, true, sc.mem, &op, status, s));
+    return oz_gemm_tiled(A, op, alpha, beta, C0, ldc0, D, ldd, false, status, s, nb.partial, nb.pcap);
+}
+
+int OzScratch::ensure(size_t need) {
+    if (bytes >= need) return EDA_OK;
+    void* old = mem;
+    mem = nullptr;
+    bytes = 0;
+    EDA_TRY(dev_free_idle(old));   // earlier products may still read it
+    EDA_TRY(dev_alloc(&mem, need));
+    bytes = need;
     return EDA_OK;
 }
 

@@ -120,27 +120,21 @@ struct SolveWs {
     int* olist = nullptr;            // d + 1 ints: rows of VN to split afresh
 };
 
-// tc products with the split basis, 32 columns at a time: C (cols x p, ldc) = V^T X, and X -= V C
+// tc products with the split basis: C (cols x p, ldc) = V^T X, and X -= V C
 template <class T>
 int oz_basis_tn(eda_ctx* h, SolveWs<T>& w, int cols, int p, const double* X, int64_t ldx, double* C, int ldc,
                 cudaStream_t s) {
     OzOperand A = w.VT;
     A.M = cols;
     A.mtiles = ceil_div(cols, 128);
-    for (int c0 = 0; c0 < p; c0 += 32)
-        EDA_TRY(oz_gemm(A, h->oznb, std::min(32, p - c0), X + (size_t)c0 * ldx, ldx, 1.0, 0.0, nullptr, 0,
-                        C + (size_t)c0 * ldc, ldc, h->status, s));
-    return EDA_OK;
+    return oz_gemm_wide(A, h->oznb, h->ozwide, p, X, ldx, 1.0, 0.0, nullptr, 0, C, ldc, h->status, s);
 }
 template <class T>
 int oz_basis_nn(eda_ctx* h, SolveWs<T>& w, int cols, int p, const double* C, int ldc, double alpha, double beta,
                 const double* X0, int64_t ldx0, double* X, int64_t ldx, cudaStream_t s) {
     OzOperand A = w.VN;
     A.K = cols;
-    for (int c0 = 0; c0 < p; c0 += 32)
-        EDA_TRY(oz_gemm(A, h->oznb, std::min(32, p - c0), C + (size_t)c0 * ldc, ldc, alpha, beta,
-                        X0 ? X0 + (size_t)c0 * ldx0 : nullptr, ldx0, X + (size_t)c0 * ldx, ldx, h->status, s));
-    return EDA_OK;
+    return oz_gemm_wide(A, h->oznb, h->ozwide, p, C, ldc, alpha, beta, X0, ldx0, X, ldx, h->status, s);
 }
 
 // The basis has grown from cols0 to cols1 columns: append their column-scaled digit planes and split the
@@ -475,10 +469,7 @@ int m_apply_composed(eda_ctx* h, int p, const double* Y, int64_t ldy, double* MY
     auto nn = [&](const OzOperand* oz, const double* M, const double* X, double beta, const double* C0,
                   double* D) -> int {
         if (!oz) return gemm_small_f64(false, false, n, p, n, 1.0, M, n, X, nk, beta, D, nk, s);
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(*oz, h->oznb, std::min(32, p - c0), X + (size_t)c0 * nk, nk, 1.0, beta,
-                            C0 ? C0 + (size_t)c0 * nk : nullptr, nk, D + (size_t)c0 * nk, nk, h->status, s));
-        return EDA_OK;
+        return oz_gemm_wide(*oz, h->oznb, h->ozwide, p, X, nk, 1.0, beta, C0, nk, D, nk, h->status, s);
     };
     const OzOperand* okw = h->ozsmall ? &h->ozKW : nullptr;
     const OzOperand* ogw = h->ozsmall ? &h->ozGW : nullptr;
@@ -492,15 +483,11 @@ int m_apply_composed(eda_ctx* h, int p, const double* Y, int64_t ldy, double* MY
 }
 
 // PQ ((n + k) x p) = Z^T Y, Z = [H_W H_B]: the first sweep of a composed product; FP64-accurate tensor-core
-// products (error-free splitting, 32 columns at a time) for prec EDA_F64_TC, FP64 otherwise.
+// products (error-free splitting) for prec EDA_F64_TC, FP64 otherwise.
 int sweep_zt(eda_ctx* h, int p, const double* Y, int64_t ldy, double* PQ, double* part, size_t pcap, cudaStream_t s) {
     const int nk = (int)h->n + h->k;
-    if (h->cfg.prec == EDA_F64_TC && h->ozblock) {
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(h->ozT, h->oznb, std::min(32, p - c0), Y + (size_t)c0 * ldy, ldy, 1.0, 0.0, nullptr, 0,
-                            PQ + (size_t)c0 * nk, nk, h->status, s));
-        return EDA_OK;
-    }
+    if (h->cfg.prec == EDA_F64_TC && h->ozblock)
+        return oz_gemm_wide(h->ozT, h->oznb, h->ozwide, p, Y, ldy, 1.0, 0.0, nullptr, 0, PQ, nk, h->status, s);
     return gemm_tn_f64(h->d, nk, p, 1.0, h->HW, h->d, Y, ldy, 0.0, PQ, nk, part, pcap, s);
 }
 
@@ -508,12 +495,8 @@ int sweep_zt(eda_ctx* h, int p, const double* Y, int64_t ldy, double* PQ, double
 int sweep_z(eda_ctx* h, int p, const double* U, const double* Y, int64_t ldy, double* OUT, int64_t ldo,
             cudaStream_t s) {
     const int nk = (int)h->n + h->k;
-    if (h->cfg.prec == EDA_F64_TC && h->ozblock) {
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(h->ozN, h->oznb, std::min(32, p - c0), U + (size_t)c0 * nk, nk, 1.0, 1.0,
-                            Y + (size_t)c0 * ldy, ldy, OUT + (size_t)c0 * ldo, ldo, h->status, s));
-        return EDA_OK;
-    }
+    if (h->cfg.prec == EDA_F64_TC && h->ozblock)
+        return oz_gemm_wide(h->ozN, h->oznb, h->ozwide, p, U, nk, 1.0, 1.0, Y, ldy, OUT, ldo, h->status, s);
     return gemm_nn_f64(h->d, nk, p, 1.0, h->HW, h->d, U, nk, 1.0, Y, ldy, OUT, ldo, s);
 }
 
@@ -530,10 +513,7 @@ int fin_tn(eda_ctx* h, SolveWs<T>& w, int m, int p, const double* A, const doubl
     if (w.oz && m <= w.oz_cap) {
         OzOperand op;
         EDA_TRY(oz_operand_make(A, d, m, d, true, w.VT.tiles, &op, h->status, s));
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(op, h->oznb, std::min(32, p - c0), B + (size_t)c0 * ldb, ldb, 1.0, 0.0, nullptr, 0,
-                            C + (size_t)c0 * ldc, ldc, h->status, s));
-        return EDA_OK;
+        return oz_gemm_wide(op, h->oznb, h->ozwide, p, B, ldb, 1.0, 0.0, nullptr, 0, C, ldc, h->status, s);
     }
     return gemm_tn_f64(d, m, p, 1.0, A, d, B, ldb, 0.0, C, ldc, static_cast<double*>(w.part), w.pcap, s);
 }
@@ -545,10 +525,7 @@ int fin_nn(eda_ctx* h, SolveWs<T>& w, int m, int p, double alpha, const double* 
     if (w.oz && m <= w.oz_cap) {
         OzOperand op;
         EDA_TRY(oz_operand_make(A, d, d, m, false, w.VN.tiles, &op, h->status, s));
-        for (int c0 = 0; c0 < p; c0 += 32)
-            EDA_TRY(oz_gemm(op, h->oznb, std::min(32, p - c0), Bs + (size_t)c0 * ldbs, ldbs, alpha, beta,
-                            X0 ? X0 + (size_t)c0 * d : nullptr, d, OUT + (size_t)c0 * d, d, h->status, s));
-        return EDA_OK;
+        return oz_gemm_wide(op, h->oznb, h->ozwide, p, Bs, ldbs, alpha, beta, X0, d, OUT, d, h->status, s);
     }
     return gemm_nn_f64(d, m, p, alpha, A, d, Bs, ldbs, beta, X0, d, OUT, d, s);
 }
@@ -828,19 +805,12 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
         AT.M = n;
         AT.mtiles = ceil_div(n, 128);
         AN.K = n;
-        for (int c0 = 0; c0 < t; c0 += 32)
-            EDA_TRY(oz_gemm(AT, h->oznb, std::min(32, t - c0), w.Y2 + (size_t)c0 * d, d, 1.0, 0.0, nullptr, 0,
-                            w.P + (size_t)c0 * n, n, h->status, s));
-        if (h->ozsmall) {
-            for (int c0 = 0; c0 < t; c0 += 32)
-                EDA_TRY(oz_gemm(h->ozKW, h->oznb, std::min(32, t - c0), w.P + (size_t)c0 * n, n, 1.0, 0.0, nullptr,
-                                0, w.Q + (size_t)c0 * n, n, h->status, s));
-        } else {
+        EDA_TRY(oz_gemm_wide(AT, h->oznb, h->ozwide, t, w.Y2, d, 1.0, 0.0, nullptr, 0, w.P, n, h->status, s));
+        if (h->ozsmall)
+            EDA_TRY(oz_gemm_wide(h->ozKW, h->oznb, h->ozwide, t, w.P, n, 1.0, 0.0, nullptr, 0, w.Q, n, h->status, s));
+        else
             EDA_TRY(gemm_small_f64(false, false, n, t, n, 1.0, h->KW, n, w.P, n, 0.0, w.Q, n, s));
-        }
-        for (int c0 = 0; c0 < t; c0 += 32)
-            EDA_TRY(oz_gemm(AN, h->oznb, std::min(32, t - c0), w.Q + (size_t)c0 * n, n, 1.0, 1.0,
-                            w.Y2 + (size_t)c0 * d, d, w.Xt + (size_t)c0 * d, d, h->status, s));
+        EDA_TRY(oz_gemm_wide(AN, h->oznb, h->ozwide, t, w.Q, n, 1.0, 1.0, w.Y2, d, w.Xt, d, h->status, s));
     } else {
         EDA_TRY(exp_apply<double>(d, h->HW, h->KW, n, "exp_apply_w", t, w.Y2, d, w.Xt, d, w.P, w.Q, w.part, w.pcap,
                                   s));

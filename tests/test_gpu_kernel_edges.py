@@ -117,3 +117,27 @@ def test_nearly_dependent_blocks(eda, seed, b, prec_name):
             assert code == 0
             assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
             assert O.sin_angle(ref["V"], V.cpu().numpy().T) <= 1e-8
+
+
+# tensor-core FP64 products with more than 32 right-hand sides (one launch over all 32-column blocks): the edges of a block
+# and of a 128-row band, K splits on and off, and an operand with room for more columns than it holds (the Krylov basis)
+@pytest.mark.parametrize("d,k,nj,b", [(1000, 34, 3, 8), (4097, 66, 2, 16), (700, 65, 4, 33), (9000, 45, 12, 40)])
+def test_wide_right_hand_sides(eda, d, k, nj, b):
+    p = synth.gaussian_clusters(d=d, k=k, n_per_class=nj, seed=d + k)
+    cfg = eda.config(prec=eda.EDA_F64_TC, block_b=b, tau=8.0, tc_min_mi=-1)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, cfg) as h:
+        rng = np.random.default_rng(k)
+        f = O.scatter_factors(p.X, p.labels, p.k)
+        for m in (33, 64, 65, 129):
+            X = rng.standard_normal((d, m))
+            Y = h.apply_exp(eda.OP_M, _dev(X.T)).cpu().numpy().T
+            Yr = O.m_apply(f["HW"], f["HB"], h.c2, X)
+            assert (np.abs(Y - Yr).max(0) <= 1e-12 * np.abs(Yr).max(0)).all()
+        ref = O.eda(p.X, p.labels, p.k, p.k - 1, c2=h.c2, tier="projected")
+        for V, lam, code in ((lambda r: (r[0], r[1], r[4]))(h.solve(p.k - 1, 1e-11)),
+                             (lambda r: (r[0], r[1], r[3]))(h.solve_direct(p.k - 1))):
+            assert code == 0
+            V = V.cpu().numpy().T
+            assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
+            assert O.sin_angle(ref["V"], V) <= 1e-8
+            assert np.abs(V.T @ V - np.eye(p.k - 1)).max() <= 1e-12

@@ -142,6 +142,9 @@ int gemm_nn_f64(int64_t d, int m, int p, double alpha, const double* A, int64_t 
 // Small dense C (m x p) = alpha * op(A) op(B) + beta * C with op = N or T (all column-major).
 int gemm_small_f64(bool ta, bool tb, int m, int p, int kk, double alpha, const double* A, int lda,
                    const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s);
+// The same (no transposes) for an m x m product that is symmetric, with symmetric C: one triangle in 32-row blocks, mirrored.
+int gemm_small_sym_f64(int m, double alpha, const double* A, int lda, const double* B, int ldb, double beta, double* C,
+                       int ldc, cudaStream_t s);
 // In-place upper Cholesky of a b x b SPD matrix G = R^T R (R stored in the upper triangle, the
 // strict lower triangle zeroed) and Rinv = R^{-1} (b x b, ld b). A pivot (squared) at or below
 // max(rank_tol * max diag, piv_min2) marks rank loss: that row of R and of Rinv is set to zero
@@ -377,7 +380,7 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
 
 // D (A.M x B.M, ldd) = alpha A B^T + beta C0 for two split operands over the same K (both in the
 // column-scaled layout: D_ij = sum_k A_ik B_jk), one launch over (128-row band of A, 32-row block of B).
-// upper (A and B the same operand, beta = 0): only the blocks meeting the upper triangle are computed and
+// upper (for a symmetric product, and C0): only the blocks meeting the upper triangle are computed and
 // the others mirrored; the product of an operand with itself is exactly symmetric. part (pcap doubles,
 // optional): K-split partials, used when the output grid alone leaves SMs idle (not with upper).
 int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double beta, const double* C0, int64_t ldc0,

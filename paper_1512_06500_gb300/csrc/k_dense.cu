@@ -342,7 +342,10 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double
 // eight independent chains (eight loads of A in flight per lane: at these sizes the product is bound
 // by load latency, then by the FP64 pipe), and the eighths are added in a fixed order through shared
 // memory.
+// SYM (m = p, a symmetric product and C): entries i >= j only, each written to (i, j) and (j, i); the grid's x runs over
+// the CTAs that hold such entries, column after column.
 constexpr int kSplitkWarps = 8;
+template <bool SYM>
 __global__ void __launch_bounds__(32 * kSplitkWarps) k_gemm_small_nn_splitk(int m, int p, int kk, double alpha,
                                                                            const double* __restrict__ A, int lda,
                                                                            const double* __restrict__ B, int ldb,
@@ -350,8 +353,17 @@ __global__ void __launch_bounds__(32 * kSplitkWarps) k_gemm_small_nn_splitk(int 
                                                                            int ldc) {
     __shared__ double part[kSplitkWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + lane;
-    const int j = blockIdx.y;
+    int ib = blockIdx.x, j = blockIdx.y;
+    if (SYM) {
+        // blocks of 32 columns from the right: column block c has nb - c row blocks a column
+        const int nb = (m + 31) / 32;
+        int c = 0, e = blockIdx.x;
+        while (e >= 32 * (nb - c)) e -= 32 * (nb - c), ++c;
+        ib = c + e % (nb - c);
+        j = 32 * c + e / (nb - c);
+        if (j >= m) return;   // uniform over the CTA
+    }
+    const int i = ib * 32 + lane;
     const int q = (kk + kSplitkWarps - 1) / kSplitkWarps;
     const int lb = w * q, le = min(kk, lb + q);
     double a[8];
@@ -371,9 +383,11 @@ __global__ void __launch_bounds__(32 * kSplitkWarps) k_gemm_small_nn_splitk(int 
     if (w == 0 && i < m) {
         const double acc = ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane])) +
                            ((part[4][lane] + part[5][lane]) + (part[6][lane] + part[7][lane]));
+        if (SYM && i < j) return;
         double v = alpha * acc;
         if (beta != 0.0) v = fma(beta, C[(int64_t)j * ldc + i], v);
         C[(int64_t)j * ldc + i] = v;
+        if (SYM) C[(int64_t)i * ldc + j] = v;
     }
 }
 
@@ -932,7 +946,7 @@ int gemm_small_f64(bool ta, bool tb, int m, int p, int kk, double alpha, const d
                    int ldb, double beta, double* C, int ldc, cudaStream_t s) {
     if (m <= 0 || p <= 0) return EDA_OK;
     if (!ta && !tb && kk >= 64) {
-        k_gemm_small_nn_splitk<<<dim3(ceil_div(m, 32), p), 32 * kSplitkWarps, 0, s>>>(m, p, kk, alpha, A, lda, B, ldb,
+        k_gemm_small_nn_splitk<false><<<dim3(ceil_div(m, 32), p), 32 * kSplitkWarps, 0, s>>>(m, p, kk, alpha, A, lda, B, ldb,
                                                                                   beta, C, ldc);
         EDA_LAUNCHED();
         return EDA_OK;
@@ -940,6 +954,16 @@ int gemm_small_f64(bool ta, bool tb, int m, int p, int kk, double alpha, const d
     // one warp per CTA (32 rows of one column): FP64 work spreads over all SMs
     dim3 blk(32, 1), grid(ceil_div(m, 32), p);
     k_gemm_small<<<grid, blk, 0, s>>>(ta, tb, m, p, kk, alpha, A, lda, B, ldb, beta, C, ldc);
+    EDA_LAUNCHED();
+    return EDA_OK;
+}
+
+int gemm_small_sym_f64(int m, double alpha, const double* A, int lda, const double* B, int ldb, double beta, double* C,
+                       int ldc, cudaStream_t s) {
+    if (m < 64) return gemm_small_f64(false, false, m, m, m, alpha, A, lda, B, ldb, beta, C, ldc, s);
+    const int nb = ceil_div(m, 32);
+    k_gemm_small_nn_splitk<true><<<32 * (nb * (nb + 1) / 2), 32 * kSplitkWarps, 0, s>>>(m, m, m, alpha, A, lda, B, ldb,
+                                                                                      beta, C, ldc);
     EDA_LAUNCHED();
     return EDA_OK;
 }

@@ -715,7 +715,7 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
 
 // D[i, j] = alpha sum_k A_ik B_jk + beta C0[i, j] for two split operands with the same K (i < A.M, j < B.M):
 // one launch over (A band, B 32-row block); upper: only the blocks meeting the upper triangle i <= j, the
-// rest filled by the mirror image (A and B the same operand: the product is then exactly symmetric).
+// rest filled by the mirror image (for products that are symmetric; blocks on the diagonal are computed whole).
 __global__ void k_oz_mirror_lower(int n, double* D, int64_t ldd) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)n * n) return;
@@ -726,7 +726,7 @@ __global__ void k_oz_mirror_lower(int n, double* D, int64_t ldd) {
 int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double beta, const double* C0, int64_t ldc0,
                   double* D, int64_t ldd, bool upper, int* status, cudaStream_t s, double* part, size_t pcap) {
     if (A.K != B.K || A.M < 1 || B.M < 1) return EDA_ERR_INVALID_ARG;
-    if (upper && (A.tiles != B.tiles || beta != 0.0)) return EDA_ERR_INVALID_ARG;
+    if (upper && A.M != B.M) return EDA_ERR_INVALID_ARG;
     EDA_TRY(oz_attr());
     const int kst = ceil_div(A.K, TC_KS);   // an operand with room for more (a growing basis) has more tiles a band
     const int nblk = ceil_div(B.M, OZ_N);

@@ -360,12 +360,10 @@ int oz_operand_make(const double* A, int64_t lda, int64_t M, int64_t K, bool row
                     OzOperand* op, int* status, cudaStream_t s);
 // A growing operand (the Krylov basis): room for Mcap rows and Kcap reduction values, planes zeroed.
 // oz_append_cols: split columns i0 .. i1 of A (d x ., lda) as rows i0 .. i1 of a column-scaled operand
-// (K = d). oz_resplit_rows: split all of A (M x K) afresh as a row-scaled operand (row scales over the K
-// columns present).
+// (K = d).
 int oz_operand_init(int64_t Mcap, int64_t Kcap, void* mem, OzOperand* op, cudaStream_t s);
 int oz_append_cols(const double* A, int64_t lda, int i0, int i1, int64_t K, OzOperand* op, int* status,
                    cudaStream_t s);
-int oz_resplit_rows(const double* A, int64_t lda, int64_t M, int64_t K, OzOperand* op, int* status, cudaStream_t s);
 // Grow a row-scaled operand (made by oz_operand_init, grown only by this call) from k0 to k1 columns of A:
 // new digits for the rows whose scale the new columns leave unchanged, a full re-split of the others.
 // list: M + 1 ints of scratch.

@@ -75,13 +75,24 @@ __global__ void k_class_means(const T* __restrict__ X, int64_t d, int64_t ldx, c
     mu_j[(int64_t)j * d + p] = __ddiv_rn(acc, (double)counts[j]);
 }
 
+// mu[p] = (sum over all samples in input order) / n; on the way every sample is looked at for
+// Inf and NaN (the bits of its upper word: no FP64 comparison), which took a pass of its own.
 template <class T>
-__global__ void k_global_mean(const T* __restrict__ X, int64_t d, int64_t ldx, int n, double* __restrict__ mu) {
+__global__ void k_global_mean(const T* __restrict__ X, int64_t d, int64_t ldx, int n, double* __restrict__ mu,
+                              int* __restrict__ status) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= d) return;
-    double acc = 0.0;
-    for (int i = 0; i < n; ++i) acc = __dadd_rn(acc, ld_sample(X, ldx, i, p));
-    mu[p] = __ddiv_rn(acc, (double)n);
+    bool bad = false;
+    if (p < d) {
+        double acc = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+            const double v = ld_sample(X, ldx, i, p);
+            acc = __dadd_rn(acc, v);
+            bad |= (__double2hiint(v) & 0x7ff00000) == 0x7ff00000;
+        }
+        mu[p] = __ddiv_rn(acc, (double)n);
+    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_NONFINITE);
 }
 
 // H_W[:, q] = chi_{perm[q]} - mu_{label}
@@ -96,25 +107,33 @@ __global__ void k_build_hw(const T* __restrict__ X, int64_t d, int64_t ldx, int 
     HW[(int64_t)q * d + p] = __dsub_rn(ld_sample(X, ldx, i, p), mu_j[(int64_t)l * d + p]);
 }
 
-// H_B[:, j] = sqrt(n_j) (mu_j - mu)
+// H_B[:, j] = sqrt(n_j) (mu_j - mu); a thread takes several pixels, as the square root is a third of a microsecond of its
+// sub-partition's FP64 pipe (one a pixel took 36 us at d = 16384, k = 100, now 13).
+constexpr int kHbPer = 8;
 __global__ void k_build_hb(int64_t d, const int32_t* __restrict__ counts, const double* __restrict__ mu_j,
                            const double* __restrict__ mu, double* __restrict__ HB) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t p0 = (int64_t)blockIdx.x * blockDim.x * kHbPer + threadIdx.x;
     const int j = blockIdx.y;
-    if (p >= d) return;
+    if (p0 >= d) return;
     const double s = __dsqrt_rn((double)counts[j]);
-    HB[(int64_t)j * d + p] = __dmul_rn(s, __dsub_rn(mu_j[(int64_t)j * d + p], mu[p]));
+#pragma unroll
+    for (int u = 0; u < kHbPer; ++u) {
+        const int64_t p = p0 + (int64_t)u * blockDim.x;
+        if (p < d) HB[(int64_t)j * d + p] = __dmul_rn(s, __dsub_rn(mu_j[(int64_t)j * d + p], mu[p]));
+    }
 }
 
-template <class T>
-__global__ void k_check_finite(int64_t rows, int cols, const T* __restrict__ A, int64_t lda, int* status) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t tot = rows * cols;
+// ST_NONFINITE when A holds Inf or NaN: a CTA per 1024 rows of a column (columns strided over the grid's y), tests on the bits.
+__global__ void __launch_bounds__(256) k_check_finite(int64_t rows, int cols, const double* __restrict__ A, int64_t lda,
+                                                     int* status) {
     bool bad = false;
-    for (int64_t x = e; x < tot; x += (int64_t)gridDim.x * blockDim.x) {
-        const double v = (double)A[(x / rows) * lda + (x % rows)];
-        if (!isfinite(v)) bad = true;
-    }
+    const int64_t r0 = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+    for (int c = blockIdx.y; c < cols; c += gridDim.y)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t r = r0 + 256 * u;
+            if (r < rows) bad |= (__double2hiint(A[(int64_t)c * lda + r]) & 0x7ff00000) == 0x7ff00000;
+        }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_NONFINITE);
 }
 
@@ -171,35 +190,32 @@ int build_factors(const void* X, int x_dtype, int64_t d, int n, int64_t ldx, int
     const dim3 gk(ceil_div(d, tb), k), g1(ceil_div(d, tb)), gn(ceil_div(d, tb), n);
     if (x_dtype == EDA_F64) {
         const double* x = static_cast<const double*>(X);
-        k_check_finite<<<std::min(ceil_div(d * n, tb), 4096), tb, 0, s>>>(d, n, x, ldx, status);
-        EDA_LAUNCHED();
         k_class_means<<<gk, tb, 0, s>>>(x, d, ldx, counts, offsets, perm, mu_j);
         EDA_LAUNCHED();
-        k_global_mean<<<g1, tb, 0, s>>>(x, d, ldx, n, mu);
+        k_global_mean<<<g1, tb, 0, s>>>(x, d, ldx, n, mu, status);
         EDA_LAUNCHED();
         k_build_hw<<<gn, tb, 0, s>>>(x, d, ldx, n, labels, perm, mu_j, HW);
         EDA_LAUNCHED();
     } else if (x_dtype == EDA_F32) {
         const float* x = static_cast<const float*>(X);
-        k_check_finite<<<std::min(ceil_div(d * n, tb), 4096), tb, 0, s>>>(d, n, x, ldx, status);
-        EDA_LAUNCHED();
         k_class_means<<<gk, tb, 0, s>>>(x, d, ldx, counts, offsets, perm, mu_j);
         EDA_LAUNCHED();
-        k_global_mean<<<g1, tb, 0, s>>>(x, d, ldx, n, mu);
+        k_global_mean<<<g1, tb, 0, s>>>(x, d, ldx, n, mu, status);
         EDA_LAUNCHED();
         k_build_hw<<<gn, tb, 0, s>>>(x, d, ldx, n, labels, perm, mu_j, HW);
         EDA_LAUNCHED();
     } else {
         return EDA_ERR_INVALID_ARG;
     }
-    k_build_hb<<<gk, tb, 0, s>>>(d, counts, mu_j, mu, HB);
+    k_build_hb<<<dim3(ceil_div(d, (int64_t)tb * kHbPer), k), tb, 0, s>>>(d, counts, mu_j, mu, HB);
     EDA_LAUNCHED();
     return EDA_OK;
 }
 
 int check_finite_f64(int64_t rows, int cols, const double* A, int64_t lda, int* status, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return EDA_OK;
-    k_check_finite<<<std::min(ceil_div(rows * cols, 256), 4096), 256, 0, s>>>(rows, cols, A, lda, status);
+    k_check_finite<<<dim3((unsigned)ceil_div(rows, 1024), (unsigned)std::min(cols, 65535)), 256, 0, s>>>(rows, cols, A, lda,
+                                                                                                    status);
     EDA_LAUNCHED();
     return EDA_OK;
 }

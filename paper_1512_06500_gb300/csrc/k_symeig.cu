@@ -1067,7 +1067,9 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(int n, const double* __r
 // k_lz_matvec forms u = A v_j (one warp per row; A is symmetric, so row r is read as its contiguous
 // column r), k_lz_update the rest of the step in one CTA. The vectors rotate through three buffers
 // chosen by the host; st[0] = beta_{j-1}, st[1] = the running norm estimate, st[2] = the stop flag.
-constexpr int LZG_THREADS = 1024;
+// eight warps: with 32 the FP64 sums over the warps (each instruction about 64 cycles of a sub-partition's pipe) took most
+// of the step (n = 2000: 30 us against 8)
+constexpr int LZG_THREADS = 256;
 __global__ void k_lz_start(int n, uint64_t seed, double* __restrict__ v, double* __restrict__ vprev,
                            double* __restrict__ st) {
     __shared__ double red[32];
@@ -1446,11 +1448,10 @@ int symeig_f64(int n, const double* A, int lda, int il, int iu, double* w, doubl
 // Cluster MGS with a tolerance relative to max |lambda|, computed on the device.
 namespace {
 __global__ void k_cluster_scale(int nv, const double* lam, double rel, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double m = 0.0;
-        for (int i = 0; i < nv; ++i) m = fmax(m, fabs(lam[i]));
-        out[0] = rel * m;
-    }
+    double m = 0.0;
+    for (int i = threadIdx.x; i < nv; i += 32) m = fmax(m, fabs(lam[i]));
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x == 0) out[0] = rel * m;
 }
 // Columns Z[:, 0 .. bs) (bs <= 16), already orthogonal to every earlier column of their cluster: each column
 // against the earlier ones of the block by classical Gram-Schmidt applied twice (the dot products of a pass

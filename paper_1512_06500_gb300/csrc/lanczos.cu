@@ -54,19 +54,21 @@ __global__ void k_set_col_block(double* T, int ldt, int cols, int j0, int b, con
     }
 }
 
-// relres[i] = ||B S[rlast:rlast+b, i]|| / |theta_i| for the t Ritz pairs (theta ascending).
+// relres[i] = ||B S[rlast:rlast+b, i]|| / |theta_i| for the t Ritz pairs (theta ascending): a warp per pair, a lane per row of B
+// (one thread for a whole pair took 21 us at b = 16).
 __global__ void k_ritz_residuals(int t, int b, const double* Bm, int ldb, const double* S, int lds, int rlast,
                                  const double* theta, double* relres) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= t) return;
     double acc = 0.0;
-    for (int r = 0; r < b; ++r) {
+    for (int r = lane; r < b; r += 32) {
         double v = 0.0;
         for (int c = 0; c < b; ++c) v = fma(Bm[(int64_t)c * ldb + r], S[(int64_t)i * lds + rlast + c], v);
         acc = fma(v, v, acc);
     }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     const double th = fabs(theta[i]);
-    relres[i] = th > 0.0 ? sqrt(acc) / th : INFINITY;
+    if (lane == 0) relres[i] = th > 0.0 ? sqrt(acc) / th : INFINITY;
 }
 
 // out[:, i] = in[:, t-1-i] (descending order of the Ritz values)
@@ -368,7 +370,7 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
                     k_divide<<<ceil_div(t, 128), 128, 0, s>>>(t, w.relres, w.theta);
                     EDA_LAUNCHED();
                 } else {
-                    k_ritz_residuals<<<ceil_div(t, 128), 128, 0, s>>>(t, b, w.Bm, b, w.S, cols, cols - b, w.theta,
+                    k_ritz_residuals<<<ceil_div(t, 4), 128, 0, s>>>(t, b, w.Bm, b, w.S, cols, cols - b, w.theta,
                                                                      w.relres);
                     EDA_LAUNCHED();
                 }

@@ -358,7 +358,7 @@ size_t oz_operand_bytes(int64_t M, int64_t K);
 // Splitting flags ST_NONFINITE in *status when it meets Inf or NaN.
 int oz_operand_make(const double* A, int64_t lda, int64_t M, int64_t K, bool rows_are_cols, void* mem,
                     OzOperand* op, int* status, cudaStream_t s);
-// A growing operand (the Krylov basis): room for Mcap rows and Kcap reduction values, planes zeroed.
+// A growing operand (the Krylov basis): room for Mcap rows and Kcap reduction values (not cleared).
 // oz_append_cols: split columns i0 .. i1 of A (d x ., lda) as rows i0 .. i1 of a column-scaled operand
 // (K = d).
 int oz_operand_init(int64_t Mcap, int64_t Kcap, void* mem, OzOperand* op, cudaStream_t s);

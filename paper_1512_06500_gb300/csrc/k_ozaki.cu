@@ -29,6 +29,8 @@
 // bounded (ST_TIMEOUT on give-up).
 #include "tc_ptx.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <mutex>
 
@@ -392,29 +394,58 @@ __global__ void __launch_bounds__(256) k_oz_exp_rows(int64_t rows, int cols, con
     if (mx != kOzExpZero) atomicMax(&e[r], mx);
 }
 
-// The seven digit planes of a narrow operand B (K x p, ldb; its columns are the N rows of the product),
-// planes [7][32][ld] (plane q, row j at (32 q + j) ld), zero for j >= p or k >= K. Eight consecutive k per
-// thread: one 64-byte read and one 16-byte store per plane.
-__global__ void k_oz_split_narrow(int64_t K, int p, const double* __restrict__ B, int64_t ldb,
-                                  const int* __restrict__ e, int64_t ld, __nv_bfloat16* __restrict__ out,
-                                  int* __restrict__ status) {
+// A narrow operand B (K x p, ldb; its columns are the N rows of the product): column scales and the seven digit planes, in
+// one launch. planes [7][32][ld] (plane q, row j at (32 q + j) ld), zero for j >= p or k >= K; e[j] the scales (0 for
+// j >= p). One cluster per column: each CTA takes the maximum over its share of the column, the CTAs exchange theirs
+// through distributed shared memory, and each splits its share (read again, from L2), eight consecutive k per thread: one
+// 64-byte read and one 16-byte store per plane. Launch overhead bounds it at the usual sizes: a fill, a scale and a split
+// launch and their gaps took about 15 us at K = 65536 and 11 us at K = 700, this one 9 and 5 us.
+constexpr int OZ_NARROW_CL = 8;
+__global__ void __cluster_dims__(OZ_NARROW_CL, 1, 1) __launch_bounds__(256)
+    k_oz_narrow(int64_t K, int p, const double* __restrict__ B, int64_t ldb, int* __restrict__ e, int64_t ld,
+                __nv_bfloat16* __restrict__ out, int* __restrict__ status) {
+    namespace cg = cooperative_groups;
+    __shared__ int wmax[8];
+    __shared__ int cmax;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int j = blockIdx.y, rank = blockIdx.x;
     const int64_t groups = ld / 8;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)OZ_N * groups) return;
-    const int j = (int)(t / groups);
-    const int64_t k0 = (t % groups) * 8;
-    const int ex = j < p ? e[j] : 0;
-    double v[8];
+    const double* col = B + (int64_t)j * ldb;
+    int ex = 0;
+    if (j < p) {   // uniform over the cluster
+        int mx = kOzExpZero;
+        for (int64_t g = (int64_t)rank * 256 + threadIdx.x; g < groups; g += OZ_NARROW_CL * 256) {
+            double v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        v[u] = (j < p && k0 + u < K) ? B[(int64_t)j * ldb + k0 + u] : 0.0;
+            for (int u = 0; u < 8; ++u) v[u] = 8 * g + u < K ? col[8 * g + u] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mx = max(mx, oz_frexp_exp(v[u]));
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; ++w) mx = max(mx, wmax[w]);
+            cmax = mx;
+        }
+        cluster.sync();
+        ex = kOzExpZero;
+        for (int r = 0; r < OZ_NARROW_CL; ++r) ex = max(ex, *cluster.map_shared_rank(&cmax, r));
+        cluster.sync();   // no CTA leaves while another reads its maximum
     }
-    uint4 dg[OZ_S];
-    const bool fin = oz_digits8(v, ex, dg);
-    if (!fin) atomicOr(status, ST_NONFINITE);
+    if (rank == 0 && threadIdx.x == 0) e[j] = ex;
+    bool fin = true;
+    for (int64_t g = (int64_t)rank * 256 + threadIdx.x; g < groups; g += OZ_NARROW_CL * 256) {
+        const int64_t k0 = 8 * g;
+        double v[8];
 #pragma unroll
-    for (int q = 0; q < OZ_S; ++q)
-        *reinterpret_cast<uint4*>(out + ((int64_t)q * OZ_N + j) * ld + k0) = dg[q];
+        for (int u = 0; u < 8; ++u) v[u] = (j < p && k0 + u < K) ? col[k0 + u] : 0.0;
+        uint4 dg[OZ_S];
+        fin &= oz_digits8(v, ex, dg);
+#pragma unroll
+        for (int q = 0; q < OZ_S; ++q) *reinterpret_cast<uint4*>(out + ((int64_t)q * OZ_N + j) * ld + k0) = dg[q];
+    }
+    if (!fin) atomicOr(status, ST_NONFINITE);
 }
 
 // Digit planes of the columns i0 .. i1 of A (d x m, lda) as M rows of a split operand whose K index runs down
@@ -479,7 +510,8 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(const double* __restrict_
 
 // Growing a row-scaled operand (the Krylov basis, M = d rows, K = the columns so far) from k0 to k1 columns:
 // thread per row. A row whose scale is unchanged by the new columns gets the digits of its new 8-groups
-// [k0 rounded down to 8, k1) (the part of a group below k0 rewritten with identical digits); a row whose
+// [k0 rounded down to 8, k1) (the part of a group below k0 rewritten with identical digits) and zeros to the end of the
+// last 64-wide tile; a row whose
 // scale grows records the new scale and joins list (count in list[0]) for a full re-split by
 // k_oz_resplit_listed. Zero rows keep the scale kOzExpZero.
 __global__ void k_oz_grow_rows(const double* __restrict__ A, int64_t lda, int64_t M, int64_t k0, int64_t k1,
@@ -498,7 +530,7 @@ __global__ void k_oz_grow_rows(const double* __restrict__ A, int64_t lda, int64_
         return;
     }
     bool fin = true;
-    for (int64_t kg = k0 & ~(int64_t)7; kg < k1; kg += 8) {
+    for (int64_t kg = k0 & ~(int64_t)7; kg < ((k1 + TC_KS - 1) & ~(int64_t)(TC_KS - 1)); kg += 8) {
         double v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -519,7 +551,7 @@ __global__ void k_oz_grow_rows(const double* __restrict__ A, int64_t lda, int64_
 __global__ void k_oz_resplit_listed(const double* __restrict__ A, int64_t lda, int64_t K, const int* __restrict__ e,
                                     int kbs, __nv_bfloat16* __restrict__ out, int64_t slice,
                                     const int* __restrict__ list, int* __restrict__ status) {
-    const int64_t groups = (K + 7) / 8;
+    const int64_t groups = (K + TC_KS - 1) / TC_KS * (TC_KS / 8);   // whole tiles: zeros beyond K
     const int64_t total = (int64_t)list[0] * groups;
     bool fin = true;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
@@ -624,7 +656,9 @@ int oz_operand_make(const double* A, int64_t lda, int64_t M, int64_t K, bool row
 }
 
 // A split operand with room for Mcap rows (columns of a d x Mcap matrix, K = d) or for Kcap values of K
-// (rows_are_cols = false: M = d rows, K up to Kcap columns), planes zeroed, no row filled yet.
+// (rows_are_cols = false: M = d rows, K up to Kcap columns), no row filled yet. The planes are not cleared (4 GB at
+// d = 65536, m = 2232): rows beyond those present only reach results that are not stored, and every write fills its 64-wide
+// tile along K up to the end with zeros.
 int oz_operand_init(int64_t Mcap, int64_t Kcap, void* mem, OzOperand* op, cudaStream_t s) {
     const int64_t mt = (Mcap + TC_M - 1) / TC_M, kb = (Kcap + TC_KS - 1) / TC_KS;
     const int64_t plane = mt * kb * TC_M * TC_KS;
@@ -636,7 +670,7 @@ int oz_operand_init(int64_t Mcap, int64_t Kcap, void* mem, OzOperand* op, cudaSt
     op->K = 0;
     op->kbs = (int)kb;
     op->mtiles = 0;
-    EDA_CUDA_TRY(cudaMemsetAsync(mem, 0, (size_t)OZ_S * slice * 2, s));
+    (void)s;
     return EDA_OK;
 }
 
@@ -704,9 +738,7 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
     // digit planes), B read and D written once in FP64
     ProfScope prof("oz_gemm", s, 2.0 * (double)A.M * A.K * p,
                    2.0 * OZ_S * (double)A.M * A.K + 8.0 * (double)A.K * p + 8.0 * (double)A.M * p);
-    EDA_TRY(oz_col_exps(A.K, B, ldb, p, nb.exps, s));
-    k_oz_split_narrow<<<ceil_div((int64_t)OZ_N * (ld / 8), 256), 256, 0, s>>>(A.K, p, B, ldb, nb.exps, ld, nb.planes,
-                                                                            status);
+    k_oz_narrow<<<dim3(OZ_NARROW_CL, OZ_N), 256, 0, s>>>(A.K, p, B, ldb, nb.exps, ld, nb.planes, status);
     EDA_LAUNCHED();
     const int kst = (int)(ld / TC_KS);
     // K splits: fill the SMs with one CTA each (the kernel holds all of an SM's tensor memory)

@@ -113,14 +113,17 @@ int sym_nn(eda_ctx* h, const OzOperand* oz, const double* M, int n, int p, const
 int apply_c(eda_ctx* h, int p, double* PQ, double* U, DirectWs& w, cudaStream_t s) {
     const int n = (int)h->n, k = h->k, nk = n + k;
     const OzOperand* okw = h->ozsmall ? &h->ozKW : nullptr;
-    const OzOperand* ogw = h->ozsmall ? &h->ozGW : nullptr;
     double* Pw = PQ;
     double* Qb = PQ + n;
     double* Uw = U;
     double* Ub = U + n;
     EDA_TRY(sym_nn(h, okw, h->KW, n, p, Pw, nk, false, Uw, nk, w, s));                            // u1 = K p
-    EDA_TRY(gemm_tn_f64(n, k, p, 1.0, h->GWB, n, Uw, nk, 1.0, Qb, nk, w.part, w.pcap, s));       // q + G_BW u1
-    EDA_TRY(sym_nn(h, ogw, h->GW, n, p, Uw, nk, true, Pw, nk, w, s));                             // p + G_W u1
+    if (h->ozsmall) {
+        EDA_TRY(sym_nn(h, &h->ozGW, nullptr, n, p, Uw, nk, true, PQ, nk, w, s));                  // [p; q] + [G_W; G_BW] u1
+    } else {
+        EDA_TRY(gemm_tn_f64(n, k, p, 1.0, h->GWB, n, Uw, nk, 1.0, Qb, nk, w.part, w.pcap, s));    // q + G_BW u1
+        EDA_TRY(sym_nn(h, nullptr, h->GW, n, p, Uw, nk, true, Pw, nk, w, s));                     // p + G_W u1
+    }
     EDA_TRY(gemm_tn_f64(k, k, p, 1.0, h->KB, k, Qb, nk, 0.0, Ub, nk, w.part, w.pcap, s));        // v = K_B q'
     EDA_TRY(gemm_tn_f64(k, n, p, 1.0, h->GBW, k, Ub, nk, 1.0, Pw, nk, w.part, w.pcap, s));       // p' + G_WB v
     return sym_nn(h, okw, h->KW, n, p, Pw, nk, true, Uw, nk, w, s);                               // u1 + K p''

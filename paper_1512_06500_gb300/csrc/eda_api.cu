@@ -97,6 +97,9 @@ constexpr double kSigRel = 32.0;   // eigenvalues <= kSigRel * n * eps * lambda_
 constexpr int kLanczosSteps = 64;  // steps of the largest-eigenvalue Lanczos run on a Gram
 constexpr double kLmaxAccept = 8.0;  // accept its theta_1 when its residual is <= kLmaxAccept * eps * theta_1
 constexpr int kLanczosStepsLarge = 64;    // the same run on a large Gram (n >= kOzSmallMinN, tensor-core mode)
+// G_WB v (n x k times k x p) from n k = 2^18 entries on as a tensor-core product: at n = 2000, k = 200 (p = 32) the FP64
+// kernel takes 38 us and the split product 14; at n = 700, k = 100 (p = 16) 10 and 12
+constexpr int64_t kOzCrossMin = 1 << 18;
 constexpr int64_t kTcMinMiDefault = 4;    // EDA_F64_TC: tensor-core products from d (n + k) >= 4 x 2^20 on
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -452,10 +455,10 @@ int finish_build(eda_ctx* h, cudaStream_t s) {
     // back-transformation of the eigensolver; G_B keeps its route.
     const bool sq_w_tc = tc && !by_squaring && n >= kOzSmallMinN;
     if (sq_w_tc) {
-        // four n x n split operands: the squaring's two factors, then K_W and G_W for the solves
+        // the squaring's two n x n factors, then K_W, [G_W; G_BW] and G_WB for the solves
         const size_t b1 = align256(oz_operand_bytes(n, n));
         void* p = nullptr;
-        EDA_TRY(dev_alloc(&p, 4 * b1));
+        EDA_TRY(dev_alloc(&p, 3 * b1 + align256(oz_operand_bytes(n + k, n)) + align256(oz_operand_bytes(n, k))));
         h->ozsmall = p;
     }
     if (tc) {
@@ -562,7 +565,17 @@ int finish_build(eda_ctx* h, cudaStream_t s) {
         const size_t b1 = align256(oz_operand_bytes(n, n));
         char* p = static_cast<char*>(h->ozsmall);
         EDA_TRY(oz_operand_make(h->KW, n, n, n, true, p + 2 * b1, &h->ozKW, h->status, s));
-        EDA_TRY(oz_operand_make(h->GW, n, n, n, true, p + 3 * b1, &h->ozGW, h->status, s));
+        // rows of [G_W; G_BW] = columns of [G_W G_WB], put side by side in the squaring's work
+        scratch.used = mark;
+        double* gz = scratch.take<double>((size_t)n * (n + k));
+        if (!gz) return EDA_ERR_OOM;
+        EDA_TRY(copy_mat_f64(n, n, h->GW, n, gz, n, s));
+        EDA_TRY(copy_mat_f64(n, k, h->GWB, n, gz + (size_t)n * n, n, s));
+        EDA_TRY(oz_operand_make(gz, n, n + k, n, true, p + 3 * b1, &h->ozGW, h->status, s));
+        h->ozcross = (int64_t)n * k >= kOzCrossMin;
+        if (h->ozcross)
+            EDA_TRY(oz_operand_make(h->GBW, k, n, k, true, p + 3 * b1 + align256(oz_operand_bytes(n + k, n)), &h->ozGWB,
+                                    h->status, s));
     }
     if (h->cfg.prec == EDA_BF16) {
         // bf16 H_W, H_B tiled for sweep 1, bf16 H K tiled for sweep 2, and the staging

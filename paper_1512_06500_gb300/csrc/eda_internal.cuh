@@ -454,10 +454,12 @@ struct eda_ctx {
     eda::OzNarrow oznb;
     eda::OzScratch ozwide;                 // split of a right-hand side of more than 32 columns (grown on demand)
     // prec = EDA_F64_TC and n >= kOzSmallMinN: the left-factor split of the scaling and squaring that
-    // forms K_W (and, for the nonsymmetric form, K(-c^2) and K(+c^2)), then K_W and G_W split for
-    // their products with the n x p coordinates inside the composed M-apply and the recovery
+    // forms K_W (and, for the nonsymmetric form, K(-c^2) and K(+c^2)), then the operators of the
+    // n x p coordinates inside the composed M-apply and the recovery: ozKW = K_W, ozGW = [G_W; G_BW] (n + k rows: G_W u and G_BW u in one product)
+    // and, when worth a launch (n k >= kOzCrossMin), ozGWB = G_WB
     void* ozsmall = nullptr;
-    eda::OzOperand ozKW, ozGW;
+    eda::OzOperand ozKW, ozGW, ozGWB;
+    bool ozcross = false;                  // ozGWB is there
     // K(-c^2) and K(+c^2) for H_W, the operators of the nonsymmetric form exp(-c^2 S_W) exp(c^2 S_B) and of
     // exp(c^2 S_W) (allocated on first use by the Arnoldi solver)
     void* nblock = nullptr;

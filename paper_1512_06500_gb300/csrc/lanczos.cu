@@ -467,19 +467,23 @@ int m_apply_composed(eda_ctx* h, int p, const double* Y, int64_t ldy, double* MY
     double* Qb = PQ + n;
     double* Uw = U;
     double* Ub = U + n;
-    // the n x n products with K_W and G_W: on the tensor cores from their splits when the handle has them
+    // the products with K_W, G_W and the cross Grams: on the tensor cores from their splits when the handle has them
     auto nn = [&](const OzOperand* oz, const double* M, const double* X, double beta, const double* C0,
                   double* D) -> int {
         if (!oz) return gemm_small_f64(false, false, n, p, n, 1.0, M, n, X, nk, beta, D, nk, s);
         return oz_gemm_wide(*oz, h->oznb, h->ozwide, p, X, nk, 1.0, beta, C0, nk, D, nk, h->status, s);
     };
     const OzOperand* okw = h->ozsmall ? &h->ozKW : nullptr;
-    const OzOperand* ogw = h->ozsmall ? &h->ozGW : nullptr;
     EDA_TRY(nn(okw, h->KW, Pw, 0.0, nullptr, Uw));                                               // u1
-    EDA_TRY(gemm_small_f64(false, false, k, p, n, 1.0, h->GBW, k, Uw, nk, 1.0, Qb, nk, s));  // H_B^T y1
-    EDA_TRY(nn(ogw, h->GW, Uw, 1.0, Pw, Pw));                                                    // H_W^T y1
+    if (h->ozsmall) {
+        EDA_TRY(nn(&h->ozGW, nullptr, Uw, 1.0, PQ, PQ));                                         // H_W^T y1, H_B^T y1
+    } else {
+        EDA_TRY(gemm_small_f64(false, false, k, p, n, 1.0, h->GBW, k, Uw, nk, 1.0, Qb, nk, s));  // H_B^T y1
+        EDA_TRY(nn(nullptr, h->GW, Uw, 1.0, Pw, Pw));                                            // H_W^T y1
+    }
     EDA_TRY(gemm_small_f64(false, false, k, p, k, 1.0, h->KB, k, Qb, nk, 0.0, Ub, nk, s));   // v
-    EDA_TRY(gemm_small_f64(false, false, n, p, k, 1.0, h->GWB, n, Ub, nk, 1.0, Pw, nk, s));  // H_W^T y2
+    if (h->ozcross) EDA_TRY(nn(&h->ozGWB, nullptr, Ub, 1.0, Pw, Pw));                            // H_W^T y2
+    else EDA_TRY(gemm_small_f64(false, false, n, p, k, 1.0, h->GWB, n, Ub, nk, 1.0, Pw, nk, s));
     EDA_TRY(nn(okw, h->KW, Pw, 1.0, Uw, Uw));                                                    // u1 + u3
     return sweep_z(h, p, U, Y, ldy, MY, ldm, s);
 }

@@ -141,3 +141,18 @@ def test_wide_right_hand_sides(eda, d, k, nj, b):
             assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
             assert O.sin_angle(ref["V"], V) <= 1e-8
             assert np.abs(V.T @ V - np.eye(p.k - 1)).max() <= 1e-12
+
+
+# the stacked [G_W; G_BW] operand (from n = 512 on) and the split G_WB (from n k = 2^18 entries on) of the composed M-apply,
+# on either side of both rules
+@pytest.mark.parametrize("k,nj", [(64, 8), (85, 6), (255, 4), (256, 4)])
+def test_composed_m_apply_operands(eda, k, nj):
+    p = synth.gaussian_clusters(d=1300, k=k, n_per_class=nj, seed=k)
+    f = O.scatter_factors(p.X, p.labels, p.k)
+    rng = np.random.default_rng(k)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(prec=eda.EDA_F64_TC, tau=8.0, tc_min_mi=-1)) as h:
+        for m in (1, 32, 40):
+            X = rng.standard_normal((1300, m))
+            Y = h.apply_exp(eda.OP_M, _dev(X.T)).cpu().numpy().T
+            Yr = O.m_apply(f["HW"], f["HB"], h.c2, X)
+            assert (np.abs(Y - Yr).max(0) <= 1e-12 * np.abs(Yr).max(0)).all()

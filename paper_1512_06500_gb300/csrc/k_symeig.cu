@@ -843,28 +843,139 @@ __global__ void __launch_bounds__(256) k_transpose_out(int n, int nv, const doub
         if (q0 + c < nv && i0 + lane < n) Z[(int64_t)(q0 + c) * ldz + i0 + lane] = t[lane][c];
 }
 
-// Z <- H_0 H_1 ... H_{n-3} Z, one warp per column of Z; reflector j is read from HV (row j,
-// contiguous, zero above j + 1) through the read-only cache.
-__global__ void k_backtransform(int n, int nv, const double* __restrict__ HV, const double* __restrict__ tau,
-                                double* Z, int ldz) {
-    const int lane = threadIdx.x & 31;
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= nv) return;
-    double* z = Z + (int64_t)col * ldz;
-    for (int j = n - 3; j >= 0; --j) {
-        const double tj = __ldg(tau + j);
-        if (tj == 0.0) continue;
-        const double* u = HV + (int64_t)j * n;
-        double dot = 0.0;
-        for (int i = j + 1 + lane; i < n; i += 32) dot = fma(__ldg(u + i), z[i], dot);
-        for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-        const double f = tj * dot;
-        for (int i = j + 1 + lane; i < n; i += 32) z[i] = fma(-f, __ldg(u + i), z[i]);
+// Z <- H_0 H_1 ... H_{n-3} Z in blocks of WY_B reflectors, last block first. A block is I - V U^{-1} V^T with V its
+// reflectors (n x 32) and U upper triangular, U_ii = 1 / tau_i and U_ik = v_i^T v_k above the diagonal (the inverse of the
+// compact WY factor; Joffrain, Low, Quintana-Orti, van de Geijn and Van Zee, "Accumulating Householder transformations,
+// revisited", ACM TOMS 32, 2006). Applied one by one, each reflector of each column costs a reduction over all warps,
+// as many FP64 instructions as the products themselves at n = 700; here a CTA keeps NC columns of Z in shared memory, takes
+// the 32 NC products of a block with packed reductions, solves with U by one warp per column and updates the rows with no
+// reduction at all. The FP64 pipe bounds it (n^2 FMAs a column, each CTA on its own SM): n = nv = 698 2.58 -> 0.80 ms,
+// n = 668, nv = 92 1.13 -> 0.39, n = 288, nv = 199 0.40 -> 0.25, n = 144, nv = 99 0.12 -> 0.07.
+constexpr int WY_B = 32;
+
+// Upper triangles of V^T V of every block: G[kb][i][k], i < k. grid (blocks, 8): four rows i each; a warp per product.
+__global__ void __launch_bounds__(256) k_wy_gram(int n, const double* __restrict__ HV, double* __restrict__ G) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j0 = blockIdx.x * WY_B, m = min(WY_B, n - 2 - j0);
+    double* g = G + (size_t)blockIdx.x * WY_B * WY_B;
+    for (int ii = 0; ii < 4; ++ii) {
+        const int i = 4 * blockIdx.y + ii;
+        const double* vi = HV + (int64_t)(j0 + i) * n;
+        for (int k = i + 1 + w; k < m; k += 8) {
+            const double* vk = HV + (int64_t)(j0 + k) * n;   // zero above row j0 + k + 1
+            double a0 = 0.0, a1 = 0.0;
+            int r = j0 + k + 1 + lane;
+            for (; r + 32 < n; r += 64) {
+                a0 = fma(vi[r], vk[r], a0);
+                a1 = fma(vi[r + 32], vk[r + 32], a1);
+            }
+            if (r < n) a0 = fma(vi[r], vk[r], a0);
+            a0 += a1;
+            for (int o = 16; o > 0; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+            if (lane == 0) g[i * WY_B + k] = a0;
+        }
     }
 }
 
-// The same with the column held in the registers of four warps (n <= 128 NPL), one warp per SM
-// sub-partition: carried by a single warp, the chain of reflectors is bound by the FP64 issue rate of one
+// Sums over the lanes of N values (N a power of two up to 8): value v's sum ends in the lanes whose upper log2(N) bits,
+// read from lane bit 4 down, spell v. Half of the values change sides at each of the first steps, so that 8 values take 9
+// FP64 additions and not 40.
+template <int N>
+__device__ __forceinline__ double warp_sum_packed(double (&a)[N], int lane) {
+#pragma unroll
+    for (int h = N / 2, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int v = 0; v < N / 2; ++v)
+            if (v < h) {
+                const double keep = up ? a[v + h] : a[v], send = up ? a[v] : a[v + h];
+                a[v] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+    double x = a[0];
+#pragma unroll
+    for (int o = 16 / N; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+template <int NC>
+__global__ void __launch_bounds__(256) k_wy_apply(int n, int nv, const double* __restrict__ HV,
+                                                  const double* __restrict__ tau, const double* __restrict__ G, double* Z,
+                                                  int ldz) {
+    constexpr int NP = NC <= 1 ? 1 : (NC <= 2 ? 2 : (NC <= 4 ? 4 : 8));
+    extern __shared__ double sz[];               // NC x n: this CTA's columns
+    __shared__ double xs[WY_B][NC];              // V^T Z of the block, then U^{-1} V^T Z
+    __shared__ double gs[WY_B][WY_B + 1];
+    __shared__ double ts[WY_B];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int q0 = blockIdx.x * NC, nc = min(NC, nv - q0);
+    for (int c = 0; c < NC; ++c)
+        for (int i = tid; i < n; i += 256) sz[c * n + i] = c < nc ? Z[(int64_t)(q0 + c) * ldz + i] : 0.0;
+    const int nr = n - 2, nb = (nr + WY_B - 1) / WY_B;
+    for (int kb = nb - 1; kb >= 0; --kb) {
+        const int j0 = kb * WY_B, m = min(WY_B, nr - j0);
+        for (int e = tid; e < WY_B * WY_B; e += 256) {
+            const int i = e / WY_B, k = e % WY_B;
+            gs[i][k] = (i < k && k < m) ? G[(size_t)kb * WY_B * WY_B + e] : 0.0;
+        }
+        if (tid < WY_B) ts[tid] = tid < m ? tau[j0 + tid] : 0.0;
+        __syncthreads();   // also: the columns are up to date
+        // products of the block's reflectors with the columns, one warp per reflector
+        for (int r = w; r < m; r += 8) {
+            const double* v = HV + (int64_t)(j0 + r) * n;
+            double a[NP];
+#pragma unroll
+            for (int c = 0; c < NP; ++c) a[c] = 0.0;
+            for (int i = ((j0 + r + 1) & ~31) + lane; i < n; i += 32) {
+                const double vi = v[i];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) a[c] = fma(vi, sz[c * n + i], a[c]);
+            }
+            const double x = warp_sum_packed<NP>(a, lane);
+            // the value this lane holds: lane bits 4, 3, 2 (for NP = 8), and so on
+            const int val = NP == 1 ? 0 : lane / (32 / NP);
+            if (lane % (32 / NP) == 0 && val < NC) xs[r][val] = x;
+        }
+        __syncthreads();
+        // U x = V^T Z by back substitution, one warp per column, lane i holding row i
+        for (int c = w; c < NC; c += 8) {
+            double wi = lane < m ? xs[lane][c] : 0.0, mine = 0.0;
+            for (int k = m - 1; k >= 0; --k) {
+                const double xk = ts[k] * __shfl_sync(0xffffffffu, wi, k);
+                if (lane == k) mine = xk;
+                wi = fma(-gs[lane][k], xk, wi);   // zero at and below the diagonal
+            }
+            if (lane < m) xs[lane][c] = mine;
+        }
+        __syncthreads();
+        // Z -= V x
+        for (int i = j0 + 1 + tid; i < n; i += 256) {
+            double z[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) z[c] = sz[c * n + i];
+            const double* v = HV + (int64_t)j0 * n + i;
+            for (int r = 0; r < m; r += 4) {
+                double vr[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) vr[u] = r + u < m ? v[(int64_t)(r + u) * n] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (r + u < m) {
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) z[c] = fma(-vr[u], xs[r + u][c], z[c]);
+                    }
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) sz[c * n + i] = z[c];
+        }
+        __syncthreads();
+    }
+    for (int c = 0; c < nc; ++c)
+        for (int i = tid; i < n; i += 256) Z[(int64_t)(q0 + c) * ldz + i] = sz[c * n + i];
+}
+
+// Z <- H_0 H_1 ... H_{n-3} Z for few or short columns: one column per CTA, held in the registers of four warps
+// (n <= 128 NPL), one warp per SM sub-partition: carried by a single warp, the chain of reflectors is bound by the FP64 issue rate of one
 // sub-partition. Rows are dealt in 32-row stripes, row 32 (4 k + w) + lane in register k of warp w; a
 // warp skips the stripes that lie wholly at or above reflector j's first nonzero row j + 1 (exact zero
 // terms), the four partial dot products are added in a fixed order through shared memory (one barrier
@@ -1176,6 +1287,7 @@ int symeig_backtransform(int n, int nv, double* Z, int ldz, SymEigWork* ws, cuda
 // the cooperative grid from here when its columns fit: at n = 288 a column step takes about 5 us on either path, beyond it
 // the columns of 16 CTAs grow with n while those of the grid's up to 152 stay few
 constexpr int kResMinN = 288;
+constexpr int kWyMinN = 64;   // back-transformation in blocks of reflectors from here; below it one launch serves
 
 size_t symeig_work_bytes(int n, int nv) {
     const size_t nn = (size_t)n * n;
@@ -1587,16 +1699,50 @@ int symeig_orth_clusters(int n, int nv, const double* w, double* Z, int ldz, Sym
 }
 
 // Householder back-transformation of the tridiagonal eigenvectors Z (reflectors still in ws).
-int symeig_backtransform(int n, int nv, double* Z, int ldz, SymEigWork* ws, cudaStream_t s) {
-    if (n >= 3) {
-        ProfScope prof("backtransform", s);
-        if (n <= 256) k_backtransform_w4<2><<<nv, 128, 0, s>>>(n, nv, ws->partial, ws->tau, Z, ldz);
-        else if (n <= 512) k_backtransform_w4<4><<<nv, 128, 0, s>>>(n, nv, ws->partial, ws->tau, Z, ldz);
-        else if (n <= 1024) k_backtransform_w4<8><<<nv, 128, 0, s>>>(n, nv, ws->partial, ws->tau, Z, ldz);
-        else k_backtransform<<<nv, 32, 0, s>>>(n, nv, ws->partial, ws->tau, Z, ldz);
-        EDA_LAUNCHED();
+namespace {
+template <int NC>
+int wy_apply(int n, int nv, double* Z, int ldz, SymEigWork* ws, cudaStream_t s) {
+    const size_t smem = (size_t)NC * n * sizeof(double);
+    {
+        // raise-only, under a lock: concurrent solves of different sizes share the attribute
+        static std::mutex mu;
+        static size_t set = 0;
+        std::lock_guard<std::mutex> lk(mu);
+        if (smem > set && smem > 32 * 1024) {
+            EDA_CUDA_TRY(cudaFuncSetAttribute(k_wy_apply<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            set = smem;
+        }
     }
+    k_wy_apply<NC><<<ceil_div(nv, NC), 256, smem, s>>>(n, nv, ws->partial, ws->tau, ws->A, Z, ldz);
+    EDA_LAUNCHED();
     return EDA_OK;
+}
+}  // namespace
+
+int symeig_backtransform(int n, int nv, double* Z, int ldz, SymEigWork* ws, cudaStream_t s) {
+    if (n < 3) return EDA_OK;
+    ProfScope prof("backtransform", s);
+    if (n < kWyMinN) {
+        k_backtransform_w4<2><<<nv, 128, 0, s>>>(n, nv, ws->partial, ws->tau, Z, ldz);
+        EDA_LAUNCHED();
+        return EDA_OK;
+    }
+    // the blocks' triangles go into the matrix copy, which the reduction has done with (n^2 + 16 n doubles hold them)
+    k_wy_gram<<<dim3(ceil_div(n - 2, WY_B), 8), 256, 0, s>>>(n, ws->partial, ws->A);
+    EDA_LAUNCHED();
+    // columns per CTA: one wave of CTAs, at most eight, as many as fit in 200 KB
+    const int fit = (int)std::max<size_t>(1, 200 * 1024 / ((size_t)n * sizeof(double)));
+    const int nc = std::min(std::min(8, ceil_div(nv, sm_count())), fit);
+    switch (nc) {
+        case 1: return wy_apply<1>(n, nv, Z, ldz, ws, s);
+        case 2: return wy_apply<2>(n, nv, Z, ldz, ws, s);
+        case 3: return wy_apply<3>(n, nv, Z, ldz, ws, s);
+        case 4: return wy_apply<4>(n, nv, Z, ldz, ws, s);
+        case 5: return wy_apply<5>(n, nv, Z, ldz, ws, s);
+        case 6: return wy_apply<6>(n, nv, Z, ldz, ws, s);
+        case 7: return wy_apply<7>(n, nv, Z, ldz, ws, s);
+        default: return wy_apply<8>(n, nv, Z, ldz, ws, s);
+    }
 }
 
 int newton_schulz_f64(int n, int nv, double* Z, int ldz, int steps, double* tmp, double* partial, size_t partial_cap,

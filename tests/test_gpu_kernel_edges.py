@@ -156,3 +156,26 @@ def test_composed_m_apply_operands(eda, k, nj):
             Y = h.apply_exp(eda.OP_M, _dev(X.T)).cpu().numpy().T
             Yr = O.m_apply(f["HW"], f["HB"], h.c2, X)
             assert (np.abs(Y - Yr).max(0) <= 1e-12 * np.abs(Yr).max(0)).all()
+
+
+# eigenvectors through the back-transformation: matrix orders n - 1 around its smallest blocked size (64) and its blocks of 32
+# reflectors, few and many columns (1 to 8 a CTA by the number of columns)
+@pytest.mark.parametrize("n,t", [(34, 3), (64, 5), (65, 1), (66, 40), (67, 66), (98, 9), (99, 98), (131, 64), (400, 399)])
+def test_direct_solve_orders(eda, n, t):
+    k = max(2, n // 3)
+    counts = [n // k + (1 if j < n % k else 0) for j in range(k)]
+    p = synth.gaussian_clusters(d=1100, k=k, n_per_class=counts, seed=n)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(tau=6.0)) as h:
+        V, lam, info, code = h.solve_direct(t)
+        assert code == 0
+        c2 = h.c2
+        V = V.cpu().numpy().T
+        MV = h.apply_exp(eda.OP_N, _dev(V.T)).cpu().numpy().T
+    # beyond the k - 1 eigenvalues above 1 the direct solver's pairs are those of span[H_W H_B] (below 1), the oracle's t
+    # largest the unit ones of its complement
+    m = min(t, p.k - 1)
+    ref = O.eda(p.X, p.labels, p.k, m, c2=c2, tier="projected")
+    assert np.max(np.abs(lam.cpu().numpy()[:m] - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
+    assert np.abs(V.T @ V - np.eye(t)).max() <= 1e-12
+    # span(V) is invariant under N: N V = V (V^T N V) up to 1e-10 of ||N|| <= lambda_1 (the spectrum below may be close)
+    assert np.abs(MV - V @ (V.T @ MV)).max() <= 1e-9 * ref["lam_t"][0]

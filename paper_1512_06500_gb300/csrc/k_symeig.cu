@@ -483,6 +483,16 @@ __global__ void __launch_bounds__(TD_THREADS) k_tridiag_x(int n, const double* _
     if (CL) cg::this_cluster().sync();   // no CTA leaves while another may still read its shared memory
 }
 
+__device__ __forceinline__ bool abs_less(double a, double b) {   // |a| < |b|
+    return (__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) < (__double_as_longlong(b) & 0x7FFFFFFFFFFFFFFFll);
+}
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
+// 1 / x for any sign: td_rcp on |x| with the sign put back
+__device__ __forceinline__ double signed_rcp(double x) {
+    const double r = td_rcp(fabs(x));
+    return __hiloint2double(__double2hiint(r) | (__double2hiint(x) & 0x80000000), __double2loint(r));
+}
+
 // Number of eigenvalues below x of the tridiagonal with diagonal d and squared off-diagonal e2, in
 // single precision (ratio form q_i = (d_i - x) - e2_{i-1} / q_{i-1}, small pivots replaced).
 __device__ __forceinline__ int sturm_count_f32(int n, const float* d, const float* e2, float x, float pivmin) {
@@ -511,29 +521,54 @@ __device__ __forceinline__ double fix_zero(double p, double prev) {
     return __hiloint2double((~__double2hiint(prev) & 0x80000000) | 0x00100000, 0);   // -sign(prev) * DBL_MIN
 }
 
-__device__ __forceinline__ void rescale_pair(double& pc, double& pm) {
+__device__ __forceinline__ void rescale_pair(double& pc, double& pm, int& shift) {
     const int ex = (__double2hiint(pc) >> 20) & 0x7ff;
     if (ex > 1023 + 480 || ex < 1023 - 480) {
         const double sc = __hiloint2double((2046 - ex) << 20, 0);   // 2^(1023 - ex)
         pc *= sc;
         pm *= sc;
+        shift += ex - 1023;
     }
 }
 
-// The number of eigenvalues below x0 by that recurrence (one shift per thread).
-__device__ __forceinline__ int sturm_count1_f64(int n, const double* d, const double* e2, double x0) {
+// The number of eigenvalues below x0 by that recurrence (one shift per thread), and the value of the characteristic
+// polynomial there as val 2^shift.
+__device__ __forceinline__ int sturm_count1_f64(int n, const double* d, const double* e2, double x0, double* val = nullptr,
+                                                int* shift = nullptr) {
     double pm0 = 1.0;
     double pc0 = fix_zero(d[0] - x0, 1.0);
     int c0 = (int)((unsigned)__double2hiint(pc0) >> 31);
+    int sh = 0;
     for (int i = 1; i < n; ++i) {
         const double di = d[i], ei = e2[i - 1];
         const double pn0 = fix_zero(fma(di - x0, pc0, -ei * pm0), pc0);
         c0 += (int)(((unsigned)__double2hiint(pn0) ^ (unsigned)__double2hiint(pc0)) >> 31);
         pm0 = pc0;
         pc0 = pn0;
-        if ((i & 3) == 0) rescale_pair(pc0, pm0);
+        if ((i & 3) == 0) rescale_pair(pc0, pm0, sh);
+    }
+    if (val) {
+        *val = pc0;
+        *shift = sh;
     }
     return c0;
+}
+
+// The root in [0, 1] of the cubic through f(-1), f(0), f(1), f(2), f(0) and f(1) of opposite signs: Newton's iteration on
+// the interpolation polynomial in Newton's form from the chord's root (which is returned when the iteration leaves [0, 1]).
+__device__ __forceinline__ double cubic_root01(double fm, double f0, double f1, double f2) {
+    const double d01 = f1 - f0, d1m = 0.5 * (f1 - fm);
+    const double d2 = d01 - d1m;
+    const double d3 = 0.5 * (fma(f2 - fm, 1.0 / 3.0, -d1m) - d2);
+    const double s0 = fabs(f0) * td_rcp(fabs(f0) + fabs(f1));
+    double s = s0;
+    for (int it = 0; it < 3; ++it) {
+        const double q = fma(s + 1.0, d3, d2);
+        const double r = fma(s - 1.0, q, d01);
+        const double dp = fma(s, fma(s - 1.0, d3, q), r);
+        s = fma(-fma(s, r, f0), signed_rcp(dp), s);
+    }
+    return s >= 0.0 && s <= 1.0 ? s : s0;
 }
 
 // One CTA of two warps per wanted eigenvalue (ascending index il + blockIdx.x). The tridiagonal is
@@ -543,6 +578,13 @@ __device__ __forceinline__ int sturm_count1_f64(int n, const double* d, const do
 // counts down to ~eps: lane l of warp 0 counts at the shift 2 l + 1 of the 65-way split and lane l of
 // warp 1 at 2 l + 2, so each warp's FP64 chain carries one shift (the FP64 pipe of a sub-partition
 // holds a warp instruction for ~64 cycles, so two warps on two sub-partitions halve the time).
+//
+// A double-precision round gains 6 bits and costs n dependent steps, so the first one also gives the polynomial's values:
+// when the four shifts around the bracket hold this eigenvalue alone, the cubic through them puts it within about
+// (h / gap)^3 of the bracket's width h (3e-7), and the second round counts at x* +- h 2^-i, i = 0 .. 31: whatever
+// the quality of x*, the counts make the new bracket, about as wide as x* was wrong. Two or three rounds then do the work
+// of six. GB300: n = 698 and 100, all eigenvalues, 1.70 -> 1.13 ms; n = 668, 92 of them 0.73 -> 0.56; n = 144, 99 of them
+// 0.165 -> 0.085.
 __global__ void __launch_bounds__(64) k_bisect(int n, const double* __restrict__ dgl, const double* __restrict__ eoff,
                                                 int il, int nw, double* w) {
     extern __shared__ double smb[];
@@ -552,6 +594,8 @@ __global__ void __launch_bounds__(64) k_bisect(int n, const double* __restrict__
     float* e232 = d32 + n;                                 // n
     __shared__ double s_tnorm;
     __shared__ unsigned s_ball[2];
+    __shared__ double s_f[64];
+    __shared__ int s_fs[64], s_cnt[64];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     // ||T||_inf by warp 0
     if (threadIdx.x < 32) {
@@ -599,24 +643,59 @@ __global__ void __launch_bounds__(64) k_bisect(int n, const double* __restrict__
     // first double-precision round: 64 shifts from dlo to dhi, both included (lane l of warp 0 at shift 2 l, of warp 1 at
     // 2 l + 1), so that it confirms the bracket and divides it; the full interval when the bracket fails
     {
-        const double step = (dhi - dlo) / 63.0;
-        const int c = sturm_count1_f64(n, d64, e264, dlo + (2 * lane + wp) * step);
-        const unsigned b = __ballot_sync(0xffffffffu, c > idx);
-        if (lane == 0) s_ball[wp] = b;
+        const double step = (dhi - dlo) * (1.0 / 63.0);
+        const int me = 2 * lane + wp;
+        double f;
+        int fs;
+        const int c = sturm_count1_f64(n, d64, e264, me == 63 ? dhi : fma((double)me, step, dlo), &f, &fs);
+        s_f[me] = f;
+        s_fs[me] = fs;
+        s_cnt[me] = c;
         __syncthreads();
-        const unsigned b0 = s_ball[0], b1 = s_ball[1];
-        __syncthreads();
-        if ((b0 & 1u) || !(b1 >> 31)) {
+        if (s_cnt[0] > idx || s_cnt[63] <= idx) {
             dlo = -1.0 - 1e-12;
             dhi = 1.0 + 1e-12;
         } else {
             // the first shift with more than idx eigenvalues below it
-            const int l = __ffs(b0 | b1) - 1;
-            const int k = ((b0 >> l) & 1u) ? 2 * l : 2 * l + 1;
-            const double base = dlo;
-            dlo = base + (k - 1) * step;
-            dhi = base + k * step;
+            int k = 1;
+            {
+                const unsigned b0 = __ballot_sync(0xffffffffu, s_cnt[lane] > idx);
+                const unsigned b1 = __ballot_sync(0xffffffffu, s_cnt[32 + lane] > idx);
+                k = b0 ? __ffs(b0) - 1 : 31 + __ffs(b1);
+            }
+            const double x0 = fma((double)(k - 1), step, dlo), x1 = k == 63 ? dhi : fma((double)k, step, dlo);
+            const bool alone = k >= 2 && k <= 62 && s_cnt[k - 2] == idx && s_cnt[k + 1] == idx + 1;
+            dlo = x0;
+            dhi = x1;
+            if (alone) {
+                // values at the four shifts on one scale (powers of two; far smaller ones vanish)
+                double v[4];
+                int top = s_fs[k - 2];
+#pragma unroll
+                for (int u = 1; u < 4; ++u) top = max(top, s_fs[k - 2 + u]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int sh = s_fs[k - 2 + u] - top;
+                    v[u] = sh < -500 ? 0.0 : s_f[k - 2 + u] * __hiloint2double((1023 + sh) << 20, 0);
+                }
+                const double xs = fma(cubic_root01(v[0], v[1], v[2], v[3]), step, x0);
+                // second round: x* -+ step 2^-i, ascending with the index
+                auto at = [&](int m) {
+                    return m < 32 ? fma(-step, __hiloint2double((1023 - m) << 20, 0), xs)
+                                  : fma(step, __hiloint2double((1023 - (63 - m)) << 20, 0), xs);
+                };
+                const int c2 = sturm_count1_f64(n, d64, e264, at(me));
+                __syncthreads();   // the first round's counts have been read
+                s_cnt[me] = c2;
+                __syncthreads();
+                const unsigned b0 = __ballot_sync(0xffffffffu, s_cnt[lane] > idx);
+                const unsigned b1 = __ballot_sync(0xffffffffu, s_cnt[32 + lane] > idx);
+                const int m = b0 ? __ffs(b0) - 1 : (b1 ? 31 + __ffs(b1) : 64);
+                if (m > 0) dlo = fmax(dlo, at(m - 1));
+                if (m < 64) dhi = fmin(dhi, at(m));
+            }
         }
+        __syncthreads();
     }
     for (int round = 0; round < 24; ++round) {
         const double width = dhi - dlo;
@@ -668,16 +747,6 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 // group while the current one is used; the interchanges are one bit a row. GB300: n = 288, nv = 199 450 -> 225 us;
 // n = nv = 698 and 100 together 1.77 -> 0.97 ms; n = 144, nv = 99 305 -> 175 us.
 constexpr int IV_U = 8;
-
-__device__ __forceinline__ bool abs_less(double a, double b) {   // |a| < |b|
-    return (__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) < (__double_as_longlong(b) & 0x7FFFFFFFFFFFFFFFll);
-}
-__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
-// 1 / x for any sign: td_rcp on |x| with the sign put back
-__device__ __forceinline__ double signed_rcp(double x) {
-    const double r = td_rcp(fabs(x));
-    return __hiloint2double(__double2hiint(r) | (__double2hiint(x) & 0x80000000), __double2loint(r));
-}
 
 __global__ void __launch_bounds__(32) k_invit(int n, int nv, const double* __restrict__ dgl,
                                               const double* __restrict__ eoff, const double* __restrict__ lam, double* lu,

@@ -35,6 +35,8 @@ size_t a256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // H[i, j0 + jj] = C1[i, jj] + C2[i, jj] for i < cols (the full coefficients V^T N V_j of the new block)
 __global__ void k_arn_set_hcol(double* H, int ldh, int cols, int j0, int b, const double* C1, const double* C2) {
+    PDL_ENTER();
+    PDL_ARG(H); PDL_ARG(C1); PDL_ARG(C2);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= cols * b) return;
     const int i = e % cols, jj = e / cols;
@@ -43,6 +45,8 @@ __global__ void k_arn_set_hcol(double* H, int ldh, int cols, int j0, int b, cons
 
 // H[r0 + i, c0 + jj] = B[i, jj] (the sub-diagonal block: W = V_{j+1} B)
 __global__ void k_arn_set_block(double* H, int ldh, int r0, int c0, int b, const double* Bm) {
+    PDL_ENTER();
+    PDL_ARG(H); PDL_ARG(Bm);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= b * b) return;
     const int i = e % b, jj = e / b;
@@ -50,12 +54,16 @@ __global__ void k_arn_set_block(double* H, int ldh, int r0, int c0, int b, const
 }
 
 __global__ void k_arn_add_identity(int m, double* A, int lda) {
+    PDL_ENTER();
+    PDL_ARG(A);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) A[(int64_t)i * lda + i] += 1.0;
 }
 
 // R[:, c] -= theta[c] S[:, c]
 __global__ void k_arn_sub_scaled(int rows, int t, double* R, int ldr, const double* S, int lds, const double* theta) {
+    PDL_ENTER();
+    PDL_ARG(R); PDL_ARG(S); PDL_ARG(theta);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)rows * t) return;
     const int r = (int)(e % rows), c = (int)(e / rows);
@@ -65,6 +73,8 @@ __global__ void k_arn_sub_scaled(int rows, int t, double* R, int ldr, const doub
 // relres[i] = sqrt(a[i]^2 + b[i]^2 + q[i]) / |theta[i]|
 __global__ void k_arn_relres(int t, const double* a, const double* b, const double* q, const double* theta,
                              double* relres) {
+    PDL_ENTER();
+    PDL_ARG(a); PDL_ARG(b); PDL_ARG(q); PDL_ARG(theta); PDL_ARG(relres);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= t) return;
     const double den = fabs(theta[i]);
@@ -73,6 +83,8 @@ __global__ void k_arn_relres(int t, const double* a, const double* b, const doub
 
 // q[c] = sum_r X[r, c] Y[r, c] (one warp per column)
 __global__ void k_arn_coldot(int rows, int t, const double* X, int ldx, const double* Y, int ldy, double* q) {
+    PDL_ENTER();
+    PDL_ARG(X); PDL_ARG(Y); PDL_ARG(q);
     const int c = blockIdx.x;
     const int lane = threadIdx.x;
     double acc = 0.0;
@@ -82,6 +94,8 @@ __global__ void k_arn_coldot(int rows, int t, const double* X, int ldx, const do
 }
 
 __global__ void k_arn_reverse_cols(int64_t rows, int t, const double* in, int64_t ldi, double* out, int64_t ldo) {
+    PDL_ENTER();
+    PDL_ARG(in); PDL_ARG(out);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= rows * t) return;
     const int64_t r = e % rows;
@@ -90,6 +104,8 @@ __global__ void k_arn_reverse_cols(int64_t rows, int t, const double* in, int64_
 }
 
 __global__ void k_arn_reverse_vec(int t, const double* in, double* out) {
+    PDL_ENTER();
+    PDL_ARG(in); PDL_ARG(out);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < t) out[i] = in[t - 1 - i];
 }
@@ -146,10 +162,8 @@ int arn_ritz(eda_ctx* h, int m, int ldh, int t, int b, ArnWs& w, std::vector<dou
     EDA_TRY(gemm_tn_f64(n, m, m, 1.0, QW, nk, w.T1, n, 0.0, w.AW, m, w.part, w.pcap, s));
     EDA_TRY(gemm_small_f64(false, false, k, m, k, 1.0, h->KB, k, QB, nk, 0.0, w.T1, k, s));
     EDA_TRY(gemm_tn_f64(k, m, m, 1.0, QB, nk, w.T1, k, 0.0, w.AB, m, w.part, w.pcap, s));
-    k_arn_add_identity<<<ceil_div(m, 128), 128, 0, s>>>(m, w.AW, m);
-    EDA_LAUNCHED();
-    k_arn_add_identity<<<ceil_div(m, 128), 128, 0, s>>>(m, w.AB, m);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_arn_add_identity, dim3(ceil_div(m, 128)), dim3(128), 0, s, m, w.AW, m)));
+    EDA_CUDA_TRY((launch_chained(k_arn_add_identity, dim3(ceil_div(m, 128)), dim3(128), 0, s, m, w.AB, m)));
     EDA_TRY(symmetrize_f64(m, w.AW, m, s));
     EDA_TRY(symmetrize_f64(m, w.AB, m, s));
     // A_W = R^T R; the symmetric C = R^{-T} A_B R^{-1} has the pencil's eigenvalues; s = R^{-1} y
@@ -161,8 +175,8 @@ int arn_ritz(eda_ctx* h, int m, int ldh, int t, int b, ArnWs& w, std::vector<dou
     EDA_TRY(gemm_small_f64(false, false, m, t, m, 1.0, w.Ri, m, w.T1, m, 0.0, w.S, m, s));
     // residuals in the exp(c^2 S_W) norm: ||H s - theta s||^2 + ||W s_last||^2 + (H_W^T r)^T K_W(c^2) (H_W^T r)
     EDA_TRY(gemm_small_f64(false, false, m, t, m, 1.0, w.H, ldh, w.S, m, 0.0, w.HS, m, s));
-    k_arn_sub_scaled<<<ceil_div((int64_t)m * t, 256), 256, 0, s>>>(m, t, w.HS, m, w.S, m, w.theta);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_arn_sub_scaled, dim3(ceil_div((int64_t)m * t, 256)), dim3(256), 0, s, m, t, w.HS, m,
+        w.S, m, w.theta)));
     EDA_TRY(col_norms_f64(m, t, w.HS, m, w.n1, s));
     EDA_TRY(gemm_nn_f64(d, b, t, 1.0, w.W, d, w.S + (m - b), m, 0.0, nullptr, 0, w.X, d, s));
     EDA_TRY(col_norms_f64(d, t, w.X, d, w.n2, s));
@@ -170,10 +184,9 @@ int arn_ritz(eda_ctx* h, int m, int ldh, int t, int b, ArnWs& w, std::vector<dou
     EDA_TRY(gemm_small_f64(false, false, n, t, m, 1.0, QW, nk, w.HS, m, 0.0, w.T2, n, s));
     EDA_TRY(gemm_small_f64(false, false, n, t, b, 1.0, w.ZW, nk, w.S + (m - b), m, 1.0, w.T2, n, s));
     EDA_TRY(gemm_small_f64(false, false, n, t, n, 1.0, h->KWp, n, w.T2, n, 0.0, w.T3, n, s));
-    k_arn_coldot<<<t, 32, 0, s>>>(n, t, w.T2, n, w.T3, n, w.sn);
-    EDA_LAUNCHED();
-    k_arn_relres<<<ceil_div(t, 128), 128, 0, s>>>(t, w.n1, w.n2, w.sn, w.theta, w.relres);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_arn_coldot, dim3(t), dim3(32), 0, s, n, t, w.T2, n, w.T3, n, w.sn)));
+    EDA_CUDA_TRY((launch_chained(k_arn_relres, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.n1, w.n2, w.sn, w.theta,
+        w.relres)));
     EDA_TRY(read_back(relres_h.data(), w.relres, t * sizeof(double), s));
     return EDA_OK;
 }
@@ -193,16 +206,15 @@ int arn_true_residuals(eda_ctx* h, int m, int t, int b, ArnWs& w, std::vector<do
         EDA_TRY(n_apply_composed(h, cb, w.X + (size_t)c0 * d, d, w.X2 + (size_t)c0 * d, d, w.PQ, w.U, nullptr, w.part,
                                  w.pcap, s));
     }
-    k_arn_sub_scaled<<<ceil_div(d * t, 256), 256, 0, s>>>((int)d, t, w.X2, (int)d, w.X, (int)d, w.theta);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_arn_sub_scaled, dim3(ceil_div(d * t, 256)), dim3(256), 0, s, (int)d, t, w.X2, (int)d,
+        w.X, (int)d, w.theta)));
     EDA_TRY(col_norms_f64(d, t, w.X2, d, w.n1, s));
     EDA_TRY(sweep_zt(h, t, w.X2, d, w.T1, w.part, w.pcap, s));   // Z^T r: its first n rows are H_W^T r
     EDA_TRY(gemm_tn_f64(n, n, t, 1.0, h->KWp, n, w.T1, nk, 0.0, w.T2, n, w.part, w.pcap, s));
-    k_arn_coldot<<<t, 32, 0, s>>>(n, t, w.T1, nk, w.T2, n, w.sn);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_arn_coldot, dim3(t), dim3(32), 0, s, n, t, w.T1, nk, w.T2, n, w.sn)));
     EDA_CUDA_TRY(cudaMemsetAsync(w.n2, 0, t * sizeof(double), s));
-    k_arn_relres<<<ceil_div(t, 128), 128, 0, s>>>(t, w.n1, w.n2, w.sn, w.theta, w.relres);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_arn_relres, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.n1, w.n2, w.sn, w.theta,
+        w.relres)));
     EDA_TRY(read_back(relres_h.data(), w.relres, t * sizeof(double), s));
     return EDA_OK;
 }
@@ -367,9 +379,12 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
             double* C1 = w.C;
             double* C2 = w.C + (size_t)m_max * b;
             if ((rc = cgs2_f64(d, cols, b, w.V, w.W, C1, C2, w, s)) != EDA_OK) break;
-            k_arn_set_hcol<<<ceil_div(cols * b, 256), 256, 0, s>>>(w.H, m_max, cols, j0, b, C1, C2);
-            launch_counter()++;
-            if (cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
+            if (launch_chained(k_arn_set_hcol, dim3(ceil_div(cols * b, 256)), dim3(256), 0, s, w.H, m_max, cols, j0, b,
+                C1, C2) !=
+                cudaSuccess) {
+                rc = EDA_ERR_CUDA;
+                break;
+            }
             // W1 = W R1^{-1} (the remainder W itself stays for the residuals)
             if ((rc = cholqr_once(d, b, w.W, w.W1, w.R1, w.R1i, piv_min2, h->status, w.lost, w, s)) != EDA_OK) break;
             int lw[2] = {0, 0};   // lost and nearly lost columns
@@ -403,12 +418,15 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
                     rc = copy_mat_f64(b, b, w.Bm, b, w.R1, b, s);
                 }
                 if (rc != EDA_OK) break;
-                if (cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
                 if ((rc = cholqr_once(d, b, w.W1, Vn, w.R2, w.R2i, 0.0, h->status, w.lost, w, s)) != EDA_OK) break;
                 if ((rc = gemm_small_f64(false, false, b, b, b, 1.0, w.R2, b, w.R1, b, 0.0, w.Bm, b, s)) != EDA_OK)
                     break;
-                k_arn_set_block<<<ceil_div(b * b, 256), 256, 0, s>>>(w.H, m_max, cols, j0, b, w.Bm);
-                launch_counter()++;
+                if (launch_chained(k_arn_set_block, dim3(ceil_div(b * b, 256)), dim3(256), 0, s, w.H, m_max, cols, j0, b,
+                    w.Bm) !=
+                    cudaSuccess) {
+                    rc = EDA_ERR_CUDA;
+                    break;
+                }
             }
             const bool last = !room;
             if ((cols >= next_check && cols >= t + 1) || (last && cols >= t)) {
@@ -463,10 +481,17 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
             if (rc == EDA_OK) rc = copy_mat_f64(d, t, w.X2, d, w.X, d, s);
         }
         if (rc != EDA_OK) break;
-        k_arn_reverse_cols<<<ceil_div((int64_t)d * t, 256), 256, 0, s>>>(d, t, w.X, d, Vout, d);
-        launch_counter()++;
-        k_arn_reverse_vec<<<ceil_div(t, 128), 128, 0, s>>>(t, w.theta, w.lamd);
-        launch_counter()++;
+        if (launch_chained(k_arn_reverse_cols, dim3(ceil_div((int64_t)d * t, 256)), dim3(256), 0, s, d, t, w.X, d, Vout,
+            d) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
+        if (launch_chained(k_arn_reverse_vec, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.theta, w.lamd) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
         if (cudaMemcpyAsync(lambda, w.lamd, t * sizeof(double), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             rc = EDA_ERR_CUDA;
     } while (false);

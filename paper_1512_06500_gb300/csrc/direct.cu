@@ -37,6 +37,8 @@ size_t a256(size_t b) { return (b + 255) & ~size_t(255); }
 // Out[i, j] = A[rows ? rows[i] : i, cols[j]] for i < m, j < c (Out ld m; A ld lda).
 __global__ void k_gather(int m, int c, const double* __restrict__ A, int64_t lda, const int* __restrict__ rows,
                          const int* __restrict__ cols, double* __restrict__ Out) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(rows); PDL_ARG(cols); PDL_ARG(Out);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * c) return;
     const int i = (int)(e % m), j = (int)(e / m);
@@ -47,6 +49,8 @@ __global__ void k_gather(int m, int c, const double* __restrict__ A, int64_t lda
 // Out (nk x t, zero outside the kept rows): Out[keep[i], j] = A[i, j] for i < r (A ld r).
 __global__ void k_scatter_rows(int nk, int r, int t, const double* __restrict__ A, const int* __restrict__ keep,
                                double* __restrict__ Out) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(keep); PDL_ARG(Out);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)r * t) return;
     const int i = (int)(e % r), j = (int)(e / r);
@@ -55,6 +59,8 @@ __global__ void k_scatter_rows(int nk, int r, int t, const double* __restrict__ 
 
 // Columns in reverse order: Out[:, j] = A[:, t - 1 - j] (ld rows each).
 __global__ void k_reverse_cols(int64_t rows, int t, const double* __restrict__ A, double* __restrict__ Out) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(Out);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= rows * t) return;
     const int64_t r = e % rows;
@@ -65,6 +71,8 @@ __global__ void k_reverse_cols(int64_t rows, int t, const double* __restrict__ A
 // Rank check of the Cholesky factor R (upper, ld r) of the kept columns' Gram: a pivot R_jj^2 at or below
 // 1e-13 of the largest (or not finite) means the kept columns are dependent (samples not affinely independent).
 __global__ void k_rank_check(int r, const double* __restrict__ R, int* status) {
+    PDL_ENTER();
+    PDL_ARG(R); PDL_ARG(status);
     __shared__ double smax;
     double mx = 0.0;
     for (int j = threadIdx.x; j < r; j += blockDim.x) {
@@ -87,6 +95,8 @@ __global__ void k_rank_check(int r, const double* __restrict__ R, int* status) {
 
 // lambda[j] = 1 + mu[t - 1 - j] (descending; mu ascending)
 __global__ void k_lambda_desc(int t, const double* __restrict__ mu, double* __restrict__ lam) {
+    PDL_ENTER();
+    PDL_ARG(mu); PDL_ARG(lam);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < t) lam[j] = 1.0 + mu[t - 1 - j];
 }
@@ -220,13 +230,24 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
         if ((rc = copy_mat_f64(n, k, h->GWB, n, w.G + (size_t)n * nk, nk, s)) != EDA_OK) break;
         if ((rc = copy_mat_f64(k, k, h->GB, k, w.G + (size_t)n * nk + n, nk, s)) != EDA_OK) break;
         // G' = S^T G S = R^T R, F = G S
-        k_gather<<<ceil_div((int64_t)r * r, 256), 256, 0, s>>>(r, r, w.G, nk, w.keep, w.keep, w.Gs);
-        launch_counter()++;
-        k_gather<<<ceil_div((int64_t)nk * r, 256), 256, 0, s>>>(nk, r, w.G, nk, nullptr, w.keep, w.PQ);
-        launch_counter()++;
+        if (launch_chained(k_gather, dim3(ceil_div((int64_t)r * r, 256)), dim3(256), 0, s, r, r, w.G, nk, w.keep, w.keep,
+            w.Gs) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
+        if (launch_chained(k_gather, dim3(ceil_div((int64_t)nk * r, 256)), dim3(256), 0, s, nk, r, w.G, nk, nullptr,
+            w.keep, w.PQ) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
         if ((rc = chol_inv_blocked(r, w.Gs, r, w.Ri, r, 1e-13, h->status, w.CW, w.part, w.pcap, s)) != EDA_OK) break;
-        k_rank_check<<<1, 256, 0, s>>>(r, w.Gs, h->status);
-        launch_counter()++;
+        if (launch_chained(k_rank_check, dim3(1), dim3(256), 0, s, r, w.Gs, h->status) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
         // P = F R^{-1} = Z^T Q
         if ((rc = gemm_nn_f64(nk, r, r, 1.0, w.PQ, nk, w.Ri, r, 0.0, nullptr, 0, w.P, nk, s)) != EDA_OK) break;
         // B = P^T C P
@@ -241,8 +262,12 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
         // y = Z a, a = S R^{-1} w
         if ((rc = gemm_nn_f64(r, r, t, 1.0, w.Ri, r, w.Wv, r, 0.0, nullptr, 0, w.As, r, s)) != EDA_OK) break;
         if (cudaMemsetAsync(w.a, 0, (size_t)nk * t * 8, s) != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
-        k_scatter_rows<<<ceil_div((int64_t)r * t, 256), 256, 0, s>>>(nk, r, t, w.As, w.keep, w.a);
-        launch_counter()++;
+        if (launch_chained(k_scatter_rows, dim3(ceil_div((int64_t)r * t, 256)), dim3(256), 0, s, nk, r, t, w.As, w.keep,
+            w.a) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
         // x = exp(-c^2 S_W / 2) y: coordinates a + [K (G_W a_W + G_WB a_B); 0]
         if ((rc = sym_nn(h, nullptr, h->GW, n, t, w.a, nk, false, w.T1, n, w, s)) != EDA_OK) break;
         if ((rc = gemm_tn_f64(k, n, t, 1.0, h->GBW, k, w.a + n, nk, 1.0, w.T1, n, w.part, w.pcap, s)) != EDA_OK) break;
@@ -254,15 +279,21 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
         if ((rc = chol_inv_auto(t, w.Gv, t, w.Rvi, 1e-28, h->status, w.CW, w.part, w.pcap, s)) != EDA_OK) break;
         if ((rc = gemm_nn_f64(nk, t, t, 1.0, w.a, nk, w.Rvi, t, 0.0, nullptr, 0, w.bco, nk, s)) != EDA_OK) break;
         // descending order, then V = Z b R_v^{-1}
-        k_reverse_cols<<<ceil_div((int64_t)nk * t, 256), 256, 0, s>>>(nk, t, w.bco, w.brev);
-        launch_counter()++;
+        if (launch_chained(k_reverse_cols, dim3(ceil_div((int64_t)nk * t, 256)), dim3(256), 0, s, nk, t, w.bco, w.brev) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
         if ((rc = z_times(h, t, w.brev, w.X, s)) != EDA_OK) break;
         // one CholQR pass on V itself
         if ((rc = syrk_f64(d, t, 1.0, w.X, d, 0.0, w.Rv, t, w.part, w.pcap, s)) != EDA_OK) break;
         if ((rc = chol_inv_auto(t, w.Rv, t, w.Rvi, 1e-28, h->status, w.CW, w.part, w.pcap, s)) != EDA_OK) break;
         if ((rc = gemm_nn_f64(d, t, t, 1.0, w.X, d, w.Rvi, t, 0.0, nullptr, 0, Vout, d, s)) != EDA_OK) break;
-        k_lambda_desc<<<ceil_div(t, 128), 128, 0, s>>>(t, w.mu, lambda);
-        launch_counter()++;
+        if (launch_chained(k_lambda_desc, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.mu, lambda) !=
+            cudaSuccess) {
+            rc = EDA_ERR_CUDA;
+            break;
+        }
         if (cudaPeekAtLastError() != cudaSuccess) { rc = EDA_ERR_CUDA; break; }
     } while (false);
     float ms = 0.f;

@@ -65,6 +65,8 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
 namespace {
 // B (k x n) = A^T for A (n x k), both column-major.
 __global__ void k_transpose_nk(int n, int k, const double* __restrict__ A, double* __restrict__ B) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(B);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)n * k) return;
     const int i = (int)(e % n), j = (int)(e / n);
@@ -85,8 +87,8 @@ int ensure_cross_gram(eda_ctx* h, double* part, size_t pcap, cudaStream_t s) {
     h->GWB = static_cast<double*>(xp);
     h->GBW = reinterpret_cast<double*>(static_cast<char*>(xp) + xb);
     EDA_TRY(gemm_tn_f64(h->d, n, k, 1.0, h->HW, h->d, h->HB, h->d, 0.0, h->GWB, n, part, pcap, s));
-    k_transpose_nk<<<ceil_div((int64_t)n * k, 256), 256, 0, s>>>(n, k, h->GWB, h->GBW);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_transpose_nk, dim3(ceil_div((int64_t)n * k, 256)), dim3(256), 0, s, n, k, h->GWB,
+        h->GBW)));
     return EDA_OK;
 }
 

@@ -41,6 +41,55 @@ std::atomic<uint64_t>& launch_counter();   // kernels launched by this process (
         EDA_CUDA_TRY(cudaPeekAtLastError());          \
     } while (0)
 
+// ---------------------------------------------------------------- chained launches
+// The solvers issue hundreds of kernels of a few microseconds one after another. Launched with programmatic stream
+// serialisation, the CTAs of a kernel are set up while its predecessor still runs and wait (griddepcontrol.wait) until that
+// one has completed and its writes are visible. A kernel that is launched this way starts with PDL_WAIT, before anything
+// else, and lets its own successor be set up with PDL_NEXT: at once (PDL_ENTER) when it is short, after its main loop when it
+// runs long, so that waiting CTAs do not hold room that other streams could use. PDL_ARG adds a zero that the compiler sees
+// only after the wait to every pointer the kernel takes: a load through a const __restrict__ one counts as invariant, and the
+// wait alone would not keep it from being moved up. Every other kind of operation before or after (copies, fills, events,
+// kernels without PDL_WAIT, other streams) orders as without it.
+#define PDL_WAIT()    \
+    int64_t pdl_zero; \
+    asm volatile("griddepcontrol.wait;\n\tmov.u64 %0, 0;" : "=l"(pdl_zero)::"memory")
+#define PDL_NEXT() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
+#define PDL_ENTER() \
+    PDL_NEXT();     \
+    PDL_WAIT()
+#define PDL_ARG(p) (p) += pdl_zero
+
+// CTAs that are set up early go to whichever SMs have room at that moment, several to one SM when a large predecessor drains
+// unevenly, and stay there. For a kernel that fills the chip and is bound by the FP64 pipe of each SM that costs more than the
+// launch it hides (k_gemm_tn_partial<16>, 16384 x 100 blocks: 0.15 -> 0.36 ms): launch_spread therefore chains only grids of
+// at most half the SMs and starts the others when the chip is empty.
+int sm_count();   // of the current device
+
+template <class... P, class... A>
+cudaError_t launch_after(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    launch_counter()++;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    return launch_after(true, kernel, grid, block, smem, s, args...);
+}
+template <class... P, class... A>
+cudaError_t launch_spread(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    const bool small = (uint64_t)grid.x * grid.y * grid.z <= (uint64_t)sm_count() / 8;
+    return launch_after(small, kernel, grid, block, smem, s, args...);
+}
+
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // Device status word bits (written by kernels, read by the host).
@@ -134,7 +183,6 @@ int gemm_tn_f64(int64_t d, int m, int p, double alpha, const double* A, int64_t 
 int syrk_f64(int64_t d, int m, double alpha, const double* A, int64_t lda, double beta, double* C, int ldc,
              double* partial, size_t partial_cap, cudaStream_t s);
 // Streaming multiprocessors of the current device (queried once per process).
-int sm_count();
 // C (d x p) = beta * C0 + alpha * A B, A: d x m (lda), B: m x p (ldb); C may equal C0 (same ld).
 int gemm_nn_f64(int64_t d, int m, int p, double alpha, const double* A, int64_t lda,
                 const double* B, int ldb, double beta, const double* C0, int64_t ldc0,

@@ -14,6 +14,8 @@ namespace {
 // in input order, 32 samples at a time, with equal labels ranked by lane order.
 __global__ void k_segment(const int32_t* __restrict__ labels, int n, int k, int32_t* counts, int32_t* offsets,
                           int32_t* perm, int* status) {
+    PDL_ENTER();
+    PDL_ARG(labels); PDL_ARG(counts); PDL_ARG(offsets); PDL_ARG(perm); PDL_ARG(status);
     extern __shared__ int cnt[];
     for (int j = threadIdx.x; j < k; j += blockDim.x) cnt[j] = 0;
     __syncthreads();
@@ -67,6 +69,8 @@ template <class T>
 __global__ void k_class_means(const T* __restrict__ X, int64_t d, int64_t ldx, const int32_t* __restrict__ counts,
                               const int32_t* __restrict__ offsets, const int32_t* __restrict__ perm,
                               double* __restrict__ mu_j) {
+    PDL_WAIT();
+    PDL_ARG(X); PDL_ARG(counts); PDL_ARG(offsets); PDL_ARG(perm); PDL_ARG(mu_j);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (p >= d) return;
@@ -80,6 +84,8 @@ __global__ void k_class_means(const T* __restrict__ X, int64_t d, int64_t ldx, c
 template <class T>
 __global__ void k_global_mean(const T* __restrict__ X, int64_t d, int64_t ldx, int n, double* __restrict__ mu,
                               int* __restrict__ status) {
+    PDL_WAIT();
+    PDL_ARG(X); PDL_ARG(mu); PDL_ARG(status);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool bad = false;
     if (p < d) {
@@ -99,6 +105,8 @@ __global__ void k_global_mean(const T* __restrict__ X, int64_t d, int64_t ldx, i
 template <class T>
 __global__ void k_build_hw(const T* __restrict__ X, int64_t d, int64_t ldx, int n, const int32_t* __restrict__ labels,
                            const int32_t* __restrict__ perm, const double* __restrict__ mu_j, double* __restrict__ HW) {
+    PDL_WAIT();
+    PDL_ARG(X); PDL_ARG(labels); PDL_ARG(perm); PDL_ARG(mu_j); PDL_ARG(HW);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int q = blockIdx.y;
     if (p >= d) return;
@@ -112,6 +120,8 @@ __global__ void k_build_hw(const T* __restrict__ X, int64_t d, int64_t ldx, int 
 constexpr int kHbPer = 8;
 __global__ void k_build_hb(int64_t d, const int32_t* __restrict__ counts, const double* __restrict__ mu_j,
                            const double* __restrict__ mu, double* __restrict__ HB) {
+    PDL_WAIT();
+    PDL_ARG(counts); PDL_ARG(mu_j); PDL_ARG(mu); PDL_ARG(HB);
     const int64_t p0 = (int64_t)blockIdx.x * blockDim.x * kHbPer + threadIdx.x;
     const int j = blockIdx.y;
     if (p0 >= d) return;
@@ -126,6 +136,8 @@ __global__ void k_build_hb(int64_t d, const int32_t* __restrict__ counts, const 
 // ST_NONFINITE when A holds Inf or NaN: a CTA per 1024 rows of a column (columns strided over the grid's y), tests on the bits.
 __global__ void __launch_bounds__(256) k_check_finite(int64_t rows, int cols, const double* __restrict__ A, int64_t lda,
                                                      int* status) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(status);
     bool bad = false;
     const int64_t r0 = (int64_t)blockIdx.x * 1024 + threadIdx.x;
     for (int c = blockIdx.y; c < cols; c += gridDim.y)
@@ -140,6 +152,8 @@ __global__ void __launch_bounds__(256) k_check_finite(int64_t rows, int cols, co
 // tmp[:, s] = coef_s W[:, first + s],  coef_s = alpha (phi(alpha lam_s) - 1),  phi(z) = expm1(z) / z.
 __global__ void k_phi_scale(int n, int ns, const double* __restrict__ lam, const double* __restrict__ W, int ldw,
                             double alpha, double* __restrict__ tmp) {
+    PDL_ENTER();
+    PDL_ARG(lam); PDL_ARG(W); PDL_ARG(tmp);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)n * ns) return;
     const int i = (int)(e % n), s = (int)(e / n);
@@ -149,6 +163,8 @@ __global__ void k_phi_scale(int n, int ns, const double* __restrict__ lam, const
 }
 
 __global__ void k_add_diag(int n, double alpha, double* K) {
+    PDL_ENTER();
+    PDL_ARG(K);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) K[(int64_t)i * n + i] += alpha;
 }
@@ -156,6 +172,8 @@ __global__ void k_add_diag(int n, double alpha, double* K) {
 // D = c0 I + c1 P1 + c2 P2 + c3 P3 (m x m, ld m); a null P contributes nothing.
 __global__ void k_lincomb4(int m, double c0, double c1, const double* P1, double c2, const double* P2, double c3,
                            const double* P3, double* D) {
+    PDL_ENTER();
+    PDL_ARG(P1); PDL_ARG(P2); PDL_ARG(P3); PDL_ARG(D);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * m) return;
     const int i = (int)(e % m), j = (int)(e / m);
@@ -168,6 +186,8 @@ __global__ void k_lincomb4(int m, double c0, double c1, const double* P1, double
 
 // D = a S (m x m)
 __global__ void k_scale_sq(int m, double a, const double* S, double* D) {
+    PDL_ENTER();
+    PDL_ARG(S); PDL_ARG(D);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e < (int64_t)m * m) D[e] = a * S[e];
 }
@@ -178,8 +198,7 @@ int segment_labels(const int32_t* labels, int n, int k, int32_t* counts, int32_t
                    int* status, cudaStream_t s) {
     const size_t smem = (size_t)k * sizeof(int);
     if (smem > 48 * 1024) return EDA_ERR_INVALID_ARG;
-    k_segment<<<1, 1024, smem, s>>>(labels, n, k, counts, offsets, perm, status);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_segment, dim3(1), dim3(1024), smem, s, labels, n, k, counts, offsets, perm, status)));
     return EDA_OK;
 }
 
@@ -190,47 +209,40 @@ int build_factors(const void* X, int x_dtype, int64_t d, int n, int64_t ldx, int
     const dim3 gk(ceil_div(d, tb), k), g1(ceil_div(d, tb)), gn(ceil_div(d, tb), n);
     if (x_dtype == EDA_F64) {
         const double* x = static_cast<const double*>(X);
-        k_class_means<<<gk, tb, 0, s>>>(x, d, ldx, counts, offsets, perm, mu_j);
-        EDA_LAUNCHED();
-        k_global_mean<<<g1, tb, 0, s>>>(x, d, ldx, n, mu, status);
-        EDA_LAUNCHED();
-        k_build_hw<<<gn, tb, 0, s>>>(x, d, ldx, n, labels, perm, mu_j, HW);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_spread(k_class_means<double>, gk, dim3(tb), 0, s, x, d, ldx, counts, offsets, perm, mu_j)));
+        EDA_CUDA_TRY((launch_spread(k_global_mean<double>, g1, dim3(tb), 0, s, x, d, ldx, n, mu, status)));
+        EDA_CUDA_TRY((launch_spread(k_build_hw<double>, gn, dim3(tb), 0, s, x, d, ldx, n, labels, perm, mu_j, HW)));
     } else if (x_dtype == EDA_F32) {
         const float* x = static_cast<const float*>(X);
-        k_class_means<<<gk, tb, 0, s>>>(x, d, ldx, counts, offsets, perm, mu_j);
-        EDA_LAUNCHED();
-        k_global_mean<<<g1, tb, 0, s>>>(x, d, ldx, n, mu, status);
-        EDA_LAUNCHED();
-        k_build_hw<<<gn, tb, 0, s>>>(x, d, ldx, n, labels, perm, mu_j, HW);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_spread(k_class_means<float>, gk, dim3(tb), 0, s, x, d, ldx, counts, offsets, perm, mu_j)));
+        EDA_CUDA_TRY((launch_spread(k_global_mean<float>, g1, dim3(tb), 0, s, x, d, ldx, n, mu, status)));
+        EDA_CUDA_TRY((launch_spread(k_build_hw<float>, gn, dim3(tb), 0, s, x, d, ldx, n, labels, perm, mu_j, HW)));
     } else {
         return EDA_ERR_INVALID_ARG;
     }
-    k_build_hb<<<dim3(ceil_div(d, (int64_t)tb * kHbPer), k), tb, 0, s>>>(d, counts, mu_j, mu, HB);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_spread(k_build_hb, dim3(ceil_div(d, (int64_t)tb * kHbPer), k), dim3(tb), 0, s, d, counts, mu_j,
+        mu, HB)));
     return EDA_OK;
 }
 
 int check_finite_f64(int64_t rows, int cols, const double* A, int64_t lda, int* status, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return EDA_OK;
-    k_check_finite<<<dim3((unsigned)ceil_div(rows, 1024), (unsigned)std::min(cols, 65535)), 256, 0, s>>>(rows, cols, A, lda,
-                                                                                                    status);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_check_finite, dim3((unsigned)ceil_div(rows, 1024), (unsigned)std::min(cols, 65535)),
+        dim3(256), 0, s, rows, cols, A, lda,
+            status)));
     return EDA_OK;
 }
 
 int phi_operator(int n, int ns, const double* lam, const double* W, int ldw, double alpha, double* K, double* tmp,
                  cudaStream_t s) {
     if (ns > 0) {
-        k_phi_scale<<<ceil_div((int64_t)n * ns, 256), 256, 0, s>>>(n, ns, lam, W, ldw, alpha, tmp);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_phi_scale, dim3(ceil_div((int64_t)n * ns, 256)), dim3(256), 0, s, n, ns, lam, W,
+            ldw, alpha, tmp)));
         EDA_TRY(gemm_small_f64(false, true, n, n, ns, 1.0, tmp, n, W, ldw, 0.0, K, n, s));
     } else {
         EDA_CUDA_TRY(cudaMemsetAsync(K, 0, (size_t)n * n * sizeof(double), s));
     }
-    k_add_diag<<<ceil_div(n, 256), 256, 0, s>>>(n, alpha, K);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_add_diag, dim3(ceil_div(n, 256)), dim3(256), 0, s, n, alpha, K)));
     return EDA_OK;
 }
 
@@ -277,29 +289,27 @@ int phi_by_squaring(int m, const double* G, double alpha, double lmax, double* K
         return oz_gemm_tiled(oa, ob, alpha_, beta, beta != 0.0 ? C : nullptr, m, C, m, true, oz->status, s);
     };
     auto mul = [&](const double* A, const double* B, double beta, double* C) { return mulab(1.0, A, B, beta, C); };
-    k_scale_sq<<<eb, 256, 0, s>>>(m, std::ldexp(alpha, -sq), G, P1);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_scale_sq, dim3(eb), dim3(256), 0, s, m, std::ldexp(alpha, -sq), G, P1)));
     EDA_TRY(mul(P1, P1, 0.0, P2));
     EDA_TRY(mul(P2, P1, 0.0, P3));
     EDA_TRY(mul(P3, P1, 0.0, P4));
     // Horner in B^4 over the blocks c_{4i} .. c_{4i+3}, i = 4 (c_16, c_17) down to 0
-    k_lincomb4<<<eb, 256, 0, s>>>(m, c[16], c[17], P1, 0.0, nullptr, 0.0, nullptr, F);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_lincomb4, dim3(eb), dim3(256), 0, s, m, c[16], c[17], P1, 0.0, nullptr, 0.0, nullptr,
+        F)));
     for (int i = 3; i >= 0; --i) {
-        k_lincomb4<<<eb, 256, 0, s>>>(m, c[4 * i], c[4 * i + 1], P1, c[4 * i + 2], P2, c[4 * i + 3], P3, T);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_lincomb4, dim3(eb), dim3(256), 0, s, m, c[4 * i], c[4 * i + 1], P1, c[4 * i + 2],
+            P2, c[4 * i + 3], P3, T)));
         EDA_TRY(mul(F, P4, 1.0, T));               // T = F B^4 + Q_i
         std::swap(F, T);
     }
     // E = I + B phi(B) (in P2; B^2 and B^3 are no longer needed)
     double* E = P2;
     double* E2 = P3;
-    k_lincomb4<<<eb, 256, 0, s>>>(m, 1.0, 0.0, nullptr, 0.0, nullptr, 0.0, nullptr, E);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_lincomb4, dim3(eb), dim3(256), 0, s, m, 1.0, 0.0, nullptr, 0.0, nullptr, 0.0, nullptr,
+        E)));
     EDA_TRY(mul(P1, F, 1.0, E));
     for (int q = 0; q < sq; ++q) {
-        k_scale_sq<<<eb, 256, 0, s>>>(m, 0.5, F, T);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_scale_sq, dim3(eb), dim3(256), 0, s, m, 0.5, F, T)));
         EDA_TRY(mulab(0.5, F, E, 1.0, T));                                                 // phi(2B)
         std::swap(F, T);
         if (q + 1 < sq) {
@@ -307,8 +317,7 @@ int phi_by_squaring(int m, const double* G, double alpha, double lmax, double* K
             std::swap(E, E2);
         }
     }
-    k_scale_sq<<<eb, 256, 0, s>>>(m, alpha, F, K);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_scale_sq, dim3(eb), dim3(256), 0, s, m, alpha, F, K)));
     return symmetrize_f64(m, K, m, s);
 }
 

@@ -34,6 +34,8 @@ template <int TP, class T, bool SYM = false>
 __global__ void __launch_bounds__(TN_THREADS) k_gemm_tn_partial(int64_t d, int m, int p, const T* __restrict__ A,
                                                                 int64_t lda, const T* __restrict__ B, int64_t ldb,
                                                                 int64_t rows_per_split, T* __restrict__ partial) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(B); PDL_ARG(partial);
     __shared__ T As[TN_KB][TN_TM + 1];
     __shared__ T Bs[TN_KB][TP + 1];
     int bx = blockIdx.x, by = blockIdx.y;
@@ -107,6 +109,7 @@ __global__ void __launch_bounds__(TN_THREADS) k_gemm_tn_partial(int64_t d, int m
         }
         __syncthreads();
     }
+    PDL_NEXT();
     T* out = partial + (int64_t)s * m * p;
 #pragma unroll
     for (int a = 0; a < TMT; ++a)
@@ -131,6 +134,8 @@ constexpr int SN_MAXM = 32;
 template <int ACC, int CH, int MC, class T>
 __global__ void __launch_bounds__(SN_THREADS, 2) k_syrk_narrow(int64_t d, int m, const T* __restrict__ A, int64_t lda,
                                                             int64_t rows_per_split, int R, T* __restrict__ partial) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(partial);
     constexpr int LD = MC | 1;   // odd: the columns of a row and the rows of a column fall into different banks
     __shared__ T As[CH][LD];
     __shared__ T tot[32 * ACC];
@@ -191,6 +196,7 @@ __global__ void __launch_bounds__(SN_THREADS, 2) k_syrk_narrow(int64_t d, int m,
         }
         __syncthreads();
     }
+    PDL_NEXT();
     for (int v = 0; v < SN_THREADS / 32; ++v) {
         if (w == v) {
 #pragma unroll
@@ -227,6 +233,8 @@ __device__ __forceinline__ void tn_store(double* C, int ldc, int i, int j, doubl
 template <class T>
 __global__ void k_gemm_tn_reduce(int m, int p, int splits, const T* __restrict__ partial, double alpha,
                                  double beta, double* __restrict__ C, int ldc, bool sym) {
+    PDL_ENTER();
+    PDL_ARG(partial); PDL_ARG(C);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * p) return;
     const int i = (int)(e % m), j = (int)(e / m);
@@ -239,6 +247,8 @@ __global__ void k_gemm_tn_reduce(int m, int p, int splits, const T* __restrict__
 template <class T>
 __global__ void k_gemm_tn_reduce_warp(int m, int p, int splits, const T* __restrict__ partial, double alpha,
                                       double beta, double* __restrict__ C, int ldc, bool sym) {
+    PDL_ENTER();
+    PDL_ARG(partial); PDL_ARG(C);
     const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (e >= (int64_t)m * p) return;
@@ -268,6 +278,8 @@ template <int NC, class T>
 __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double alpha, const T* __restrict__ A,
                                                  int64_t lda, const double* __restrict__ B, int ldb, double beta,
                                                  const T* C0, int64_t ldc0, T* C, int64_t ldc, int ub) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(B); PDL_ARG(C0); PDL_ARG(C);
     constexpr int LCH = 256;                 // rows of B staged per pass
     __shared__ T Bs[LCH][NC];
     __shared__ T red[7][32][NC];
@@ -320,6 +332,7 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double
             for (int c = 0; c < NC; ++c) acc[c] = fma(a0, Bs[l][c], acc[c]);
         }
     }
+    PDL_NEXT();
     if (w > 0) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) red[w - 1][lane][c] = acc[c];
@@ -351,6 +364,8 @@ __global__ void __launch_bounds__(32 * kSplitkWarps) k_gemm_small_nn_splitk(int 
                                                                            const double* __restrict__ B, int ldb,
                                                                            double beta, double* __restrict__ C,
                                                                            int ldc) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(B); PDL_ARG(C);
     __shared__ double part[kSplitkWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int ib = blockIdx.x, j = blockIdx.y;
@@ -378,6 +393,7 @@ __global__ void __launch_bounds__(32 * kSplitkWarps) k_gemm_small_nn_splitk(int 
         }
         for (; l < le; ++l) a[0] = fma(A[(int64_t)l * lda + i], Bj[l], a[0]);
     }
+    PDL_NEXT();
     part[w][lane] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
     __syncthreads();
     if (w == 0 && i < m) {
@@ -394,6 +410,8 @@ __global__ void __launch_bounds__(32 * kSplitkWarps) k_gemm_small_nn_splitk(int 
 __global__ void k_gemm_small(bool ta, bool tb, int m, int p, int kk, double alpha, const double* __restrict__ A,
                              int lda, const double* __restrict__ B, int ldb, double beta, double* __restrict__ C,
                              int ldc) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(B); PDL_ARG(C);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= m || j >= p) return;
@@ -453,6 +471,8 @@ constexpr double kCholWeak = 1e-10;
 template <int NC>
 __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg, double* Rinv, double rank_tol,
                                                        double piv_min2, int* status, int* lost) {
+    PDL_ENTER();
+    PDL_ARG(G); PDL_ARG(Rinv); PDL_ARG(status); PDL_ARG(lost);
     constexpr int NR = 4 * NC;               // rows per warp
     __shared__ double urow[2][32 * NC];      // the pivot row: G's part c >= j, the inverse's part c < j
     __shared__ double ginv[2];               // 1 / pivot, 0 where the pivot is lost
@@ -587,6 +607,8 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
 // The same by one CTA in global memory, for any b: two divisions a column and a back substitution.
 __global__ void k_chol_inv(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2, int* status,
                            int* lost) {
+    PDL_WAIT();
+    PDL_ARG(G); PDL_ARG(Rinv); PDL_ARG(status); PDL_ARG(lost);
     __shared__ double maxdiag;
     __shared__ int nlost;
     __shared__ double piv;
@@ -673,6 +695,8 @@ constexpr int kCholPairMax = 96;
 template <class Ti, class To>
 __global__ void k_copy(int64_t rows, int cols, const Ti* __restrict__ A, int64_t lda, To* __restrict__ B,
                        int64_t ldb) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(B);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= rows * cols) return;
     const int64_t r = e % rows, c = e / rows;
@@ -680,6 +704,8 @@ __global__ void k_copy(int64_t rows, int cols, const Ti* __restrict__ A, int64_t
 }
 
 __global__ void k_symmetrize(int m, double* A, int lda) {
+    PDL_ENTER();
+    PDL_ARG(A);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * m) return;
     const int r = (int)(e % m), c = (int)(e / m);
@@ -700,6 +726,8 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 
 template <class T>
 __global__ void k_fill_gaussian(int64_t rows, int cols, T* A, int64_t lda, uint64_t seed, uint64_t sid) {
+    PDL_ENTER();
+    PDL_ARG(A);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= rows * cols) return;
     const int64_t r = e % rows, c = e / rows;
@@ -712,6 +740,8 @@ __global__ void k_fill_gaussian(int64_t rows, int cols, T* A, int64_t lda, uint6
 
 template <class T>
 __global__ void k_col_norms(int64_t rows, const T* __restrict__ A, int64_t lda, double* out) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(out);
     const int c = blockIdx.x;
     double acc = 0.0;
     for (int64_t r = threadIdx.x; r < rows; r += blockDim.x) {
@@ -761,17 +791,20 @@ int gemm_tn_impl(int64_t d, int m, int p, double alpha, const T* A, int64_t lda,
         const int cap = 32 * (m <= 8 ? 9 : (m <= 16 ? 17 : 33));
         int R = 32;
         while (R * tri > cap) R >>= 1;
-        if (m <= 8) k_syrk_narrow<9, 256, 8, T><<<(unsigned)G, SN_THREADS, 0, s>>>(d, m, A, lda, rw, R, partial);
-        else if (m <= 16) k_syrk_narrow<17, 128, 16, T><<<(unsigned)G, SN_THREADS, 0, s>>>(d, m, A, lda, rw, R, partial);
-        else k_syrk_narrow<33, 64, 32, T><<<(unsigned)G, SN_THREADS, 0, s>>>(d, m, A, lda, rw, R, partial);
-        EDA_LAUNCHED();
+        if (m <= 8) EDA_CUDA_TRY((launch_spread(k_syrk_narrow<9, 256, 8, T>, dim3((unsigned)G), dim3(SN_THREADS), 0, s,
+            d, m, A, lda, rw, R, partial)));
+        else if (m <= 16) EDA_CUDA_TRY((launch_spread(k_syrk_narrow<17, 128, 16, T>, dim3((unsigned)G), dim3(SN_THREADS),
+            0, s, d, m, A, lda, rw, R, partial)));
+        else EDA_CUDA_TRY((launch_spread(k_syrk_narrow<33, 64, 32, T>, dim3((unsigned)G), dim3(SN_THREADS), 0, s, d, m,
+            A, lda, rw, R, partial)));
         const int64_t out = (int64_t)m * m;
         if (G >= 16)
-            k_gemm_tn_reduce_warp<T><<<ceil_div(out * 32, 256), 256, 0, s>>>(m, m, (int)G, partial, alpha, beta, C, ldc,
-                                                                            true);
+            EDA_CUDA_TRY((launch_chained(k_gemm_tn_reduce_warp<T>, dim3(ceil_div(out * 32, 256)), dim3(256), 0, s, m, m,
+                (int)G, partial, alpha, beta, C, ldc,
+            true)));
         else
-            k_gemm_tn_reduce<T><<<ceil_div(out, 256), 256, 0, s>>>(m, m, (int)G, partial, alpha, beta, C, ldc, true);
-        EDA_LAUNCHED();
+            EDA_CUDA_TRY((launch_chained(k_gemm_tn_reduce<T>, dim3(ceil_div(out, 256)), dim3(256), 0, s, m, m, (int)G,
+                partial, alpha, beta, C, ldc, true)));
         return EDA_OK;
     }
     // Split count: the kernel is FP64- or bandwidth-bound per SM, so an SM holding one CTA more than
@@ -803,24 +836,28 @@ int gemm_tn_impl(int64_t d, int m, int p, double alpha, const T* A, int64_t lda,
     if (d > 0) {
         if (sym) {
             dim3 grid(tiles, 1, splits);
-            k_gemm_tn_partial<32, T, true><<<grid, TN_THREADS, 0, s>>>(d, m, p, A, lda, B, ldb, rows, partial);
+            EDA_CUDA_TRY((launch_spread(k_gemm_tn_partial<32, T, true>, grid, dim3(TN_THREADS), 0, s, d, m, p, A, lda, B,
+                ldb, rows, partial)));
         } else {
             dim3 grid(tm, ceil_div(p, TP), splits);
-            if (TP == 8) k_gemm_tn_partial<8, T><<<grid, TN_THREADS, 0, s>>>(d, m, p, A, lda, B, ldb, rows, partial);
-            else if (TP == 16) k_gemm_tn_partial<16, T><<<grid, TN_THREADS, 0, s>>>(d, m, p, A, lda, B, ldb, rows, partial);
-            else k_gemm_tn_partial<32, T><<<grid, TN_THREADS, 0, s>>>(d, m, p, A, lda, B, ldb, rows, partial);
+            if (TP == 8) EDA_CUDA_TRY((launch_spread(k_gemm_tn_partial<8, T>, grid, dim3(TN_THREADS), 0, s, d, m, p, A,
+                lda, B, ldb, rows, partial)));
+            else if (TP == 16) EDA_CUDA_TRY((launch_spread(k_gemm_tn_partial<16, T>, grid, dim3(TN_THREADS), 0, s, d, m,
+                p, A, lda, B, ldb, rows, partial)));
+            else EDA_CUDA_TRY((launch_spread(k_gemm_tn_partial<32, T>, grid, dim3(TN_THREADS), 0, s, d, m, p, A, lda, B,
+                ldb, rows, partial)));
         }
-        EDA_LAUNCHED();
     } else {
         splits = 0;
     }
     const int64_t tot = (int64_t)m * p;
     if (splits >= 16 && tot <= 65536)
-        k_gemm_tn_reduce_warp<T><<<ceil_div(tot * 32, 256), 256, 0, s>>>(m, p, splits, partial, alpha, beta, C, ldc,
-                                                                          sym);
+        EDA_CUDA_TRY((launch_chained(k_gemm_tn_reduce_warp<T>, dim3(ceil_div(tot * 32, 256)), dim3(256), 0, s, m, p,
+            splits, partial, alpha, beta, C, ldc,
+            sym)));
     else
-        k_gemm_tn_reduce<T><<<ceil_div(tot, 256), 256, 0, s>>>(m, p, splits, partial, alpha, beta, C, ldc, sym);
-    EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_gemm_tn_reduce<T>, dim3(ceil_div(tot, 256)), dim3(256), 0, s, m, p, splits,
+            partial, alpha, beta, C, ldc, sym)));
     return EDA_OK;
 }
 
@@ -870,39 +907,41 @@ int gemm_nn(int64_t d, int m, int p, double alpha, const T* A, int64_t lda, cons
     const int rowblocks = ceil_div(d, 32);
     // columns per thread: as many as possible while at least ~one CTA per SM stays busy
     if (p >= 6 && (int64_t)rowblocks * ceil_div(p, 8) >= 120) {
-        k_gemm_nn<8, T><<<dim3(rowblocks, ceil_div(p, 8)), 256, 0, s>>>(d, m, p, alpha, A, lda, B, ldb, beta, C0, ldc0, C, ldc, ub);
+        EDA_CUDA_TRY((launch_spread(k_gemm_nn<8, T>, dim3(rowblocks, ceil_div(p, 8)), dim3(256), 0, s, d, m, p, alpha, A,
+            lda, B, ldb, beta, C0, ldc0, C, ldc, ub)));
     } else if (p >= 3 && (int64_t)rowblocks * ceil_div(p, 4) >= 120) {
-        k_gemm_nn<4, T><<<dim3(rowblocks, ceil_div(p, 4)), 256, 0, s>>>(d, m, p, alpha, A, lda, B, ldb, beta, C0, ldc0, C, ldc, ub);
+        EDA_CUDA_TRY((launch_spread(k_gemm_nn<4, T>, dim3(rowblocks, ceil_div(p, 4)), dim3(256), 0, s, d, m, p, alpha, A,
+            lda, B, ldb, beta, C0, ldc0, C, ldc, ub)));
     } else if (p >= 2) {
-        k_gemm_nn<2, T><<<dim3(rowblocks, ceil_div(p, 2)), 256, 0, s>>>(d, m, p, alpha, A, lda, B, ldb, beta, C0, ldc0, C, ldc, ub);
+        EDA_CUDA_TRY((launch_spread(k_gemm_nn<2, T>, dim3(rowblocks, ceil_div(p, 2)), dim3(256), 0, s, d, m, p, alpha, A,
+            lda, B, ldb, beta, C0, ldc0, C, ldc, ub)));
     } else {
-        k_gemm_nn<1, T><<<dim3(rowblocks, p), 256, 0, s>>>(d, m, p, alpha, A, lda, B, ldb, beta, C0, ldc0, C, ldc, ub);
+        EDA_CUDA_TRY((launch_spread(k_gemm_nn<1, T>, dim3(rowblocks, p), dim3(256), 0, s, d, m, p, alpha, A, lda, B, ldb,
+            beta, C0, ldc0, C, ldc, ub)));
     }
-    EDA_LAUNCHED();
     return EDA_OK;
 }
 
 template <class Ti, class To>
 int copy_mat(int64_t rows, int cols, const Ti* A, int64_t lda, To* B, int64_t ldb, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return EDA_OK;
-    k_copy<Ti, To><<<ceil_div(rows * cols, 256), 256, 0, s>>>(rows, cols, A, lda, B, ldb);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_copy<Ti, To>, dim3(ceil_div(rows * cols, 256)), dim3(256), 0, s, rows, cols, A, lda,
+        B, ldb)));
     return EDA_OK;
 }
 
 template <class T>
 int fill_gaussian(int64_t rows, int cols, T* A, int64_t lda, uint64_t seed, uint64_t stream_id, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return EDA_OK;
-    k_fill_gaussian<T><<<ceil_div(rows * cols, 256), 256, 0, s>>>(rows, cols, A, lda, seed, stream_id);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_fill_gaussian<T>, dim3(ceil_div(rows * cols, 256)), dim3(256), 0, s, rows, cols, A,
+        lda, seed, stream_id)));
     return EDA_OK;
 }
 
 template <class T>
 int col_norms(int64_t rows, int cols, const T* A, int64_t lda, double* out, cudaStream_t s) {
     if (cols <= 0) return EDA_OK;
-    k_col_norms<T><<<cols, 256, 0, s>>>(rows, A, lda, out);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_col_norms<T>, dim3(cols), dim3(256), 0, s, rows, A, lda, out)));
     return EDA_OK;
 }
 
@@ -946,15 +985,14 @@ int gemm_small_f64(bool ta, bool tb, int m, int p, int kk, double alpha, const d
                    int ldb, double beta, double* C, int ldc, cudaStream_t s) {
     if (m <= 0 || p <= 0) return EDA_OK;
     if (!ta && !tb && kk >= 64) {
-        k_gemm_small_nn_splitk<false><<<dim3(ceil_div(m, 32), p), 32 * kSplitkWarps, 0, s>>>(m, p, kk, alpha, A, lda, B, ldb,
-                                                                                  beta, C, ldc);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_gemm_small_nn_splitk<false>, dim3(ceil_div(m, 32), p), dim3(32 * kSplitkWarps), 0,
+            s, m, p, kk, alpha, A, lda, B, ldb,
+            beta, C, ldc)));
         return EDA_OK;
     }
     // one warp per CTA (32 rows of one column): FP64 work spreads over all SMs
     dim3 blk(32, 1), grid(ceil_div(m, 32), p);
-    k_gemm_small<<<grid, blk, 0, s>>>(ta, tb, m, p, kk, alpha, A, lda, B, ldb, beta, C, ldc);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_spread(k_gemm_small, grid, blk, 0, s, ta, tb, m, p, kk, alpha, A, lda, B, ldb, beta, C, ldc)));
     return EDA_OK;
 }
 
@@ -962,35 +1000,42 @@ int gemm_small_sym_f64(int m, double alpha, const double* A, int lda, const doub
                        int ldc, cudaStream_t s) {
     if (m < 64) return gemm_small_f64(false, false, m, m, m, alpha, A, lda, B, ldb, beta, C, ldc, s);
     const int nb = ceil_div(m, 32);
-    k_gemm_small_nn_splitk<true><<<32 * (nb * (nb + 1) / 2), 32 * kSplitkWarps, 0, s>>>(m, m, m, alpha, A, lda, B, ldb,
-                                                                                      beta, C, ldc);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_spread(k_gemm_small_nn_splitk<true>, dim3(32 * (nb * (nb + 1) / 2)), dim3(32 * kSplitkWarps), 0,
+        s, m, m, m, alpha, A, lda, B, ldb,
+            beta, C, ldc)));
     return EDA_OK;
 }
 
 int chol_inv_small(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2, int* status, int* lost,
                    cudaStream_t s) {
     if (b <= 32)
-        k_chol_inv_pair<1><<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
+        EDA_CUDA_TRY((launch_chained(k_chol_inv_pair<1>, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2,
+            status, lost)));
     else if (b <= 64)
-        k_chol_inv_pair<2><<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
+        EDA_CUDA_TRY((launch_chained(k_chol_inv_pair<2>, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2,
+            status, lost)));
     else if (b <= kCholPairMax)
-        k_chol_inv_pair<3><<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
+        EDA_CUDA_TRY((launch_chained(k_chol_inv_pair<3>, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2,
+            status, lost)));
     else
-        k_chol_inv<<<1, 256, 0, s>>>(b, G, ldg, Rinv, rank_tol, piv_min2, status, lost);
-    EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_chol_inv, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2, status,
+            lost)));
     return EDA_OK;
 }
 
 namespace {
 // B (rows x cols, ldb) = 0 below the diagonal (strict lower triangle of a square or tall block)
 __global__ void k_zero_lower(int m, double* A, int lda) {
+    PDL_ENTER();
+    PDL_ARG(A);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * m) return;
     const int r = (int)(e % m), c = (int)(e / m);
     if (r > c) A[(int64_t)c * lda + r] = 0.0;
 }
 __global__ void k_zero_all(int m, double* A, int lda) {
+    PDL_ENTER();
+    PDL_ARG(A);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * m) return;
     A[(int64_t)(e / m) * lda + e % m] = 0.0;
@@ -1010,8 +1055,7 @@ int chol_inv_blocked(int m, double* G, int ldg, double* Rinv, int ldr, double ra
     double* T = work;                          // NB x m
     double* Dinv = work + (size_t)NB * m;      // NB x NB
     // R^{-1} starts as zero: its blocks below the block diagonal are never written and are read as zeros
-    k_zero_all<<<ceil_div((int64_t)m * m, 256), 256, 0, s>>>(m, Rinv, ldr);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_zero_all, dim3(ceil_div((int64_t)m * m, 256)), dim3(256), 0, s, m, Rinv, ldr)));
     for (int j0 = 0; j0 < m; j0 += NB) {
         const int nb = std::min(NB, m - j0);
         double* G11 = G + (int64_t)j0 * ldg + j0;
@@ -1029,8 +1073,7 @@ int chol_inv_blocked(int m, double* G, int ldg, double* Rinv, int ldr, double ra
             EDA_TRY(gemm_tn_f64(nb, r, r, -1.0, G12, ldg, G12, ldg, 1.0, G22, ldg, partial, pcap, s));
         }
     }
-    k_zero_lower<<<ceil_div((int64_t)m * m, 256), 256, 0, s>>>(m, G, ldg);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_zero_lower, dim3(ceil_div((int64_t)m * m, 256)), dim3(256), 0, s, m, G, ldg)));
     // off-diagonal blocks of R^{-1}: X[:j0, j-block] = -X[:j0, :j0] (R[:j0, j-block] R_jj^{-1})
     for (int j0 = NB; j0 < m; j0 += NB) {
         const int nb = std::min(NB, m - j0);
@@ -1055,8 +1098,7 @@ int copy_mat_f64(int64_t rows, int cols, const double* A, int64_t lda, double* B
 
 int symmetrize_f64(int m, double* A, int lda, cudaStream_t s) {
     if (m <= 1) return EDA_OK;
-    k_symmetrize<<<ceil_div((int64_t)m * m, 256), 256, 0, s>>>(m, A, lda);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_symmetrize, dim3(ceil_div((int64_t)m * m, 256)), dim3(256), 0, s, m, A, lda)));
     return EDA_OK;
 }
 

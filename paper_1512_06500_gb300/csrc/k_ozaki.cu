@@ -86,6 +86,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
               const OzBTiles bt, const int* __restrict__ expA, const int* __restrict__ expB, int M, int N, int kst,
               int kps, double alpha, double beta, const double* C0, int64_t ldc0, double* D, int64_t ldd,
               int64_t split_stride, int* status) {
+    PDL_WAIT();
+    PDL_ARG(At); PDL_ARG(expA); PDL_ARG(expB); PDL_ARG(C0); PDL_ARG(D); PDL_ARG(status);
     extern __shared__ unsigned char smraw[];
     OzRing& sm = oz_ring(smraw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -242,6 +244,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             mbar_wait(&sm.fullB[i % OZ_BST], (i / OZ_BST) & 1, status);
     }
     __syncthreads();
+    PDL_NEXT();
     if (warp >= 4) {
         const int i = band * TC_M + 32 * (warp - 4) + lane;
         if (i < M) {
@@ -351,6 +354,8 @@ constexpr int kOzExpPer = 8;
 constexpr int kOzExpChunk = kOzExpThreads * kOzExpPer;
 __global__ void __launch_bounds__(kOzExpThreads) k_oz_exp_cols(int64_t rows, const double* __restrict__ A,
                                                               int64_t lda, int* __restrict__ e) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(e);
     __shared__ int wmax[kOzExpThreads / 32];
     const int c = blockIdx.x;
     const double* col = A + (int64_t)c * lda;
@@ -380,6 +385,8 @@ __global__ void __launch_bounds__(kOzExpThreads) k_oz_exp_cols(int64_t rows, con
 constexpr int kOzRowChunk = 64;
 __global__ void __launch_bounds__(256) k_oz_exp_rows(int64_t rows, int cols, const double* __restrict__ A, int64_t lda,
                                                     int* __restrict__ e) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(e);
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
     const int c0 = blockIdx.y * kOzRowChunk, c1 = min(cols, c0 + kOzRowChunk);
@@ -404,6 +411,8 @@ constexpr int OZ_NARROW_CL = 8;
 __global__ void __cluster_dims__(OZ_NARROW_CL, 1, 1) __launch_bounds__(256)
     k_oz_narrow(int64_t K, int p, const double* __restrict__ B, int64_t ldb, int* __restrict__ e, int64_t ld,
                 __nv_bfloat16* __restrict__ out, int* __restrict__ status) {
+    PDL_ENTER();
+    PDL_ARG(B); PDL_ARG(e); PDL_ARG(out); PDL_ARG(status);
     namespace cg = cooperative_groups;
     __shared__ int wmax[8];
     __shared__ int cmax;
@@ -455,6 +464,8 @@ __global__ void __cluster_dims__(OZ_NARROW_CL, 1, 1) __launch_bounds__(256)
 __global__ void k_oz_split_cols8(const double* __restrict__ A, int64_t lda, int i0, int i1, int Mvalid, int64_t K,
                                  const int* __restrict__ e, int kbs, int64_t ld, __nv_bfloat16* __restrict__ out,
                                  int64_t slice, int* __restrict__ status) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(e); PDL_ARG(out); PDL_ARG(status);
     const int64_t groups = ld / 8;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)(i1 - i0) * groups) return;
@@ -486,6 +497,8 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(const double* __restrict_
                                                       const int* __restrict__ e, int kbs, int kst,
                                                       __nv_bfloat16* __restrict__ out, int64_t slice,
                                                       int* __restrict__ status) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(e); PDL_ARG(out); PDL_ARG(status);
     __shared__ __align__(16) uint4 img[OZ_S][32 * 8];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t i0 = (int64_t)(blockIdx.x / kst) * 32, i = i0 + lane;
@@ -517,6 +530,8 @@ __global__ void __launch_bounds__(256) k_oz_split_rows(const double* __restrict_
 __global__ void k_oz_grow_rows(const double* __restrict__ A, int64_t lda, int64_t M, int64_t k0, int64_t k1,
                                int* __restrict__ e, int kbs, __nv_bfloat16* __restrict__ out, int64_t slice,
                                int* __restrict__ list, int* __restrict__ status) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(e); PDL_ARG(out); PDL_ARG(list); PDL_ARG(status);
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M) return;
     int mnew = kOzExpZero;
@@ -551,6 +566,8 @@ __global__ void k_oz_grow_rows(const double* __restrict__ A, int64_t lda, int64_
 __global__ void k_oz_resplit_listed(const double* __restrict__ A, int64_t lda, int64_t K, const int* __restrict__ e,
                                     int kbs, __nv_bfloat16* __restrict__ out, int64_t slice,
                                     const int* __restrict__ list, int* __restrict__ status) {
+    PDL_WAIT();
+    PDL_ARG(A); PDL_ARG(e); PDL_ARG(out); PDL_ARG(list); PDL_ARG(status);
     const int64_t groups = (K + TC_KS - 1) / TC_KS * (TC_KS / 8);   // whole tiles: zeros beyond K
     const int64_t total = (int64_t)list[0] * groups;
     bool fin = true;
@@ -577,6 +594,8 @@ __global__ void k_oz_resplit_listed(const double* __restrict__ A, int64_t lda, i
 // D[i, j] = alpha * sum_s P[s][j][i] + beta * D[i, j], splits added in order (deterministic).
 __global__ void k_oz_reduce(int M, int N, int splits, const double* __restrict__ P, int64_t sstride, double alpha,
                             double beta, const double* C0, int64_t ldc0, double* D, int64_t ldd) {
+    PDL_ENTER();
+    PDL_ARG(P); PDL_ARG(C0); PDL_ARG(D);
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)M * N) return;
     const int i = (int)(t % M), j = (int)(t / M);
@@ -614,8 +633,7 @@ static int oz_col_exps(int64_t K, const double* A, int64_t lda, int ncols, int* 
     if (ncols <= 0) return EDA_OK;
     EDA_CUDA_TRY(cudaMemsetAsync(e, 0xC0, (size_t)ncols * sizeof(int), s));   // kOzExpZero in every entry
     const dim3 grid((unsigned)ncols, (unsigned)ceil_div(std::max<int64_t>(K, 1), kOzExpChunk));
-    k_oz_exp_cols<<<grid, kOzExpThreads, 0, s>>>(K, A, lda, e);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_oz_exp_cols, grid, dim3(kOzExpThreads), 0, s, K, A, lda, e)));
     return EDA_OK;
 }
 
@@ -624,8 +642,8 @@ static int oz_row_exps(int64_t M, int64_t K, const double* A, int64_t lda, int* 
     if (M <= 0) return EDA_OK;
     EDA_CUDA_TRY(cudaMemsetAsync(e, 0xC0, (size_t)M * sizeof(int), s));   // kOzExpZero in every entry
     if (K <= 0) return EDA_OK;
-    k_oz_exp_rows<<<dim3((unsigned)ceil_div(M, 256), (unsigned)ceil_div(K, kOzRowChunk)), 256, 0, s>>>(M, (int)K, A, lda, e);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_oz_exp_rows, dim3((unsigned)ceil_div(M, 256), (unsigned)ceil_div(K, kOzRowChunk)),
+        dim3(256), 0, s, M, (int)K, A, lda, e)));
     return EDA_OK;
 }
 
@@ -644,14 +662,15 @@ int oz_operand_make(const double* A, int64_t lda, int64_t M, int64_t K, bool row
     const int64_t ld = kb * TC_KS, mpad = mt * TC_M;
     if (rows_are_cols) {
         EDA_TRY(oz_col_exps(K, A, lda, (int)M, op->exps, s));
-        k_oz_split_cols8<<<ceil_div(mpad * (ld / 8), 256), 256, 0, s>>>(A, lda, 0, (int)mpad, (int)M, K, op->exps,
-                                                                        (int)kb, ld, op->tiles, slice, status);
+        EDA_CUDA_TRY((launch_chained(k_oz_split_cols8, dim3(ceil_div(mpad * (ld / 8), 256)), dim3(256), 0, s, A, lda, 0,
+            (int)mpad, (int)M, K, op->exps,
+            (int)kb, ld, op->tiles, slice, status)));
     } else {
         EDA_TRY(oz_row_exps(M, K, A, lda, op->exps, s));
-        k_oz_split_rows<<<(unsigned)(mpad / 32 * kb), 256, 0, s>>>(A, lda, M, K, op->exps, (int)kb, (int)kb, op->tiles,
-                                                                   slice, status);
+        EDA_CUDA_TRY((launch_chained(k_oz_split_rows, dim3((unsigned)(mpad / 32 * kb)), dim3(256), 0, s, A, lda, M, K,
+            op->exps, (int)kb, (int)kb, op->tiles,
+            slice, status)));
     }
-    EDA_LAUNCHED();
     return EDA_OK;
 }
 
@@ -679,9 +698,8 @@ int oz_append_cols(const double* A, int64_t lda, int i0, int i1, int64_t K, OzOp
     if (i1 <= i0) return EDA_OK;
     EDA_TRY(oz_col_exps(K, A + (int64_t)i0 * lda, lda, i1 - i0, op->exps + i0, s));
     const int64_t ld = (int64_t)op->kbs * TC_KS;
-    k_oz_split_cols8<<<ceil_div((int64_t)(i1 - i0) * (ld / 8), 256), 256, 0, s>>>(
-        A, lda, i0, i1, i1, K, op->exps + i0, op->kbs, ld, op->tiles, op->slice, status);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_oz_split_cols8, dim3(ceil_div((int64_t)(i1 - i0) * (ld / 8), 256)), dim3(256), 0, s,
+        A, lda, i0, i1, i1, K, op->exps + i0, op->kbs, ld, op->tiles, op->slice, status)));
     op->M = i1;
     op->K = K;
     op->mtiles = ceil_div(i1, TC_M);
@@ -692,12 +710,12 @@ int oz_grow_rows(const double* A, int64_t lda, int64_t M, int64_t k0, int64_t k1
                  int* status, cudaStream_t s) {
     if (k1 <= k0) return EDA_OK;
     EDA_CUDA_TRY(cudaMemsetAsync(list, 0, sizeof(int), s));
-    k_oz_grow_rows<<<ceil_div(M, 256), 256, 0, s>>>(A, lda, M, k0, k1, op->exps, op->kbs, op->tiles, op->slice, list,
-                                                    status);
-    EDA_LAUNCHED();
-    k_oz_resplit_listed<<<2 * sm_count(), 256, 0, s>>>(A, lda, k1, op->exps, op->kbs, op->tiles, op->slice, list,
-                                                        status);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_oz_grow_rows, dim3(ceil_div(M, 256)), dim3(256), 0, s, A, lda, M, k0, k1, op->exps,
+        op->kbs, op->tiles, op->slice, list,
+            status)));
+    EDA_CUDA_TRY((launch_chained(k_oz_resplit_listed, dim3(2 * sm_count()), dim3(256), 0, s, A, lda, k1, op->exps,
+        op->kbs, op->tiles, op->slice, list,
+            status)));
     op->M = M;
     op->K = k1;
     op->mtiles = ceil_div(M, TC_M);
@@ -738,8 +756,8 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
     // digit planes), B read and D written once in FP64
     ProfScope prof("oz_gemm", s, 2.0 * (double)A.M * A.K * p,
                    2.0 * OZ_S * (double)A.M * A.K + 8.0 * (double)A.K * p + 8.0 * (double)A.M * p);
-    k_oz_narrow<<<dim3(OZ_NARROW_CL, OZ_N), 256, 0, s>>>(A.K, p, B, ldb, nb.exps, ld, nb.planes, status);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_oz_narrow, dim3(OZ_NARROW_CL, OZ_N), dim3(256), 0, s, A.K, p, B, ldb, nb.exps, ld,
+        nb.planes, status)));
     const int kst = (int)(ld / TC_KS);
     // K splits: fill the SMs with one CTA each (the kernel holds all of an SM's tensor memory)
     const int nsm = sm_count();
@@ -756,19 +774,20 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
                         2.0 * OZ_S * ((double)A.M * A.K + (double)A.K * p) + 8.0 * (double)A.M * p);
         const OzBTiles none{};
         if (splits == 1)
-            k_oz_gemm<false><<<grid, OZ_THREADS, oz_smem_bytes(), s>>>(A.tiles, A.slice, A.kbs, nb.map, none, A.exps,
-                                                                       nb.exps, (int)A.M, p, kst, kps, alpha, beta, C0,
-                                                                       ldc0, D, ldd, 0, status);
+            EDA_CUDA_TRY((launch_chained(k_oz_gemm<false>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
+                A.kbs, nb.map, none, A.exps,
+            nb.exps, (int)A.M, p, kst, kps, alpha, beta, C0,
+            ldc0, D, ldd, 0, status)));
         else
-            k_oz_gemm<false><<<grid, OZ_THREADS, oz_smem_bytes(), s>>>(A.tiles, A.slice, A.kbs, nb.map, none, A.exps,
-                                                                       nb.exps, (int)A.M, p, kst, kps, 1.0, 0.0,
-                                                                       nullptr, 0, nb.partial, A.M, sstride, status);
-        EDA_LAUNCHED();
+            EDA_CUDA_TRY((launch_chained(k_oz_gemm<false>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
+                A.kbs, nb.map, none, A.exps,
+            nb.exps, (int)A.M, p, kst, kps, 1.0, 0.0,
+            nullptr, 0, nb.partial, A.M, sstride, status)));
     }
     if (splits == 1) return EDA_OK;
-    k_oz_reduce<<<ceil_div((int64_t)A.M * p, 256), 256, 0, s>>>((int)A.M, p, splits, nb.partial, sstride, alpha,
-                                                                 beta, C0, ldc0, D, ldd);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_oz_reduce, dim3(ceil_div((int64_t)A.M * p, 256)), dim3(256), 0, s, (int)A.M, p,
+        splits, nb.partial, sstride, alpha,
+            beta, C0, ldc0, D, ldd)));
     return EDA_OK;
 }
 
@@ -776,6 +795,8 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
 // one launch over (A band, B 32-row block); upper: only the blocks meeting the upper triangle i <= j, the
 // rest filled by the mirror image (for products that are symmetric; blocks on the diagonal are computed whole).
 __global__ void k_oz_mirror_lower(int n, double* D, int64_t ldd) {
+    PDL_ENTER();
+    PDL_ARG(D);
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)n * n) return;
     const int i = (int)(t % n), j = (int)(t / n);
@@ -823,23 +844,24 @@ int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double b
         // tmB is not read in this mode; the operand's planes are passed in bt
         static const CUtensorMap unused{};
         if (splits == 1)
-            k_oz_gemm<true><<<grid, OZ_THREADS, oz_smem_bytes(), s>>>(A.tiles, A.slice, A.kbs, unused, bt, A.exps,
-                                                                      B.exps, (int)A.M, (int)B.M, kst, kps, alpha, beta,
-                                                                      C0, ldc0, D, ldd, 0, status);
+            EDA_CUDA_TRY((launch_chained(k_oz_gemm<true>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
+                A.kbs, unused, bt, A.exps,
+            B.exps, (int)A.M, (int)B.M, kst, kps, alpha, beta,
+            C0, ldc0, D, ldd, 0, status)));
         else
-            k_oz_gemm<true><<<grid, OZ_THREADS, oz_smem_bytes(), s>>>(A.tiles, A.slice, A.kbs, unused, bt, A.exps,
-                                                                      B.exps, (int)A.M, (int)B.M, kst, kps, 1.0, 0.0,
-                                                                      nullptr, 0, part, A.M, (int64_t)A.M * B.M, status);
-        EDA_LAUNCHED();
+            EDA_CUDA_TRY((launch_chained(k_oz_gemm<true>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
+                A.kbs, unused, bt, A.exps,
+            B.exps, (int)A.M, (int)B.M, kst, kps, 1.0, 0.0,
+            nullptr, 0, part, A.M, (int64_t)A.M * B.M, status)));
     }
     if (splits > 1) {
-        k_oz_reduce<<<ceil_div((int64_t)A.M * B.M, 256), 256, 0, s>>>((int)A.M, (int)B.M, splits, part,
-                                                                     (int64_t)A.M * B.M, alpha, beta, C0, ldc0, D, ldd);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_oz_reduce, dim3(ceil_div((int64_t)A.M * B.M, 256)), dim3(256), 0, s, (int)A.M,
+            (int)B.M, splits, part,
+            (int64_t)A.M * B.M, alpha, beta, C0, ldc0, D, ldd)));
     }
     if (upper) {
-        k_oz_mirror_lower<<<ceil_div((int64_t)A.M * A.M, 256), 256, 0, s>>>((int)A.M, D, ldd);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_oz_mirror_lower, dim3(ceil_div((int64_t)A.M * A.M, 256)), dim3(256), 0, s,
+            (int)A.M, D, ldd)));
     }
     return EDA_OK;
 }

@@ -587,6 +587,8 @@ __device__ __forceinline__ double cubic_root01(double fm, double f0, double f1, 
 // 0.165 -> 0.085.
 __global__ void __launch_bounds__(64) k_bisect(int n, const double* __restrict__ dgl, const double* __restrict__ eoff,
                                                 int il, int nw, double* w) {
+    PDL_WAIT();
+    PDL_ARG(dgl); PDL_ARG(eoff); PDL_ARG(w);
     extern __shared__ double smb[];
     double* d64 = smb;                                     // n
     double* e264 = smb + n;                                // n
@@ -751,6 +753,8 @@ constexpr int IV_U = 8;
 __global__ void __launch_bounds__(32) k_invit(int n, int nv, const double* __restrict__ dgl,
                                               const double* __restrict__ eoff, const double* __restrict__ lam, double* lu,
                                               double* Zt, uint64_t seed) {
+    PDL_WAIT();
+    PDL_ARG(dgl); PDL_ARG(eoff); PDL_ARG(lam); PDL_ARG(lu); PDL_ARG(Zt);
     const int lane = threadIdx.x;
     // ||T||_inf, by the whole warp
     double tn = 0.0;
@@ -902,6 +906,8 @@ __global__ void __launch_bounds__(32) k_invit(int n, int nv, const double* __res
 // Zt (row-major n x nv) times its column factors -> Z (column-major, ldz), by 32 x 32 tiles through shared memory
 __global__ void __launch_bounds__(256) k_transpose_out(int n, int nv, const double* __restrict__ Zt,
                                                        const double* __restrict__ fac, double* __restrict__ Z, int ldz) {
+    PDL_ENTER();
+    PDL_ARG(Zt); PDL_ARG(fac); PDL_ARG(Z);
     __shared__ double t[32][33];
     const int q0 = blockIdx.y * 32, i0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const double f = q0 + lane < nv ? fac[q0 + lane] : 0.0;
@@ -924,6 +930,8 @@ constexpr int WY_B = 32;
 
 // Upper triangles of V^T V of every block: G[kb][i][k], i < k. grid (blocks, 8): four rows i each; a warp per product.
 __global__ void __launch_bounds__(256) k_wy_gram(int n, const double* __restrict__ HV, double* __restrict__ G) {
+    PDL_WAIT();
+    PDL_ARG(HV); PDL_ARG(G);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int j0 = blockIdx.x * WY_B, m = min(WY_B, n - 2 - j0);
     double* g = G + (size_t)blockIdx.x * WY_B * WY_B;
@@ -971,6 +979,8 @@ template <int NC>
 __global__ void __launch_bounds__(256) k_wy_apply(int n, int nv, const double* __restrict__ HV,
                                                   const double* __restrict__ tau, const double* __restrict__ G, double* Z,
                                                   int ldz) {
+    PDL_WAIT();
+    PDL_ARG(HV); PDL_ARG(tau); PDL_ARG(G); PDL_ARG(Z);
     constexpr int NP = NC <= 1 ? 1 : (NC <= 2 ? 2 : (NC <= 4 ? 4 : 8));
     extern __shared__ double sz[];               // NC x n: this CTA's columns
     __shared__ double xs[WY_B][NC];              // V^T Z of the block, then U^{-1} V^T Z
@@ -1039,6 +1049,7 @@ __global__ void __launch_bounds__(256) k_wy_apply(int n, int nv, const double* _
         }
         __syncthreads();
     }
+    PDL_NEXT();
     for (int c = 0; c < nc; ++c)
         for (int i = tid; i < n; i += 256) Z[(int64_t)(q0 + c) * ldz + i] = sz[c * n + i];
 }
@@ -1053,6 +1064,8 @@ __global__ void __launch_bounds__(256) k_wy_apply(int n, int nv, const double* _
 template <int NPL>
 __global__ void __launch_bounds__(128) k_backtransform_w4(int n, int nv, const double* __restrict__ HV,
                                                           const double* __restrict__ tau, double* Z, int ldz) {
+    PDL_WAIT();
+    PDL_ARG(HV); PDL_ARG(tau); PDL_ARG(Z);
     __shared__ double red[2][4];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int col = blockIdx.x;
@@ -1252,6 +1265,8 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(int n, const double* __r
 constexpr int LZG_THREADS = 256;
 __global__ void k_lz_start(int n, uint64_t seed, double* __restrict__ v, double* __restrict__ vprev,
                            double* __restrict__ st) {
+    PDL_ENTER();
+    PDL_ARG(v); PDL_ARG(vprev); PDL_ARG(st);
     __shared__ double red[32];
     double ss = 0.0;
     for (int c = threadIdx.x; c < n; c += blockDim.x) {
@@ -1273,6 +1288,8 @@ __global__ void k_lz_start(int n, uint64_t seed, double* __restrict__ v, double*
 
 __global__ void k_lz_matvec(int n, const double* __restrict__ A, int lda, const double* __restrict__ v,
                             double* __restrict__ u, const double* __restrict__ st) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(v); PDL_ARG(u); PDL_ARG(st);
     if (st[2] != 0.0) return;
     const int row = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (row >= n) return;
@@ -1288,6 +1305,8 @@ __global__ void k_lz_matvec(int n, const double* __restrict__ A, int lda, const 
 __global__ void __launch_bounds__(LZG_THREADS) k_lz_update(int n, int j, double* __restrict__ u,
                                                            const double* __restrict__ v, double* __restrict__ vprev,
                                                            double* __restrict__ st, double* dgl, double* eoff) {
+    PDL_ENTER();
+    PDL_ARG(u); PDL_ARG(v); PDL_ARG(vprev); PDL_ARG(st); PDL_ARG(dgl); PDL_ARG(eoff);
     __shared__ double red[32];
     if (st[2] != 0.0) {
         if (threadIdx.x == 0) {
@@ -1331,6 +1350,8 @@ __global__ void __launch_bounds__(LZG_THREADS) k_lz_update(int n, int j, double*
 // (z: the inverse-iteration vector before its normalisation by *fac).
 __global__ void k_lanczos_pack(int m, const double* w, const double* z, const double* fac, const double* eoff,
                                double* out) {
+    PDL_ENTER();
+    PDL_ARG(w); PDL_ARG(z); PDL_ARG(fac); PDL_ARG(eoff); PDL_ARG(out);
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     out[0] = w[m >= 2 ? 1 : 0];
     out[1] = (m >= 2) ? w[0] : -DBL_MAX;
@@ -1339,6 +1360,8 @@ __global__ void k_lanczos_pack(int m, const double* w, const double* z, const do
 }
 
 __global__ void k_copy_sq(int n, const double* A, int lda, double* B) {
+    PDL_ENTER();
+    PDL_ARG(A); PDL_ARG(B);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)n * n) return;
     const int r = (int)(e % n), c = (int)(e / n);
@@ -1554,8 +1577,7 @@ int symeig_values(int n, const double* A, int lda, int il, int iu, double* w, Sy
     ctas = std::min(ctas, std::max(1, per_sm * sms));
     double* pglob = ws->vbuf;
     EDA_CUDA_TRY(cudaMemsetAsync(ws->bar.count, 0, sizeof(unsigned), s));
-    k_copy_sq<<<ceil_div((int64_t)n * n, 256), 256, 0, s>>>(n, A, lda, ws->A);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_copy_sq, dim3(ceil_div((int64_t)n * n, 256)), dim3(256), 0, s, n, A, lda, ws->A)));
     {
         ProfScope prof("tridiag", s, 4.0 / 3.0 * (double)n * n * n);
         int nn = n;
@@ -1587,8 +1609,7 @@ int symeig_values(int n, const double* A, int lda, int il, int iu, double* w, Sy
     {
         ProfScope prof("bisect", s);
         // one warp per CTA: the FP64 pipe of one SM is narrow, so the warps are spread over SMs
-        k_bisect<<<nv, 64, bsm, s>>>(n, ws->dgl, ws->eoff, il, nv, w);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_bisect, dim3(nv), dim3(64), bsm, s, n, ws->dgl, ws->eoff, il, nv, w)));
     }
     return EDA_OK;
 }
@@ -1600,12 +1621,12 @@ int invit_vectors(int n, int nv, const double* w, double* Z, int ldz, SymEigWork
     double* Zt = ws->lu + 5 * (size_t)n * nv;
     {
         ProfScope prof("invit", s);
-        k_invit<<<ceil_div(nv, 32), 32, 0, s>>>(n, nv, ws->dgl, ws->eoff, w, lu, Zt, seed);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_invit, dim3(ceil_div(nv, 32)), dim3(32), 0, s, n, nv, ws->dgl, ws->eoff, w, lu,
+            Zt, seed)));
     }
     // the normalisation factors: row 0 of the reciprocal pivots
-    k_transpose_out<<<dim3(ceil_div(n, 32), ceil_div(nv, 32)), 256, 0, s>>>(n, nv, Zt, lu + (size_t)n * nv, Z, ldz);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_transpose_out, dim3(ceil_div(n, 32), ceil_div(nv, 32)), dim3(256), 0, s, n, nv, Zt,
+        lu + (size_t)n * nv, Z, ldz)));
     return EDA_OK;
 }
 }  // namespace
@@ -1629,6 +1650,8 @@ int symeig_f64(int n, const double* A, int lda, int il, int iu, double* w, doubl
 // Cluster MGS with a tolerance relative to max |lambda|, computed on the device.
 namespace {
 __global__ void k_cluster_scale(int nv, const double* lam, double rel, double* out) {
+    PDL_ENTER();
+    PDL_ARG(lam); PDL_ARG(out);
     double m = 0.0;
     for (int i = threadIdx.x; i < nv; i += 32) m = fmax(m, fabs(lam[i]));
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -1641,6 +1664,8 @@ __global__ void k_cluster_scale(int nv, const double* lam, double rel, double* o
 // vectors of a tight cluster keep their content above the rounding level.
 constexpr int kClusterBlock = 16;
 __global__ void __launch_bounds__(512) k_cluster_block_cgs2(int n, double* Z, int ldz, int bs) {
+    PDL_WAIT();
+    PDL_ARG(Z);
     __shared__ double dots[kClusterBlock];
     __shared__ double red[16];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1683,6 +1708,8 @@ __global__ void __launch_bounds__(512) k_cluster_block_cgs2(int n, double* Z, in
 // one warp per run; runs of maxc or more columns are left to the block path.
 __global__ void k_cluster_mgs_dev(int n, int nv, const double* lam, const double* ctol_dev, double* Z, int ldz,
                                   int maxc) {
+    PDL_ENTER();
+    PDL_ARG(lam); PDL_ARG(ctol_dev); PDL_ARG(Z);
     const double ctol = ctol_dev[0];
     const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -1723,10 +1750,9 @@ __global__ void k_cluster_mgs_dev(int n, int nv, const double* lam, const double
 int symeig_orth_clusters(int n, int nv, const double* w, double* Z, int ldz, SymEigWork* ws, double cluster_rel,
                          int maxc, cudaStream_t s) {
     double* ctol = ws->vbuf + 2 * n;
-    k_cluster_scale<<<1, 32, 0, s>>>(nv, w, cluster_rel, ctol);
-    EDA_LAUNCHED();
-    k_cluster_mgs_dev<<<ceil_div((int64_t)nv * 32, 256), 256, 0, s>>>(n, nv, w, ctol, Z, ldz, maxc);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_cluster_scale, dim3(1), dim3(32), 0, s, nv, w, cluster_rel, ctol)));
+    EDA_CUDA_TRY((launch_chained(k_cluster_mgs_dev, dim3(ceil_div((int64_t)nv * 32, 256)), dim3(256), 0, s, n, nv, w,
+        ctol, Z, ldz, maxc)));
     if (maxc == INT_MAX || nv < maxc) return EDA_OK;
     std::vector<double> wh(nv);
     EDA_TRY(read_back(wh.data(), w, nv * sizeof(double), s));
@@ -1760,8 +1786,7 @@ int symeig_orth_clusters(int n, int nv, const double* w, double* Z, int ldz, Sym
                 EDA_TRY(gemm_tn_f64(n, prev, bs, 1.0, Zq, ldz, Zj, ldz, 0.0, C, prev, part, pcap, s));
                 EDA_TRY(gemm_nn_f64(n, prev, bs, -1.0, Zq, ldz, C, prev, 1.0, Zj, ldz, Zj, ldz, s));
             }
-            k_cluster_block_cgs2<<<1, 512, 0, s>>>(n, Zj, ldz, bs);
-            EDA_LAUNCHED();
+            EDA_CUDA_TRY((launch_chained(k_cluster_block_cgs2, dim3(1), dim3(512), 0, s, n, Zj, ldz, bs)));
         }
     }
     return EDA_OK;
@@ -1782,8 +1807,8 @@ int wy_apply(int n, int nv, double* Z, int ldz, SymEigWork* ws, cudaStream_t s) 
             set = smem;
         }
     }
-    k_wy_apply<NC><<<ceil_div(nv, NC), 256, smem, s>>>(n, nv, ws->partial, ws->tau, ws->A, Z, ldz);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_spread(k_wy_apply<NC>, dim3(ceil_div(nv, NC)), dim3(256), smem, s, n, nv, ws->partial, ws->tau,
+        ws->A, Z, ldz)));
     return EDA_OK;
 }
 }  // namespace
@@ -1792,13 +1817,11 @@ int symeig_backtransform(int n, int nv, double* Z, int ldz, SymEigWork* ws, cuda
     if (n < 3) return EDA_OK;
     ProfScope prof("backtransform", s);
     if (n < kWyMinN) {
-        k_backtransform_w4<2><<<nv, 128, 0, s>>>(n, nv, ws->partial, ws->tau, Z, ldz);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_spread(k_backtransform_w4<2>, dim3(nv), dim3(128), 0, s, n, nv, ws->partial, ws->tau, Z, ldz)));
         return EDA_OK;
     }
     // the blocks' triangles go into the matrix copy, which the reduction has done with (n^2 + 16 n doubles hold them)
-    k_wy_gram<<<dim3(ceil_div(n - 2, WY_B), 8), 256, 0, s>>>(n, ws->partial, ws->A);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_spread(k_wy_gram, dim3(ceil_div(n - 2, WY_B), 8), dim3(256), 0, s, n, ws->partial, ws->A)));
     // columns per CTA: one wave of CTAs, at most eight, as many as fit in 200 KB
     const int fit = (int)std::max<size_t>(1, 200 * 1024 / ((size_t)n * sizeof(double)));
     const int nc = std::min(std::min(8, ceil_div(nv, sm_count())), fit);
@@ -1836,27 +1859,24 @@ int lanczos_top(int n, const double* A, int lda, int m, uint64_t seed, SymEigWor
         double* st = ws->lu;
         {
             ProfScope prof("lanczos", s);
-            k_lz_start<<<1, LZG_THREADS, 0, s>>>(n, seed, buf[0], buf[1], st);
-            EDA_LAUNCHED();
+            EDA_CUDA_TRY((launch_chained(k_lz_start, dim3(1), dim3(LZG_THREADS), 0, s, n, seed, buf[0], buf[1], st)));
             // v_j in buf[j % 2], v_{j-1} (then v_{j+1}) in buf[(j + 1) % 2], u in buf[2]
             for (int j = 0; j < m; ++j) {
                 double* v = buf[j & 1];
                 double* vp = buf[(j + 1) & 1];
-                k_lz_matvec<<<ceil_div((int64_t)n * 32, 256), 256, 0, s>>>(n, A, lda, v, buf[2], st);
-                EDA_LAUNCHED();
-                k_lz_update<<<1, LZG_THREADS, 0, s>>>(n, j, buf[2], v, vp, st, ws->dgl, ws->eoff);
-                EDA_LAUNCHED();
+                EDA_CUDA_TRY((launch_chained(k_lz_matvec, dim3(ceil_div((int64_t)n * 32, 256)), dim3(256), 0, s, n, A,
+                    lda, v, buf[2], st)));
+                EDA_CUDA_TRY((launch_chained(k_lz_update, dim3(1), dim3(LZG_THREADS), 0, s, n, j, buf[2], v, vp, st,
+                    ws->dgl, ws->eoff)));
             }
         }
         const int nv = m >= 2 ? 2 : 1;
         double* w = ws->vbuf + 3 * (size_t)n;       // nv values (vbuf holds 4 n doubles)
         double* zt = ws->lu + 5 * (size_t)m;        // the eigenvector after the 5 m factor entries
-        k_bisect<<<nv, 64, 3 * (size_t)m * sizeof(double), s>>>(m, ws->dgl, ws->eoff, m - nv, nv, w);
-        EDA_LAUNCHED();
-        k_invit<<<1, 32, 0, s>>>(m, 1, ws->dgl, ws->eoff, w + nv - 1, ws->lu, zt, seed);   // st is dead here
-        EDA_LAUNCHED();
-        k_lanczos_pack<<<1, 32, 0, s>>>(m, w, zt, ws->lu + m, ws->eoff, out);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_bisect, dim3(nv), dim3(64), 3 * (size_t)m * sizeof(double), s, m, ws->dgl,
+            ws->eoff, m - nv, nv, w)));
+        EDA_CUDA_TRY((launch_chained(k_invit, dim3(1), dim3(32), 0, s, m, 1, ws->dgl, ws->eoff, w + nv - 1, ws->lu, zt, seed)));   // st is dead here
+        EDA_CUDA_TRY((launch_chained(k_lanczos_pack, dim3(1), dim3(32), 0, s, m, w, zt, ws->lu + m, ws->eoff, out)));
         return EDA_OK;
     }
     const int C = (n + LZ_ROWS - 1) / LZ_ROWS;
@@ -1888,12 +1908,10 @@ int lanczos_top(int n, const double* A, int lda, int m, uint64_t seed, SymEigWor
     const int nv = m >= 2 ? 2 : 1;
     double* w = ws->vbuf;                       // nv values
     double* zt = ws->lu + 5 * (size_t)m;        // the eigenvector (m entries) after the 5 m factor entries
-    k_bisect<<<nv, 64, 3 * (size_t)m * sizeof(double), s>>>(m, ws->dgl, ws->eoff, m - nv, nv, w);
-    EDA_LAUNCHED();
-    k_invit<<<1, 32, 0, s>>>(m, 1, ws->dgl, ws->eoff, w + nv - 1, ws->lu, zt, seed);
-    EDA_LAUNCHED();
-    k_lanczos_pack<<<1, 32, 0, s>>>(m, w, zt, ws->lu + m, ws->eoff, out);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_bisect, dim3(nv), dim3(64), 3 * (size_t)m * sizeof(double), s, m, ws->dgl, ws->eoff,
+        m - nv, nv, w)));
+    EDA_CUDA_TRY((launch_chained(k_invit, dim3(1), dim3(32), 0, s, m, 1, ws->dgl, ws->eoff, w + nv - 1, ws->lu, zt, seed)));
+    EDA_CUDA_TRY((launch_chained(k_lanczos_pack, dim3(1), dim3(32), 0, s, m, w, zt, ws->lu + m, ws->eoff, out)));
     return EDA_OK;
 }
 

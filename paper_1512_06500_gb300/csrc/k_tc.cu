@@ -429,25 +429,6 @@ __global__ void k_tile_bf16(int64_t d, int m, const double* __restrict__ H, int 
     out[e] = __float2bfloat16_rn((float)v);
 }
 
-// Launch with programmatic stream serialisation: the kernel may start while the preceding kernel of
-// the stream drains; it orders its dependent reads with griddepcontrol.wait.
-template <class... KArgs, class... Args>
-int launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    EDA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
-    launch_counter()++;
-    return EDA_OK;
-}
-
 template <int N, int MODE>
 int set_smem_attr() {
     static std::mutex mu;
@@ -486,13 +467,13 @@ int launch_tc(const TcFactor& f, const TcBuffers& bufs, int b, const float* X, i
     if ((size_t)splits * m * b > partial_cap) return EDA_ERR_INVALID_ARG;
     const int rows = ceil_div(kst, splits) * TC_KS;
     splits = ceil_div(f.ldh, rows);
-    EDA_TRY(launch_pdl(k_tc_sweep1<N>, dim3(tiles, splits), dim3(128), smem, s, f.A1, (int)(f.ldh / TC_KS),
-                       bufs.mapXh[nb], bufs.mapXl[nb], m, b, rows, (int)f.ldh, partial, status));
-    EDA_TRY(launch_pdl(k_reduce_split, dim3(ceil_div(bufs.ldq, 32), b), dim3(256), 0, s, m, b, splits,
-                       (const float*)partial, bufs.ldq, bufs.Qhi, bufs.Qlo));
-    EDA_TRY(launch_pdl(k_tc_sweep2<N, 0>, dim3(ceil_div(f.d, TC_M)), dim3(128), smem, s, f.A2, bufs.mapQh[nb],
+    EDA_CUDA_TRY((launch_chained(k_tc_sweep1<N>, dim3(tiles, splits), dim3(128), smem, s, f.A1, (int)(f.ldh / TC_KS),
+                       bufs.mapXh[nb], bufs.mapXl[nb], m, b, rows, (int)f.ldh, partial, status)));
+    EDA_CUDA_TRY((launch_chained(k_reduce_split, dim3(ceil_div(bufs.ldq, 32), b), dim3(256), 0, s, m, b, splits,
+                       (const float*)partial, bufs.ldq, bufs.Qhi, bufs.Qlo)));
+    EDA_CUDA_TRY((launch_chained(k_tc_sweep2<N, 0>, dim3(ceil_div(f.d, TC_M)), dim3(128), smem, s, f.A2, bufs.mapQh[nb],
                        bufs.mapQl[nb], f.d, f.ldm, b, X, ldx, Y, ldy, emit_split ? bufs.Xhi : nullptr,
-                       emit_split ? bufs.Xlo : nullptr, f.ldh, (__nv_bfloat16*)nullptr, 0, 0, status));
+                       emit_split ? bufs.Xlo : nullptr, f.ldh, (__nv_bfloat16*)nullptr, 0, 0, status)));
     return EDA_OK;
 }
 

@@ -28,6 +28,8 @@ namespace {
 size_t a256(size_t b) { return (b + 255) & ~size_t(255); }
 
 __global__ void k_set_block(double* T, int ldt, int r0, int c0, int b, const double* Bm, int ldb, bool transpose) {
+    PDL_ENTER();
+    PDL_ARG(T); PDL_ARG(Bm);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= b * b) return;
     const int i = e % b, j = e / b;
@@ -40,6 +42,8 @@ __global__ void k_set_block(double* T, int ldt, int r0, int c0, int b, const dou
 // block symmetrised. Keeping every coupling (not only the block-tridiagonal ones) makes the
 // Rayleigh-Ritz step exact on span(V) even after lost directions were replaced by fresh ones.
 __global__ void k_set_col_block(double* T, int ldt, int cols, int j0, int b, const double* C1, const double* C2) {
+    PDL_ENTER();
+    PDL_ARG(T); PDL_ARG(C1); PDL_ARG(C2);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= cols * b) return;
     const int i = e % cols, jj = e / cols;
@@ -58,6 +62,8 @@ __global__ void k_set_col_block(double* T, int ldt, int cols, int j0, int b, con
 // (one thread for a whole pair took 21 us at b = 16).
 __global__ void k_ritz_residuals(int t, int b, const double* Bm, int ldb, const double* S, int lds, int rlast,
                                  const double* theta, double* relres) {
+    PDL_ENTER();
+    PDL_ARG(Bm); PDL_ARG(S); PDL_ARG(theta); PDL_ARG(relres);
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= t) return;
     double acc = 0.0;
@@ -73,6 +79,8 @@ __global__ void k_ritz_residuals(int t, int b, const double* Bm, int ldb, const 
 
 // out[:, i] = in[:, t-1-i] (descending order of the Ritz values)
 __global__ void k_reverse_cols(int64_t rows, int t, const double* in, int64_t ldi, double* out, int64_t ldo) {
+    PDL_ENTER();
+    PDL_ARG(in); PDL_ARG(out);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= rows * t) return;
     const int64_t r = e % rows;
@@ -81,6 +89,8 @@ __global__ void k_reverse_cols(int64_t rows, int t, const double* in, int64_t ld
 }
 
 __global__ void k_reverse_vec(int t, const double* in, double* out) {
+    PDL_ENTER();
+    PDL_ARG(in); PDL_ARG(out);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < t) out[i] = in[t - 1 - i];
 }
@@ -88,6 +98,8 @@ __global__ void k_reverse_vec(int t, const double* in, double* out) {
 // R = MY - Y diag(theta), written over MY
 __global__ void k_sub_scaled(int64_t d, int t, double* MY, int64_t ldm, const double* Y, int64_t ldy,
                              const double* theta) {
+    PDL_ENTER();
+    PDL_ARG(MY); PDL_ARG(Y); PDL_ARG(theta);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= d * t) return;
     const int64_t r = e % d;
@@ -96,6 +108,8 @@ __global__ void k_sub_scaled(int64_t d, int t, double* MY, int64_t ldm, const do
 }
 
 __global__ void k_divide(int t, double* num, const double* den) {
+    PDL_ENTER();
+    PDL_ARG(num); PDL_ARG(den);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < t) num[i] = fabs(den[i]) > 0.0 ? num[i] / fabs(den[i]) : INFINITY;
 }
@@ -319,10 +333,9 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
         double* C1 = w.C;
         double* C2 = w.C + (size_t)m_max * tw;
         EDA_TRY(cgs2<T>(d, cols, b, w.V, w.W, d, C1, C2, w, s, h));
-        k_set_col_block<<<ceil_div(cols * b, 256), 256, 0, s>>>(w.Tm, m_max, cols, j0, b, C1, C2);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_set_col_block, dim3(ceil_div(cols * b, 256)), dim3(256), 0, s, w.Tm, m_max, cols,
+            j0, b, C1, C2)));
         // CholQR2 of W with rank detection: W = V_{j+1} B_{j+1}
-        EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s));
         EDA_TRY(cholqr_pass<T>(d, b, w.W, d, w.R1, w.R1i, w.W1, piv_min2, h->status, w.lost, w, s));
         int lw[2] = {0, 0};   // lost and nearly lost columns
         EDA_TRY(read_back(lw, w.lost + b, sizeof(lw), s));
@@ -344,7 +357,6 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
             T* Vn = w.V + (size_t)cols * d;
             if (lw[1] > 0 && std::is_same<T, double>::value)
                 EDA_TRY(strengthen<T>(h, d, cols, b, Vn, w.C + (size_t)m_max * tw * 2, w, s));
-            EDA_CUDA_TRY(cudaMemsetAsync(w.lost, 0, (b + 2) * sizeof(int), s));
             EDA_TRY(cholqr_pass<T>(d, b, w.W1, d, w.R2, w.R2i, Vn, 0.0, h->status, w.lost, w, s));
             EDA_TRY(oz_basis_grow<T>(w, d, cols, cols + b, h->status, s));
             EDA_TRY(gemm_small_f64(false, false, b, b, b, 1.0, w.R2, b, w.R1, b, 0.0, w.Bm, b, s));   // B = R2 R1
@@ -367,12 +379,11 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
                 if (lostc > 0) {
                     EDA_TRY(gemm_nn<T>(d, b, t, 1.0, w.W, d, w.S + (cols - b), cols, 0.0, nullptr, 0, w.Yt, d, s));
                     EDA_TRY(col_norms<T>(d, t, w.Yt, d, w.relres, s));
-                    k_divide<<<ceil_div(t, 128), 128, 0, s>>>(t, w.relres, w.theta);
-                    EDA_LAUNCHED();
+                    EDA_CUDA_TRY((launch_chained(k_divide, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.relres, w.theta)));
                 } else {
-                    k_ritz_residuals<<<ceil_div(t, 4), 128, 0, s>>>(t, b, w.Bm, b, w.S, cols, cols - b, w.theta,
-                                                                     w.relres);
-                    EDA_LAUNCHED();
+                    EDA_CUDA_TRY((launch_chained(k_ritz_residuals, dim3(ceil_div(t, 4)), dim3(128), 0, s, t, b, w.Bm, b,
+                        w.S, cols, cols - b, w.theta,
+            w.relres)));
                 }
                 EDA_TRY(read_back(st.relres.data(), w.relres, t * sizeof(double), s));
                 st.max_rel = 0.0;
@@ -427,10 +438,10 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
             next_check = cols + gap;
         }
         if (st.converged || last) break;
-        k_set_block<<<ceil_div(b * b, 256), 256, 0, s>>>(w.Tm, m_max, cols, j0, b, w.Bm, b, false);
-        EDA_LAUNCHED();
-        k_set_block<<<ceil_div(b * b, 256), 256, 0, s>>>(w.Tm, m_max, j0, cols, b, w.Bm, b, true);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_set_block, dim3(ceil_div(b * b, 256)), dim3(256), 0, s, w.Tm, m_max, cols, j0, b,
+            w.Bm, b, false)));
+        EDA_CUDA_TRY((launch_chained(k_set_block, dim3(ceil_div(b * b, 256)), dim3(256), 0, s, w.Tm, m_max, j0, cols, b,
+            w.Bm, b, true)));
         cols += b;
     }
     if (st.rr_cols == 0) return EDA_ERR_NOT_CONVERGED;
@@ -556,6 +567,8 @@ int cholqr_f64(eda_ctx* h, int p, double* X, double* tmpX, SolveWs<T>& w, int pa
 
 __global__ void k_gather_cols(int64_t d, int r, const int* idx, const double* src, int64_t lds, double* dst,
                               int64_t ldd) {
+    PDL_ENTER();
+    PDL_ARG(idx); PDL_ARG(src); PDL_ARG(dst);
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= d * r) return;
     const int64_t i = e % d;
@@ -567,11 +580,10 @@ __global__ void k_gather_cols(int64_t d, int r, const int* idx, const double* sr
 template <class T>
 int ritz_residuals(int64_t d, int t, SolveWs<T>& w, std::vector<double>& relres_h, double* max_rel, cudaStream_t s) {
     EDA_TRY(copy_mat_f64(d, t, w.Z, d, w.R, d, s));
-    k_sub_scaled<<<ceil_div((int64_t)d * t, 256), 256, 0, s>>>(d, t, w.R, d, w.Y, d, w.theta);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_sub_scaled, dim3(ceil_div((int64_t)d * t, 256)), dim3(256), 0, s, d, t, w.R, d, w.Y,
+        d, w.theta)));
     EDA_TRY(col_norms_f64(d, t, w.R, d, w.relres, s));
-    k_divide<<<ceil_div(t, 128), 128, 0, s>>>(t, w.relres, w.theta);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_divide, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.relres, w.theta)));
     EDA_TRY(read_back(relres_h.data(), w.relres, t * sizeof(double), s));
     *max_rel = 0.0;
     for (int i = 0; i < t; ++i) *max_rel = std::max(*max_rel, relres_h[i]);
@@ -618,8 +630,8 @@ int refine_f64(eda_ctx* h, int t, double tol, SolveWs<T>& w, int max_iter, int* 
         const int tr = t + r;
         // R_u: the unconverged residual columns, packed right after Y ([Y R_u] adjacent)
         EDA_CUDA_TRY(cudaMemcpyAsync(w.idx, idx.data(), r * sizeof(int), cudaMemcpyHostToDevice, s));
-        k_gather_cols<<<ceil_div(d * r, 256), 256, 0, s>>>(d, r, w.idx, w.R, d, w.Y2, d);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_gather_cols, dim3(ceil_div(d * r, 256)), dim3(256), 0, s, d, r, w.idx, w.R, d,
+            w.Y2, d)));
         EDA_TRY(copy_mat_f64(d, r, w.Y2, d, w.R, d, s));
         for (int pass = 0; pass < 2; ++pass) {
             EDA_TRY(fin_tn(h, w, t, r, w.Y, w.R, d, w.Gt, t, s));
@@ -789,10 +801,9 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
     if (stw & ST_NONFINITE) return EDA_ERR_NONFINITE;
 
     // ---- descending order, recovery and orthonormalisation (FP64) ----
-    k_reverse_cols<<<ceil_div((int64_t)d * t, 256), 256, 0, s>>>(d, t, w.Y, d, w.Y2, d);
-    EDA_LAUNCHED();
-    k_reverse_vec<<<ceil_div(t, 128), 128, 0, s>>>(t, w.theta, w.lamd);
-    EDA_LAUNCHED();
+    EDA_CUDA_TRY((launch_chained(k_reverse_cols, dim3(ceil_div((int64_t)d * t, 256)), dim3(256), 0, s, d, t, w.Y, d,
+        w.Y2, d)));
+    EDA_CUDA_TRY((launch_chained(k_reverse_vec, dim3(ceil_div(t, 128)), dim3(128), 0, s, t, w.theta, w.lamd)));
     EDA_CUDA_TRY(cudaMemcpyAsync(lambda, w.lamd, t * sizeof(double), cudaMemcpyDeviceToDevice, s));
     if (Yout) EDA_CUDA_TRY(cudaMemcpyAsync(Yout, w.Y2, (size_t)d * t * 8, cudaMemcpyDeviceToDevice, s));
     // x = exp(-c^2 S_W / 2) y = y + H_W K_W (H_W^T y)
@@ -800,8 +811,8 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
         // H_W^T Y is already known (the first n rows of the tracked coordinates Z^T Y): one sweep
         EDA_TRY(gemm_small_f64(false, false, n, t, n, 1.0, h->KW, n, w.ZY, n + k, 0.0, w.PQ, n, s));
         EDA_TRY(gemm_nn_f64(d, n, t, 1.0, h->HW, d, w.PQ, n, 1.0, w.Y, d, w.Z2, d, s));
-        k_reverse_cols<<<ceil_div((int64_t)d * t, 256), 256, 0, s>>>(d, t, w.Z2, d, w.Xt, d);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_reverse_cols, dim3(ceil_div((int64_t)d * t, 256)), dim3(256), 0, s, d, t, w.Z2, d,
+            w.Xt, d)));
     } else if (h->cfg.prec == EDA_F64_TC && h->ozblock) {
         // the same product with the FP64-accurate tensor-core sweeps: H_W is the first n columns of the
         // split Z (the first n rows of its column-scaled operand, the first n of the reduction index of the
@@ -832,8 +843,8 @@ int solve_t(eda_ctx* h, int t, double tol, const double* V0, int b0, double* Vou
             EDA_TRY(m_apply_t<double>(h, cb, w.Y2 + (size_t)c0 * d, d, MY + (size_t)c0 * d, d, w.tmp64, w.P, w.Q,
                                       w.part, w.pcap, s, /*allow_composed=*/false));
         }
-        k_sub_scaled<<<ceil_div((int64_t)d * t, 256), 256, 0, s>>>(d, t, MY, d, w.Y2, d, w.lamd);
-        EDA_LAUNCHED();
+        EDA_CUDA_TRY((launch_chained(k_sub_scaled, dim3(ceil_div((int64_t)d * t, 256)), dim3(256), 0, s, d, t, MY, d,
+            w.Y2, d, w.lamd)));
         EDA_TRY(col_norms_f64(d, t, MY, d, w.relres, s));
         std::vector<double> rn(t), lam_h(t);
         EDA_TRY(read_back(rn.data(), w.relres, t * 8, s));

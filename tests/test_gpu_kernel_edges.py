@@ -179,3 +179,41 @@ def test_direct_solve_orders(eda, n, t):
     assert np.abs(V.T @ V - np.eye(t)).max() <= 1e-12
     # span(V) is invariant under N: N V = V (V^T N V) up to 1e-10 of ||N|| <= lambda_1 (the spectrum below may be close)
     assert np.abs(MV - V @ (V.T @ MV)).max() <= 1e-9 * ref["lam_t"][0]
+
+
+# Kernels launched to be set up while their predecessor runs: long chains of short ones (small and middle sizes, with and
+# without chip-filling kernels between), with another stream keeping the SMs busy unevenly. All sums are taken in a fixed
+# order, so a kernel that read before its predecessor had finished would show as different bits.
+@pytest.mark.parametrize("mode,d,k,per", [("EDA_F64", 96, 4, 3), ("EDA_F64", 1500, 24, 5), ("EDA_F64_TC", 1500, 24, 5),
+                                          ("EDA_BF16X2", 1500, 24, 5), ("EDA_F32", 700, 9, 4)])
+def test_chained_launches_give_the_same_bits(eda, mode, d, k, per):
+    p = synth.gaussian_clusters(d=d, k=k, n_per_class=[per] * k, seed=5)
+    X, lab = _dev(p.X), _dev(p.labels)
+    other = torch.cuda.Stream()
+    busy = torch.randn(900, 900, device="cuda:0")
+    with eda.build(X, lab, k, eda.config(tau=6.0, precision=getattr(eda, mode))) as h:
+        first = None
+        for i in range(6):
+            if i % 2:
+                with torch.cuda.stream(other):
+                    for _ in range(60):
+                        busy = torch.tanh(busy @ busy / 30.0)
+            V, lam, _, _, code = h.solve(k - 1, 1e-9, check=False)
+            assert code in (0, -8)
+            if first is None:
+                first = (V.clone(), lam.clone())
+            assert torch.equal(V, first[0]) and torch.equal(lam, first[1])
+        # recorded into a graph: replayed on inputs written after the capture
+        x = torch.zeros(5, d, dtype=torch.float64, device="cuda:0")
+        y = torch.empty_like(x)
+        h.apply_exp(eda.OP_M, x, out=y)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            h.apply_exp(eda.OP_M, x, out=y, stream=torch.cuda.current_stream())
+        x.copy_(torch.randn(5, d, dtype=torch.float64, device="cuda:0"))
+        g.replay()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, h.apply_exp(eda.OP_M, x))
+    torch.cuda.synchronize()

@@ -20,7 +20,7 @@
 // so the reduction over k is exact as well; the only roundings are the final conversion to FP64 and the
 // 2^-56 truncation of the digits.
 //
-// Kernel. One CTA per (128-row band of M, split of K), 256 threads: thread 0 issues the bulk copies of
+// Kernel. A CTA works on a run of K stages of one or several 128-row bands of M, 256 threads: thread 0 issues the bulk copies of
 // the pre-tiled digit planes of A (one contiguous 16 KB swizzled tile per K stage of 64 and plane) and
 // the TMA boxes of the seven planes of B; thread 32 issues tcgen05.mma (M = 128, K = 16, N = 32 (7 - a) for
 // digit plane a of A against planes 0 .. 6 - a of B at once) into one of two accumulator sets of seven
@@ -45,6 +45,7 @@ constexpr int OZ_N = 32;              // N of every MMA: the narrow operand's co
 constexpr int OZ_AST = 8;             // A ring slots (one 16 KB tile of one plane each)
 constexpr int OZ_BST = 2;             // B ring slots (the seven 32 x 64 planes of one K stage)
 constexpr int OZ_THREADS = 256;
+constexpr int kOzJoinStages = 3;      // what k_oz_join costs, in K stages of a CTA
 constexpr int OZ_SET_COLS = 256;      // tensor-memory columns of one accumulator set (7 levels x 32)
 
 struct OzRing {
@@ -75,34 +76,93 @@ struct OzBTiles {
     int upper = 0;
 };
 
+// A narrow product with more bands than SMs (RUNS): the K stages of all bands, band after band, are dealt to the CTAs of
+// one wave in contiguous runs, one per CTA. The roles run through the bands of their run without a pause: the copies of a
+// band's first stages are in flight, and its MMAs run, while the previous band is still being folded and written. A band that
+// lies in one run is written to D; of a band that several runs share, each writes the sum over its stages to its own 128 x N
+// slot of partial (a run has at most two such pieces, its first, slot 2 c, and its last, slot 2 c + 1), and k_oz_join adds them
+// in the order of k. One CTA a band took four rounds of 152 for 3.4 rounds of work, each with its own start and end
+// (65536 x 2200 times 32 columns: 408 -> 340 us). With fewer bands than SMs the split of K stays the same for all bands: the
+// CTAs of one split read the same stages of B at the same time (2200 x 65536 times 32 columns 315 us, in runs 363).
+// unit: a run starts at a multiple of this many stages: 1, or the stages of a band (whole bands, nothing to join).
+struct OzRuns {
+    int kst;        // stages per band
+    int unit;
+    int64_t units;  // bands * kst / unit
+    __host__ __device__ int64_t begin(int c, int ctas) const { return units * c / ctas * unit; }
+    // the CTA whose run holds stage t
+    __host__ __device__ int of(int64_t t, int ctas) const {
+        return (int)(((t / unit + 1) * ctas + units - 1) / units) - 1;
+    }
+};
+
+// round((g0 2^32 + g1) 2^{e - 62}), to nearest even, by integer operations. The two conversions and two ldexp of the plain form
+// are some ten FP64 instructions, and a warp instruction of that pipe takes 64 cycles: 10 us for a warp's 32 x 32 results,
+// against 1.5 here (one rounding instead of three).
+__device__ __forceinline__ double oz_value(long long g0, long long g1, int e) {
+    unsigned long long lo = ((unsigned long long)g0 << 32) + (unsigned long long)g1;
+    long long hi = (g0 >> 32) + (g1 >> 63) + (lo < (unsigned long long)g1 ? 1 : 0);
+    const bool neg = hi < 0;
+    if (neg) {
+        lo = 0ull - lo;
+        hi = ~hi + (lo == 0 ? 1 : 0);
+    }
+    if (hi == 0) {   // g0 2^32 + g1 below 2^64
+        if (lo == 0) return 0.0;
+        hi = (long long)lo;
+        lo = 0;
+        e -= 64;
+    }
+    const int lz = __clzll(hi);
+    const unsigned long long m = ((unsigned long long)hi << lz) | ((lo >> 1) >> (63 - lz)), rest = lo << lz;
+    unsigned long long q = m >> 11;   // 53 bits, 2^{e + 13 - lz} times q
+    const unsigned rem = (unsigned)(m & 0x7ff);
+    q += (rem > 0x400u || (rem == 0x400u && (rest != 0 || (q & 1)))) ? 1 : 0;
+    const int ex = e + 65 - lz + 1023;   // biased exponent
+    const unsigned long long sign = neg ? 1ull << 63 : 0ull;
+    if (ex >= 1 && ex <= 2045) return __longlong_as_double((long long)(((unsigned long long)(ex - 1) << 52) + q | sign));
+    return ldexp(__longlong_as_double((long long)((1022ull << 52) + q | sign)), ex - 1023);   // q up to 2^53: one binade more
+}
+
 // D[i, j] (i < M, j < N) = alpha * sum_k A_ik B_jk + beta * C0[i, j]; D, C0 column-major (ld ldd, ldc0),
 // the split-th slice of D at D + split * split_stride. A: digit planes at At + q * aslice, pre-tiled
 // (128-row bands, kbs tiles of 64 along K per band), row scales expA. B: digit planes read through tmB
 // (inner = K, outer = 7 x 32 rows: plane q is rows 32 q .. 32 q + 31), or in BT mode from bt (N rows, the
-// CTA's 32 of them chosen by blockIdx.x mod nblk), row scales expB. K stages [split * kps, min(kst, (split + 1) * kps)).
-template <bool BT>
+// CTA's 32 of them chosen by blockIdx.x mod nblk), row scales expB. Without RUNS: one band a CTA, K stages
+// [split * kps, min(kst, (split + 1) * kps)), split = blockIdx.y.
+template <bool BT, bool RUNS>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(const __nv_bfloat16* __restrict__ At, int64_t aslice, int kbs, const __grid_constant__ CUtensorMap tmB,
-              const OzBTiles bt, const int* __restrict__ expA, const int* __restrict__ expB, int M, int N, int kst,
-              int kps, double alpha, double beta, const double* C0, int64_t ldc0, double* D, int64_t ldd,
-              int64_t split_stride, int* status) {
+              const OzBTiles bt, const int* __restrict__ expA, const int* __restrict__ expB, int M, int N,
+              const OzRuns runs, int kps, double alpha, double beta, const double* C0, int64_t ldc0, double* D, int64_t ldd,
+              int64_t split_stride, double* partial, int* status) {
     PDL_WAIT();
-    PDL_ARG(At); PDL_ARG(expA); PDL_ARG(expB); PDL_ARG(C0); PDL_ARG(D); PDL_ARG(status);
+    PDL_ARG(At); PDL_ARG(expA); PDL_ARG(expB); PDL_ARG(C0); PDL_ARG(D); PDL_ARG(partial); PDL_ARG(status);
     extern __shared__ unsigned char smraw[];
     OzRing& sm = oz_ring(smraw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int band = BT ? (int)blockIdx.x / bt.nblk : (int)blockIdx.x, split = blockIdx.y;
+    const int kst = runs.kst;
     const int blk = BT ? (int)blockIdx.x % bt.nblk : 0;
+    // this CTA's stages: n of them from stage k0 of band0 on, going on with stage 0 of the next band
+    int band0, k0, n;
+    if (!RUNS) {
+        band0 = BT ? (int)blockIdx.x / bt.nblk : (int)blockIdx.x;
+        k0 = blockIdx.y * kps;
+        n = max(0, min(kst, k0 + kps) - k0);
+        D += blockIdx.y * split_stride;
+    } else {
+        const int64_t t0 = runs.begin(blockIdx.x, gridDim.x), t1 = runs.begin(blockIdx.x + 1, gridDim.x);
+        band0 = (int)(t0 / kst);
+        k0 = (int)(t0 % kst);
+        n = (int)(t1 - t0);
+    }
     if (BT) {
-        if (bt.upper && blk * OZ_N + OZ_N <= band * TC_M) return;   // the whole CTA: a uniform exit
+        if (bt.upper && blk * OZ_N + OZ_N <= band0 * TC_M) return;   // the whole CTA: a uniform exit
         expB += blk * OZ_N;
         N -= blk * OZ_N;
         D += (int64_t)blk * OZ_N * ldd;
         if (C0) C0 += (int64_t)blk * OZ_N * ldc0;
     }
-    const int ks0 = split * kps;
-    const int nks = max(0, min(kst, ks0 + kps) - ks0);
-    const int nchunks = (nks + 1) >> 1;
     if (warp == 0) {
         tmem_alloc(&sm.tbase, 2 * OZ_SET_COLS);
         tmem_relinquish();
@@ -134,8 +194,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         // ---- producer ----
         constexpr uint32_t abytes = TC_M * TC_KS * 2;
         constexpr uint32_t bbytes = OZ_S * OZ_N * TC_KS * 2;
-        for (int s = 0; s < nks && ok; ++s) {
-            const int kstage = ks0 + s;
+        int band = band0, kstage = k0;
+        for (int s = 0; s < n && ok; ++s) {
             const int bslot = s % OZ_BST;
             if (s >= OZ_BST && !(ok = mbar_wait(&sm.emptyB[bslot], ((s / OZ_BST) - 1) & 1, status))) break;
             mbar_expect_tx(&sm.fullB[bslot], bbytes);
@@ -160,12 +220,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                           &sm.fullA[slot]);
                 issuedA = idx + 1;
             }
+            ++kstage;
+            if (RUNS && kstage == kst) {
+                kstage = 0;
+                ++band;
+            }
         }
     } else if (tid == 32) {
         // ---- MMA issuer ----
-        for (int s = 0; s < nks && ok; ++s) {
-            const int chunk = s >> 1, set = chunk & 1;
-            const bool first = (s & 1) == 0;
+        int kstage = k0, chunk = 0;   // chunks of two stages, cut at the end of a band
+        bool first = true;
+        for (int s = 0; s < n && ok; ++s) {
+            const int set = chunk & 1;
             if (first && chunk >= 2 && !(ok = mbar_wait(&sm.accEmpty[set], ((chunk >> 1) - 1) & 1, status))) break;
             const int bslot = s % OZ_BST;
             if (!(ok = mbar_wait(&sm.fullB[bslot], (s / OZ_BST) & 1, status))) break;
@@ -196,45 +262,85 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             }
             if (!ok) break;
             mma_commit(&sm.emptyB[bslot]);
-            if ((s & 1) || s == nks - 1) mma_commit(&sm.accFull[set]);
+            const bool band_end = RUNS && ++kstage == kst;
+            if (band_end) kstage = 0;
+            first = !first || band_end || s == n - 1;   // the chunk ends here
+            if (first) {
+                mma_commit(&sm.accFull[set]);
+                ++chunk;
+            }
         }
     }
-    // ---- epilogue: warps 4-7 fold each finished chunk into exact 64-bit integer sums ----
-    long long g0[OZ_N], g1[OZ_N];
-#pragma unroll
-    for (int c = 0; c < OZ_N; ++c) g0[c] = g1[c] = 0;
-    bool eok = true;
+    // ---- epilogue: warps 4-7 fold each finished chunk into exact 64-bit integer sums and write a band out at its end ----
     if (warp >= 4) {
         const int ew = warp - 4;
         const uint32_t lanebase = tmem + ((uint32_t)(32 * ew) << 16);
-        for (int ch = 0; ch < nchunks; ++ch) {
-            const int set = ch & 1;
-            if (!(eok = mbar_wait(&sm.accFull[set], (ch >> 1) & 1, status))) break;
-            tc_fence_after();
+        bool eok = true;   // a give-up: this band and the rest of the run become NaN
+        int chunk = 0, left = n, band = band0, kfrom = k0;
+        do {
+            const int nks = RUNS ? min(left, kst - kfrom) : n;
+            long long g0[OZ_N], g1[OZ_N];
 #pragma unroll
-            for (int c0 = 0; c0 < OZ_N; c0 += 8) {
-                uint32_t r[OZ_S][8];
+            for (int c = 0; c < OZ_N; ++c) g0[c] = g1[c] = 0;
+            for (int ch = (nks + 1) >> 1; ch > 0; --ch, ++chunk) {
+                const int set = chunk & 1;
+                if (!(eok = eok && mbar_wait(&sm.accFull[set], (chunk >> 1) & 1, status))) break;
+                tc_fence_after();
 #pragma unroll
-                for (int q = 0; q < OZ_S; ++q) tmem_ld8(lanebase + set * OZ_SET_COLS + q * OZ_N + c0, r[q]);
-                tmem_wait_ld();
+                for (int c0 = 0; c0 < OZ_N; c0 += 8) {
+                    uint32_t r[OZ_S][8];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    long long L[OZ_S];
+                    for (int q = 0; q < OZ_S; ++q) tmem_ld8(lanebase + set * OZ_SET_COLS + q * OZ_N + c0, r[q]);
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int q = 0; q < OZ_S; ++q) L[q] = (long long)__float2int_rn(__uint_as_float(r[q][c]));
-                    g0[c0 + c] += L[0] * 65536LL + L[1] * 256LL + L[2];
-                    g1[c0 + c] += ((L[3] * 256LL + L[4]) * 256LL + L[5]) * 256LL + L[6];
+                    for (int c = 0; c < 8; ++c) {
+                        long long L[OZ_S];
+#pragma unroll
+                        for (int q = 0; q < OZ_S; ++q) L[q] = (long long)__float2int_rn(__uint_as_float(r[q][c]));
+                        g0[c0 + c] += L[0] * 65536LL + L[1] * 256LL + L[2];
+                        g1[c0 + c] += ((L[3] * 256LL + L[4]) * 256LL + L[5]) * 256LL + L[6];
+                    }
+                }
+                tc_fence_before();
+                mbar_arrive(&sm.accEmpty[set]);
+            }
+            left -= nks;
+            if (!RUNS || left == 0) PDL_NEXT();
+            const int row = 32 * ew + lane, i = band * TC_M + row;
+            if (i < M) {
+                const int ea = expA[i];
+                const bool whole = !RUNS || nks == kst;
+                double* out = whole ? D + i : partial + ((int64_t)(2 * blockIdx.x + (left + nks < n ? 1 : 0)) * N) * TC_M + row;
+                const int64_t ldo = whole ? ldd : TC_M;
+#pragma unroll
+                for (int c0 = 0; c0 < OZ_N; c0 += 8) {
+                    if (c0 >= N) break;
+                    // the eight loads of C0 go out together: D may be C0, so none could pass a store
+                    double add[8];
+                    if (whole && beta != 0.0) {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) add[u] = c0 + u < N ? C0[(int64_t)(c0 + u) * ldc0 + i] : 0.0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int c = c0 + u;
+                        if (c >= N) break;
+                        double v = eok ? oz_value(g0[c], g1[c], ea + expB[c]) : nan("");
+                        if (whole) {
+                            if (alpha != 1.0) v = alpha * v;
+                            if (beta != 0.0) v = fma(beta, add[u], v);
+                        }
+                        out[c * ldo] = v;
+                    }
                 }
             }
-            tc_fence_before();
-            mbar_arrive(&sm.accEmpty[set]);
-        }
+            kfrom = 0;
+            ++band;
+        } while (RUNS && left > 0);
+        if (!eok) sm.fail = 1;
     }
-    __shared__ int s_ok;
     if ((tid == 0 || tid == 32) && !ok) sm.fail = 1;
-    if (warp >= 4 && !eok) sm.fail = 1;
     __syncthreads();
-    if (tid == 0) s_ok = sm.fail == 0 ? 1 : 0;
     if (tid == 0 && sm.fail) {
         // after a give-up, wait (bounded again) for this CTA's copies that may still be in flight, so
         // that none lands after the CTA's shared memory is released
@@ -242,25 +348,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             mbar_wait(&sm.fullA[i % OZ_AST], (i / OZ_AST) & 1, status);
         for (int i = max(0, issuedB - OZ_BST); i < issuedB; ++i)
             mbar_wait(&sm.fullB[i % OZ_BST], (i / OZ_BST) & 1, status);
-    }
-    __syncthreads();
-    PDL_NEXT();
-    if (warp >= 4) {
-        const int i = band * TC_M + 32 * (warp - 4) + lane;
-        if (i < M) {
-            const int ea = expA[i];
-            double* Ds = D + (int64_t)split * split_stride;
-#pragma unroll
-            for (int c = 0; c < OZ_N; ++c) {
-                if (c >= N) break;
-                const int e = ea + expB[c];
-                double v = (s_ok && nks > 0) ? ldexp((double)g0[c], e - 30) + ldexp((double)g1[c], e - 62) : 0.0;
-                if (!s_ok) v = nan("");
-                double out = alpha * v;
-                if (beta != 0.0) out = fma(beta, C0[(int64_t)c * ldc0 + i], out);
-                Ds[(int64_t)c * ldd + i] = out;
-            }
-        }
     }
     tc_fence_before();
     __syncthreads();
@@ -606,13 +693,42 @@ __global__ void k_oz_reduce(int M, int N, int splits, const double* __restrict__
     D[(int64_t)j * ldd + i] = v;
 }
 
+// The bands that several runs share: D = alpha * (the sum of their slots, in the order of k) + beta * C0. Block row c > 0 takes
+// the band in which run c begins, if it is the first run to begin inside that band; 256 of the band's 128 x N entries a CTA.
+__global__ void __launch_bounds__(256) k_oz_join(const OzRuns runs, int ctas, int M, int N, const double* __restrict__ P,
+                                                 double alpha, double beta, const double* C0, int64_t ldc0, double* D,
+                                                 int64_t ldd) {
+    PDL_ENTER();
+    PDL_ARG(P); PDL_ARG(C0); PDL_ARG(D);
+    const int c = blockIdx.y + 1;
+    const int64_t t = runs.begin(c, ctas);
+    const int band = (int)(t / runs.kst);
+    const int64_t b0 = (int64_t)band * runs.kst;
+    if (t == b0 || runs.begin(c - 1, ctas) > b0) return;
+    const int e = blockIdx.x * 256 + threadIdx.x, row = e % TC_M, j = e / TC_M, i = band * TC_M + row;
+    if (j >= N || i >= M) return;
+    const int last = runs.of(b0 + runs.kst - 1, ctas);
+    // run c - 1 holds the band's first stages: as its first piece if it begins with the band, else as its last
+    const double* src = P + (int64_t)j * TC_M + row;
+    const int64_t slot = (int64_t)N * TC_M;
+    double acc = src[(2 * (c - 1) + (runs.begin(c - 1, ctas) == b0 ? 0 : 1)) * slot];
+    for (int q = c; q <= last; ++q) acc += src[2 * q * slot];
+    double v = alpha * acc;
+    if (beta != 0.0) v = fma(beta, C0[(int64_t)j * ldc0 + i], v);
+    D[(int64_t)j * ldd + i] = v;
+}
+
 int oz_attr() {
     static std::once_flag once;
     static cudaError_t rc = cudaSuccess;
     std::call_once(once, [] {
-        rc = cudaFuncSetAttribute(k_oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_smem_bytes());
+        rc = cudaFuncSetAttribute(k_oz_gemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)oz_smem_bytes());
         if (rc == cudaSuccess)
-            rc = cudaFuncSetAttribute(k_oz_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            rc = cudaFuncSetAttribute(k_oz_gemm<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)oz_smem_bytes());
+        if (rc == cudaSuccess)
+            rc = cudaFuncSetAttribute(k_oz_gemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)oz_smem_bytes());
 
     });
@@ -722,10 +838,14 @@ int oz_grow_rows(const double* A, int64_t lda, int64_t M, int64_t k0, int64_t k1
     return EDA_OK;
 }
 
+// doubles of the partial buffer: max_splits copies of a result, and two 128-row slots for each run of a narrow product
+static size_t oz_partial_cap(int max_splits, int64_t Mmax) {
+    return (size_t)max_splits * OZ_N * (size_t)std::max<int64_t>(Mmax, 2 * TC_M);
+}
+
 size_t oz_narrow_bytes(int64_t Kmax, int max_splits, int64_t Mmax) {
     const int64_t ld = (Kmax + TC_KS - 1) / TC_KS * TC_KS;
-    return ((size_t)OZ_S * OZ_N * ld * 2 + 255) / 256 * 256 + 256 +
-           ((size_t)max_splits * OZ_N * Mmax * 8 + 255) / 256 * 256;
+    return ((size_t)OZ_S * OZ_N * ld * 2 + 255) / 256 * 256 + 256 + (oz_partial_cap(max_splits, Mmax) * 8 + 255) / 256 * 256;
 }
 
 int oz_narrow_make(int64_t Kmax, int max_splits, int64_t Mmax, void* mem, OzNarrow* nb) {
@@ -736,7 +856,7 @@ int oz_narrow_make(int64_t Kmax, int max_splits, int64_t Mmax, void* mem, OzNarr
     nb->exps = reinterpret_cast<int*>(p);
     p += 256;
     nb->partial = reinterpret_cast<double*>(p);
-    nb->pcap = (size_t)max_splits * OZ_N * Mmax;
+    nb->pcap = oz_partial_cap(max_splits, Mmax);
     nb->ldmax = ld;
     nb->map_ld = 0;
     return EDA_OK;
@@ -759,35 +879,39 @@ int oz_gemm(const OzOperand& A, OzNarrow& nb, int p, const double* B, int64_t ld
     EDA_CUDA_TRY((launch_chained(k_oz_narrow, dim3(OZ_NARROW_CL, OZ_N), dim3(256), 0, s, A.K, p, B, ldb, nb.exps, ld,
         nb.planes, status)));
     const int kst = (int)(ld / TC_KS);
-    // K splits: fill the SMs with one CTA each (the kernel holds all of an SM's tensor memory)
+    // One CTA an SM at most (the kernel holds all of an SM's tensor memory). Up to one band an SM: K splits that fill the SMs.
+    // More: runs; of whole bands, which need no join, unless even ones are shorter by more than the join costs.
     const int nsm = sm_count();
-    int splits = std::max(1, std::min(kst / 2, nsm / std::max(1, A.mtiles)));
-    while (splits > 1 && (size_t)splits * p * A.M > nb.pcap) --splits;
-    const int kps = ceil_div(kst, splits);
-    splits = ceil_div(kst, kps);
-    const dim3 grid((unsigned)A.mtiles, (unsigned)splits);
-    const int64_t sstride = splits == 1 ? 0 : (int64_t)p * A.M;
+    OzRuns runs{kst, kst, A.mtiles};
+    int ctas = std::min(nsm, A.mtiles), splits = 1, kps = 0;
+    if (A.mtiles <= nsm) {
+        splits = std::max(1, std::min(kst / 2, nsm / std::max(1, A.mtiles)));
+        while (splits > 1 && (size_t)splits * p * A.M > nb.pcap) --splits;
+        kps = ceil_div(kst, splits);
+        splits = ceil_div(kst, kps);
+    } else if ((size_t)2 * TC_M * p * nsm <= nb.pcap &&
+               (int64_t)ceil_div(A.mtiles, nsm) * kst > (int64_t)A.mtiles * kst / nsm + kOzJoinStages) {
+        runs.unit = 1;
+        runs.units = (int64_t)A.mtiles * kst;
+    }
+    const bool add = splits > 1;   // the splits' sums go to partial
+    const bool join = kps == 0 && runs.unit == 1;
     {
         // the tensor-core kernel alone: it must read the seven digit planes of A and of B once and write D
         // tensor work: the 28 digit-plane products of 2 M K p flops each
         ProfScope kprof("oz_kernel", s, 56.0 * (double)A.M * A.K * p,
                         2.0 * OZ_S * ((double)A.M * A.K + (double)A.K * p) + 8.0 * (double)A.M * p);
         const OzBTiles none{};
-        if (splits == 1)
-            EDA_CUDA_TRY((launch_chained(k_oz_gemm<false>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
-                A.kbs, nb.map, none, A.exps,
-            nb.exps, (int)A.M, p, kst, kps, alpha, beta, C0,
-            ldc0, D, ldd, 0, status)));
-        else
-            EDA_CUDA_TRY((launch_chained(k_oz_gemm<false>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
-                A.kbs, nb.map, none, A.exps,
-            nb.exps, (int)A.M, p, kst, kps, 1.0, 0.0,
-            nullptr, 0, nb.partial, A.M, sstride, status)));
+        EDA_CUDA_TRY((launch_chained(kps ? k_oz_gemm<false, false> : k_oz_gemm<false, true>, dim3((unsigned)ctas, (unsigned)splits), dim3(OZ_THREADS), oz_smem_bytes(),
+            s, A.tiles, A.slice, A.kbs, nb.map, none, A.exps, nb.exps, (int)A.M, p, runs, kps, add ? 1.0 : alpha,
+            add ? 0.0 : beta, C0, ldc0, add ? nb.partial : D, add ? A.M : ldd, add ? (int64_t)p * A.M : 0, nb.partial, status)));
     }
-    if (splits == 1) return EDA_OK;
-    EDA_CUDA_TRY((launch_chained(k_oz_reduce, dim3(ceil_div((int64_t)A.M * p, 256)), dim3(256), 0, s, (int)A.M, p,
-        splits, nb.partial, sstride, alpha,
-            beta, C0, ldc0, D, ldd)));
+    if (add)
+        EDA_CUDA_TRY((launch_chained(k_oz_reduce, dim3(ceil_div((int64_t)A.M * p, 256)), dim3(256), 0, s, (int)A.M, p, splits,
+            nb.partial, (int64_t)p * A.M, alpha, beta, C0, ldc0, D, ldd)));
+    if (!join) return EDA_OK;
+    EDA_CUDA_TRY((launch_chained(k_oz_join, dim3(ceil_div(TC_M * p, 256), (unsigned)(ctas - 1)), dim3(256), 0, s, runs, ctas,
+        (int)A.M, p, nb.partial, alpha, beta, C0, ldc0, D, ldd)));
     return EDA_OK;
 }
 
@@ -843,16 +967,17 @@ int oz_gemm_tiled(const OzOperand& A, const OzOperand& B, double alpha, double b
                         2.0 * OZ_S * ((double)A.M * A.K + (double)A.K * B.M) + 8.0 * (double)A.M * B.M);
         // tmB is not read in this mode; the operand's planes are passed in bt
         static const CUtensorMap unused{};
+        const OzRuns runs{kst, kst, A.mtiles};
         if (splits == 1)
-            EDA_CUDA_TRY((launch_chained(k_oz_gemm<true>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
+            EDA_CUDA_TRY((launch_chained(k_oz_gemm<true, false>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
                 A.kbs, unused, bt, A.exps,
-            B.exps, (int)A.M, (int)B.M, kst, kps, alpha, beta,
-            C0, ldc0, D, ldd, 0, status)));
+            B.exps, (int)A.M, (int)B.M, runs, kps, alpha, beta,
+            C0, ldc0, D, ldd, 0, nullptr, status)));
         else
-            EDA_CUDA_TRY((launch_chained(k_oz_gemm<true>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
+            EDA_CUDA_TRY((launch_chained(k_oz_gemm<true, false>, grid, dim3(OZ_THREADS), oz_smem_bytes(), s, A.tiles, A.slice,
                 A.kbs, unused, bt, A.exps,
-            B.exps, (int)A.M, (int)B.M, kst, kps, 1.0, 0.0,
-            nullptr, 0, part, A.M, (int64_t)A.M * B.M, status)));
+            B.exps, (int)A.M, (int)B.M, runs, kps, 1.0, 0.0,
+            nullptr, 0, part, A.M, (int64_t)A.M * B.M, nullptr, status)));
     }
     if (splits > 1) {
         EDA_CUDA_TRY((launch_chained(k_oz_reduce, dim3(ceil_div((int64_t)A.M * B.M, 256)), dim3(256), 0, s, (int)A.M,

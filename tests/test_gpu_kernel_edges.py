@@ -158,6 +158,21 @@ def test_composed_m_apply_operands(eda, k, nj):
             assert (np.abs(Y - Yr).max(0) <= 1e-12 * np.abs(Yr).max(0)).all()
 
 
+# narrow products with more 128-row bands than SMs (152), dealt to the CTAs in runs: of whole bands for short rows, even ones
+# for longer (a run's pieces joined); bands of one row, one column and a full block of 32
+@pytest.mark.parametrize("d,k,nj", [(19457, 8, 3), (19585, 66, 3), (40000, 40, 10)])
+def test_narrow_product_runs(eda, d, k, nj):
+    p = synth.gaussian_clusters(d=d, k=k, n_per_class=nj, seed=d)
+    f = O.scatter_factors(p.X, p.labels, p.k)
+    rng = np.random.default_rng(k)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(prec=eda.EDA_F64_TC, tau=8.0, tc_min_mi=-1)) as h:
+        for m in (1, 32):
+            X = rng.standard_normal((d, m))
+            Y = h.apply_exp(eda.OP_M, _dev(X.T)).cpu().numpy().T
+            Yr = O.m_apply(f["HW"], f["HB"], h.c2, X)
+            assert (np.abs(Y - Yr).max(0) <= 1e-12 * np.abs(Yr).max(0)).all()
+
+
 # eigenvectors through the back-transformation: matrix orders n - 1 around its smallest blocked size (64) and its blocks of 32
 # reflectors, few and many columns (1 to 8 a CTA by the number of columns)
 @pytest.mark.parametrize("n,t", [(34, 3), (64, 5), (65, 1), (66, 40), (67, 66), (98, 9), (99, 98), (131, 64), (400, 399)])
@@ -185,13 +200,13 @@ def test_direct_solve_orders(eda, n, t):
 # without chip-filling kernels between), with another stream keeping the SMs busy unevenly. All sums are taken in a fixed
 # order, so a kernel that read before its predecessor had finished would show as different bits.
 @pytest.mark.parametrize("mode,d,k,per", [("EDA_F64", 96, 4, 3), ("EDA_F64", 1500, 24, 5), ("EDA_F64_TC", 1500, 24, 5),
-                                          ("EDA_BF16X2", 1500, 24, 5), ("EDA_F32", 700, 9, 4)])
+                                          ("EDA_BF16", 1500, 24, 5), ("EDA_F32", 700, 9, 4)])
 def test_chained_launches_give_the_same_bits(eda, mode, d, k, per):
     p = synth.gaussian_clusters(d=d, k=k, n_per_class=[per] * k, seed=5)
     X, lab = _dev(p.X), _dev(p.labels)
     other = torch.cuda.Stream()
     busy = torch.randn(900, 900, device="cuda:0")
-    with eda.build(X, lab, k, eda.config(tau=6.0, precision=getattr(eda, mode))) as h:
+    with eda.build(X, lab, k, eda.config(tau=6.0, prec=getattr(eda, mode))) as h:
         first = None
         for i in range(6):
             if i % 2:

@@ -488,6 +488,14 @@ __global__ void __launch_bounds__(256) k_oz_exp_rows(int64_t rows, int cols, con
     if (mx != kOzExpZero) atomicMax(&e[r], mx);
 }
 
+// A chained launch where a memset would break the chain: the gap before it and after it came to 4 to 9 us, of which 2 are left.
+__global__ void k_oz_fill(int* __restrict__ p, int64_t n, int v) {
+    PDL_ENTER();
+    PDL_ARG(p);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n) p[t] = v;
+}
+
 // A narrow operand B (K x p, ldb; its columns are the N rows of the product): column scales and the seven digit planes, in
 // one launch. planes [7][32][ld] (plane q, row j at (32 q + j) ld), zero for j >= p or k >= K; e[j] the scales (0 for
 // j >= p). One cluster per column: each CTA takes the maximum over its share of the column, the CTAs exchange theirs
@@ -747,7 +755,7 @@ size_t oz_operand_bytes(int64_t M, int64_t K) {
 // Column scales of columns 0 .. ncols of A (K x ncols, lda) into e.
 static int oz_col_exps(int64_t K, const double* A, int64_t lda, int ncols, int* e, cudaStream_t s) {
     if (ncols <= 0) return EDA_OK;
-    EDA_CUDA_TRY(cudaMemsetAsync(e, 0xC0, (size_t)ncols * sizeof(int), s));   // kOzExpZero in every entry
+    EDA_CUDA_TRY((launch_chained(k_oz_fill, dim3(ceil_div(ncols, 256)), dim3(256), 0, s, e, ncols, kOzExpZero)));
     const dim3 grid((unsigned)ncols, (unsigned)ceil_div(std::max<int64_t>(K, 1), kOzExpChunk));
     EDA_CUDA_TRY((launch_chained(k_oz_exp_cols, grid, dim3(kOzExpThreads), 0, s, K, A, lda, e)));
     return EDA_OK;
@@ -756,7 +764,7 @@ static int oz_col_exps(int64_t K, const double* A, int64_t lda, int ncols, int* 
 // Row scales of A (M x K, lda) into e.
 static int oz_row_exps(int64_t M, int64_t K, const double* A, int64_t lda, int* e, cudaStream_t s) {
     if (M <= 0) return EDA_OK;
-    EDA_CUDA_TRY(cudaMemsetAsync(e, 0xC0, (size_t)M * sizeof(int), s));   // kOzExpZero in every entry
+    EDA_CUDA_TRY((launch_chained(k_oz_fill, dim3(ceil_div(M, 256)), dim3(256), 0, s, e, M, kOzExpZero)));
     if (K <= 0) return EDA_OK;
     EDA_CUDA_TRY((launch_chained(k_oz_exp_rows, dim3((unsigned)ceil_div(M, 256), (unsigned)ceil_div(K, kOzRowChunk)),
         dim3(256), 0, s, M, (int)K, A, lda, e)));
@@ -825,7 +833,7 @@ int oz_append_cols(const double* A, int64_t lda, int i0, int i1, int64_t K, OzOp
 int oz_grow_rows(const double* A, int64_t lda, int64_t M, int64_t k0, int64_t k1, OzOperand* op, int* list,
                  int* status, cudaStream_t s) {
     if (k1 <= k0) return EDA_OK;
-    EDA_CUDA_TRY(cudaMemsetAsync(list, 0, sizeof(int), s));
+    EDA_CUDA_TRY((launch_chained(k_oz_fill, dim3(1), dim3(32), 0, s, list, 1, 0)));
     EDA_CUDA_TRY((launch_chained(k_oz_grow_rows, dim3(ceil_div(M, 256)), dim3(256), 0, s, A, lda, M, k0, k1, op->exps,
         op->kbs, op->tiles, op->slice, list,
             status)));

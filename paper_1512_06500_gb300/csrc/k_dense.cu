@@ -271,10 +271,15 @@ __global__ void k_gemm_tn_reduce_warp(int m, int p, int splits, const T* __restr
 // (m x p). A CTA owns 32 rows and NC columns; its eight warps (two per SM sub-partition, so that
 // one issues FP64 work while the other waits on a load) split the inner dimension into eighths,
 // each thread keeps NC independent accumulators, the slice of B sits in shared memory, and the
-// partial sums of the eighths are added in a fixed pairwise order at the end. For an upper
+// partial sums of the eighths are added in a fixed pairwise order at the end, a column per warp (one
+// warp adding all of them took as long as the products of m = 64). For an upper
 // triangular B (ub) each warp stops at row c0 + NC of B, below which the CTA's columns are zero: the
 // partition of the inner dimension is unchanged and only exact zero terms are left out.
-template <int NC, class T>
+// KS = 1 (few inner rows and warps enough for every sub-partition): a warp takes 32 rows of its own over the whole inner
+// dimension; nothing is added across warps, a quarter of the FP64 instructions at m = 32. GB300, 65536 rows,
+// m = p = 32, upper triangular: 114 -> 86 us (FP64 bound 84); 4096 rows, 8 columns, m = 240, KS = 8: 23 -> 19.6 us.
+constexpr int kNnWholeM = 64;
+template <int NC, class T, int KS = 8>
 __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double alpha, const T* __restrict__ A,
                                                  int64_t lda, const double* __restrict__ B, int ldb, double beta,
                                                  const T* C0, int64_t ldc0, T* C, int64_t ldc, int ub) {
@@ -282,9 +287,9 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double
     PDL_ARG(A); PDL_ARG(B); PDL_ARG(C0); PDL_ARG(C);
     constexpr int LCH = 256;                 // rows of B staged per pass
     __shared__ T Bs[LCH][NC];
-    __shared__ T red[7][32][NC];
+    __shared__ T red[KS == 1 ? 1 : 8][NC][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t r = (int64_t)blockIdx.x * 32 + lane;
+    const int64_t r = (KS == 1 ? (int64_t)blockIdx.x * 8 + w : (int64_t)blockIdx.x) * 32 + lane;
     const int c0 = blockIdx.y * NC;
     const int nc = min(NC, p - c0);
     const int lim = ub ? min(m, c0 + NC) : m;   // rows of B that can be nonzero in these columns
@@ -301,8 +306,8 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double
             Bs[l][c] = (c < nc) ? (T)B[(int64_t)(c0 + c) * ldb + l0 + l] : T(0);
         }
         __syncthreads();
-        const int q = (lc + 7) / 8;
-        const int lb = w * q, le = min(min(lc, lb + q), lim - l0);
+        const int q = (lc + KS - 1) / KS;
+        const int lb = KS == 1 ? 0 : w * q, le = min(min(lc, lb + q), lim - l0);
         int l = lb;
         // groups of four rows of A, the next group read while the current one is multiplied
         T a[4];
@@ -333,21 +338,26 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int64_t d, int m, int p, double
         }
     }
     PDL_NEXT();
-    if (w > 0) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) red[w - 1][lane][c] = acc[c];
-    }
-    __syncthreads();
-    if (w > 0 || !live) return;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        if (c >= nc) break;
-        const T sum = ((acc[c] + red[0][lane][c]) + (red[1][lane][c] + red[2][lane][c])) +
-                      ((red[3][lane][c] + red[4][lane][c]) + (red[5][lane][c] + red[6][lane][c]));
+    auto put = [&](int c, T sum) {
         T v = (T)alpha * sum;
         if (beta != 0.0) v = fma((T)beta, C0[(int64_t)(c0 + c) * ldc0 + r], v);
         C[(int64_t)(c0 + c) * ldc + r] = v;
+    };
+    if (KS == 1) {
+        if (!live) return;
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < nc) put(c, acc[c]);
+        return;
     }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) red[w][c][lane] = acc[c];
+    __syncthreads();
+    if (w >= nc || !live) return;
+    T x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = red[KS == 1 ? 0 : u][w][lane];
+    put(w, ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7])));
 }
 
 // Small C (m x p) = alpha A B + beta C (both operands untransposed) with a long inner dimension:
@@ -906,7 +916,10 @@ int gemm_nn(int64_t d, int m, int p, double alpha, const T* A, int64_t lda, cons
     const int ub = b_upper ? 1 : 0;
     const int rowblocks = ceil_div(d, 32);
     // columns per thread: as many as possible while at least ~one CTA per SM stays busy
-    if (p >= 6 && (int64_t)rowblocks * ceil_div(p, 8) >= 120) {
+    if (p >= 6 && m <= kNnWholeM && (int64_t)rowblocks * ceil_div(p, 8) >= 4 * sm_count()) {
+        EDA_CUDA_TRY((launch_spread(k_gemm_nn<8, T, 1>, dim3(ceil_div(rowblocks, 8), ceil_div(p, 8)), dim3(256), 0, s, d, m, p,
+            alpha, A, lda, B, ldb, beta, C0, ldc0, C, ldc, ub)));
+    } else if (p >= 6 && (int64_t)rowblocks * ceil_div(p, 8) >= 120) {
         EDA_CUDA_TRY((launch_spread(k_gemm_nn<8, T>, dim3(rowblocks, ceil_div(p, 8)), dim3(256), 0, s, d, m, p, alpha, A,
             lda, B, ldb, beta, C0, ldc0, C, ldc, ub)));
     } else if (p >= 3 && (int64_t)rowblocks * ceil_div(p, 4) >= 120) {

@@ -42,6 +42,21 @@ def test_solve_block_width_edges(eda, b):
     assert O.sin_angle(ref["V"], V) <= 1e-8
 
 
+# block products with few inner rows, from the row count on at which a warp takes them whole (rows / 32 times blocks of 8
+# columns >= 608 warps, up to 64 inner rows), just below it and beyond 64
+@pytest.mark.parametrize("d,b", [(4831, 32), (4865, 32), (9001, 17), (2600, 64), (2600, 65)])
+def test_solve_block_products(eda, d, b):
+    p = synth.gaussian_clusters(d=d, k=20, n_per_class=5, seed=b)
+    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(block_b=b, tau=8.0)) as h:
+        V, lam, _, info, code = h.solve(p.k - 1, 1e-11)
+        assert code == 0, info
+        ref = O.eda(p.X, p.labels, p.k, p.k - 1, c2=h.c2, tier="projected")
+    V = V.cpu().numpy().T
+    assert np.abs(V.T @ V - np.eye(p.k - 1)).max() <= 1e-13
+    assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
+    assert O.sin_angle(ref["V"], V) <= 1e-8
+
+
 # matrix orders around the eigensolver's rules (cluster sizes double from 24 columns on, the cooperative grid starts at
 # 288, one exchange chunk holds 512 rows, the columns of 608 and more no longer come four to a CTA) and its smallest
 @pytest.mark.parametrize("n", [2, 3, 4, 5, 23, 24, 25, 48, 97, 192, 257, 287, 288, 289, 511, 513, 609, 700])

@@ -119,26 +119,6 @@ int sym_nn(eda_ctx* h, const OzOperand* oz, const double* M, int n, int p, const
     return gemm_tn_f64(n, n, p, 1.0, M, n, X, ldx, acc ? 1.0 : 0.0, D, ldd, w.part, w.pcap, s);
 }
 
-// D (m x p, ldd) = op(A) B over K, op(A) = A (m x K) or, trans, A^T (A: K x m); sym: D is symmetric, and only its upper blocks
-// are computed on the tensor cores. From kOzSquareMin multiplications on, a tensor-core handle splits both factors into its
-// scratch, six launches and some 50 us, in place of the FP64 product, which its pipe bounds (0.14 ms at the line). GB300, the
-// whole solve: d = 10305, k = 93, n = 744 10.47 -> 9.44 ms; d = 8000, k = 62, n = 496 7.30 -> 6.85.
-constexpr int64_t kOzSquareMin = 1 << 26;
-int square_product(eda_ctx* h, bool trans, bool sym, int m, int p, int K, const double* A, int lda, const double* B, int ldb,
-                   double* D, int ldd, DirectWs& w, cudaStream_t s) {
-    if (h->cfg.prec == EDA_F64_TC && h->ozblock && (int64_t)m * p * K >= kOzSquareMin) {
-        const size_t ba = (oz_operand_bytes(m, K) + 255) / 256 * 256;
-        if (h->ozwide.ensure(ba + oz_operand_bytes(p, K)) == EDA_OK) {   // else there is no room for the splits
-            OzOperand oa, ob;
-            EDA_TRY(oz_operand_make(A, lda, m, K, trans, h->ozwide.mem, &oa, h->status, s));
-            EDA_TRY(oz_operand_make(B, ldb, p, K, true, static_cast<char*>(h->ozwide.mem) + ba, &ob, h->status, s));
-            return oz_gemm_tiled(oa, ob, 1.0, 0.0, nullptr, 0, D, ldd, sym, h->status, s, w.part, w.pcap);
-        }
-    }
-    if (trans) return gemm_tn_f64(K, m, p, 1.0, A, lda, B, ldb, 0.0, D, ldd, w.part, w.pcap, s);
-    return gemm_nn_f64(m, K, p, 1.0, A, lda, B, ldb, 0.0, nullptr, 0, D, ldd, s);
-}
-
 // U = C PQ for p columns (both (n + k) x p, ld nk); PQ is overwritten (the chain of the composed M-apply).
 int apply_c(eda_ctx* h, int p, double* PQ, double* U, DirectWs& w, cudaStream_t s) {
     const int n = (int)h->n, k = h->k, nk = n + k;
@@ -269,11 +249,11 @@ int direct_impl(eda_ctx* h, int t, double* Vout, double* lambda, eda_solve_info*
             break;
         }
         // P = F R^{-1} = Z^T Q
-        if ((rc = square_product(h, false, false, nk, r, r, w.PQ, nk, w.Ri, r, w.P, nk, w, s)) != EDA_OK) break;
+        if ((rc = gemm_nn_f64(nk, r, r, 1.0, w.PQ, nk, w.Ri, r, 0.0, nullptr, 0, w.P, nk, s)) != EDA_OK) break;
         // B = P^T C P
         if ((rc = copy_mat_f64(nk, r, w.P, nk, w.PQ, nk, s)) != EDA_OK) break;
         if ((rc = apply_c(h, r, w.PQ, w.U, w, s)) != EDA_OK) break;
-        if ((rc = square_product(h, true, true, r, r, nk, w.P, nk, w.U, nk, w.B, r, w, s)) != EDA_OK) break;
+        if ((rc = gemm_tn_f64(nk, r, r, 1.0, w.P, nk, w.U, nk, 0.0, w.B, r, w.part, w.pcap, s)) != EDA_OK) break;
         if ((rc = symmetrize_f64(r, w.B, r, s)) != EDA_OK) break;
         // the t largest eigenpairs of P^T C P (ascending)
         if ((rc = symeig_f64(r, w.B, r, r - t, r - 1, w.mu, w.Wv, r, &w.eig, h->status, h->cfg.seed + 29, 1e-7, s)) !=

@@ -211,22 +211,6 @@ def test_direct_solve_orders(eda, n, t):
     assert np.abs(MV - V @ (V.T @ MV)).max() <= 1e-9 * ref["lam_t"][0]
 
 
-# direct solve with a tensor-core handle: its two square products below and above the order from which they run there
-# ((n + k) (n + k - 1)^2 = 2^26 near n + k = 407)
-@pytest.mark.parametrize("n,k", [(320, 80), (336, 84), (560, 70)])
-def test_direct_solve_square_products(eda, n, k):
-    p = synth.gaussian_clusters(d=4200, k=k, n_per_class=n // k, seed=n)
-    with eda.build(_dev(p.X), _dev(p.labels), p.k, eda.config(prec=eda.EDA_F64_TC, tau=6.0, tc_min_mi=-1)) as h:
-        V, lam, info, code = h.solve_direct(k - 1)
-        assert code == 0
-        c2 = h.c2
-    V = V.cpu().numpy().T
-    ref = O.eda(p.X, p.labels, p.k, k - 1, c2=c2, tier="projected")
-    assert np.max(np.abs(lam.cpu().numpy() - ref["lam_t"]) / ref["lam_t"]) <= 1e-10
-    assert np.abs(V.T @ V - np.eye(k - 1)).max() <= 1e-12
-    assert O.sin_angle(ref["V"], V) <= 1e-8
-
-
 # Kernels launched to be set up while their predecessor runs: long chains of short ones (small and middle sizes, with and
 # without chip-filling kernels between), with another stream keeping the SMs busy unevenly. All sums are taken in a fixed
 # order, so a kernel that read before its predecessor had finished would show as different bits.

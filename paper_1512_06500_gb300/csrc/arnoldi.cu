@@ -123,9 +123,9 @@ struct ArnWs {
 
 // X <- orth(X) in place by CholQR (one pass); X2: d x p scratch; R, Ri: p x p.
 int cholqr_once(int64_t d, int p, double* X, double* X2, double* R, double* Ri, double piv_min2, int* status, int* lost,
-                ArnWs& w, cudaStream_t s) {
+                ArnWs& w, cudaStream_t s, const NoteRef& note = {}) {
     EDA_TRY(syrk_f64(d, p, 1.0, X, d, 0.0, R, p, w.part, w.pcap, s));
-    if (lost || piv_min2 > 0.0) EDA_TRY(chol_inv_small(p, R, p, Ri, 1e-28, piv_min2, status, lost, s));
+    if (lost || piv_min2 > 0.0) EDA_TRY(chol_inv_small(p, R, p, Ri, 1e-28, piv_min2, status, lost, s, note));
     else EDA_TRY(chol_inv_auto(p, R, p, Ri, 1e-28, status, w.CW, w.part, w.pcap, s));
     EDA_TRY(gemm_nn_f64(d, p, p, 1.0, X, d, Ri, p, 0.0, nullptr, 0, X2, d, s));
     return EDA_OK;
@@ -358,6 +358,8 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
     const size_t t1_cap = std::max<size_t>((size_t)m_max * m_max, (size_t)n * m_max);
     double max_rel = INFINITY;
     std::vector<double> relres_h(t, INFINITY);
+    Note note;
+    EDA_TRY(note.open(s));
     do {
         // rank threshold of a new direction: 64 eps ||N|| with ||N|| <= exp(c^2 lmax(G_B)) (||exp(-c^2 S_W)|| <= 1)
         const double normN = std::exp(std::min(700.0, h->c2 * h->lmax_b));
@@ -386,9 +388,11 @@ int arnoldi_impl(eda_ctx* h, int t, double tol, double* Vout, double* lambda, ed
                 break;
             }
             // W1 = W R1^{-1} (the remainder W itself stays for the residuals)
-            if ((rc = cholqr_once(d, b, w.W, w.W1, w.R1, w.R1i, piv_min2, h->status, w.lost, w, s)) != EDA_OK) break;
+            if ((rc = cholqr_once(d, b, w.W, w.W1, w.R1, w.R1i, piv_min2, h->status, w.lost, w, s, note.next())) !=
+                EDA_OK)
+                break;
             int lw[2] = {0, 0};   // lost and nearly lost columns
-            if ((rc = read_back(lw, w.lost + b, sizeof(lw), s)) != EDA_OK) break;
+            if ((rc = note.wait(lw, w.lost + b)) != EDA_OK) break;
             const int lostc = lw[0];
             const bool room = cols + b <= m_max;
             if (room) {

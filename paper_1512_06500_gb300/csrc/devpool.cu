@@ -253,6 +253,45 @@ void host_kit_give(HostKit* k) {
     host_kit_destroy(k);
 }
 
+int Note::open(cudaStream_t stream) {
+    s = stream;
+    if (hold.open() != EDA_OK) {
+        hold.kit = nullptr;
+        cudaGetLastError();
+        return EDA_OK;
+    }
+    std::memset(hold.kit->page, 0, 3 * sizeof(int));
+    return EDA_OK;
+}
+
+Note::~Note() {
+    if (pending) cudaStreamSynchronize(s);
+}
+
+NoteRef Note::next() {
+    if (!hold.kit) return {};
+    pending = true;
+    return {static_cast<int*>(hold.kit->page), ++tag};
+}
+
+int Note::wait(int out[2], const int* dev) {
+    if (!hold.kit) return read_back(out, dev, 2 * sizeof(int), s);
+    const int* w = static_cast<const int*>(hold.kit->page);
+    for (bool done = false;;) {
+        for (int i = 0; i < 4096; ++i)
+            if (__atomic_load_n(w + 2, __ATOMIC_ACQUIRE) == tag) {
+                out[0] = w[0];
+                out[1] = w[1];
+                pending = false;
+                return EDA_OK;
+            }
+        if (done) return EDA_ERR_CUDA;   // the stream ran dry without the note
+        const cudaError_t q = cudaStreamQuery(s);
+        if (q == cudaSuccess) done = true;
+        else if (q != cudaErrorNotReady) EDA_CUDA_TRY(q);
+    }
+}
+
 int read_back(void* host, const void* dev, size_t bytes, cudaStream_t s) {
     HostHold hold;
     if (bytes <= kHostPage && hold.open() == EDA_OK) {

@@ -160,6 +160,38 @@ struct HostHold {
     HostHold& operator=(const HostHold&) = delete;
     ~HostHold() { host_kit_give(kit); }
 };
+// Two integers that a kernel writes to pinned host memory, followed by a tag, while the kernels queued behind it go on: the
+// host learns how a factorisation went, and queues what follows from it, beside the product that uses the factor. A copy and
+// a wait in the stream left the GPU idle for 8 us a block of a Krylov basis, and 5 more until the next kernel ran.
+struct NoteRef {
+    int* words = nullptr;   // {first, second, tag}; null: no note
+    int tag = 0;
+};
+class Note {
+  public:
+    int open(cudaStream_t s);   // without a pinned page there are no notes (next() gives none)
+    ~Note();                    // a note not waited for: its kernel is, before the page goes back
+    Note() = default;
+    Note(const Note&) = delete;
+    Note& operator=(const Note&) = delete;
+    NoteRef next();             // for one launch on the stream
+    // the two integers of the last next(), or, without a page, of `dev` after the work queued so far
+    int wait(int out[2], const int* dev);
+
+  private:
+    HostHold hold;
+    cudaStream_t s = nullptr;
+    int tag = 0;
+    bool pending = false;
+};
+__device__ __forceinline__ void note_write(const NoteRef& n, int first, int second) {
+    if (!n.words) return;
+    volatile int* w = n.words;
+    w[0] = first;
+    w[1] = second;
+    __threadfence_system();
+    w[2] = n.tag;
+}
 // Copy `bytes` from the device once the work queued on s is done, and wait for it (through a pinned page when it fits).
 int read_back(void* host, const void* dev, size_t bytes, cudaStream_t s);
 
@@ -199,7 +231,7 @@ int gemm_small_sym_f64(int m, double alpha, const double* A, int lda, const doub
 // and ST_RANKLOSS is or-ed into *status; lost pivots are listed in lost[0..], lost[b] = count, and
 // lost[b + 1] counts the kept pivots below 1e-10 of their column's squared norm.
 int chol_inv_small(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2,
-                   int* status, int* lost, cudaStream_t s);
+                   int* status, int* lost, cudaStream_t s, const NoteRef& note = {});
 // The same factorisation for any m, blocked: one-CTA factorisations of kCholBlock x kCholBlock diagonal
 // blocks and multi-CTA products for the panels, trailing updates and the inverse. Rank detection
 // (rank_tol) applies within each diagonal block; no lost list. work: chol_inv_blocked_doubles(m) doubles;

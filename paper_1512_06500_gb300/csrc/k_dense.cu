@@ -480,7 +480,7 @@ __device__ __forceinline__ double newton_rcp(double x) {
 constexpr double kCholWeak = 1e-10;
 template <int NC>
 __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg, double* Rinv, double rank_tol,
-                                                       double piv_min2, int* status, int* lost) {
+                                                       double piv_min2, int* status, int* lost, const NoteRef note) {
     PDL_ENTER();
     PDL_ARG(G); PDL_ARG(Rinv); PDL_ARG(status); PDL_ARG(lost);
     constexpr int NR = 4 * NC;               // rows per warp
@@ -611,12 +611,13 @@ __global__ void __launch_bounds__(256) k_chol_inv_pair(int b, double* G, int ldg
     if (threadIdx.x == 0 && lost) {
         lost[b] = s_nlost;
         lost[b + 1] = s_nweak;
+        note_write(note, s_nlost, s_nweak);
     }
 }
 
 // The same by one CTA in global memory, for any b: two divisions a column and a back substitution.
 __global__ void k_chol_inv(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2, int* status,
-                           int* lost) {
+                           int* lost, const NoteRef note) {
     PDL_WAIT();
     PDL_ARG(G); PDL_ARG(Rinv); PDL_ARG(status); PDL_ARG(lost);
     __shared__ double maxdiag;
@@ -696,7 +697,10 @@ __global__ void k_chol_inv(int b, double* G, int ldg, double* Rinv, double rank_
         if (p > 0.0 && p * p < kCholWeak * sum) atomicAdd(&nweak, 1);
     }
     __syncthreads();
-    if (threadIdx.x == 0) lost[b + 1] = nweak;
+    if (threadIdx.x == 0) {
+        lost[b + 1] = nweak;
+        note_write(note, nlost, nweak);
+    }
 }
 
 // the register-resident factorisation up to this size (three 32-column slices a lane)
@@ -1020,19 +1024,19 @@ int gemm_small_sym_f64(int m, double alpha, const double* A, int lda, const doub
 }
 
 int chol_inv_small(int b, double* G, int ldg, double* Rinv, double rank_tol, double piv_min2, int* status, int* lost,
-                   cudaStream_t s) {
+                   cudaStream_t s, const NoteRef& note) {
     if (b <= 32)
         EDA_CUDA_TRY((launch_chained(k_chol_inv_pair<1>, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2,
-            status, lost)));
+            status, lost, note)));
     else if (b <= 64)
         EDA_CUDA_TRY((launch_chained(k_chol_inv_pair<2>, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2,
-            status, lost)));
+            status, lost, note)));
     else if (b <= kCholPairMax)
         EDA_CUDA_TRY((launch_chained(k_chol_inv_pair<3>, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2,
-            status, lost)));
+            status, lost, note)));
     else
         EDA_CUDA_TRY((launch_chained(k_chol_inv, dim3(1), dim3(256), 0, s, b, G, ldg, Rinv, rank_tol, piv_min2, status,
-            lost)));
+            lost, note)));
     return EDA_OK;
 }
 

@@ -166,9 +166,9 @@ int oz_basis_grow(SolveWs<T>& w, int64_t d, int cols0, int cols1, int* status, c
 
 template <class T>
 int cholqr_pass(int64_t d, int b, T* X, int64_t ldx, double* Rm, double* Rinv, T* out, double piv_min2, int* status,
-                int* lost, SolveWs<T>& w, cudaStream_t s) {
+                int* lost, SolveWs<T>& w, cudaStream_t s, const NoteRef& note = {}) {
     EDA_TRY(syrk_tn<T>(d, b, 1.0, X, ldx, 0.0, Rm, b, w.part, w.pcap, s));
-    EDA_TRY(chol_inv_small(b, Rm, b, Rinv, 1e-28, piv_min2, status, lost, s));
+    EDA_TRY(chol_inv_small(b, Rm, b, Rinv, 1e-28, piv_min2, status, lost, s, note));
     // R^{-1} is upper triangular with its zeros stored: the product skips the zero rows of each column slice
     EDA_TRY(gemm_nn<T>(d, b, b, 1.0, X, ldx, Rinv, b, 0.0, nullptr, 0, out, ldx, s, true));
     return EDA_OK;
@@ -305,12 +305,14 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
         EDA_TRY(fill_gaussian<T>(d, b, w.V, d, h->cfg.seed, 0, s));
     }
     EDA_TRY(cholqr_pass<T>(d, b, w.V, d, w.R1, w.R1i, w.W1, 0.0, h->status, w.lost, w, s));
-    EDA_TRY(cholqr_pass<T>(d, b, w.W1, d, w.R2, w.R2i, w.V, 0.0, h->status, w.lost, w, s));
+    Note note;
+    EDA_TRY(note.open(s));
+    EDA_TRY(cholqr_pass<T>(d, b, w.W1, d, w.R2, w.R2i, w.V, 0.0, h->status, w.lost, w, s, note.next()));
     EDA_TRY(oz_basis_grow<T>(w, d, 0, b, h->status, s));
     {
-        int lostc = 0;
-        EDA_TRY(read_back(&lostc, w.lost + b, sizeof(int), s));
-        if (lostc) return EDA_ERR_BREAKDOWN;   // the start block itself is rank deficient
+        int lw[2] = {0, 0};
+        EDA_TRY(note.wait(lw, w.lost + b));
+        if (lw[0]) return EDA_ERR_BREAKDOWN;   // the start block itself is rank deficient
     }
 
     int cols = b;
@@ -336,9 +338,9 @@ int run_lanczos(eda_ctx* h, int t, double tol, const double* V0, int b0, int m_m
         EDA_CUDA_TRY((launch_chained(k_set_col_block, dim3(ceil_div(cols * b, 256)), dim3(256), 0, s, w.Tm, m_max, cols,
             j0, b, C1, C2)));
         // CholQR2 of W with rank detection: W = V_{j+1} B_{j+1}
-        EDA_TRY(cholqr_pass<T>(d, b, w.W, d, w.R1, w.R1i, w.W1, piv_min2, h->status, w.lost, w, s));
+        EDA_TRY(cholqr_pass<T>(d, b, w.W, d, w.R1, w.R1i, w.W1, piv_min2, h->status, w.lost, w, s, note.next()));
         int lw[2] = {0, 0};   // lost and nearly lost columns
-        EDA_TRY(read_back(lw, w.lost + b, sizeof(lw), s));
+        EDA_TRY(note.wait(lw, w.lost + b));
         const int lostc = lw[0];
         const bool room = cols + b <= m_max;
         if (room) {

@@ -362,8 +362,12 @@ __global__ void __launch_bounds__(TD_THREADS) k_tridiag_x(int n, const double* _
             const double alpha = s_alpha;
             const double sig = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
             double beta = alpha, t = 0.0, v1 = 0.0;
-            if (__double_as_longlong(sig) != 0) {   // tests on the bits: a comparison would take the FP64 pipe
-                const double ab = td_sqrt(fma(alpha, alpha, sig));
+            // Tests on the bits: a comparison would take the FP64 pipe. A column below 2^-450 ends the coupling (graded matrices
+            // come down to 1e-160 where their eigenvectors have converged): its tau, the square's reciprocal, times the
+            // matrix would leave the exponent range.
+            const double nn = fma(alpha, alpha, sig);
+            if (__double_as_longlong(sig) != 0 && __double2hiint(nn) >= (1023 - 900) << 20) {
+                const double ab = td_sqrt(nn);
                 const double av = fabs(alpha) + ab;   // |alpha - beta|: beta has the other sign
                 t = td_rcp(ab * av);
                 const int sg = __double2hiint(alpha) & 0x80000000;

@@ -211,6 +211,25 @@ def test_direct_solve_orders(eda, n, t):
     assert np.abs(MV - V @ (V.T @ MV)).max() <= 1e-9 * ref["lam_t"][0]
 
 
+# Gram matrices whose columns all but decouple: classes of two opposite samples in pixels of their own, with one pixel in
+# common that couples them by 1e-60 and 1e-140 (squares of the coupling in range) and 1e-160 (out of range); cluster and grid
+@pytest.mark.parametrize("k", [6, 40, 150, 170])
+@pytest.mark.parametrize("c", [1e-30, 1e-70, 1e-80])
+def test_gram_eigenvalues_tiny_couplings(eda, k, c):
+    n, d = 2 * k, k + 40
+    X = np.zeros((n, d))
+    for j in range(k):
+        X[2 * j, j] = 1.0 + j / k
+        X[2 * j, d - 1] = c
+        X[2 * j + 1] = -X[2 * j]
+    lab = np.repeat(np.arange(k), 2).astype(np.int32)
+    with eda.build(_dev(X), _dev(lab), k, eda.config(tau=2.0, c2=0.1)) as h:
+        f = h.factors()
+    G, ev = f["GW"].cpu().numpy(), f["evals_w"].cpu().numpy()
+    ref = np.linalg.eigvalsh(G)
+    assert np.abs(ev - ref).max() <= 4 * n * np.finfo(float).eps * ref[-1]
+
+
 # Kernels launched to be set up while their predecessor runs: long chains of short ones (small and middle sizes, with and
 # without chip-filling kernels between), with another stream keeping the SMs busy unevenly. All sums are taken in a fixed
 # order, so a kernel that read before its predecessor had finished would show as different bits.

@@ -418,7 +418,7 @@ def run_gpu_batched(args, rank, world, local_rank):
                             "time (launches of 64 problems overlap on many streams): a lower bound")
         roofline.pop("avg_launch_us", None)
     tridiag = {
-        "kernel": "k_tridiag_res / k_tridiag_cluster / k_tridiag: Householder tridiagonalisation (4/3 n^3 flops) of the FP64 "
+        "kernel": "k_tridiag_x / k_tridiag: Householder tridiagonalisation (4/3 n^3 flops) of the FP64 "
                   "Grams and Rayleigh-Ritz matrices, summed over concurrent problems",
         "bound": "alu", "achieved": tri_tf, "peak": NOMINAL_FP64_TFLOPS, "unit": "TFLOP/s",
         "frac": tri_tf / NOMINAL_FP64_TFLOPS, "traffic": None,
@@ -718,7 +718,7 @@ def run_gpu(args, rank, world, local_rank):
     tri_ms, tri_calls = regions["tridiag"]
     tri_flops, _ = r["work"]["tridiag"]
     latency_bound = {
-        "kernel": "k_tridiag_res / k_tridiag_cluster / k_tridiag: Householder tridiagonalisation (4/3 n^3 flops) of the Rayleigh-Ritz "
+        "kernel": "k_tridiag_x / k_tridiag: Householder tridiagonalisation (4/3 n^3 flops) of the Rayleigh-Ritz "
                   "matrices (and of a Gram taking the eigensolver route)",
         "achieved_tflops": rate(tri_flops, tri_ms) if tri_ms > 0 else None,
         "avg_call_us": tri_ms * 1e3 / max(tri_calls, 1), "calls": tri_calls,

@@ -81,8 +81,8 @@ typedef struct {
                                  /* form one after another (Eq. (3.16)); 1 = their composed  */
                                  /* form M = I + Z C Z^T, Z = [H_W H_B] (Theorem 3.1 for each  */
                                  /* factor; two sweeps over Z instead of six over H_W, H_B)   */
-    int32_t wait_limit;          /* polls of a grid-wide barrier wait (the cooperative        */
-                                 /* symmetric eigensolver, n > 512) before it gives up and    */
+    int32_t wait_limit;          /* polls of a grid-wide wait (the cooperative symmetric      */
+                                 /* eigensolver, n >= 288) before it gives up and             */
                                  /* the call returns EDA_ERR_TIMEOUT; <= 0: the default,      */
                                  /* 20,000,000 (about 1-2 s)                                  */
     int32_t tc_min_mi;           /* EDA_F64_TC: the size of Z = [H_W H_B], d (n + k), in units  */

@@ -61,8 +61,10 @@ std::atomic<uint64_t>& launch_counter();   // kernels launched by this process (
 
 // CTAs that are set up early go to whichever SMs have room at that moment, several to one SM when a large predecessor drains
 // unevenly, and stay there. For a kernel that fills the chip and is bound by the FP64 pipe of each SM that costs more than the
-// launch it hides (k_gemm_tn_partial<16>, 16384 x 100 blocks: 0.15 -> 0.36 ms): launch_spread therefore chains only grids of
-// at most half the SMs and starts the others when the chip is empty.
+// launch it hides (k_gemm_tn_partial<16> in an Arnoldi solve at d = 16384: 0.15 -> 0.36 ms): launch_spread therefore chains
+// only grids of at most an eighth of the SMs and starts the others when the chip is empty. With half the SMs as the line
+// the 18 k_gemm_tn_partial<32> of a direct solve took 1.43 ms, with an eighth 1.31, unchained 1.26; below it, d = 256 gains
+// (35 k_gemm_tn_partial<8> 0.29 -> 0.22 ms).
 int sm_count();   // of the current device
 
 template <class... P, class... A>
